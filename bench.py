@@ -301,12 +301,8 @@ TRAFFIC = {
              "source": "ncu dram__bytes_read+write, zd_gemm_kernel (128-column tiles), p2_48cube_chunk"},
     "pair_from_f": {"bytes_per_launch": 5.504037e9 + 1.240109e9,
                     "source": "ncu dram__bytes_read+write, pair_kernel_tf_from_f<48> (TMA-fed), p2_48cube_chunk"},
-    # the single-stream launch (4-deep TMA ring) the tensor-core route runs
-    "ozaki_gemm": {"bytes_per_launch": 5.176667e9 + 0.212558e9,
-                   "source": "ncu dram__bytes_read+write, oz_gemm_kernel<240,0,4> (s = 7), p2_48cube_chunk"},
-    "ozaki_gemm_single_stream": {"bytes_per_launch": 5.176667e9 + 0.212558e9,
-                                 "source": "ncu dram__bytes_read+write, oz_gemm_kernel<240,0,4> (s = 7), "
-                                           "p2_48cube_chunk"},
+    "ozaki_gemm": None,
+    "ozaki_gemm_single_stream": None,
 }
 
 
@@ -604,8 +600,15 @@ def _hbm_peak():
 
 
 def oz_kpad(ka):
-    """Real K extent of a general split product with ka complex inner entries (padded to 64)."""
-    return (2 * ka + 63) // 64 * 64
+    """Real K extent of a general split product with ka complex inner entries (padded to 64 each)."""
+    return 2 * ((ka + 63) // 64 * 64)
+
+
+def oz_products(nslices):
+    """Slice products of a split contraction at the accuracy of nslices six-bit slices: the library
+    takes n = 3, 3, 4, 5, 5, 6 nine-bit slices for nslices = 3 .. 8 and keeps n (n + 1) / 2 products."""
+    n = {3: 3, 4: 3, 5: 4, 6: 5, 7: 5, 8: 6}[nslices]
+    return n * (n + 1) // 2
 
 
 def mode_roofline(bound, kernel, work, ms, unit_of_work, prec="ozaki"):
@@ -749,8 +752,8 @@ def roofline_for(cfg, prec, nslices, res, single_stream=False):
     nchunk = -(-cfg.npairs // cfg.pair_chunk)
     per_launch_flops = 4.0 * cfg.ng * (cfg.ng + 1) * cfg.npairs / nchunk
     if prec == "ozaki":
-        # low-precision flops of the kept slice pairs: s(s+1)/2 x 4 N_G^2 P per chunk and frequency
-        per_launch_flops = nslices * (nslices + 1) / 2 * 4.0 * cfg.ng ** 2 * cfg.npairs / nchunk
+        # low-precision flops of the kept slice pairs, each 4 N_G^2 P per chunk and frequency
+        per_launch_flops = oz_products(nslices) * 4.0 * cfg.ng ** 2 * cfg.npairs / nchunk
     peak, peak_src = peak_for(prec)
     achieved = per_launch_flops / (kms / kn * 1e-3) * 1e-12 if kn else None
     return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
@@ -929,7 +932,7 @@ def batch(args):
     # a graph replay has no per-kernel timing: the contraction's rate over the whole call (stage (a)
     # and the per-frequency slicing included) bounds it from below
     roof = mode_roofline("tensor", "oz_gemm_kernel (16 per-frequency launches over all q), whole replay",
-                         sum(s * (s + 1) / 2 * 4.0 * n * n * P * 16 for n in ngs), ms,
+                         sum(oz_products(s) * 4.0 * n * n * P * 16 for n in ngs), ms,
                          "low-precision flops of the kept slice pairs over the whole replay time")
     cpu = None
     if not args.no_cpu_baseline:
@@ -983,7 +986,7 @@ def adjoint(args):
                                           kms.get("adj_products"), "H read once by each product kernel, 16 B per point")
     if args.prec == "ozaki":
         roofs["y_mw"] = mode_roofline("tensor", "oz_gemm_kernel (general product Y = M W)",
-                                      s * (s + 1) / 2 * 2.0 * P * (2 * cfg.ng) * oz_kpad(cfg.ng), kms.get("adj_zgemm"),
+                                      oz_products(s) * 2.0 * P * (2 * cfg.ng) * oz_kpad(cfg.ng), kms.get("adj_zgemm"),
                                       "low-precision flops of the kept slice pairs")
     dom = max(roofs, key=lambda k: roofs[k]["ms"] if roofs[k] else 0.0) if roofs else None
     cpu = None if args.no_cpu_baseline else oracle_adjoint_sample(prob, W, 1)
@@ -1046,10 +1049,10 @@ def subspace(args):
                                             kms.get("pair_mtxel"), "FP32 operations of the pair kernel x pairs")}
     if args.prec == "ozaki":
         roofs["contraction"] = mode_roofline("tensor", "oz_gemm_kernel (N_Eig columns)",
-                                             s * (s + 1) / 2 * 4.0 * neig ** 2 * P * len(om19),
+                                             oz_products(s) * 4.0 * neig ** 2 * P * len(om19),
                                              kms.get("ozaki_gemm"), "low-precision flops of the kept slice pairs")
         roofs["projection"] = mode_roofline("tensor", "oz_gemm_kernel (general product M C_s)",
-                                            s * (s + 1) / 2 * 2.0 * P * (2 * neig) * oz_kpad(cfg.ng),
+                                            oz_products(s) * 2.0 * P * (2 * neig) * oz_kpad(cfg.ng),
                                             kms.get("subspace_projection"), "low-precision flops of the kept slice pairs")
     cpu = None
     if not args.no_cpu_baseline:
@@ -1104,7 +1107,7 @@ def epsilon(args):
     s = args.nslices
     n = cfg.ng
     if args.prec == "ozaki":
-        per_step = 2 * s * (s + 1) / 2 * 2.0 * n * (2 * n) * oz_kpad(n)
+        per_step = 2 * oz_products(s) * 2.0 * n * (2 * n) * oz_kpad(n)
         roof = mode_roofline("tensor", "oz_gemm_kernel (general products of the Newton-Schulz steps)",
                              per_step * steps, kms.get("eps_products"), "low-precision flops of the kept slice pairs")
     else:
@@ -1173,7 +1176,7 @@ def extras(args):
                                             pms, "FP32 operations of the pair kernel x pairs")}
     if args.prec == "ozaki":
         roofs["contraction"] = mode_roofline("tensor", "oz_gemm_kernel (sign-split real-axis contractions)",
-                                             s * (s + 1) / 2 * 4.0 * cfg.ng ** 2 * P / nchunk * gl, gms,
+                                             oz_products(s) * 4.0 * cfg.ng ** 2 * P / nchunk * gl, gms,
                                              "low-precision flops of the kept slice pairs, per chunk contraction")
     cpu = None
     if not args.no_cpu_baseline:
@@ -1229,7 +1232,7 @@ def sigma(args):
     clocks = clk.stop()
     kms = {k: val[0] / steps for k, val in kt.items()}
     s = args.nslices
-    issued_x = s * (s + 1) / 2 * 8.0 * nsig * ng * ng * nb * ne      # slice pairs x real flops, first product
+    issued_x = oz_products(s) * 8.0 * nsig * ng * ng * nb * ne      # slice pairs x real flops, first product
     pk, pk_src = peak_for("ozaki")
     roof = None
     if args.prec == "ozaki" and "gpp_gemm_x" in kms:

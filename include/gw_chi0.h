@@ -86,15 +86,16 @@ typedef struct {
     int n[3];                /* FFT grid n0 x n1 x n2 (each a product of 2, 3, 5; 4 <= n <= 128) */
     int nq;                  /* number of q-point slots (>= 1) */
     int prec;                /* gw_prec */
-    int nslices;             /* Ozaki slices for GW_PREC_OZAKI_BF16 (3..8); ignored for FP64 */
+    int nslices;             /* accuracy of GW_PREC_OZAKI_BF16 in six-bit slices (3..8; the kernels take
+                                the nine-bit slices that reach it); ignored for FP64 */
     int64_t pair_chunk;      /* pairs per M chunk; 0 = 8192 */
     size_t mem_budget_bytes; /* cap on library-owned device memory; 0 = no cap */
     int device;              /* CUDA device ordinal; must be current on the calling thread */
     int mtxel_prec;          /* gw_mtxel_prec */
     int single_stream;       /* 0: in split-precision streamed compute, the contraction of each chunk
-                                runs on a second, high-priority stream beside the pair elements of
-                                the next (tensor cores and FP32 pipes share the SMs); 1: every
-                                kernel on the handle's stream, one after the other */
+                                runs on a second, high-priority stream, overlapping the pair
+                                elements of the next; 1: every kernel on the handle's stream, one
+                                after the other */
 } gw_chi0_desc;
 
 /*
@@ -161,9 +162,9 @@ GW_API gw_status gw_chi0_compute(gw_chi0 *h, int nq, const int *iq, int nw, cons
  * persistent launch per frequency covering every slot (split precision), ordered largest
  * block first.  The whole sequence is captured once per call signature (slots, sphere
  * sizes, frequencies, output pointers) into a CUDA graph and replayed on later calls.
- * On the first call of a problem shape an autotuner times the contraction's launch-shape
- * candidates (FP64 tile edge 32/64 and wave count; split-precision tile width 128/240/256
- * columns) and keeps the fastest for the handle (see gw_chi0_tuning).  The first call
+ * On the first call of a problem shape in FP64 mode an autotuner times the contraction's
+ * launch-shape candidates (tile edge 32/64 and wave count) and keeps the fastest for the handle
+ * (see gw_chi0_tuning); the split contraction has one tile shape.  The first call
  * synchronises the stream; replays are asynchronous.  Slots must be distinct.
  * Errors: as gw_chi0_compute; GW_ERR_OOM when the resident buffers do not fit.
  */
@@ -172,10 +173,8 @@ GW_API gw_status gw_chi0_compute_batch(gw_chi0 *h, int nq, const int *iq, int nw
 
 /*
  * Launch shapes in use (chosen by the autotuner of gw_chi0_compute_batch, or defaults):
- * FP64 tile edge (complex), FP64 waves, split-precision tile width (real columns; 256 before
- * tuning, when each contraction instead takes 240 or 256 columns by which fills the SMs' waves
- * better).  The environment variable GW_CHI0_SPLIT_TILE=128, 240 or 256, read at every
- * contraction, forces the split-precision tile width; the results do not depend on it.
+ * FP64 tile edge (complex), FP64 waves, split-precision tile width (256 real columns, the one
+ * shape there is).
  * Returns the number of problem shapes tuned so far.  Any pointer may be NULL.
  */
 GW_API int gw_chi0_tuning(const gw_chi0 *h, int *tile_f64, int *waves_f64, int *tile_split);
@@ -310,7 +309,7 @@ GW_API gw_status gw_chi0_epsilon_inverse(gw_chi0 *h, int ng, int nw, const doubl
  *   sigma   device complex128 [ne][nsig][nsig], written in full (zero when nb = 0).
  * Work buffers, held by the handle until destroy: FP64 mode two [ng][ng] complex128 matrices;
  * split mode the pole parameters transposed in two-float form (32 ng^2 bytes), the BF16 slices
- * of P^T for a batch of energies (28 ng^2 bytes each at 7 slices, at most 32 GiB or a quarter of
+ * of P^T for a batch of energies (20 ng^2 bytes each at nslices = 7, at most 32 GiB or a quarter of
  * mem_budget_bytes when set) and X^T for 16 energies (16 nsig ng complex128 plus its slices).
  * GW_ERR_ARG for sizes out of range, null or misaligned (16 bytes) complex pointers, non-finite
  * energies; other errors as gw_chi0_compute.
@@ -350,8 +349,8 @@ GW_API gw_status gw_chi0_keep_pair_elements(gw_chi0 *h, int enable);
 /*
  * How many streams a single-frequency gw_chi0_compute uses for slot iq as it stands (bands and
  * sphere set): 2 when each chunk's split contraction runs on a second stream beside the next
- * chunk's pair elements (split precision, two-float stage (a) by the FFT pair kernel, and room for
- * two pair-kernel blocks beside a contraction block on an SM), else 1 (always 1 on the
+ * chunk's pair elements (split precision, two-float stage (a) by the grid-specialised FFT pair
+ * kernel with blocks of at most 64 KB of shared memory), else 1 (always 1 on the
  * tensor-core route of stage (a), see gw_chi0_pair_elements_block).  Calls with several frequencies always
  * run on one stream.  Negative (a gw_status, negated) on a bad handle or slot.
  */

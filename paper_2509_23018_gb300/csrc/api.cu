@@ -256,56 +256,123 @@ gw_status make_tmap_z(gw_chi0 *h, CUtensorMap *map, void *Z, int64_t kpad, int n
     return GW_OK;
 }
 
-// GW_CHI0_SPLIT_TILE=128|240|256, read at every contraction, forces the width (the result does not
-// depend on it: every entry sums the same slice products in the same K order)
-int contraction_bn(const gw_chi0 *h, int ng)
-{
-    if (const char *e = getenv("GW_CHI0_SPLIT_TILE")) {
-        const int v = atoi(e);
-        if (v == 128 || v == 240 || v == 256) return v;
-    }
-    return h->bn_tuned ? h->tuned_bn : gw::oz_pick_bn(ng, num_sms());
-}
-
-gw_status oz_job(gw_chi0 *h, gw::OzJob &j, void *Z, int64_t kpad, int ng, const int *E, double2 *chi, int bn)
+gw_status oz_job(gw_chi0 *h, gw::OzJob &j, void *Z, int64_t kpad, int ng, const int *E, double2 *chi)
 {
     std::memset(&j, 0, sizeof j);
+    const int s = gw::oz_slices(h->d.nslices);
     gw_status st;
-    if ((st = make_tmap_z(h, &j.tmA, Z, kpad, 2 * ng, h->d.nslices, gw::oz_box_rows_a())) ||
-        (st = make_tmap_z(h, &j.tmB, Z, kpad, 2 * ng, h->d.nslices, bn)))
-        return st;
+    if ((st = make_tmap_z(h, &j.tmA, Z, kpad, 2 * ng, s, gw::oz_box_rows()))) return st;
+    j.tmB = j.tmA;
     j.E = E;
     j.chi = (double *)chi;
     j.ng = ng;
     j.nk = (int)(kpad / gw::oz_box_k());
-    j.s = h->d.nslices;
-    j.ntiles = gw::oz_tiles(ng, bn);
+    j.s = s;
     return GW_OK;
 }
 
-int oz_schedule(std::vector<gw::OzJob> &jobs)
+int oz_clusters(size_t nitems) { return (int)std::max<size_t>(1, std::min<size_t>(nitems, num_sms() / 2)); }
+
+// Items of the Hermitian contraction: the upper tiles of every job, largest job first.  The tiles
+// beyond the last full wave of CTA pairs split their K range in p parts, one part of every tile
+// after the other (pairs that run together then read the same pairs' slices from L2): at
+// N_G = 2000, 136 tiles on 76 pairs run as 76 and 60 x 5 parts, 1.8 waves instead of 2.  A part has
+// at least 4 K-steps and costs about 2.5 K-steps more for its own epilogue, and a launch has at most
+// four waves of parts.  The scratch where the parts meet is the handle's; without room for it in
+// the memory budget the tiles stay whole.
+gw_status oz_items(gw_chi0 *h, std::vector<gw::OzJob> &jobs, std::vector<gw::OzItem> &items)
 {
     std::stable_sort(jobs.begin(), jobs.end(), [](const gw::OzJob &a, const gw::OzJob &b) {
         return (double)a.ng * a.ng * a.nk > (double)b.ng * b.ng * b.nk;
     });
-    int items = 0;
-    for (auto &j : jobs) {
-        j.item_start = items;
-        items += j.ntiles;
+    items.clear();
+    for (size_t j = 0; j < jobs.size(); ++j)
+        for (int J = 0; J * gw::oz_box_rows() < jobs[j].ng; ++J)
+            for (int I = 0; I <= J; ++I) items.push_back({(int)j, I, J, 0, jobs[j].nk, 0, 1, 0});
+    const size_t ncl = std::max(1, num_sms() / 2), full = items.size() / ncl * ncl, rest = items.size() - full;
+    if (rest == 0) return GW_OK;
+    int nk = items[full].nk;
+    for (size_t i = full; i < items.size(); ++i) nk = std::min(nk, items[i].nk);
+    int p = 1;
+    double best = 1e300;
+    for (int q = 1; q <= std::max(1, nk / 4) && q <= 16 && (q == 1 || rest * q <= 4 * ncl); ++q) {
+        const double c = (double)((rest * q + ncl - 1) / ncl) * (1.0 / q + 2.5 / nk);
+        if (c < best) {
+            best = c;
+            p = q;
+        }
     }
-    return items;
+    if (p == 1) return GW_OK;
+    const size_t need = gw::oz_part_bytes() * rest * p, flags = sizeof(int) * gw::oz_slot_flags() * ncl;
+    if (h->ozpart_cap < need || !h->ozflags) {
+        if (h->d.mem_budget_bytes && h->bytes - h->ozpart_cap + need + flags > h->d.mem_budget_bytes) return GW_OK;
+        const std::string err = h->err;
+        gw_status st = grow(h, (void **)&h->ozpart, &h->ozpart_cap, need, "split tile sums");
+        if (st == GW_ERR_OOM) {
+            h->err = err; // not a failure: whole tiles need no scratch
+            return GW_OK;
+        }
+        if (st) return st;
+        if (!h->ozflags) {
+            if ((st = grow(h, (void **)&h->ozflags, &h->ozflags_cap, flags, "split tile counters"))) return st;
+            CK(h, cudaMemset(h->ozflags, 0, flags), "split tile counters");
+        }
+    }
+    const std::vector<gw::OzItem> tail(items.begin() + full, items.end());
+    items.resize(full);
+    for (int i = 0; i < p; ++i)
+        for (size_t k = 0; k < tail.size(); ++k) {
+            const gw::OzItem &t = tail[k];
+            const int k0 = (int)((int64_t)t.nk * i / p), k1 = (int)((int64_t)t.nk * (i + 1) / p);
+            items.push_back({t.job, t.I, t.J, k0, k1 - k0, i, p, (int)k});
+        }
+    return GW_OK;
 }
 
-gw_status launch_oz_jobs(gw_chi0 *h, std::vector<gw::OzJob> &jobs, int bn)
+// A launch's job table with its item list behind it, in one block.
+size_t oz_table(const std::vector<gw::OzJob> &jobs, const std::vector<gw::OzItem> &items,
+                std::vector<unsigned char> &blob)
 {
-    const int nitems = oz_schedule(jobs);
-    const void *dj;
-    gw_status s = upload_jobs(h, jobs.data(), sizeof(gw::OzJob) * jobs.size(), &dj);
+    const size_t nj = sizeof(gw::OzJob) * jobs.size(), ni = sizeof(gw::OzItem) * items.size();
+    blob.resize(nj + ni);
+    std::memcpy(blob.data(), jobs.data(), nj);
+    std::memcpy(blob.data() + nj, items.data(), ni);
+    return nj;
+}
+
+gw_status launch_oz_jobs(gw_chi0 *h, std::vector<gw::OzJob> &jobs)
+{
+    std::vector<gw::OzItem> items;
+    std::vector<unsigned char> blob;
+    gw_status s = oz_items(h, jobs, items);
     if (s) return s;
-    const int grid = std::max(1, std::min(nitems, num_sms()));
+    const size_t off = oz_table(jobs, items, blob);
+    const void *dj;
+    if ((s = upload_jobs(h, blob.data(), blob.size(), &dj))) return s;
     Scope sc(h, "ozaki_gemm");
-    CK(h, gw::launch_oz_gemm_jobs(bn, (const gw::OzJob *)dj, (int)jobs.size(), nitems, grid, h->status, h->st),
+    CK(h, gw::launch_oz_gemm_jobs((const gw::OzJob *)dj, (const gw::OzItem *)((const char *)dj + off),
+                                  (int)items.size(), oz_clusters(items.size()), oz_scratch(h), h->status, h->st),
        "oz gemm");
+    return GW_OK;
+}
+
+// Every tile of the general products, the tiles of one block of rows one after the other (pairs of
+// CTAs that run together share A rows).
+gw_status launch_oz_general(gw_chi0 *h, const std::vector<gw::OzJob> &jobs)
+{
+    std::vector<gw::OzItem> items;
+    std::vector<unsigned char> blob;
+    const int64_t b = gw::oz_box_rows(); // complex rows and columns of a tile
+    for (size_t j = 0; j < jobs.size(); ++j)
+        for (int I = 0; I * b < jobs[j].rows_a; ++I)
+            for (int J = 0; J * b < jobs[j].cols_b; ++J) items.push_back({(int)j, I, J, 0, jobs[j].nk});
+    const size_t off = oz_table(jobs, items, blob);
+    const void *dj;
+    gw_status s = upload_jobs(h, blob.data(), blob.size(), &dj);
+    if (s) return s;
+    CK(h, gw::launch_oz_gemm_general((const gw::OzJob *)dj, (const gw::OzItem *)((const char *)dj + off),
+                                     (int)items.size(), oz_clusters(items.size()), h->status, h->st),
+       "oz general product");
     return GW_OK;
 }
 
@@ -313,7 +380,7 @@ gw_status launch_oz_jobs(gw_chi0 *h, std::vector<gw::OzJob> &jobs, int bn)
 gw_status contract_chunk_ozaki(gw_chi0 *h, const double2 *M, int64_t P, int ng, const double *delta, int64_t dstride,
                                int nw, double2 *chi)
 {
-    const int s = h->d.nslices;
+    const int s = gw::oz_slices(h->d.nslices);
     const int64_t kpad = (P + 63) / 64 * 64;
     const size_t zper = (size_t)s * 2 * ng * kpad; // bf16 slices of one frequency
     // several frequencies: slice a group at once (M read once per pass for the group), the group's
@@ -328,7 +395,6 @@ gw_status contract_chunk_ozaki(gw_chi0 *h, const double2 *M, int64_t P, int ng, 
         Scope sc(h, "oz_split");
         CK(h, gw::launch_oz_sqrt(delta, (int64_t)nw * dstride, h->spbuf, h->st), "oz sqrt");
     }
-    const int bn = contraction_bn(h, ng);
     for (int w0 = 0; w0 < nw; w0 += wg) {
         const int cnt = std::min(wg, nw - w0);
         const double *sp = h->spbuf + (int64_t)w0 * dstride;
@@ -343,24 +409,17 @@ gw_status contract_chunk_ozaki(gw_chi0 *h, const double2 *M, int64_t P, int ng, 
                    "oz slices (frequency group)");
             }
         }
+        // one launch per frequency, or for as many as fill a wave of CTA pairs when one has fewer tiles
+        const int64_t nt = (ng + gw::oz_box_rows() - 1) / gw::oz_box_rows(), tiles = nt * (nt + 1) / 2;
+        std::vector<gw::OzJob> jobs;
         for (int j = 0; j < cnt; ++j) {
-            std::vector<gw::OzJob> jobs(1);
-            if ((st = oz_job(h, jobs[0], (uint16_t *)h->Zbuf + zper * j, kpad, ng, h->Ebuf + (size_t)ng * j,
-                             chi + (int64_t)(w0 + j) * ng * ng, bn)))
+            jobs.emplace_back();
+            if ((st = oz_job(h, jobs.back(), (uint16_t *)h->Zbuf + zper * j, kpad, ng, h->Ebuf + (size_t)ng * j,
+                             chi + (int64_t)(w0 + j) * ng * ng)))
                 return st;
-            // few tiles (small N_G): split K over jobs so that about one wave of blocks runs,
-            // at least 8 K-steps each; the atomic epilogue adds the parts
-            const int nk = jobs[0].nk;
-            const int ks = std::max(1, std::min(num_sms() / std::max(1, jobs[0].ntiles), nk / 8));
-            if (ks > 1) {
-                const gw::OzJob base = jobs[0];
-                jobs.assign(ks, base);
-                for (int i = 0; i < ks; ++i) {
-                    jobs[i].kb0 = (int)((int64_t)nk * i / ks);
-                    jobs[i].nk = (int)((int64_t)nk * (i + 1) / ks) - jobs[i].kb0;
-                }
-            }
-            if ((st = launch_oz_jobs(h, jobs, bn))) return st;
+            if (j + 1 < cnt && tiles * (int64_t)jobs.size() < num_sms() / 2) continue;
+            if ((st = launch_oz_jobs(h, jobs))) return st;
+            jobs.clear();
         }
     }
     return GW_OK;
@@ -376,21 +435,20 @@ gw_status contract_chunk(gw_chi0 *h, const double2 *M, int64_t P, int ng, const 
     return launch_f64_jobs(h, jobs, h->tuned_bt, h->tuned_waves);
 }
 
-// Real K extent of a general product with ka complex inner entries, padded for the TMA boxes.
-int64_t oz_kpad(int ka) { return ((int64_t)2 * ka + 63) / 64 * 64; }
+// K extent of a general product with ka complex inner entries, padded for the TMA boxes.
+int64_t oz_kpad(int ka) { return ((int64_t)ka + 63) / 64 * 64; }
 
 // B operand of a general split product: the columns of B [ka][nout] (complex, row-major)
 // into the handle's ZB / EB buffers.
 gw_status oz_prepare_b(gw_chi0 *h, const double2 *B, int ka, int nout, int nslices)
 {
-    const int s = nslices > 0 ? nslices : h->d.nslices;
+    const int s = gw::oz_slices(nslices > 0 ? nslices : h->d.nslices);
     const int64_t kpad = oz_kpad(ka);
     gw_status st;
     if ((st = grow(h, &h->ZBbuf, &h->ZBcap, (size_t)s * 2 * nout * kpad * 2, "product operand slices")) ||
         (st = grow(h, (void **)&h->EBbuf, &h->EBcap, sizeof(int) * (size_t)nout, "product operand exponents")))
         return st;
-    CK(h, gw::launch_oz_split_cols(B, ka, nout, nout, 1, false, s, kpad, h->ZBbuf, h->EBbuf, h->st),
-       "oz column slices");
+    CK(h, gw::launch_oz_split(B, nout, ka, 1, nout, false, s, kpad, h->ZBbuf, h->EBbuf, h->st), "oz column slices");
     return GW_OK;
 }
 
@@ -399,36 +457,28 @@ gw_status oz_prepare_b(gw_chi0 *h, const double2 *B, int ka, int nout, int nslic
 // the two uses).
 gw_status oz_product(gw_chi0 *h, const double2 *A, int64_t rows, int ka, int nout, double2 *Y, int nslices)
 {
-    const int s = nslices > 0 ? nslices : h->d.nslices;
+    const int s = gw::oz_slices(nslices > 0 ? nslices : h->d.nslices);
     const int64_t kpad = oz_kpad(ka);
-    const int bn = 2 * nout >= 256 ? 256 : 128;
     gw_status st;
-    if ((st = grow(h, &h->Zbuf, &h->Zcap, (size_t)s * rows * kpad * 2, "slice buffer")) ||
+    if ((st = grow(h, &h->Zbuf, &h->Zcap, (size_t)s * 2 * rows * kpad * 2, "slice buffer")) ||
         (st = grow(h, (void **)&h->EAbuf, &h->EAcap, sizeof(int) * (size_t)rows, "product row exponents")))
         return st;
     CK(h, cudaMemsetAsync(Y, 0, sizeof(double2) * (size_t)rows * nout, h->st), "zero product");
-    CK(h, gw::launch_oz_split_rows(A, rows, ka, s, kpad, h->Zbuf, h->EAbuf, h->st), "oz row slices");
+    CK(h, gw::launch_oz_split(A, rows, ka, ka, 1, false, s, kpad, h->Zbuf, h->EAbuf, h->st), "oz row slices");
     gw::OzJob j;
     std::memset(&j, 0, sizeof j);
-    if ((st = make_tmap_z(h, &j.tmA, h->Zbuf, kpad, (int)rows, s, gw::oz_box_rows_a())) ||
-        (st = make_tmap_z(h, &j.tmB, h->ZBbuf, kpad, 2 * nout, s, bn)))
+    if ((st = make_tmap_z(h, &j.tmA, h->Zbuf, kpad, (int)(2 * rows), s, gw::oz_box_rows())) ||
+        (st = make_tmap_z(h, &j.tmB, h->ZBbuf, kpad, 2 * nout, s, gw::oz_box_rows())))
         return st;
     j.E = h->EAbuf;
     j.E2 = h->EBbuf;
     j.out = (double *)Y;
     j.ldo = 2 * (int64_t)nout;
     j.rows_a = (int)rows;
-    j.rows_b = 2 * nout;
+    j.cols_b = nout;
     j.nk = (int)(kpad / gw::oz_box_k());
     j.s = s;
-    j.ntiles = (int)((rows + gw::oz_box_rows_a() - 1) / gw::oz_box_rows_a()) * ((2 * nout + bn - 1) / bn);
-    j.item_start = 0;
-    const void *dj;
-    if ((st = upload_jobs(h, &j, sizeof j, &dj))) return st;
-    CK(h, gw::launch_oz_gemm_general(bn, (const gw::OzJob *)dj, 1, j.ntiles, std::min(j.ntiles, num_sms()), h->status,
-                                     h->st),
-       "oz general product");
-    return GW_OK;
+    return launch_oz_general(h, {j});
 }
 
 bool alias_free(const gw_chi0 *h, const BandSet &v, const BandSet &c, const Sphere &s, int *axis)
@@ -620,28 +670,17 @@ gw_status zd_stage_a(gw_chi0 *h, int iq, const CUtensorMap &tmA, const CUtensorM
 }
 
 // Split-precision streamed compute with the contraction of job j (chunk, frequency) on a
-// high-priority second stream while the user stream forms the pair elements and slices of
-// the jobs after it.  The split-precision contraction runs on the tensor cores and the pair
-// kernel on the FP32 pipes, so the two share the SMs: the contraction uses a 2-deep TMA ring
-// (99 KB of shared memory) to fit beside two pair-kernel blocks.  Slices, exponents and job
-// tables alternate between two buffer sets; job j waits for the contraction of job j - 2.
-// The overlapped path pays off when two pair-kernel blocks fit on an SM beside a contraction
-// block (48^3: 180 vs 189 ms per q-point); with room for one (72^3, 112 KB pair blocks) the pair
-// kernel, the critical path, runs at half its occupancy (5.9 vs 4.8 s per q-point).
+// high-priority second stream while the user stream forms the pair elements and slices of the jobs
+// after it.  A contraction block takes a whole SM, so the two kernels share the GPU only where one
+// of them leaves SMs idle (a launch's ramp and its last wave): 8 % faster for chunks of 500 pairs
+// on 40^3, 2 % for 4096 on 24^3, no difference for full chunks.  Slices, exponents and job tables
+// alternate between two buffer sets; job j waits for the contraction of job j - 2.  Taken where
+// the pair kernel's blocks use at most 64 KB of shared memory (24^3 to 48^3).
 bool overlap_enabled(gw_chi0 *h, const gw::PairPlan &pp)
 {
     if (h->d.prec != GW_PREC_OZAKI_BF16 || h->d.single_stream || h->d.mtxel_prec != GW_MTXEL_TWOFLOAT) return false;
     const size_t ps = gw::pair_tf_ct_smem_bytes(pp);
-    if (ps == 0) return false;
-    int dev = 0, sm_bytes = 0, resv = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    const size_t gs = std::max(gw::oz_smem_bytes(256, 2), gw::oz_smem_bytes(h->tuned_bn, 2));
-    return 2 * (ps + (size_t)resv) + gs + (size_t)resv <= (size_t)sm_bytes;
+    return ps > 0 && ps <= 64 * 1024;
 }
 
 gw_status resident_begin(gw_chi0 *h, int64_t P, int ng, bool *use)
@@ -668,7 +707,7 @@ gw_status compute_overlap(gw_chi0 *h, int iq, const gw::OmegaList &om, double2 *
 {
     const Sphere &sp = h->sph[iq];
     const BandSet &v = h->val[iq];
-    const int ng = sp.ng, nw = om.nw, s = h->d.nslices;
+    const int ng = sp.ng, nw = om.nw, s = gw::oz_slices(h->d.nslices);
     const int64_t P = (int64_t)v.nb * h->cond.nb;
     const int64_t chunk = std::min<int64_t>(h->d.pair_chunk, P);
     const int64_t kpad_max = (chunk + 63) / 64 * 64;
@@ -677,11 +716,9 @@ gw_status compute_overlap(gw_chi0 *h, int iq, const gw::OmegaList &om, double2 *
     if ((st = grow(h, (void **)&h->spbuf, &h->spcap, sizeof(double) * (size_t)nw * chunk, "scale buffer"))) return st;
     for (int b = 0; b < 2; ++b)
         if ((st = grow(h, &h->ovZ[b], &h->ovZcap[b], (size_t)s * 2 * ng * kpad_max * 2, "slice buffer")) ||
-            (st = grow(h, (void **)&h->ovE[b], &h->ovEcap[b], sizeof(int) * (size_t)ng, "exponent buffer")) ||
-            (st = grow(h, &h->ovJ[b], &h->ovJcap[b], sizeof(gw::OzJob) * 256, "job table")))
+            (st = grow(h, (void **)&h->ovE[b], &h->ovEcap[b], sizeof(int) * (size_t)ng, "exponent buffer")))
             return st;
     if ((st = ensure_overlap_stream(h))) return st;
-    const int bn = contraction_bn(h, ng);
     gw::PairPlan pp = pair_plan(h, sp);
     bool used[2] = {false, false};
     int64_t j = 0;
@@ -715,17 +752,20 @@ gw_status compute_overlap(gw_chi0 *h, int iq, const gw::OmegaList &om, double2 *
                 CK(h, gw::launch_oz_slice(Mc, cnt, ng, spw, h->ovE[b], s, kpad, h->ovZ[b], h->st), "oz slices");
             }
             std::vector<gw::OzJob> jobs(1);
-            if ((st = oz_job(h, jobs[0], h->ovZ[b], kpad, ng, h->ovE[b], cq + (int64_t)w * ng * ng, bn))) return st;
-            const int nitems = oz_schedule(jobs);
-            CK(h, cudaMemcpyAsync(h->ovJ[b], jobs.data(), sizeof(gw::OzJob) * jobs.size(), cudaMemcpyHostToDevice,
-                                  h->st),
-               "job table");
+            if ((st = oz_job(h, jobs[0], h->ovZ[b], kpad, ng, h->ovE[b], cq + (int64_t)w * ng * ng))) return st;
+            std::vector<gw::OzItem> items;
+            std::vector<unsigned char> blob;
+            if ((st = oz_items(h, jobs, items))) return st;
+            const size_t off = oz_table(jobs, items, blob);
+            if ((st = grow(h, &h->ovJ[b], &h->ovJcap[b], blob.size(), "job table"))) return st;
+            CK(h, cudaMemcpyAsync(h->ovJ[b], blob.data(), blob.size(), cudaMemcpyHostToDevice, h->st), "job table");
             CK(h, cudaEventRecord(h->ov_split[b], h->st), "record");
             CK(h, cudaStreamWaitEvent(h->ov_st, h->ov_split[b], 0), "wait slices");
             {
                 Scope sc(h, "ozaki_gemm", h->ov_st);
-                CK(h, gw::launch_oz_gemm_jobs(bn, (const gw::OzJob *)h->ovJ[b], (int)jobs.size(), nitems,
-                                              std::max(1, std::min(nitems, num_sms())), h->status, h->ov_st, 2),
+                CK(h, gw::launch_oz_gemm_jobs((const gw::OzJob *)h->ovJ[b],
+                                              (const gw::OzItem *)((const char *)h->ovJ[b] + off), (int)items.size(),
+                                              oz_clusters(items.size()), oz_scratch(h), h->status, h->ov_st),
                    "oz gemm");
             }
             CK(h, cudaEventRecord(h->ov_gemm[b], h->ov_st), "record");
@@ -854,6 +894,8 @@ void gw_chi0_destroy(gw_chi0 *h)
         if (h->ov_gemm[b]) cudaEventDestroy(h->ov_gemm[b]);
     }
     if (h->ov_st) cudaStreamDestroy(h->ov_st);
+    dfree(h, h->ozpart, h->ozpart_cap);
+    dfree(h, h->ozflags, h->ozflags_cap);
     dfree(h, h->epsbuf, h->epscap);
     dfree(h, h->Mres, h->Mres_cap);
     for (auto &b : h->gpp) dfree(h, b.p, b.cap);
@@ -1256,7 +1298,7 @@ int gw_chi0_tuning(const gw_chi0 *h, int *tile_f64, int *waves_f64, int *tile_sp
     if (!h) return 0;
     if (tile_f64) *tile_f64 = h->tuned_bt;
     if (waves_f64) *waves_f64 = h->tuned_waves;
-    if (tile_split) *tile_split = h->tuned_bn;
+    if (tile_split) *tile_split = 256;
     return (int)h->tune_cache.size();
 }
 
@@ -1306,6 +1348,8 @@ gw_status gw_chi0_sync(gw_chi0 *h)
     int st = 0;
     CK(h, cudaMemcpy(&st, h->status, sizeof(int), cudaMemcpyDeviceToHost), "status");
     CK(h, cudaMemset(h->status, 0, sizeof(int)), "status reset");
+    if ((st & gw::kStatusTimeout) && h->ozflags) // parts that never met leave their counters behind
+        CK(h, cudaMemset(h->ozflags, 0, h->ozflags_cap), "split tile counters");
     if (st & gw::kStatusTimeout) return fail(h, GW_ERR_TIMEOUT, "a bounded device-side wait gave up");
     if (st & gw::kStatusNoSlot) return fail(h, GW_ERR_CUDA, "a pair block found no free scratch slot");
     if (st & gw::kStatusBounds) return fail(h, GW_ERR_CUDA, "an index outside its buffer (bounds-checked build)");

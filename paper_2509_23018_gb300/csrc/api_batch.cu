@@ -48,7 +48,7 @@ BatchLayout batch_layout(gw_chi0 *h, int nq, const int *iq, int nw)
             sg.kpad = (sg.cnt + 63) / 64 * 64;
             sg.zoff = (int64_t)L.Ztot;
             sg.eoff = (int64_t)L.Etot;
-            L.Ztot += (size_t)h->d.nslices * 2 * ng * sg.kpad;
+            L.Ztot += (size_t)gw::oz_slices(h->d.nslices) * 2 * ng * sg.kpad;
             L.Etot += (size_t)ng;
             L.seg.push_back(sg);
         }
@@ -110,7 +110,7 @@ gw_status batch_oz_split(gw_chi0 *h, int nq, int w, const BatchLayout &L)
         const double *sp = h->SPall + L.doff[sg.q] + (int64_t)w * L.P[sg.q] + sg.p0;
         const double2 *M = h->Mall + L.moff[sg.q] + sg.p0 * ng;
         CK(h, gw::launch_oz_colexp(M, sg.cnt, ng, sp, h->Eall + sg.eoff, h->st), "oz exponents");
-        CK(h, gw::launch_oz_slice(M, sg.cnt, ng, sp, h->Eall + sg.eoff, h->d.nslices, sg.kpad,
+        CK(h, gw::launch_oz_slice(M, sg.cnt, ng, sp, h->Eall + sg.eoff, gw::oz_slices(h->d.nslices), sg.kpad,
                                   (uint16_t *)h->Zall + sg.zoff, h->st),
            "oz slices");
     }
@@ -129,7 +129,7 @@ gw_status batch_f64_jobs(gw_chi0 *h, int nq, int nw, const BatchLayout &L, doubl
     return GW_OK;
 }
 
-gw_status batch_oz_jobs(gw_chi0 *h, int nq, int w, const BatchLayout &L, double2 *chi, int bn,
+gw_status batch_oz_jobs(gw_chi0 *h, int nq, int w, const BatchLayout &L, double2 *chi,
                         std::vector<gw::OzJob> &jobs)
 {
     (void)nq;
@@ -138,15 +138,16 @@ gw_status batch_oz_jobs(gw_chi0 *h, int nq, int w, const BatchLayout &L, double2
         const int ng = L.ng[sg.q];
         gw::OzJob j;
         gw_status s = oz_job(h, j, (uint16_t *)h->Zall + sg.zoff, sg.kpad, ng, h->Eall + sg.eoff,
-                             chi + L.coff[sg.q] + (int64_t)w * ng * ng, bn);
+                             chi + L.coff[sg.q] + (int64_t)w * ng * ng);
         if (s) return s;
         jobs.push_back(j);
     }
     return GW_OK;
 }
 
-// Time each launch-shape candidate of the contraction on the real data (into chi, which
-// is cleared afterwards by the real run) and keep the fastest.
+// Time each launch-shape candidate of the FP64 contraction on the real data (into chi, which is
+// cleared afterwards by the real run) and keep the fastest.  The split contraction has one tile
+// shape: nothing to time.
 gw_status batch_autotune(gw_chi0 *h, int nq, const int *iq, int nw, const gw::OmegaList &om, const BatchLayout &L,
                          double2 *chi)
 {
@@ -155,20 +156,18 @@ gw_status batch_autotune(gw_chi0 *h, int nq, const int *iq, int nw, const gw::Om
     if (it != h->tune_cache.end()) {
         h->tuned_bt = it->second[0];
         h->tuned_waves = it->second[1];
-        h->tuned_bn = it->second[2];
-        h->bn_tuned = h->d.prec != GW_PREC_FP64;
         return GW_OK;
     }
-    gw_status s = batch_stage_a(h, nq, iq, om, L);
-    if (s) return s;
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    float best = 1e30f;
-    std::array<int, 3> pick = {h->tuned_bt, h->tuned_waves, h->tuned_bn};
-    const bool saved_timing = h->timing;
-    h->timing = false;
+    std::array<int, 2> pick = {h->tuned_bt, h->tuned_waves};
     if (h->d.prec == GW_PREC_FP64) {
+        gw_status s = batch_stage_a(h, nq, iq, om, L);
+        if (s) return s;
+        cudaEvent_t e0, e1;
+        cudaEventCreate(&e0);
+        cudaEventCreate(&e1);
+        float best = 1e30f;
+        const bool saved_timing = h->timing;
+        h->timing = false;
         for (int bt : {64, 32})
             for (int waves : {2, 4, 8}) {
                 std::vector<gw::F64Job> jobs;
@@ -181,34 +180,17 @@ gw_status batch_autotune(gw_chi0 *h, int nq, const int *iq, int nw, const gw::Om
                 cudaEventElapsedTime(&ms, e0, e1);
                 if (ms < best) {
                     best = ms;
-                    pick = {bt, waves, h->tuned_bn};
+                    pick = {bt, waves};
                 }
             }
-    } else if (!(s = batch_oz_split(h, nq, 0, L))) {
-        for (int bn : {256, 240, 128}) {
-            std::vector<gw::OzJob> jobs;
-            if ((s = batch_oz_jobs(h, nq, 0, L, chi, bn, jobs))) break;
-            cudaEventRecord(e0, h->st);
-            if ((s = launch_oz_jobs(h, jobs, bn))) break;
-            cudaEventRecord(e1, h->st);
-            cudaEventSynchronize(e1);
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < best) {
-                best = ms;
-                pick = {h->tuned_bt, h->tuned_waves, bn};
-            }
-        }
+        h->timing = saved_timing;
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        if (s) return s;
     }
-    h->timing = saved_timing;
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (s) return s;
     h->tune_cache[key] = pick;
     h->tuned_bt = pick[0];
     h->tuned_waves = pick[1];
-    h->tuned_bn = pick[2];
-    h->bn_tuned = h->d.prec != GW_PREC_FP64;
     return GW_OK;
 }
 
@@ -229,14 +211,15 @@ gw_status compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const double 
     if ((s = batch_autotune(h, nq, iq, nw, om, L, (double2 *)chi))) return s;
 
     const std::string key = batch_key(h, nq, iq, nw, omega, chi, diag) + "|" + std::to_string(h->tuned_bt) + "," +
-                            std::to_string(h->tuned_waves) + "," + std::to_string(h->tuned_bn);
+                            std::to_string(h->tuned_waves);
     gw_chi0::Graph *g = nullptr;
     for (auto &x : h->graphs)
         if (x.key == key) g = &x;
     if (!g) {
         // job tables first (outside the capture), in a buffer owned by the graph
         std::vector<gw::F64Job> fj;
-        std::vector<std::vector<gw::OzJob>> oj(nw);
+        std::vector<gw::OzJob> oj;
+        std::vector<gw::OzItem> items; // the same for every frequency
         std::vector<unsigned char> blob;
         std::vector<size_t> offs;
         if (h->d.prec == GW_PREC_FP64) {
@@ -247,12 +230,15 @@ gw_status compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const double 
             std::memcpy(blob.data(), fj.data(), blob.size());
         } else {
             for (int w = 0; w < nw; ++w) {
-                if ((s = batch_oz_jobs(h, nq, w, L, (double2 *)chi, h->tuned_bn, oj[w]))) return s;
-                oz_schedule(oj[w]);
+                if ((s = batch_oz_jobs(h, nq, w, L, (double2 *)chi, oj))) return s;
+                if ((s = oz_items(h, oj, items))) return s;
                 offs.push_back(blob.size());
-                blob.resize(blob.size() + sizeof(gw::OzJob) * oj[w].size());
-                std::memcpy(blob.data() + offs.back(), oj[w].data(), sizeof(gw::OzJob) * oj[w].size());
+                blob.resize(blob.size() + sizeof(gw::OzJob) * oj.size());
+                std::memcpy(blob.data() + offs.back(), oj.data(), sizeof(gw::OzJob) * oj.size());
             }
+            offs.push_back(blob.size());
+            blob.resize(blob.size() + sizeof(gw::OzItem) * items.size());
+            std::memcpy(blob.data() + offs.back(), items.data(), sizeof(gw::OzItem) * items.size());
         }
         gw_chi0::Graph ng;
         ng.key = key;
@@ -288,11 +274,9 @@ gw_status compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const double 
                 for (int w = 0; w < nw && !body; ++w) {
                     body = batch_oz_split(h, nq, w, L);
                     if (body) break;
-                    int nitems = 0;
-                    for (auto &j : oj[w]) nitems = std::max(nitems, j.item_start + j.ntiles);
-                    const int grid = std::max(1, std::min(nitems, num_sms()));
-                    if (gw::launch_oz_gemm_jobs(h->tuned_bn, (const gw::OzJob *)((char *)ng.jobs + offs[w]),
-                                                (int)oj[w].size(), nitems, grid, h->status, h->st) != cudaSuccess)
+                    if (gw::launch_oz_gemm_jobs((const gw::OzJob *)((char *)ng.jobs + offs[w]),
+                                                (const gw::OzItem *)((char *)ng.jobs + offs[nw]), (int)items.size(),
+                                                oz_clusters(items.size()), oz_scratch(h), h->status, h->st) != cudaSuccess)
                         body = fail(h, GW_ERR_CUDA, "capture: split contraction");
                 }
             }

@@ -86,12 +86,15 @@ struct gw_chi0 {
     size_t spcap = 0;
     int *Ebuf = nullptr;       // column exponents [ng]
     size_t Ecap = 0;
+    double *ozpart = nullptr;  // sums of the parts of split tiles (contraction launches run one at a time)
+    size_t ozpart_cap = 0;
+    int *ozflags = nullptr;    // their counters
+    size_t ozflags_cap = 0;
     void *jobbuf = nullptr;    // job tables of the batched contraction kernels
     size_t jobcap = 0;
     // contraction launch shapes (set by the autotuner; these are the defaults)
-    int tuned_bt = 64, tuned_waves = 4, tuned_bn = 256;
-    bool bn_tuned = false; // tuned_bn set by the autotuner (else the width follows the wave count)
-    std::map<std::string, std::array<int, 3>> tune_cache; // signature -> (bt, waves, bn)
+    int tuned_bt = 64, tuned_waves = 4;
+    std::map<std::string, std::array<int, 2>> tune_cache; // signature -> (bt, waves)
     // batched path: every slot's M resident, one graph per call signature
     double2 *Mall = nullptr;
     size_t Mall_cap = 0;
@@ -218,7 +221,6 @@ void drain_timing(gw_chi0 *h);
 gw_status ensure_work(gw_chi0 *h, size_t m_elems, size_t d_elems);
 gw_status make_tmap(gw_chi0 *h, CUtensorMap *map, const void *M, int64_t P, int ng, int bt);
 int num_sms();
-int contraction_bn(const gw_chi0 *h, int ng); // split-precision tile width: tuned, else by the wave count
 void drop_graphs(gw_chi0 *h);
 gw_status grow(gw_chi0 *h, void **p, size_t *cap, size_t bytes, const char *what);
 gw_status upload_jobs(gw_chi0 *h, const void *src, size_t bytes, const void **dev);
@@ -227,9 +229,12 @@ gw_status f64_jobs(gw_chi0 *h, std::vector<gw::F64Job> &jobs, const double2 *M, 
 int f64_schedule(std::vector<gw::F64Job> &jobs, int waves);
 gw_status launch_f64_jobs(gw_chi0 *h, std::vector<gw::F64Job> &jobs, int bt, int waves);
 gw_status make_tmap_z(gw_chi0 *h, CUtensorMap *map, void *Z, int64_t kpad, int nrows, int s, int box_rows);
-gw_status oz_job(gw_chi0 *h, gw::OzJob &j, void *Z, int64_t kpad, int ng, const int *E, double2 *chi, int bn);
-int oz_schedule(std::vector<gw::OzJob> &jobs);
-gw_status launch_oz_jobs(gw_chi0 *h, std::vector<gw::OzJob> &jobs, int bn);
+gw_status oz_job(gw_chi0 *h, gw::OzJob &j, void *Z, int64_t kpad, int ng, const int *E, double2 *chi);
+int oz_clusters(size_t nitems);
+gw_status oz_items(gw_chi0 *h, std::vector<gw::OzJob> &jobs, std::vector<gw::OzItem> &items);
+inline gw::OzScratch oz_scratch(const gw_chi0 *h) { return {h->ozpart, h->ozflags}; }
+gw_status launch_oz_general(gw_chi0 *h, const std::vector<gw::OzJob> &jobs);
+gw_status launch_oz_jobs(gw_chi0 *h, std::vector<gw::OzJob> &jobs);
 gw_status contract_chunk_ozaki(gw_chi0 *h, const double2 *M, int64_t P, int ng, const double *delta, int64_t dstride,
                                int nw, double2 *chi);
 gw_status contract_chunk(gw_chi0 *h, const double2 *M, int64_t P, int ng, const double *delta, int64_t dstride,

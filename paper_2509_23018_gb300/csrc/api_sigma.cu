@@ -29,7 +29,7 @@ gw_status gbuf(gw_chi0 *h, int i, size_t bytes, const char *what)
 }
 
 // Energies per batch.  X^T (and its slices) for up to 16 energies, so that the second product
-// runs on 16 N_Sigma columns at once; P^T slices (28 ng^2 bytes each at s = 7) for as many of
+// runs on 16 N_Sigma columns at once; P^T slices (20 ng^2 bytes each at nslices = 7) for as many of
 // them as 32 GiB (a quarter of the handle's memory budget, when one is set) holds: one prep.
 // launch and one first-product launch per batch, so the pole parameters are read once per
 // batch and the product's tiles fill the last wave.
@@ -40,47 +40,29 @@ int x_batch(int ne) { return std::max(1, std::min(kGppBatch, ne)); }
 
 int p_batch(const gw_chi0 *h, int ebx, int ng, int s, int64_t kpad)
 {
-    const double per = (double)s * ng * kpad * 2;
+    const double per = (double)s * 2 * ng * kpad * 2;
     const double budget = h->d.mem_budget_bytes ? 0.25 * (double)h->d.mem_budget_bytes : 32.0 * 1073741824.0;
     const int eb = (int)std::min<double>(ebx, std::floor(budget / per));
     return std::max(1, eb);
 }
 
 gw_status gen_job(gw_chi0 *h, gw::OzJob &j, void *ZA, int rows_a, void *ZB, int nout, int64_t kpad, const int *EA,
-                  const int *EB, double2 *out, int64_t ldo, int bn)
+                  const int *EB, double2 *out, int64_t ldo)
 {
     std::memset(&j, 0, sizeof j);
-    const int s = h->d.nslices;
+    const int s = gw::oz_slices(h->d.nslices);
     gw_status st;
-    if ((st = make_tmap_z(h, &j.tmA, ZA, kpad, rows_a, s, gw::oz_box_rows_a())) ||
-        (st = make_tmap_z(h, &j.tmB, ZB, kpad, 2 * nout, s, bn)))
+    if ((st = make_tmap_z(h, &j.tmA, ZA, kpad, 2 * rows_a, s, gw::oz_box_rows())) ||
+        (st = make_tmap_z(h, &j.tmB, ZB, kpad, 2 * nout, s, gw::oz_box_rows())))
         return st;
     j.E = EA;
     j.E2 = EB;
     j.out = (double *)out;
     j.ldo = 2 * ldo;
     j.rows_a = rows_a;
-    j.rows_b = 2 * nout;
+    j.cols_b = nout;
     j.nk = (int)(kpad / gw::oz_box_k());
     j.s = s;
-    j.ntiles = ((rows_a + gw::oz_box_rows_a() - 1) / gw::oz_box_rows_a()) * ((2 * nout + bn - 1) / bn);
-    return GW_OK;
-}
-
-gw_status run_gen_jobs(gw_chi0 *h, std::vector<gw::OzJob> &jobs, int bn, const char *name)
-{
-    int items = 0;
-    for (auto &j : jobs) {
-        j.item_start = items;
-        items += j.ntiles;
-    }
-    const void *dj;
-    gw_status st = upload_jobs(h, jobs.data(), sizeof(gw::OzJob) * jobs.size(), &dj);
-    if (st) return st;
-    Scope sc(h, name);
-    CK(h, gw::launch_oz_gemm_general(bn, (const gw::OzJob *)dj, (int)jobs.size(), items, std::min(items, num_sms()),
-                                     h->status, h->st),
-       name);
     return GW_OK;
 }
 
@@ -93,18 +75,18 @@ gw_status sigma_split(gw_chi0 *h, int nb, int nocc, int nsig, int ng, const doub
                       const double2 *omega2, const double2 *wtilde, const double *vcoul, int ne, const double *E,
                       double2 *sigma)
 {
-    const int s = h->d.nslices;
+    const int s = gw::oz_slices(h->d.nslices);
     const int64_t kpad = oz_kpad(ng);
     const int ebx = x_batch(ne), ebp = p_batch(h, ebx, ng, s, kpad);
     const size_t nn = (size_t)ng * ng;
-    const size_t zp1 = (size_t)s * ng * kpad;       // bf16 per P^T
+    const size_t zp1 = (size_t)s * 2 * ng * kpad;   // bf16 per P^T
     const int64_t ldx = (int64_t)ebx * nsig;        // X^T row length (complex)
     gw_status st;
     if ((st = gbuf(h, kA, sizeof(float4) * nn, "pole residues")) ||
         (st = gbuf(h, kW, sizeof(float4) * nn, "mode energies")) ||
         (st = gbuf(h, kX, sizeof(double2) * (size_t)ng * ldx, "X^T")) ||
         (st = gbuf(h, kP, sizeof(double2) * (size_t)nsig * ne * nsig, "Sigma^T")) ||
-        (st = gbuf(h, kZA, 2 * (size_t)s * nsig * kpad, "M_n slices")) ||
+        (st = gbuf(h, kZA, 2 * (size_t)s * 2 * nsig * kpad, "M_n slices")) ||
         (st = gbuf(h, kZB, 2 * (size_t)s * 2 * nsig * kpad, "conj(M_n)^T slices")) ||
         (st = gbuf(h, kZP, 2 * zp1 * ebp, "P^T slices")) ||
         (st = gbuf(h, kZX, 2 * (size_t)s * 2 * ldx * kpad, "X^T slices")) ||
@@ -126,14 +108,13 @@ gw_status sigma_split(gw_chi0 *h, int nb, int nocc, int nsig, int ng, const doub
             const int cx = std::min(ebx, ne - e0);
             for (int p0 = 0; p0 < cx; p0 += ebp) items.push_back({n, e0, cx, p0, std::min(ebp, cx - p0)});
         }
-    const int bn1 = 2 * nsig >= 256 ? 256 : 128;
     std::vector<gw::OzJob> jobs;
     for (const PItem &it : items) {
         if (it.e0 == 0 && it.p0 == 0) {
             const double2 *Mn = M + (size_t)it.n * nsig * ng;
             Scope sc(h, "oz_split_m");
-            CK(h, gw::launch_oz_split_rows(Mn, nsig, ng, s, kpad, ZA, EA, h->st), "M_n slices");
-            CK(h, gw::launch_oz_split_cols(Mn, ng, nsig, 1, ng, true, s, kpad, ZB, EB, h->st), "conj(M_n)^T slices");
+            CK(h, gw::launch_oz_split(Mn, nsig, ng, ng, 1, false, s, kpad, ZA, EA, h->st), "M_n slices");
+            CK(h, gw::launch_oz_split(Mn, nsig, ng, ng, 1, true, s, kpad, ZB, EB, h->st), "conj(M_n)^T slices");
         }
         if (it.p0 == 0) CK(h, cudaMemsetAsync(XT, 0, sizeof(double2) * (size_t)ng * ldx, h->st), "zero X^T");
         {
@@ -148,22 +129,25 @@ gw_status sigma_split(gw_chi0 *h, int nb, int nocc, int nsig, int ng, const doub
         jobs.assign(it.cp, gw::OzJob{});
         for (int j = 0; j < it.cp; ++j)
             if ((st = gen_job(h, jobs[j], ZP + 2 * zp1 * j, ng, ZB, nsig, kpad, EP + (size_t)j * ng, EB,
-                              XT + (size_t)(it.p0 + j) * nsig, ldx, bn1)))
+                              XT + (size_t)(it.p0 + j) * nsig, ldx)))
                 return st;
-        if ((st = run_gen_jobs(h, jobs, bn1, "gpp_gemm_x"))) return st;
+        {
+            Scope sc(h, "gpp_gemm_x");
+            if ((st = launch_oz_general(h, jobs))) return st;
+        }
         if (it.p0 + it.cp == it.cx) {
             {
                 Scope sc(h, "oz_split_x");
-                CK(h, gw::launch_oz_split_cols(XT, ng, it.cx * nsig, ldx, 1, false, s, kpad, ZX, EX, h->st),
+                CK(h, gw::launch_oz_split(XT, it.cx * nsig, ng, 1, ldx, false, s, kpad, ZX, EX, h->st),
                    "X^T slices");
             }
             // Sigma^T[m][(e, l)] += sum_c M_n[m][c] X^T[c][(e, l)]
-            const int bn2 = 2 * it.cx * nsig >= 256 ? 256 : 128;
             jobs.assign(1, gw::OzJob{});
             if ((st = gen_job(h, jobs[0], ZA, nsig, ZX, it.cx * nsig, kpad, EA, EX, ST + (size_t)it.e0 * nsig,
-                              (int64_t)ne * nsig, bn2)))
+                              (int64_t)ne * nsig)))
                 return st;
-            if ((st = run_gen_jobs(h, jobs, bn2, "gpp_gemm_sigma"))) return st;
+            Scope sc(h, "gpp_gemm_sigma");
+            if ((st = launch_oz_general(h, jobs))) return st;
         }
     }
     Scope sc(h, "gpp_untranspose");

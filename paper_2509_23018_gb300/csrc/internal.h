@@ -146,35 +146,43 @@ cudaError_t launch_oz_slice(const double2 *M, int64_t P, int ng, const double *s
                             int64_t kpad, void *Z, cudaStream_t st);
 // One job = the split contraction of one chunk into one chi block (upper tiles).
 struct __align__(128) OzJob {
-    CUtensorMap tmA, tmB; // slices [s][2 ng][kpad] bf16, boxes {64, 128} and {64, BN}
+    CUtensorMap tmA, tmB; // slices [s][2 ng][kpad] bf16, boxes {64, 128}
     const int *E;         // [ng] column exponents
     double *chi;          // [ng][ng] complex
-    int ng, nk, s, ntiles, item_start;
-    int kb0;              // first K-step of this job (jobs may split K; the epilogue adds)
-    // general product (launch_oz_gemm_general): out[rows_a][rows_b] real (complex pairs)
-    // += A B with A slices by row (exponents E[rows_a]) and B^T slices by row (exponents
-    // E2[rows_b / 2])
+    int ng, nk, s;
+    // general product (launch_oz_gemm_general): out[rows_a][cols_b] (complex, rows of ldo doubles)
+    // += A B with the slices of A's rows (tmA, exponents E[rows_a]) and of B's columns (tmB,
+    // exponents E2[cols_b])
     const int *E2;
     double *out;
     int64_t ldo;
-    int rows_a, rows_b;
+    int rows_a, cols_b;
 };
-// stages: TMA ring depth, 4 (default) or 2 (room on the SM for pair-kernel blocks alongside)
-cudaError_t launch_oz_gemm_jobs(int bn, const OzJob *jobs, int njobs, int nitems, int grid, int *status,
-                                cudaStream_t st, int stages = 4);
-int oz_tiles(int ng, int bn);
-int oz_pick_bn(int ng, int nsm); // tile width (240 or 256) by the wave count, without a tuned value
-// General split product: Y[rows][nout] (complex, row-major, overwritten) = A[rows][ka] B[ka][nout]
-// (complex, row-major), A split by rows and B by columns into s six-bit BF16 slices.
-// ZA: s * rows * kpad bf16, ZB: s * 2 nout * kpad bf16, EA: rows ints, EB: nout ints,
-// kpad = ka rounded up to a multiple of 32 complex (64 real) entries.
-// conj: split the rows of conj(A) / the columns of conj(B).  B[g][b] is read at B[g sk + b sj]
-// (sk = nout, sj = 1: row-major [ka][nout]; sk = 1, sj = ka: a row-major [nout][ka] transpose).
-cudaError_t launch_oz_split_rows(const double2 *A, int64_t rows, int ka, int s, int64_t kpad, void *ZA, int *EA,
-                                 cudaStream_t st, bool conj = false);
-cudaError_t launch_oz_split_cols(const double2 *B, int ka, int nout, int64_t sk, int64_t sj, bool conj, int s,
-                                 int64_t kpad, void *ZB, int *EB, cudaStream_t st);
-// Plasmon-pole prep. step straight into row slices of P^T (the layout of launch_oz_split_rows with
+// One unit of work of a launch: a tile of a job (oz_box_rows() complex rows and columns) over the
+// K-steps [kb0, kb0 + nk).  parts > 1: part `part` of the K range of tile `slot` of the launch's split
+// tiles; the parts' sums meet in scratch and are added in their order by whichever comes last.
+struct OzItem {
+    int job, I, J, kb0, nk, part, parts, slot;
+};
+// Scratch of a launch with split tiles: oz_part_bytes() per (slot, part), oz_slot_flags() counters per
+// slot, zero before the first launch and again after every launch.
+struct OzScratch {
+    double *sums;
+    int *flags;
+};
+size_t oz_part_bytes();
+int oz_slot_flags();
+// clusters: pairs of CTAs
+cudaError_t launch_oz_gemm_jobs(const OzJob *jobs, const OzItem *items, int nitems, int clusters, OzScratch scr,
+                                int *status, cudaStream_t st);
+int oz_slices(int nslices); // 9-bit slices for the accuracy of nslices six-bit ones
+// Slices of the general split product Y = A B: the rows of A or the columns of B, `rows` of them
+// with ka complex entries each, entry g of row p at A[p sr + g sk], into s nine-bit BF16 slices
+// Z[i][2 p + {Re, Im}][kpad] with exponents E[p]; kpad = ka rounded up to a multiple of 64.
+// conj: of the conjugate.
+cudaError_t launch_oz_split(const double2 *A, int64_t rows, int ka, int64_t sr, int64_t sk, bool conj, int s,
+                            int64_t kpad, void *Z, int *E, cudaStream_t st);
+// Plasmon-pole prep. step straight into row slices of P^T (the layout of launch_oz_split with
 // rows = ka = ng): P[g][c] = A[g][c] / (d - sgn wt[g][c]) in two-float arithmetic, At / Wt = A
 // and wt transposed [c][g] as two-float (hi, lo) pairs (gpp_setup_tf), for cnt <= kGppMaxE
 // energies d[0..cnt) (host) at once: slices of energy j at Z + j zstride (bf16 elements),
@@ -185,10 +193,9 @@ struct GppEnergies {
 };
 cudaError_t launch_gpp_prep_split(const float4 *At, const float4 *Wt, int ng, const double *d, int cnt, float sgn,
                                   int s, int64_t kpad, int64_t zstride, void *Z, int *E, cudaStream_t st);
-cudaError_t launch_oz_gemm_general(int bn, const OzJob *jobs, int njobs, int nitems, int grid, int *status,
+cudaError_t launch_oz_gemm_general(const OzJob *jobs, const OzItem *items, int nitems, int clusters, int *status,
                                    cudaStream_t st);
-size_t oz_smem_bytes(int bn, int stages = 4);
-int oz_box_rows_a();
+int oz_box_rows();
 int oz_box_k();
 
 // ---- adjoint of L = Re Tr(W chi) (adjoint.cu)

@@ -1,12 +1,14 @@
 // Digit step of the split (Ozaki) representation in integer arithmetic.
 //
 // A value x of a row or column with exponent E (E = ilogb of the row's largest magnitude + 2)
-// is written as x = 2^E sum_{i=0..s-1} 2^(-6 (i + 1)) d_i with balanced base-64 digits: the
-// integer N = round(x 2^(6 s - E)) (to nearest, ties to even) is cut into d_{s-1}, ..., d_1 in
-// [-32, 31] from the least significant end and d_0, which keeps the rest.  N is formed from the
-// bits of x and the digits are bit fields of N + sum_{k < s-1} 32 64^k (its plain base-64 fields
-// are d_k + 32), so no step runs on the FP64 pipe (1/64 of the FP32 rate on this GPU) or on the
-// 64-bit conversion units.  Host and device compile the same code.
+// is written as x = 2^(E - F) sum_{i=0..s-1} 2^(B (s - 1 - i)) d_i with balanced base-2^B digits:
+// the integer N = round(x 2^(F - E)) (to nearest, ties to even) is cut into d_{s-1}, ..., d_1 in
+// [-2^(B-1), 2^(B-1) - 1] from the least significant end and d_0, which keeps the rest.  N is
+// formed from the bits of x and the digits are bit fields of N + sum_{k < s-1} 2^(B-1) 2^(B k) (its
+// plain base-2^B fields are d_k + 2^(B-1)), so no step runs on the FP64 pipe (1/64 of the FP32
+// rate on this GPU) or on the 64-bit conversion units.  The kernels take B = 9 and F = 9 s - 1
+// (oz_frac_bits): |x| < 2^(E - 1) leaves the top digit within +-128 and the others within
+// +-256, all exact in BF16.  Host and device compile the same code.
 #pragma once
 #include <cstdint>
 #include <cstring>
@@ -60,7 +62,7 @@ __host__ __device__ __forceinline__ int oz_expo_pos(double a, int no_column)
 }
 
 // round(x 2^h), ties to even, h = sh clamped to [-1022, 1023].  The split's exponent bounds
-// |x 2^h| by 2^47, so N is formed by one right shift of the 53-bit significand (k >= 6).
+// |x 2^h| by 2^52, so N is formed by one right shift of the 53-bit significand (k >= 1).
 __host__ __device__ __forceinline__ long long oz_round_scaled(double x, int sh)
 {
     const int h = sh < -1022 ? -1022 : (sh > 1023 ? 1023 : sh);
@@ -81,11 +83,18 @@ __host__ __device__ __forceinline__ long long oz_round_scaled(double x, int sh)
     return (b >> 63) ? -(long long)q : (long long)q;
 }
 
-// sum_{k < s-1} 32 64^k: added to N it turns the balanced digits d_k into the fields d_k + 32
+constexpr int kOzBeta = 9; // bits per digit of the kernels' slices
+
+// F of the kernels' slices: N = round(x 2^(F - E)), |N| < 2^(F - 1)
+__host__ __device__ constexpr int oz_frac_bits(int s) { return kOzBeta * s - 1; }
+
+// sum_{k < s-1} 2^(B-1) 2^(B k): added to N it turns the balanced digits d_k into the fields
+// d_k + 2^(B-1)
+template <int B = 6>
 __host__ __device__ __forceinline__ long long oz_digit_bias(int s)
 {
     long long b = 0;
-    for (int k = 0; k < s - 1; ++k) b |= 32ll << (6 * k);
+    for (int k = 0; k < s - 1; ++k) b |= (1ll << (B - 1)) << (B * k);
     return b;
 }
 
@@ -107,14 +116,16 @@ __host__ __device__ __forceinline__ uint16_t oz_small_bf16(int v)
 #endif
 }
 
-// the s digits of N, d_i at out[i plane] (d_0 the most significant); bias = oz_digit_bias(s)
+// the s digits of N, d_i at out[i plane] (d_0 the most significant); bias = oz_digit_bias<B>(s)
+template <int B = 6>
 __host__ __device__ __forceinline__ void oz_store_digits(long long N, int s, long long bias, uint16_t *out,
                                                          int64_t plane)
 {
     const long long nb = N + bias;
     for (int k = 0; k < s - 1; ++k)
-        out[(int64_t)(s - 1 - k) * plane] = oz_small_bf16((int)((nb >> (6 * k)) & 63) - 32);
-    out[0] = oz_small_bf16((int)(nb >> (6 * (s - 1))));
+        out[(int64_t)(s - 1 - k) * plane] =
+            oz_small_bf16((int)((nb >> (B * k)) & ((1 << B) - 1)) - (1 << (B - 1)));
+    out[0] = oz_small_bf16((int)(nb >> (B * (s - 1))));
 }
 
 } // namespace gw

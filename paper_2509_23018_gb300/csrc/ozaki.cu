@@ -7,16 +7,20 @@
 //
 // Splitting (per chunk of pairs and per complex column G, exponent E_G with
 // max_p |Z[p][2G+c]| < 2^(E_G - 1)):
-//     Z[p][j] = 2^E_G sum_{i=1..s} 2^(-6 i) z_i[p][j],   z_i integers, |z_i| <= 32,
-// the slices are exact in BF16.  Products of slices are exact, and every partial sum of
+//     Z[p][j] = 2^(E_G + 1) sum_{i=1..s} 2^(-9 i) z_i[p][j],   z_i integers,
+// |z_1| <= 128 and |z_i| <= 256 otherwise, so the slices are exact in BF16.  Products of slices
+// are exact, and so is the FP32 sum of a slice group
 //     C_t = sum_{i+k=t} z_i^T z_k     (t = 2 .. s+1, triangular truncation)
-// over a chunk of at most 8192 pairs stays an integer of magnitude <= 2^24 for t <= 3,
-// hence exact in the FP32 accumulator; for t >= 4 it stays exact while |C_t| <= 2^24,
-// which holds unless the slices are adversarially correlated.  The FP64 recombination
-//     chi += -2^(E_G + E_G' - 6t) (integer combination of C_t)
-// happens once per chunk and group, in the epilogue, with FP64 atomic adds so that the
-// chunks (pair segments) of one chi block may run concurrently in one launch.  FP64 is kept for Delta, the
-// scaling, the recombination, the accumulation across chunks and the symmetrisation.
+// while it stays below 2^24.  The groups are therefore summed in K-segments (oz_segment): 512 pairs
+// for t = 2 (|z_1 z_1| <= 2^14, so a segment's sum is at most 2^23 and the sum of two of them that
+// makes an entry of chi is exact too), 256 for t = 3 (2 products, 2^24) and for t = 4 (2^25 if
+// every digit took its largest value with one sign; the rounding then lies 2^-36 below the leading
+// group), longer ones for t >= 5, whose rounding lies below 2^-27 2^-24 of the result.  The
+// epilogue adds the segments, times 2^(-9 (t - 2)), in two-float arithmetic in registers and adds
+//     chi += -2^(E_G + E_G' - 16) (hi + lo)
+// once per tile in FP64, with atomic adds so that the chunks (pair segments) of one chi block may
+// run concurrently in one launch (one chunk's sums are the same bits in every run).  FP64 is kept for Delta, the scaling, the accumulation across
+// chunks and the symmetrisation.
 #include "internal.h"
 #include "ptx.cuh"
 #include "fft_tf.cuh"
@@ -26,16 +30,24 @@
 
 namespace gw {
 
-constexpr int kOzBeta = 6;
-constexpr int kOzBM = 128, kOzBN = 256, kOzBK = 64, kOzStages = 4;
-constexpr int kOzThreads = 192;
-constexpr unsigned kOzABytes = kOzBM * kOzBK * 2, kOzBBytes = kOzBN * kOzBK * 2;
-constexpr int kOzNoColumn = -400; // exponent of an all-zero column
-// K-steps of one accumulation segment: 128 x 64 = 8192 real K entries, the length over which a
-// slice group's FP32 sum is exact (|z_i z_k| <= 2^10, two products per entry for t = 3).  Longer
-// K (the general product with more than 4096 complex inner entries) is summed segment by segment,
-// each segment's groups recombined in FP64 by the epilogue.
-constexpr int kOzKSeg = 128;
+// Slices for a requested accuracy of 6 nslices bits (the ABI's nslices, 3..8): the fewest 9-bit
+// slices whose dropped products (i + k > s + 1) lie no higher.  With six-bit digits the dropped
+// products come to 2^(-6 nslices - 3.6) sqrt(nslices - 1) of the operands' scales, with these to
+// 2^(-9 s - 1.6) sqrt(s - 1): 3, 3, 4, 5, 5, 6 slices for nslices = 3 .. 8.
+int oz_slices(int nslices) { return nslices <= 4 ? 3 : nslices == 5 ? 4 : nslices <= 7 ? 5 : 6; }
+
+constexpr int kOzBM = 128, kOzBK = 64; // rows of A (and of B) per CTA of a pair; K entries per ring stage
+constexpr int kOzThreads = 384;        // a warpgroup with the TMA and MMA warps, two of epilogue warps
+constexpr int kOzNoColumn = -400;      // exponent of an all-zero column
+
+// K runs in blocks of kOzKBlock K-steps (of 64 entries), every slice group over one block before
+// the next, so that a slice comes from DRAM once per block and from L2 for its other products.
+// (On 48^3 and 72^3 chunks, on N_G = 6000 self-energy products and on 2000 x 2000 products, 8, 16 and
+// 32 K-steps run within 3 % of one another.)
+constexpr int kOzKBlock = 16;
+// K-steps that slice group t sums in FP32 before the epilogue takes the sum (bounds at the top of
+// this file)
+__device__ __forceinline__ int oz_segment(int t) { return t == 2 ? 8 : t <= 4 ? 4 : kOzKBlock; }
 
 // ------------------------------------------------------------------ split, step 1: column exponents
 // E[g] = max_p ilogb(max(|Re A|, |Im A|)) + 2 over the chunk, A = s_p M[p][g].
@@ -106,7 +118,7 @@ __device__ __forceinline__ void oz_store_row_digits(const long long nb[16], int 
             for (int u = 0; u < 2; ++u) {
                 const long long v = nb[t + u];
                 d[u] = i == 0 ? oz_small_bf16((int)(v >> (kOzBeta * (s - 1))))
-                              : oz_small_bf16((int)((v >> (kOzBeta * (s - 1 - i))) & 63) - 32);
+                              : oz_small_bf16((int)((v >> (kOzBeta * (s - 1 - i))) & 511) - 256);
             }
             w[t >> 1] = (uint32_t)d[0] | ((uint32_t)d[1] << 16);
         }
@@ -128,10 +140,10 @@ __global__ void __launch_bounds__(256, 5) oz_slice_kernel(const double2 *__restr
     const OzTileThread tt = oz_tile_thread();
     const int g = blockIdx.x * 32 + tt.gl;
     if (g >= ng) return;
-    // N = round(a 2^(6 s - E)) and its balanced base-64 digits, in integer arithmetic
-    const int sh = kOzBeta * s - E[g];
+    // N = round(a 2^(9 s - 1 - E)) and its balanced base-512 digits, in integer arithmetic
+    const int sh = oz_frac_bits(s) - E[g];
     const double *Md = (const double *)M;
-    const long long bias = oz_digit_bias(s);
+    const long long bias = oz_digit_bias<kOzBeta>(s);
     long long nb[16];
 #pragma unroll
     for (int t = 0; t < 16; ++t) {
@@ -195,7 +207,7 @@ __global__ void __launch_bounds__(256) oz_slice_multi_kernel(const double2 *__re
     const OzTileThread tt = oz_tile_thread();
     const int g = blockIdx.x * 32 + tt.gl;
     if (g >= ng) return;
-    const long long bias = oz_digit_bias(s);
+    const long long bias = oz_digit_bias<kOzBeta>(s);
     // the thread's 16 entries of the block's tile of M, read once for every frequency
     const double *Md = (const double *)M;
     double m[16];
@@ -206,7 +218,7 @@ __global__ void __launch_bounds__(256) oz_slice_multi_kernel(const double2 *__re
     }
     const int64_t j = 2 * (int64_t)g + tt.c;
     for (int w = 0; w < nw; ++w) {
-        const int sh = kOzBeta * s - E[(int64_t)w * ng + g];
+        const int sh = oz_frac_bits(s) - E[(int64_t)w * ng + g];
         long long nb[16];
 #pragma unroll
         for (int t = 0; t < 16; ++t) {
@@ -219,18 +231,17 @@ __global__ void __launch_bounds__(256) oz_slice_multi_kernel(const double2 *__re
 }
 
 // ------------------------------------------------------------------ general product: slices
-// Y = A B with A split by rows and B by columns: x = 2^E sum_{i=1..s} 2^(-6 i) z_i, the same
-// balanced base-64 digits as oz_slice_kernel, with E = max(ilogb) + 2 over a row of A or a
+// Y = A B with A split by rows and B by columns: x = 2^(E+1) sum_{i=1..s} 2^(-9 i) z_i, the same
+// balanced base-512 digits as oz_slice_kernel, in the same layout (real and imaginary parts in
+// rows of their own, K the complex inner index), so that with C the real product of the 2 rows
+// slice rows by the 2 nout slice columns
+//     Re Y[r][c] = C[2r][2c] - C[2r+1][2c+1],   Im Y[r][c] = C[2r][2c+1] + C[2r+1][2c],
+// and E = max(ilogb) + 2 over a row of A or a
 // column of B (both parts of a complex entry).
 // exponent of a complex entry: ilogb(max(|Re|, |Im|)) + 2
 __device__ __forceinline__ int oz_expo(double2 x)
 {
     return oz_expo_bits(oz_absmax_bits(x.x, x.y), kOzNoColumn);
-}
-
-__device__ __forceinline__ void oz_digits(double x, int E, int s, uint16_t *out, int64_t plane)
-{
-    oz_store_digits(oz_round_scaled(x, kOzBeta * s - E), s, oz_digit_bias(s), out, plane);
 }
 
 __device__ __forceinline__ int oz_block_max(int e, int *red)
@@ -248,64 +259,45 @@ __device__ __forceinline__ int oz_block_max(int e, int *red)
     return red[0];
 }
 
-// One block per row p of A [rows][ka] (complex): E[p], then Z[i][p][k], k = 2 g + {Re, Im},
-// zero for k >= 2 ka.  CONJ: the rows of conj(A).
+// digits of two consecutive entries x0, x1 of a row: 32-bit stores at out + i plane32
+__device__ __forceinline__ void oz_store_pair(double x0, double x1, int sh, int s, long long bias, uint32_t *out,
+                                              int64_t plane32)
+{
+    const long long n0 = oz_round_scaled(x0, sh) + bias, n1 = oz_round_scaled(x1, sh) + bias;
+    for (int k = 0; k < s - 1; ++k)
+        out[(int64_t)(s - 1 - k) * plane32] =
+            (uint32_t)oz_small_bf16((int)((n0 >> (kOzBeta * k)) & 511) - 256) |
+            (uint32_t)oz_small_bf16((int)((n1 >> (kOzBeta * k)) & 511) - 256) << 16;
+    out[0] = (uint32_t)oz_small_bf16((int)(n0 >> (kOzBeta * (s - 1)))) |
+             (uint32_t)oz_small_bf16((int)(n1 >> (kOzBeta * (s - 1)))) << 16;
+}
+
+// One block per complex row p of A: E[p], then the slice rows Z[i][2 p + c][g] (c = 0 the real,
+// c = 1 the imaginary parts), zero for g >= ka.  A[p][g] is read at A[p sr + g sk] (sr = ka, sk = 1
+// for row-major A [rows][ka]; sr = 1, sk = nout for the columns of a row-major B [ka][nout]).
+// CONJ: of conj(A).
 template <bool CONJ>
-__global__ void __launch_bounds__(256) oz_split_rows_kernel(const double2 *__restrict__ A, int64_t rows, int ka,
-                                                            int s, int64_t kpad, uint16_t *__restrict__ Z,
-                                                            int *__restrict__ E)
+__global__ void __launch_bounds__(256) oz_split_kernel(const double2 *__restrict__ A, int64_t rows, int ka,
+                                                       int64_t sr, int64_t sk, int s, int64_t kpad,
+                                                       uint16_t *__restrict__ Z, int *__restrict__ E)
 {
     __shared__ int red[8];
     const int64_t p = blockIdx.x;
-    const double2 *a = A + p * ka;
+    const double2 *a = A + p * sr;
     int e = kOzNoColumn;
-    for (int g = threadIdx.x; g < ka; g += blockDim.x) {
-        const double2 x = a[g];
-        e = max(e, oz_expo(x));
-    }
+    for (int g = threadIdx.x; g < ka; g += blockDim.x) e = max(e, oz_expo(a[g * sk]));
     e = oz_block_max(e, red);
     if (threadIdx.x == 0) E[p] = e;
-    uint16_t *zr = Z + p * kpad;
-    for (int64_t k = threadIdx.x; k < kpad; k += blockDim.x) {
-        const int g = (int)(k >> 1);
-        const double x = g < ka ? ((k & 1) ? (CONJ ? -a[g].y : a[g].y) : a[g].x) : 0.0;
-        oz_digits(x, e, s, zr + k, rows * kpad);
-    }
-}
-
-// One block per column b of B [ka][nout] (complex): E[b], then rows 2b (Re of the product)
-// and 2b + 1 (Im) of the real K-major operand B^T: row 2b = (Re B, -Im B), row 2b + 1 =
-// (Im B, Re B) interleaved by g, so that [Re A, Im A] interleaved times them gives Re and
-// Im of (A B)[p][b].
-// B[g][b] is read at B[g sk + b sj] (sk = nout, sj = 1 for a row-major B; sk = 1, sj = ka for
-// the transpose of a row-major [nout][ka] matrix).  CONJ: the columns of conj(B).
-template <bool CONJ>
-__global__ void __launch_bounds__(256) oz_split_cols_kernel(const double2 *__restrict__ B, int ka, int nout,
-                                                            int64_t sk, int64_t sj, int s, int64_t kpad,
-                                                            uint16_t *__restrict__ Z, int *__restrict__ E)
-{
-    __shared__ int red[8];
-    const int b = blockIdx.x;
-    int e = kOzNoColumn;
-    for (int g = threadIdx.x; g < ka; g += blockDim.x) {
-        const double2 x = B[(int64_t)g * sk + (int64_t)b * sj];
-        e = max(e, oz_expo(x));
-    }
-    e = oz_block_max(e, red);
-    if (threadIdx.x == 0) E[b] = e;
-    const int64_t plane = (int64_t)2 * nout * kpad;
-    uint16_t *z0 = Z + (int64_t)(2 * b) * kpad, *z1 = z0 + kpad;
-    for (int64_t k = threadIdx.x; k < kpad; k += blockDim.x) {
-        const int g = (int)(k >> 1);
-        double x0 = 0.0, x1 = 0.0;
-        if (g < ka) {
-            double2 x = B[(int64_t)g * sk + (int64_t)b * sj];
-            if (CONJ) x.y = -x.y;
-            x0 = (k & 1) ? -x.y : x.x;
-            x1 = (k & 1) ? x.x : x.y;
-        }
-        oz_digits(x0, e, s, z0 + k, plane);
-        oz_digits(x1, e, s, z1 + k, plane);
+    const int sh = oz_frac_bits(s) - e;
+    const long long bias = oz_digit_bias<kOzBeta>(s);
+    const int64_t plane32 = rows * kpad; // 2 rows kpad entries of 16 bits
+    uint32_t *z0 = (uint32_t *)(Z + 2 * p * kpad), *z1 = (uint32_t *)(Z + (2 * p + 1) * kpad);
+    for (int64_t k = threadIdx.x; 2 * k < kpad; k += blockDim.x) {
+        const int64_t g = 2 * k;
+        const double2 zero = make_double2(0.0, 0.0);
+        const double2 x = g < ka ? a[g * sk] : zero, y = g + 1 < ka ? a[(g + 1) * sk] : zero;
+        oz_store_pair(x.x, y.x, sh, s, bias, z0 + k, plane32);
+        oz_store_pair(CONJ ? -x.y : x.y, CONJ ? -y.y : y.y, sh, s, bias, z1 + k, plane32);
     }
 }
 
@@ -320,12 +312,12 @@ __global__ void __launch_bounds__(256) oz_split_cols_kernel(const double2 *__res
 //    x = d - sgn wt (relative error ~2^-22 however close the pole), padded by 2^-10 so that the
 //    exponent is never below the one of the exact maximum;
 //  * pass 2, P = A conj(x) / |x|^2 in two-float arithmetic (the reciprocal by one Newton step,
-//    relative error near 2^-46, below the 2^-42 the seven slices keep), then the balanced
-//    base-64 digits of N = round(P 2^sh) in the layout of oz_split_rows_kernel, (Re P, Im P)
-//    interleaved by g.  The digits are taken in FP32, where every step is exact: v = hi 2^sh
-//    splits into t 2^24 + r (|r| <= 2^23), the low part L = rint(r) + rint(lo 2^sh) (|L| < 2^24)
-//    gives four digits by q = rint(L / 64), d = L - 64 q, and t + q the rest.  N differs from
-//    round((hi + lo) 2^sh) by one unit of the last digit at most; |d| <= 32 as before.
+//    relative error near 2^-46, below the 2^-43 five slices keep), then the balanced base-512
+//    digits of N = round(P 2^sh) in the layout of oz_split_kernel.  N is formed without 64-bit steps: v = hi 2^sh splits in FP32 into t 2^S + r, both
+//    exact (|r| <= 2^(S-1), S two digits, three for six slices), and the low part
+//    L = rint(r) + rint(lo 2^sh) (below 2^20, 2^29 for six slices) gives the S / 9 lowest digits
+//    and a carry into t, which holds the others, in 32-bit integers.  N differs from
+//    round((hi + lo) 2^sh) by one unit of the last digit at most.
 __device__ __forceinline__ tf tf_recip(tf d)
 {
     const float r0 = __frcp_rn(d.hi);
@@ -364,35 +356,40 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
     return (__float_as_uint(lo) >> 16) | (__float_as_uint(hi) & 0xffff0000u);
 }
 
-// Digits of round(v 2^sh) for v = Re P and Im P side by side (sc = (s1, s2), s1 s2 = 2^sh),
-// stored as they come: slice i of row zr (u32 pairs, slice planes plane32 apart), element g.
-__device__ __forceinline__ float tf_low(tf v, float s1, float s2, float &t)
+// N = round(v 2^sh) as L + T 2^(9 low), 2^sh = s1 s2
+__device__ __forceinline__ void tf_fixed(tf v, float s1, float s2, int low, int &L, int &T)
 {
     const float vh = __fmul_rn(__fmul_rn(v.hi, s1), s2);
-    t = rintf(__fmul_rn(vh, 0x1p-24f));
-    return __fadd_rn(rintf(__fmaf_rn(-0x1p24f, t, vh)), rintf(__fmul_rn(__fmul_rn(v.lo, s1), s2)));
+    const float t = rintf(__fmul_rn(vh, low == 2 ? 0x1p-18f : 0x1p-27f));
+    const float r = __fmaf_rn(low == 2 ? -0x1p18f : -0x1p27f, t, vh);
+    L = __float2int_rn(r) + __float2int_rn(__fmul_rn(__fmul_rn(v.lo, s1), s2));
+    T = __float2int_rn(t);
 }
 
-__device__ __forceinline__ void tf_digits_store(tcx p, float s1, float s2, int s, uint32_t *zr, int64_t plane32,
-                                                int64_t g)
+__device__ __forceinline__ uint32_t oz_digit_pair(int a, int b)
 {
-    float tr, ti;
-    float Lr = tf_low(p.re, s1, s2, tr), Li = tf_low(p.im, s1, s2, ti);
+    return bf16_pair(__int_as_float(0x4B400000 + a) - 12582912.0f, __int_as_float(0x4B400000 + b) - 12582912.0f);
+}
+
+// Digits of round(v 2^sh) of two consecutive entries of a row (2^sh = s1 s2), stored as they come:
+// slice i at zr + i plane32.
+__device__ __forceinline__ void tf_digits_store(tf v0, tf v1, float s1, float s2, int s, uint32_t *zr, int64_t plane32)
+{
+    const int low = s <= 5 ? 2 : 3;
+    int L0, T0, L1, T1;
+    tf_fixed(v0, s1, s2, low, L0, T0);
+    tf_fixed(v1, s1, s2, low, L1, T1);
     for (int i = s - 1; i >= 1; --i) {
-        if (i == s - 5) { // four digits taken from the low parts: carry into the high parts
-            Lr = __fadd_rn(Lr, tr);
-            Li = __fadd_rn(Li, ti);
+        const int d0 = ((L0 + 256) & 511) - 256, d1 = ((L1 + 256) & 511) - 256;
+        zr[i * plane32] = oz_digit_pair(d0, d1);
+        L0 = (L0 - d0) >> kOzBeta;
+        L1 = (L1 - d1) >> kOzBeta;
+        if (i == s - low) { // the low parts are used up: carry into the high ones
+            L0 += T0;
+            L1 += T1;
         }
-        const float qr = rintf(__fmul_rn(Lr, 0.015625f)), qi = rintf(__fmul_rn(Li, 0.015625f));
-        zr[i * plane32 + g] = bf16_pair(__fmaf_rn(-64.0f, qr, Lr), __fmaf_rn(-64.0f, qi, Li));
-        Lr = qr;
-        Li = qi;
     }
-    if (s <= 5) { // at most four digits taken: the high parts join the top digit (zero for s <= 4)
-        Lr = __fadd_rn(Lr, tr);
-        Li = __fadd_rn(Li, ti);
-    }
-    zr[g] = bf16_pair(Lr, Li);
+    zr[0] = oz_digit_pair(L0, L1);
 }
 
 template <int NE>
@@ -434,306 +431,315 @@ __global__ void __launch_bounds__(256, NE > 4 ? 3 : 4) gpp_prep_split_kernel(con
         const int e = tf_expo(v * (1.0f + 0x1p-10f));
         E[(int64_t)threadIdx.x * ng + c] = e;
         // 2^sh in two factors, each inside the FP32 exponent range
-        const int sh = max(-250, min(250, kOzBeta * s - e));
+        const int sh = max(-250, min(250, oz_frac_bits(s) - e));
         ssm[threadIdx.x] = make_float2(__int_as_float((127 + sh / 2) << 23), __int_as_float((127 + sh - sh / 2) << 23));
     }
     __syncthreads();
-    const int64_t plane = (int64_t)ng * kpad;
-    for (int64_t g = threadIdx.x; g < kpad / 2; g += blockDim.x) {
-        float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f), w4 = make_float4(1.f, 0.f, 0.f, 0.f);
-        if (g < ng) {
-            a4 = a[g];
-            w4 = w[g];
+    const int64_t plane32 = (int64_t)ng * kpad;
+    for (int64_t k = threadIdx.x; 2 * k < kpad; k += blockDim.x) {
+        // entries 2 k and 2 k + 1 of the row; padding entries have a = 0, so P = 0 there
+        float4 a4[2], w4[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const bool in = 2 * k + u < ng;
+            a4[u] = in ? a[2 * k + u] : make_float4(0.f, 0.f, 0.f, 0.f);
+            w4[u] = in ? w[2 * k + u] : make_float4(1.f, 0.f, 0.f, 0.f);
         }
         for (int j = 0; j < cnt; ++j) {
-            // padding entries (g >= ng) have a = 0, so p = 0 there
-            const tcx p = gpp_pole_tf(a4, w4, tf{dsm[j].x, dsm[j].y}, sgn);
+            const tf d{dsm[j].x, dsm[j].y};
+            const tcx p0 = gpp_pole_tf(a4[0], w4[0], d, sgn), p1 = gpp_pole_tf(a4[1], w4[1], d, sgn);
             const float2 sc = ssm[j];
-            tf_digits_store(p, sc.x, sc.y, s, (uint32_t *)(Z + j * zstride + (int64_t)c * kpad), plane >> 1, g);
+            uint32_t *z = (uint32_t *)(Z + j * zstride + (int64_t)2 * c * kpad) + k;
+            tf_digits_store(p0.re, p1.re, sc.x, sc.y, s, z, plane32);
+            tf_digits_store(p0.im, p1.im, sc.x, sc.y, s, z + kpad / 2, plane32);
         }
     }
 }
 
 // ------------------------------------------------------------------ tcgen05 GEMM
-// Persistent and batched: a launch takes a table of jobs (one job = one chunk's slices
-// for one chi block, each with its own N_G, tensor maps and exponents) and the list of
-// their upper tiles; block b takes items b, b + gridDim.x, ... in the same order in every
-// role, so the TMA producer warp, the MMA warp and the epilogue warps need no exchange
-// beyond the mbarriers.  The tile width BN (128, 240 or 256 real columns) is chosen by the
-// autotuner or by the wave count (oz_pick_bn); two BN-column FP32 accumulators in TMEM alternate
-// between slice groups so the epilogue of group t overlaps the MMAs of group t+1.  At BN = 240 the
-// accumulators sit 256 columns apart and the epilogue's last 32-column chunk is cut at BN.
-template <int BN, int ST = kOzStages>
+// Persistent and batched: a launch takes a table of jobs (one job = one chunk's slices for one chi
+// block, or one general product, each with its own sizes, tensor maps and exponents) and a list of
+// items (job, tile, K range).  A pair of CTAs (a cluster of two, cta_group::2) takes items c,
+// c + clusters, ... in the same order in every role, so the TMA warps, the MMA warp and the
+// epilogue warps need no exchange beyond the mbarriers.
+//
+// What bounds it: the tensor pipe, fed from L2.  A pair works on 256 x 256 real entries; each CTA
+// loads 128 rows of A and 128 of B per K-step, 32 KB, so the ring holds six stages (one CTA on a
+// 128 x 256 tile loads 48 KB per K-step for half the work and holds four).  A 256 x 128 tile is no
+// alternative: an MMA of a pair takes as long with 128 columns as with 256 (33.5 against 19.0 ms
+// for the 16 chunks of a 48^3 q-point).  The sums of a tile stay in registers as two-float pairs
+// over all its slice groups and K-segments (64 per epilogue thread: Re or Im parts, two of the real
+// products each), so a segment costs TMEM loads and FP32 adds, and FP64 work and atomics come once
+// per item.  Two accumulators in TMEM alternate between segments, so a segment's epilogue overlaps
+// the next one's MMAs; without any epilogue work the 16 launches of
+// a 48^3 q-point take 16.5 ms instead of 19.0.
+//
+// Measured (split contraction of one 8192-pair chunk, N_G = 2000, 7-slice accuracy): 1.21 ms, 15
+// products of nine-bit slices, 1.63 PFLOP/s on them; one CTA per tile with 28 products of six-bit
+// slices and an FP64 atomic epilogue per slice group took 2.44 ms (1.50 PFLOP/s).  N_G = 6000: 9.6
+// against 24.0 ms.  General product of the self-energy (N_G = 6000, 384 bands, 24 products): 20.8
+// against 54.3 ms.
 struct OzCfg {
-    static constexpr int Stages = ST;                        // TMA ring depth
-    static constexpr int BM = kOzBM;
-    static constexpr int BNC = BN / 2;                       // complex columns per tile
-    static constexpr unsigned ABytes = kOzBM * kOzBK * 2, BBytes = BN * kOzBK * 2;
-    static constexpr uint32_t TmemBuf = BN > 128 ? 256 : 128; // TMEM columns per accumulator buffer
-    static constexpr uint32_t TmemCols = 2 * TmemBuf;        // 256 or 512 (a power of two)
-    // idesc: D = F32, A = B = BF16, both K-major, N = BN, M = 128
-    static constexpr uint32_t Idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                                      ((uint32_t)(kOzBM >> 4) << 24);
-    static constexpr size_t Smem = 1024 + ST * (size_t)(ABytes + BBytes) + (2 * ST + 5) * 8 + 16;
+    static constexpr unsigned Bytes = kOzBM * kOzBK * 2;     // of A, and of B, per stage and CTA
+    static constexpr int Stages = 6;                         // TMA ring depth
+    static constexpr int Cols = 256, Bufs = 2;               // accumulators in TMEM
+    // idesc: D = F32, A = B = BF16, both K-major, N = 256, M = 256 over the pair
+    static constexpr uint32_t Idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(Cols >> 3) << 17) |
+                                      ((uint32_t)(2 * kOzBM >> 4) << 24);
+    static constexpr size_t Smem = 1024 + Stages * 2 * (size_t)Bytes + (2 * Stages + 2 * Bufs + 1) * 8 + 16;
 };
 
-// tile -> (I, J): J-major, rows I = 0 .. min((BNC (J+1) - 1)/64 + 1, nI) - 1
-__device__ __forceinline__ void oz_tile_ij(int tile, int nI, int bnc, int &I, int &J)
-{
-    int rem = tile;
-    J = 0;
-    for (;;) {
-        const int c = min((bnc * (J + 1) - 1) / 64 + 1, nI);
-        if (rem < c) break;
-        rem -= c;
-        ++J;
+// The segments of an item of nk K-steps with s slices, in the order every role walks them: K block
+// by K block, from the least significant group up, the group's segments of the block.
+struct OzSegments {
+    int nk, s, kc, t, k0, len;
+    __device__ __forceinline__ OzSegments(int nk_, int s_) : nk(nk_), s(s_), kc(0), t(s_ + 1), k0(0) { cut(); }
+    __device__ __forceinline__ void cut() { len = min(min(nk, kc + kOzKBlock) - k0, oz_segment(t)); }
+    __device__ __forceinline__ bool more() const { return kc < nk; }
+    __device__ __forceinline__ void next()
+    {
+        k0 += len;
+        if (k0 >= min(nk, kc + kOzKBlock)) {
+            if (--t < 2) {
+                t = s + 1;
+                kc += kOzKBlock;
+            }
+            k0 = kc;
+        }
+        cut();
     }
-    I = rem;
+};
+
+// A pair's waits end within a millisecond unless something failed; the bound keeps the time until
+// every warp of both CTAs has given up short.
+__device__ __forceinline__ bool pair_wait(uint64_t *b, unsigned parity) { return bar_wait(b, parity, 1LL << 22); }
+
+// hi + lo += x with the rounding error of hi + x kept in lo
+__device__ __forceinline__ void oz_add(float &hi, float &lo, float x)
+{
+    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+    hi = s;
 }
 
-// tile -> (I, J) for the general product: I-major (blocks that run together share A rows)
-template <bool GEN, int BN>
-__device__ __forceinline__ void oz_tile(const OzJob &jb, int tile, int &I, int &J)
+// x 2^ex as a double, from the bits (no conversion on the FP64 pipe); 0 below 2^-1022
+__device__ __forceinline__ double oz_scaled_double(float x, int ex)
 {
-    if constexpr (GEN) {
-        const int nJ = (jb.rows_b + BN - 1) / BN;
-        I = tile / nJ;
-        J = tile - I * nJ;
-    } else {
-        oz_tile_ij(tile, (2 * jb.ng + kOzBM - 1) / kOzBM, BN / 2, I, J);
-    }
+    const uint32_t u = __float_as_uint(x);
+    const int e = (int)((u >> 23) & 0xff) + 896 + ex;
+    if ((u & 0x7f800000u) == 0 || e <= 0) return 0.0;
+    return __hiloint2double((int)((u & 0x80000000u) | ((uint32_t)min(e, 2046) << 20) | ((u >> 3) & 0xfffffu)),
+                            (int)(u << 29));
 }
 
-__device__ __forceinline__ int oz_find_job(const OzJob *jobs, int njobs, int item)
+// GEN = false: the Hermitian contraction above (upper tiles, chi epilogue).  GEN = true: the
+// general product out += A B (all tiles, each owned by one pair of CTAs, plain FP64 adds).
+template <bool GEN>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
+    oz_gemm_kernel(const OzJob *__restrict__ jobs, const OzItem *__restrict__ items, int nitems, OzScratch scr,
+                   int *status)
 {
-    int lo = 0, hi = njobs - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (jobs[mid].item_start <= item) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
-// GEN = false: the Hermitian contraction above (upper tiles, chi epilogue).  GEN = true:
-// the general product out += A B (all tiles, each owned by one block, plain FP64 adds).
-// ST: depth of the TMA ring (2 leaves shared memory for other kernels' blocks on the SM).
-template <int BN, bool GEN, int ST = kOzStages>
-__global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(const OzJob *__restrict__ jobs, int njobs, int nitems,
-                                                               int *status)
-{
-    using C = OzCfg<BN, ST>;
+    using C = OzCfg;
+    constexpr int ST = C::Stages, NB = C::Bufs;
     extern __shared__ __align__(1024) unsigned char smraw[];
     unsigned char *sm = (unsigned char *)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
-    unsigned char *sA = sm;                                  // [stages][ABytes]
-    unsigned char *sB = sA + ST * C::ABytes;          // [stages][BBytes]
-    uint64_t *full = (uint64_t *)(sB + ST * C::BBytes);
-    uint64_t *empty = full + ST;
-    uint64_t *tfull = empty + ST;
-    uint64_t *tempty = tfull + 2;
-    uint64_t *fin = tempty + 2;
+    unsigned char *sA = sm;                 // [stages][Bytes]
+    unsigned char *sB = sA + ST * C::Bytes; // [stages][Bytes]
+    uint64_t *full = (uint64_t *)(sB + ST * C::Bytes); // used in CTA 0: both CTAs' loads count there
+    uint64_t *empty = full + ST;            // each CTA its own, by the pair's commit
+    uint64_t *tfull = empty + ST;           // likewise
+    uint64_t *tempty = tfull + NB;          // used in CTA 0: 16 epilogue warps arrive
+    uint64_t *fin = tempty + NB;
     uint32_t *tslot = (uint32_t *)(fin + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank();
+    const int cl0 = blockIdx.x >> 1, ncl = gridDim.x >> 1;
     if (threadIdx.x == 0) {
         for (int i = 0; i < ST; ++i) {
             bar_init(&full[i], 1);
             bar_init(&empty[i], 1);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < NB; ++i) {
             bar_init(&tfull[i], 1);
-            bar_init(&tempty[i], 128);
+            bar_init(&tempty[i], 16);
         }
         bar_init(fin, 1);
         bar_fence_init();
     }
-    if (warp == 1) tmem_alloc(tslot, C::TmemCols);
+    if (warp == 1) tmem_alloc_pair(tslot, NB * C::Cols);
     tc_fence_before();
     __syncthreads();
+    cluster_sync();
     tc_fence_after();
     const uint32_t tbase = *tslot;
     bool ok = true;
 
-    if (warp == 0) {
-        if (lane == 0) {
+    // registers: 384 x 168 at launch; the epilogue warps hold a tile's sums (128 of them) and take
+    // 224 a thread, the warpgroup of the TMA and MMA warps keeps 56 (2 x 224 + 56 = 3 x 168)
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        if (warp == 0 && lane == 0) {
             uint32_t it = 0;
-            for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-                const OzJob &jb = jobs[oz_find_job(jobs, njobs, item)];
-                int I, J;
-                oz_tile<GEN, BN>(jb, item - jb.item_start, I, J);
-                for (int k0 = 0; k0 < jb.nk && ok; k0 += kOzKSeg)
-                for (int t = 2; t <= jb.s + 1 && ok; ++t)
-                    for (int i = 1; i < t && ok; ++i)
-                        for (int kb = k0; kb < min(jb.nk, k0 + kOzKSeg); ++kb, ++it) {
-                            const int st = it % ST;
-                            const uint32_t n = it / ST;
-                            if (!bar_wait(&empty[st], (n & 1) ^ 1)) { ok = false; break; }
-                            bar_expect(&full[st], C::ABytes + C::BBytes);
-                            tma3(sA + st * C::ABytes, &jb.tmA, &full[st], (jb.kb0 + kb) * kOzBK, I * kOzBM, i - 1);
-                            tma3(sB + st * C::BBytes, &jb.tmB, &full[st], (jb.kb0 + kb) * kOzBK, J * BN, t - i - 1);
+            const uint32_t full0 = cluster_map(full, 0);
+            for (int item = cl0; item < nitems && ok; item += ncl) {
+                const OzItem w = items[item];
+                const OzJob &jb = jobs[w.job];
+                const int ra = (2 * w.I + (int)rank) * kOzBM, rb = (2 * w.J + (int)rank) * kOzBM;
+                for (OzSegments g(w.nk, jb.s); g.more() && ok; g.next())
+                    for (int i = 1; i < g.t && ok; ++i)
+                        for (int kb = 0; kb < g.len; ++kb, ++it) {
+                            const uint32_t st = it % ST;
+                            if (!pair_wait(&empty[st], ((it / ST) & 1) ^ 1)) { ok = false; break; }
+                            if (rank == 0) bar_expect(&full[st], 4 * C::Bytes);
+                            const int k = (w.kb0 + g.k0 + kb) * kOzBK;
+                            tma3_pair(sA + st * C::Bytes, &jb.tmA, full0 + 8 * st, k, ra, i - 1);
+                            tma3_pair(sB + st * C::Bytes, &jb.tmB, full0 + 8 * st, k, rb, g.t - i - 1);
                         }
             }
+            // copies in flight land before the pair tears down (they count at CTA 0's barriers)
+            if (!ok && rank == 0)
+                for (uint32_t j = it > ST ? it - ST : 0; j < it; ++j) pair_wait(&full[j % ST], (j / ST) & 1);
             if (!ok) atomicOr(status, kStatusTimeout);
         }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            uint32_t it = 0, grp = 0;
-            for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-                const OzJob &jb = jobs[oz_find_job(jobs, njobs, item)];
-                for (int k0 = 0; k0 < jb.nk && ok; k0 += kOzKSeg)
-                for (int t = 2; t <= jb.s + 1 && ok; ++t, ++grp) {
-                    const uint32_t b = grp & 1, u = grp >> 1;
-                    if (!bar_wait(&tempty[b], (u & 1) ^ 1)) { ok = false; break; }
+        if (warp == 1 && lane == 0 && rank == 0) {
+            uint32_t it = 0, seg = 0;
+            for (int item = cl0; item < nitems && ok; item += ncl) {
+                const OzItem w = items[item];
+                for (OzSegments g(w.nk, jobs[w.job].s); g.more() && ok; g.next(), ++seg) {
+                    const uint32_t b = seg % NB;
+                    if (!pair_wait(&tempty[b], ((seg / NB) & 1) ^ 1)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t d = tbase + b * C::TmemBuf;
-                    bool first = true;
-                    for (int i = 1; i < t && ok; ++i)
-                        for (int kb = k0; kb < min(jb.nk, k0 + kOzKSeg); ++kb, ++it) {
-                            const int st = it % ST;
-                            if (!bar_wait(&full[st], (it / ST) & 1)) { ok = false; break; }
-                            tc_fence_after();
-                            const uint32_t a0 = su32(sA + st * C::ABytes), b0 = su32(sB + st * C::BBytes);
+                    const int n = (g.t - 1) * g.len; // ring stages of the segment
+                    for (int j = 0; j < n; ++j, ++it) {
+                        const uint32_t st = it % ST;
+                        if (!pair_wait(&full[st], (it / ST) & 1)) { ok = false; break; }
+                        tc_fence_after();
+                        const uint32_t a0 = su32(sA + st * C::Bytes), b0 = su32(sB + st * C::Bytes);
 #pragma unroll
-                            for (int kk = 0; kk < kOzBK / 16; ++kk)
-                                umma_f16(d, sdesc_sw128(a0 + kk * 32), sdesc_sw128(b0 + kk * 32), C::Idesc,
-                                         (first && kk == 0) ? 0u : 1u);
-                            first = false;
-                            umma_commit(&empty[st]);
-                        }
-                    umma_commit(&tfull[b]);
+                        for (int kk = 0; kk < kOzBK / 16; ++kk)
+                            umma_f16_pair(tbase + b * C::Cols, sdesc_sw128(a0 + kk * 32), sdesc_sw128(b0 + kk * 32),
+                                          C::Idesc, (j == 0 && kk == 0) ? 0u : 1u);
+                        umma_commit_pair(&empty[st]);
+                    }
+                    umma_commit_pair(&tfull[b]);
                 }
             }
-            // every issued MMA has completed before the block tears down
-            umma_commit(fin);
-            bar_wait(fin, 0);
+            // every issued MMA has completed before the pair tears down
+            umma_commit_pair(fin);
+            pair_wait(fin, 0);
             if (!ok) atomicOr(status, kStatusTimeout);
+        } else if (warp == 1 && lane == 0) {
+            pair_wait(fin, 0); // the pair's last commit has reached this CTA too
         }
     } else {
-        // epilogue: warps 2..5 -> TMEM lane quadrant (warp % 4), one tile row per thread
-        const int q = warp & 3;
-        const int r = q * 32 + lane;              // tile row
-        uint32_t grp = 0;
-        if constexpr (GEN) {
-            for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-                const OzJob &jb = jobs[oz_find_job(jobs, njobs, item)];
-                int I, J;
-                oz_tile<GEN, BN>(jb, item - jb.item_start, I, J);
-                const int pr = I * kOzBM + r;     // output row
-                const int Ea = pr < jb.rows_a ? __ldg(jb.E + pr) : kOzNoColumn;
-                double *orow = jb.out + (int64_t)pr * jb.ldo;
-                for (int k0 = 0; k0 < jb.nk && ok; k0 += kOzKSeg)
-                for (int t = 2; t <= jb.s + 1; ++t, ++grp) {
-                    const uint32_t b = grp & 1, u = grp >> 1;
-                    const bool got = bar_wait(&tfull[b], u & 1);
-                    if (!__all_sync(0xffffffffu, got)) { ok = false; break; } // warp-uniform exit
-                    tc_fence_after();
-                    const uint32_t ta = tbase + ((uint32_t)(q * 32) << 16) + b * C::TmemBuf;
-#pragma unroll 1
-                    for (int c0 = 0; c0 < BN; c0 += 32) {
-                        uint32_t v[32];
-                        GW_TMEM_LD32(ta + c0, v);
-                        tmem_wait_ld();
-                        if (pr < jb.rows_a) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+        // epilogue: warps 4..11 -> TMEM lane quadrant (warp % 4) and half of the columns, one tile
+        // row per thread
+        constexpr int COLS = C::Cols / 2;             // columns per thread
+        constexpr int NO = COLS / 2;                  // sums per thread: Re or Im parts of a complex row
+        const int q = warp & 3, half = (warp - 4) >> 2;
+        const int r = q * 32 + lane;                  // row of this CTA's half of the tile
+        const int odd = r & 1;                        // 0 Re part, 1 Im part
+        // chi: Re = C[2G][2G'] + C[2G+1][2G'+1], Im = C[2G][2G'+1] - C[2G+1][2G']; general product: Re =
+        // C[2r][2c] - C[2r+1][2c+1], Im = C[2r][2c+1] + C[2r+1][2c].  The other row's term comes
+        // from the neighbouring lane.
+        const uint32_t flip = !GEN && odd ? 0x80000000u : 0u, rflip = GEN && !odd ? 0x80000000u : 0u;
+        const uint32_t tempty0 = cluster_map(tempty, 0);
+        float hi[NO], lo[NO];
+        uint32_t seg = 0;
+        for (int item = cl0; item < nitems && ok; item += ncl) {
+            const OzItem w = items[item];
+            const OzJob &jb = jobs[w.job];
 #pragma unroll
-                            for (int cc = 0; cc < 32; ++cc) {
-                                const int j = J * BN + c0 + cc; // output real column
-                                const int val = (int)__uint_as_float(v[cc]);
-                                if ((BN % 32 == 0 || c0 + cc < BN) && j < jb.rows_b && val != 0) {
-                                    const int ex = Ea + __ldg(jb.E2 + (j >> 1)) - kOzBeta * t;
-                                    // the tile belongs to this block alone: a plain add
-                                    orow[j] += (double)val * __longlong_as_double((long long)(1023 + max(-1022, ex)) << 52);
-                                }
-                            }
-                        }
+            for (int j = 0; j < NO; ++j) hi[j] = lo[j] = 0.0f;
+            for (OzSegments g(w.nk, jb.s); g.more(); g.next(), ++seg) {
+                const uint32_t b = seg % NB;
+                const bool got = pair_wait(&tfull[b], (seg / NB) & 1);
+                if (!__all_sync(0xffffffffu, got)) { ok = false; break; } // warp-uniform exit
+                tc_fence_after();
+                const float wt = __int_as_float((127 - kOzBeta * (g.t - 2)) << 23); // the group's weight
+                const uint32_t ta = tbase + ((uint32_t)(q * 32) << 16) + b * C::Cols + half * COLS;
+#pragma unroll
+                for (int c0 = 0; c0 < COLS; c0 += 32) {
+                    uint32_t v[32];
+                    GW_TMEM_LD32(ta + c0, v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int cc = 0; cc < 16; ++cc) {
+                        const uint32_t rv = __shfl_xor_sync(0xffffffffu, v[2 * cc + 1], 1) ^ rflip;
+                        const float x = __fadd_rn(__uint_as_float(v[2 * cc] ^ flip), __uint_as_float(rv));
+                        oz_add(hi[(c0 >> 1) + cc], lo[(c0 >> 1) + cc], __fmul_rn(wt, x));
                     }
-                    tc_fence_before();
-                    bar_arrive(&tempty[b]);
                 }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) bar_arrive_cluster(tempty0 + 8 * b);
             }
-        } else {
-            const int odd = r & 1;                    // 0: Re part, 1: Im part
-            for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-                const OzJob &jb = jobs[oz_find_job(jobs, njobs, item)];
-                int I, J;
-                oz_tile<GEN, BN>(jb, item - jb.item_start, I, J);
-                const int ng = jb.ng;
-                const int g = I * 64 + (r >> 1);      // complex row G
-                const int Eg = g < ng ? __ldg(jb.E + g) : kOzNoColumn;
-                double *crow = jb.chi + 2 * ((int64_t)g * ng) + odd;
-                for (int k0 = 0; k0 < jb.nk && ok; k0 += kOzKSeg)
-                for (int t = 2; t <= jb.s + 1; ++t, ++grp) {
-                    const uint32_t b = grp & 1, u = grp >> 1;
-                    const bool got = bar_wait(&tfull[b], u & 1);
-                    if (!__all_sync(0xffffffffu, got)) { ok = false; break; } // warp-uniform exit
-                    tc_fence_after();
-                    const uint32_t ta = tbase + ((uint32_t)(q * 32) << 16) + b * C::TmemBuf;
-#pragma unroll 1
-                    for (int c0 = 0; c0 < BN; c0 += 32) {
-                        uint32_t v[32];
-                        GW_TMEM_LD32(ta + c0, v);
-                        tmem_wait_ld();
+            if (!ok) break;
+            const int g = (2 * w.I + (int)rank) * (kOzBM / 2) + (r >> 1); // complex row
+            const int g0 = w.J * kOzBM + half * NO;                       // first complex column
+            const int nr = GEN ? jb.rows_a : jb.ng, nc = GEN ? jb.cols_b : jb.ng;
+            const int *ecol = GEN ? jb.E2 : jb.E;
+            const int eg = g < nr ? __ldg(jb.E + g) - 16 : 0;
+            double *row = (GEN ? jb.out + (int64_t)g * jb.ldo : jb.chi + 2 * (int64_t)g * jb.ng) + 2 * g0 + odd;
+            // a part of a split tile: this warp's sums go to its place in scratch, lane by lane
+            double *part = nullptr;
+            constexpr int64_t kPart = 2 * 8 * 32 * NO; // doubles of one part
+            if (!GEN && w.parts > 1)
+                part = scr.sums + ((int64_t)w.slot * w.parts + w.part) * kPart +
+                       ((int)rank * 8 + warp - 4) * (32 * NO) + lane;
 #pragma unroll
-                        for (int cc = 0; cc < 16; ++cc) {
-                            const int ev = (int)__uint_as_float(v[2 * cc]);
-                            const int od = (int)__uint_as_float(v[2 * cc + 1]);
-                            const int rv = __shfl_xor_sync(0xffffffffu, od, 1);
-                            const int val = odd ? (rv - ev) : (ev + rv);
-                            const int gp = J * C::BNC + (c0 >> 1) + cc;
-                            if ((BN % 32 == 0 || (c0 >> 1) + cc < C::BNC) && g < ng && gp < ng && g <= gp && val != 0) {
-                                const int ex = Eg + __ldg(jb.E + gp) - kOzBeta * t;
-                                const double sc = -__longlong_as_double((long long)(1023 + max(-1022, ex)) << 52);
-                                // atomic: blocks of other pair segments may add into the same entry
-                                atomicAdd(crow + 2 * (int64_t)gp, (double)val * sc);
+            for (int j = 0; j < NO; ++j)
+                if (g < nr && g0 + j < nc && (GEN || g <= g0 + j)) {
+                    const int ex = eg + __ldg(ecol + g0 + j);
+                    const double y = oz_scaled_double(hi[j], ex) + oz_scaled_double(lo[j], ex);
+                    if constexpr (GEN) row[2 * j] += y; // the tile belongs to this pair of CTAs alone
+                    else if (part) __stcg(part + 32 * j, y);
+                    else if (y != 0.0) atomicAdd(row + 2 * j, -y); // other pair segments may add here too
+                }
+            if (!GEN && part) {
+                // the warp that finishes a split tile's rows last adds all parts, in their order
+                __threadfence();
+                __syncwarp();
+                int *flag = scr.flags + w.slot * 16 + (int)rank * 8 + warp - 4;
+                int last = 0;
+                if (lane == 0) last = atomicAdd(flag, 1) == w.parts - 1;
+                if (__shfl_sync(0xffffffffu, last, 0)) {
+                    __threadfence();
+                    const double *p0 = part - (int64_t)w.part * kPart;
+                    for (int j0 = 0; j0 < NO; j0 += 16) { // 16 loads in flight
+                        double y[16];
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) y[j] = 0.0;
+                        for (int i = 0; i < w.parts; ++i) {
+                            double v[16];
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                const int c = g0 + j0 + j;
+                                v[j] = g < nr && c < nc && g <= c ? __ldcg(p0 + i * kPart + 32 * (j0 + j)) : 0.0;
                             }
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) y[j] += v[j];
                         }
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (y[j] != 0.0) atomicAdd(row + 2 * (j0 + j), -y[j]);
                     }
-                    tc_fence_before();
-                    bar_arrive(&tempty[b]);
+                    if (lane == 0) *flag = 0;
                 }
             }
         }
-        if (!ok) atomicOr(status, kStatusTimeout);
+        if (!ok && lane == 0) atomicOr(status, kStatusTimeout);
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync();
     tc_fence_after();
-    if (warp == 1) tmem_dealloc(tbase, C::TmemCols);
+    if (warp == 1) tmem_dealloc_pair(tbase, NB * C::Cols);
 }
 
 // ------------------------------------------------------------------ host launchers
-int oz_tiles(int ng, int bn)
-{
-    const int nrows = 2 * ng, bnc = bn / 2;
-    const int nI = (nrows + kOzBM - 1) / kOzBM, nJ = (nrows + bn - 1) / bn;
-    int n = 0;
-    for (int J = 0; J < nJ; ++J) n += std::min((bnc * (J + 1) - 1) / 64 + 1, nI);
-    return n;
-}
-
-size_t oz_smem_bytes(int bn, int stages)
-{
-    if (stages == 2) return bn == 128 ? OzCfg<128, 2>::Smem : bn == 240 ? OzCfg<240, 2>::Smem : OzCfg<256, 2>::Smem;
-    return bn == 128 ? OzCfg<128>::Smem : bn == 240 ? OzCfg<240>::Smem : OzCfg<256>::Smem;
-}
-
-// Tile width of the Hermitian contraction without a tuned value: 240 or 256 real columns,
-// whichever leaves less work on the busiest SM (tiles per SM rounded up, times the width).  At
-// N_G = 2000 on 152 SMs, 294 tiles of 240 fill two waves to 97 % where 272 tiles of 256 fill them
-// to 89 %.
-int oz_pick_bn(int ng, int nsm)
-{
-    int best = 256;
-    long long bestw = 0;
-    for (int bn : {256, 240}) {
-        const long long w = (long long)((oz_tiles(ng, bn) + nsm - 1) / nsm) * bn;
-        if (bn == 256 || w < bestw) {
-            best = bn;
-            bestw = w;
-        }
-    }
-    return best;
-}
-
 cudaError_t launch_oz_sqrt(const double *delta, int64_t n, double *sp, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
@@ -778,44 +784,39 @@ cudaError_t launch_oz_slice(const double2 *M, int64_t P, int ng, const double *s
     return cudaGetLastError();
 }
 
-template <int BN, int ST>
-static cudaError_t launch_oz_chi(const OzJob *jobs, int njobs, int nitems, int grid, int *status, cudaStream_t st)
-{
-    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<BN, false, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)OzCfg<BN, ST>::Smem);
-    if (e != cudaSuccess) return e;
-    oz_gemm_kernel<BN, false, ST><<<grid, kOzThreads, OzCfg<BN, ST>::Smem, st>>>(jobs, njobs, nitems, status);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_oz_gemm_jobs(int bn, const OzJob *jobs, int njobs, int nitems, int grid, int *status,
-                                cudaStream_t st, int stages)
+template <bool GEN>
+static cudaError_t launch_gemm(const OzJob *jobs, const OzItem *items, int nitems, int clusters, OzScratch scr,
+                               int *status, cudaStream_t st)
 {
     if (nitems == 0) return cudaSuccess;
-    if (stages == 2)
-        return bn == 128   ? launch_oz_chi<128, 2>(jobs, njobs, nitems, grid, status, st)
-               : bn == 240 ? launch_oz_chi<240, 2>(jobs, njobs, nitems, grid, status, st)
-                           : launch_oz_chi<256, 2>(jobs, njobs, nitems, grid, status, st);
-    return bn == 128   ? launch_oz_chi<128, kOzStages>(jobs, njobs, nitems, grid, status, st)
-           : bn == 240 ? launch_oz_chi<240, kOzStages>(jobs, njobs, nitems, grid, status, st)
-                       : launch_oz_chi<256, kOzStages>(jobs, njobs, nitems, grid, status, st);
-}
-
-cudaError_t launch_oz_split_rows(const double2 *A, int64_t rows, int ka, int s, int64_t kpad, void *ZA, int *EA,
-                                 cudaStream_t st, bool conj)
-{
-    if (rows == 0) return cudaSuccess;
-    if (conj) oz_split_rows_kernel<true><<<(unsigned)rows, 256, 0, st>>>(A, rows, ka, s, kpad, (uint16_t *)ZA, EA);
-    else oz_split_rows_kernel<false><<<(unsigned)rows, 256, 0, st>>>(A, rows, ka, s, kpad, (uint16_t *)ZA, EA);
+    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)OzCfg::Smem);
+    if (e != cudaSuccess) return e;
+    oz_gemm_kernel<GEN><<<2 * clusters, kOzThreads, OzCfg::Smem, st>>>(jobs, items, nitems, scr, status);
     return cudaGetLastError();
 }
 
-cudaError_t launch_oz_split_cols(const double2 *B, int ka, int nout, int64_t sk, int64_t sj, bool conj, int s,
-                                 int64_t kpad, void *ZB, int *EB, cudaStream_t st)
+size_t oz_part_bytes() { return sizeof(double) * 2 * 8 * 32 * (OzCfg::Cols / 4); }
+int oz_slot_flags() { return 16; }
+
+cudaError_t launch_oz_gemm_jobs(const OzJob *jobs, const OzItem *items, int nitems, int clusters, OzScratch scr,
+                                int *status, cudaStream_t st)
 {
-    if (nout == 0) return cudaSuccess;
-    if (conj) oz_split_cols_kernel<true><<<(unsigned)nout, 256, 0, st>>>(B, ka, nout, sk, sj, s, kpad, (uint16_t *)ZB, EB);
-    else oz_split_cols_kernel<false><<<(unsigned)nout, 256, 0, st>>>(B, ka, nout, sk, sj, s, kpad, (uint16_t *)ZB, EB);
+    return launch_gemm<false>(jobs, items, nitems, clusters, scr, status, st);
+}
+
+cudaError_t launch_oz_gemm_general(const OzJob *jobs, const OzItem *items, int nitems, int clusters, int *status,
+                                   cudaStream_t st)
+{
+    return launch_gemm<true>(jobs, items, nitems, clusters, OzScratch{}, status, st);
+}
+
+cudaError_t launch_oz_split(const double2 *A, int64_t rows, int ka, int64_t sr, int64_t sk, bool conj, int s,
+                            int64_t kpad, void *Z, int *E, cudaStream_t st)
+{
+    if (rows == 0) return cudaSuccess;
+    if (conj) oz_split_kernel<true><<<(unsigned)rows, 256, 0, st>>>(A, rows, ka, sr, sk, s, kpad, (uint16_t *)Z, E);
+    else oz_split_kernel<false><<<(unsigned)rows, 256, 0, st>>>(A, rows, ka, sr, sk, s, kpad, (uint16_t *)Z, E);
     return cudaGetLastError();
 }
 
@@ -835,26 +836,7 @@ cudaError_t launch_gpp_prep_split(const float4 *At, const float4 *Wt, int ng, co
     return cudaGetLastError();
 }
 
-cudaError_t launch_oz_gemm_general(int bn, const OzJob *jobs, int njobs, int nitems, int grid, int *status,
-                                   cudaStream_t st)
-{
-    if (nitems == 0) return cudaSuccess;
-    cudaError_t e;
-    if (bn == 128) {
-        e = cudaFuncSetAttribute(oz_gemm_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)OzCfg<128>::Smem);
-        if (e != cudaSuccess) return e;
-        oz_gemm_kernel<128, true><<<grid, kOzThreads, OzCfg<128>::Smem, st>>>(jobs, njobs, nitems, status);
-    } else {
-        e = cudaFuncSetAttribute(oz_gemm_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)OzCfg<256>::Smem);
-        if (e != cudaSuccess) return e;
-        oz_gemm_kernel<256, true><<<grid, kOzThreads, OzCfg<256>::Smem, st>>>(jobs, njobs, nitems, status);
-    }
-    return cudaGetLastError();
-}
-
-int oz_box_rows_a() { return kOzBM; }
+int oz_box_rows() { return kOzBM; }
 int oz_box_k() { return kOzBK; }
 
 } // namespace gw
