@@ -295,12 +295,10 @@ TRAFFIC = {
     # route existed; the kernel is unchanged since
     "pair_mtxel": {"bytes_per_launch": 3.112e9 + 1.486e9,
                    "source": "ncu dram__bytes_read+write, pair_kernel_tf_ct<48>, p1_48cube_onechunk"},
-    # the tensor-core route of the 48^3 workload: one 8192-pair chunk (128 valence x 64
-    # conduction bands), the launch shape the bench's step repeats 16 times
-    "zdft": {"bytes_per_launch": 0.477185e9 + 4.482903e9,
-             "source": "ncu dram__bytes_read+write, zd_gemm_kernel (128-column tiles), p2_48cube_chunk"},
-    "pair_from_f": {"bytes_per_launch": 5.504037e9 + 1.240109e9,
-                    "source": "ncu dram__bytes_read+write, pair_kernel_tf_from_f<48> (TMA-fed), p2_48cube_chunk"},
+    # the tensor-core route of the 48^3 workload: one 8192-pair block (16 valence x 512 conduction
+    # bands), the launch shape the bench's step repeats 16 times
+    "zdft": None,
+    "pair_from_f": None,
     "ozaki_gemm": None,
     "ozaki_gemm_single_stream": None,
 }
@@ -649,32 +647,34 @@ ZD_SLICES, ZD_TILE_N, ZD_TILE_M = 6, 128, 128
 
 
 def zd_ops(cfg, prob):
-    """Work of stage (a) on the tensor-core route per chunk: the low-precision flops the last-axis
-    split product executes (21 kept slice products of 128 x 128 x 2N tiles, padding included) and
-    the useful share, and the FP32 operations of the middle/first-axis kernel per pair."""
+    """Work of stage (a) on the tensor-core route per step: the low-precision flops the last-axis
+    split product executes (21 kept slice products of 128 x 128 x 2N tiles, 128 conduction bands by
+    as many valence bands as fill 128 columns, padding included) and the useful share, and the FP32
+    operations of the middle/first-axis kernel per pair."""
     n0, n1, n2 = cfg.grid
     k2 = kept_columns(prob, n2)
-    ct = min(4, ZD_TILE_N // (2 * k2))
-    cb = max(1, cfg.pair_chunk // cfg.nv)
-    tiles = n0 * n1 * -(-cfg.nv // ZD_TILE_M) * -(-cb // ct)
+    ct = max(1, min(6, ZD_TILE_N // (2 * ((k2 + 1) // 2 * 2))))
+    tiles = n0 * n1 * -(-cfg.nc // ZD_TILE_M) * -(-cfg.nv // ct)
     prods = ZD_SLICES * (ZD_SLICES + 1) // 2
     flops = prods * 2.0 * ZD_TILE_M * ZD_TILE_N * 2 * n2 * tiles
-    useful = prods * 8.0 * n2 * k2 * cfg.nv * cb * n0 * n1  # complex MACs of the kept outputs
+    useful = prods * 8.0 * n2 * k2 * cfg.npairs * n0 * n1  # complex MACs of the kept outputs
     k12 = cells(prob, cfg.grid)
     i1 = k2 * _head_ops(n1, lazy=True) + k12 * _prune_out_ops(n1)
     i0 = k12 * _head_ops(n0, lazy=True) + cfg.ng * _prune_out_ops(n0)
-    return flops, useful, n0 * i1 + i0, cb
+    return flops, useful, n0 * i1 + i0
 
 
 def roofline_zd(cfg, prob, res):
     """Rooflines of the tensor-core stage (a): the last-axis split product (tensor) and the
     middle/first-axis kernel (FP32 issue), each per launch; plus the method-level stage (a)
     numbers over both."""
-    flops, useful, ops_pair, cb = zd_ops(cfg, prob)
+    flops_step, useful_step, ops_pair = zd_ops(cfg, prob)
+    steps = max(1, round(res["total_ms"] / res["ms_per_step"]))
     out = {}
     kms, kn = res["timing"].get("zdft", (0.0, 0))
     if kn:
         peak, src = peak_for("ozaki")
+        flops, useful = flops_step * steps / kn, useful_step * steps / kn
         ach = flops / (kms / kn * 1e-3) * 1e-12
         out["zdft"] = {"bound": "tensor", "kernel": "zd_gemm_kernel", "achieved": ach, "peak": peak,
                        "unit": "TFLOP/s", "frac": ach / peak, "traffic": traffic_for("zdft", cfg)[0],
@@ -685,7 +685,7 @@ def roofline_zd(cfg, prob, res):
     kms2, kn2 = res["timing"].get("pair_from_f", (0.0, 0))
     if kn2:
         peak, src = fp32_lane_peak()
-        per_launch = ops_pair * cfg.nv * cb
+        per_launch = ops_pair * cfg.npairs * steps / kn2
         ach = per_launch / (kms2 / kn2 * 1e-3) * 1e-12
         out["pair_from_f"] = {"bound": "alu", "kernel": "pair_kernel_tf_from_f", "achieved": ach, "peak": peak,
                               "unit": "FP32 Tops/s", "frac": ach / peak,
@@ -697,8 +697,7 @@ def roofline_zd(cfg, prob, res):
     if kn and kn2:
         mbytes, mflops = method_stage_a(cfg)
         hbm, hbm_src = _hbm_peak()
-        nchunk = -(-cfg.nc // cb)
-        t_step = (kms / kn + kms2 / kn2) * 1e-3 * nchunk
+        t_step = (kms + kms2) * 1e-3 / steps
         dfma = LIVE_PEAKS.get("dfma")
         out["stage_a_method"] = {"bytes_per_step": mbytes, "flops_per_step": mflops,
                                  "hbm_frac": mbytes / t_step * 1e-9 / hbm, "hbm_peak_gbs": hbm,

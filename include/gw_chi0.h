@@ -138,9 +138,10 @@ GW_API gw_status gw_chi0_set_gsphere(gw_chi0 *h, int iq, int ng, const int32_t *
 
 /*
  * Forward chi0 for nq slots and nw imaginary frequencies (steps a1-a7 after setup).  With
- * two-float stage (a) on the 48^3 grid the last axis of the pair transform runs on the BF16
- * tensor cores (the route of gw_chi0_pair_elements_block); elsewhere stage (a) is the pruned
- * FFT pair kernel.
+ * two-float stage (a) on the 40^3 and 48^3 grids the last axis of the pair transform runs on the
+ * BF16 tensor cores where that is faster (see gw_chi0_pair_elements_block); elsewhere stage (a) is
+ * the pruned FFT pair kernel.  The other calls that form pair elements for whole valence rows choose
+ * alike.
  *   iq     host int [nq]      slots to compute.
  *   omega  host double [nw]   imaginary-axis frequencies w >= 0 (eV).
  *   chi    device complex128, packed by slot: for slot i, nw blocks of ng_i x ng_i
@@ -189,12 +190,12 @@ GW_API gw_status gw_chi0_pair_elements(gw_chi0 *h, int iq, int64_t pair_begin, i
  * Stage (a) alone for all valence bands of slot iq and the conduction bands c0 .. c0 + cb - 1,
  * on the route gw_chi0_compute takes for two-float stage (a) on the 48^3 grid: the last-axis
  * transform of the pair products as a split product on the BF16 tensor cores (the grid line's
- * valence points against the conduction points times the kept twiddles, six BF16 slices each,
- * FP32 group sums combined in two-float arithmetic), the middle and first axes as in the FFT
- * pair kernel.  Rows in that route's order: M[(c - c0) nv + v][g], device complex128
- * [cb nv][ng].  GW_ERR_UNSUPPORTED when the slot does not take the route (another grid, FP64
+ * conduction points against the conjugated valence points times the kept twiddles, six BF16 slices
+ * each, FP32 group sums combined in two-float arithmetic), the middle and first axes as in the FFT
+ * pair kernel.  Rows M[(c - c0) nv + v][g], device complex128 [cb nv][ng].  GW_ERR_UNSUPPORTED when the slot does not take the route (another grid, FP64
  * stage (a), resident pair elements kept); GW_ERR_ARG for a block outside [0, nc).  Uses the
- * handle's work buffers (the last-axis output of cb nv pairs, 16 * 48^2 * K2 bytes per pair).
+ * handle's work buffers (the slices of a block of the conduction bands and the last-axis output of
+ * some of its pairs, 16 * 48^2 * K2 bytes each).
  */
 GW_API gw_status gw_chi0_pair_elements_block(gw_chi0 *h, int iq, int c0, int cb, double *M);
 

@@ -571,101 +571,189 @@ gw_status ensure_overlap_stream(gw_chi0 *h)
 }
 
 // ------------------------------------------------------------------ stage (a) on the tensor cores
-// The last-axis transform of the pair products as a split product per grid line (zdft.cu) for
-// two-float stage (a) on the 48^3 grid; chunks are all valence bands x a block of conduction
-// bands, rows r = cl nv + v, on one stream (the last-axis product and the split contraction each
-// need whole SMs' shared memory: running the contraction on a second stream beside the next
-// chunk's FP32 stages measured slower, 163 against 142 ms per 48^3 q-point).
+// The last-axis transform of the pair products as a split product per grid line (zdft.cu), the
+// middle and first axes from its output, for two-float stage (a) on the 40^3 and 48^3 grids.  A block
+// is vb valence x cb conduction bands; the row slices of the conduction block are formed once, and the
+// valence bands run over it in sub-blocks whose transform output F fits the work buffer.  On one
+// stream: the last-axis product and the split contraction each need whole SMs.
 // GW_CHI0_STAGE_A=fft selects the FFT pair kernel instead.
-bool zd_route(gw_chi0 *h, int iq, bool resident)
+static bool zd_grid(const gw_chi0 *h, const Sphere &sp)
 {
     static const bool fft_only = [] {
         const char *e = getenv("GW_CHI0_STAGE_A");
         return e && strcmp(e, "fft") == 0;
     }();
-    if (fft_only || resident || h->d.mtxel_prec != GW_MTXEL_TWOFLOAT) return false;
-    const Sphere &sp = h->sph[iq];
     const int n = h->d.n[0];
-    if (h->d.n[1] != n || h->d.n[2] != n || sp.nslots <= 0 || !h->pscr) return false;
-    return gw::zd_supported(n, sp.K2, h->val[iq].nb) && h->d.pair_chunk >= h->val[iq].nb;
+    return !fft_only && h->d.mtxel_prec == GW_MTXEL_TWOFLOAT && h->d.n[1] == n && h->d.n[2] == n && sp.nslots > 0 &&
+           h->pscr && gw::zd_supported(n, sp.K2);
 }
 
-int zd_chunk_bands(gw_chi0 *h, int iq)
+// Whether a block of vb x cb pairs takes less time this way.  In units of one pair of the FFT kernel
+// (1.04 us on 48^3, 0.84 on 40^3; below about 600 pairs its blocks do not fill the GPU): a tile of 128
+// conduction bands x CT valence bands over all lines costs 70 (48^3) or 50 (40^3), however few of
+// its rows and columns hold bands, and the other two axes 0.25 a pair.
+static bool zd_faster(const gw_chi0 *h, const Sphere &sp, int vb, int cb)
 {
-    const int nv = h->val[iq].nb;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(h->cond.nb, h->d.pair_chunk / nv));
+    const int ct = gw::zd_valence_per_tile(sp.K2);
+    const double tiles = (double)((cb + 127) / 128) * ((vb + ct - 1) / ct), pairs = (double)vb * cb;
+    return tiles * (h->d.n[0] == 48 ? 70.0 : 50.0) + 0.25 * pairs < std::max(pairs, 600.0);
 }
 
-gw_status zd_prepare(gw_chi0 *h, int iq, CUtensorMap *tmA, CUtensorMap *tmC)
+// Room for the route's buffers beside what the call will still take: with a memory budget, the
+// pair elements of a chunk, their slices (for a group of frequencies) and the split tiles' scratch
+// come first; without one, the buffers may grow by a quarter of the free memory.
+static bool zd_room(const gw_chi0 *h, size_t grow_by, int64_t pairs, int ng, int nw)
 {
-    const BandSet &v = h->val[iq];
-    const Sphere &sp = h->sph[iq];
-    const int n = h->d.n[0], nv = v.nb, cb = zd_chunk_bands(h, iq);
-    const int64_t lines = (int64_t)n * n;
-    const size_t abytes = (size_t)gw::kZdSlices * lines * nv * 2 * n * 2;
-    const size_t fbytes = sizeof(float4) * (size_t)lines * nv * cb * sp.K2;
-    gw_status s;
-    if ((s = grow(h, &h->zdA, &h->zdAcap, abytes, "valence slices")) ||
-        (s = grow(h, (void **)&h->zdF, &h->zdFcap, fbytes, "last-axis transform")))
-        return s;
-    {
-        Scope sc(h, "zd_aslices");
-        CK(h, gw::launch_zd_aslices(v.psi, nv, n, (uint16_t *)h->zdA, h->st), "valence slices");
+    if (grow_by == 0) return true;
+    if (h->d.mem_budget_bytes) {
+        const double m = 16.0 * pairs * ng, z = 4.0 * gw::oz_slices(h->d.nslices) * ng * (pairs + 64.0);
+        const double later = 3.0 * m + z * std::min(nw, gw::oz_group_w()) + 16.0 * pairs * nw + 100e6;
+        return (double)h->bytes + grow_by + later <= (double)h->d.mem_budget_bytes;
     }
-    cuuint64_t dims[4] = {(cuuint64_t)2 * n, (cuuint64_t)nv, (cuuint64_t)lines, (cuuint64_t)gw::kZdSlices};
-    cuuint64_t strides[3] = {(cuuint64_t)2 * n * 2, (cuuint64_t)2 * n * 2 * nv, (cuuint64_t)2 * n * 2 * nv * lines};
-    cuuint32_t box[4] = {32, 128, 1, (cuuint32_t)gw::kZdSlices};
-    cuuint32_t es[4] = {1, 1, 1, 1};
-    CUresult r = h->encode(tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, h->zdA, dims, strides, box, es,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(h, GW_ERR_CUDA, "cuTensorMapEncodeTiled (valence slices) failed (%d)", (int)r);
-    // the conduction grids, line by line: box of one line of CT bands
-    cuuint64_t cd[3] = {(cuuint64_t)4 * n, (cuuint64_t)lines, (cuuint64_t)h->cond.nb};
-    cuuint64_t cst[2] = {(cuuint64_t)4 * n * 4, (cuuint64_t)16 * lines * n};
-    cuuint32_t cbox[3] = {(cuuint32_t)(4 * n), 1, (cuuint32_t)gw::zd_conduction_per_tile(sp.K2)};
-    cuuint32_t ces[3] = {1, 1, 1};
-    r = h->encode(tmC, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, h->cond.psi, cd, cst, cbox, ces, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(h, GW_ERR_CUDA, "cuTensorMapEncodeTiled (conduction grids) failed (%d)", (int)r);
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return grow_by <= free_b / 4;
+}
+
+gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw, ZdPlan &z)
+{
+    z = ZdPlan();
+    if (!zd_grid(h, sp)) return GW_OK;
+    const int n = h->d.n[0], ct = gw::zd_valence_per_tile(sp.K2);
+    // The route's pair elements carry 2e-13 (its fourth accumulator rounds in FP32), the FFT kernel's
+    // 8e-15.  At up to seven slices the contraction's own error is ten times that and more.  At eight,
+    // and with the FP64 contraction, the route serves chi on 48^3 alone (8.7e-14 at eight slices); on
+    // the other calls it would raise the error, by up to three times for the gradients.
+    if ((h->d.prec == GW_PREC_FP64 || h->d.nslices > 7) && (rows || n != 48)) return GW_OK;
+    if (rows) {
+        z.cb = nc;
+    } else { // conduction blocks of about 512: four row tiles share a valence tile's columns
+        const int nblk = (nc + 511) / 512;
+        z.cb = (nc + nblk - 1) / nblk;
+        if (nblk > 1) z.cb = (z.cb + 127) / 128 * 128;
+        z.cb = (int)std::min<int64_t>(z.cb, h->d.pair_chunk);
+    }
+    int64_t vb = std::min<int64_t>(nv, h->d.pair_chunk / z.cb);
+    if (vb < 1) return GW_OK;
+    if (vb >= ct && vb < nv) vb -= vb % ct;
+    z.vb = (int)vb;
+    if (!force && !zd_faster(h, sp, z.vb, z.cb)) return GW_OK;
+    z.n = n;
+    z.abytes = gw::zd_row_bytes(z.cb, n);
+    z.ebytes = sizeof(int) * (size_t)n * n * nv;
+    z.fper = sizeof(float4) * (size_t)n * n * z.cb * gw::zd_row_entries(sp.K2); // F of one valence band
+    // F of as many valence bands as 5 GB hold (whole tiles), fewer where memory is short
+    int vs = (int)std::min<size_t>(z.vb, std::max<size_t>(1, (size_t)5000000000 / z.fper));
+    for (;; vs = vs > ct ? std::max(ct, vs / 2) : vs / 2) {
+        if (vs < 1) return GW_OK;
+        if (vs > ct) vs -= vs % ct;
+        size_t by = 0;
+        for (int i = 0; i < sides; ++i)
+            by += (z.abytes > h->zdAcap[i] ? z.abytes - h->zdAcap[i] : 0) + (z.ebytes > h->zdEcap[i] ? z.ebytes - h->zdEcap[i] : 0);
+        by += z.fper * vs > h->zdFcap ? z.fper * vs - h->zdFcap : 0;
+        if (force || zd_room(h, by, (int64_t)z.vb * z.cb, sp.ng, nw)) break;
+    }
+    z.vs = vs;
+    const std::string err = h->err;
+    gw_status s = GW_OK;
+    for (int i = 0; i < sides && !s; ++i)
+        if (!(s = grow(h, &h->zdA[i], &h->zdAcap[i], z.abytes, "conduction slices")))
+            s = grow(h, (void **)&h->zdE[i], &h->zdEcap[i], z.ebytes, "column exponents");
+    if (!s) s = grow(h, (void **)&h->zdF, &h->zdFcap, z.fper * vs, "last-axis transform");
+    if (s == GW_ERR_OOM && !force) { // the FFT route needs none of these
+        h->err = err;
+        return GW_OK;
+    }
+    if (s) return s;
+    z.on = true;
     return GW_OK;
 }
 
-gw_status zd_stage_a(gw_chi0 *h, int iq, const CUtensorMap &tmA, const CUtensorMap &tmC, int c0, int cb,
-                     const gw::PairPlan &pp, double2 *M)
+bool zd_holds(const gw_chi0 *h, const ZdPlan &z)
 {
-    const BandSet &v = h->val[iq];
-    const Sphere &sp = h->sph[iq];
-    const int n = h->d.n[0];
+    return h->zdAcap[0] >= z.abytes && h->zdEcap[0] >= z.ebytes && h->zdFcap >= z.fper * z.vs;
+}
+
+gw_status zd_valence(gw_chi0 *h, ZdPlan &z, const Sphere &sp, const void *psiv, int nv, int side)
+{
+    const int n = z.n;
+    const int64_t lines = (int64_t)n * n;
     {
-        Scope sc(h, "zdft");
-        CK(h, gw::launch_zd_gemm(tmA, tmC, h->cond.psi, sp.kz, pp.ax[2].twf, n, v.nb, c0, cb, sp.K2, h->zdF,
-                                 h->status, h->st),
-           "last-axis transform");
+        Scope sc(h, "zd_slices");
+        CK(h, gw::launch_zd_colexp(psiv, nv, n, h->zdE[side], h->st), "column exponents");
     }
-    // F as [n^2 lines][R K2] two-float entries: the middle/first-axis kernel loads a slab pair's
-    // 2n lines of one row (K2 entries each) with one TMA box
-    const int64_t R = (int64_t)v.nb * cb;
-    CUtensorMap tmF;
-    cuuint64_t fd[2] = {(cuuint64_t)R * sp.K2 * 4, (cuuint64_t)n * n};
-    cuuint64_t fst[1] = {(cuuint64_t)R * sp.K2 * 16};
-    cuuint32_t fbox[2] = {(cuuint32_t)(sp.K2 * 4), (cuuint32_t)(2 * n)};
-    cuuint32_t fes[2] = {1, 1};
-    CUresult r = h->encode(&tmF, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->zdF, fd, fst, fbox, fes,
+    // the valence grids, line by line: box of one line of CT bands
+    cuuint64_t d[3] = {(cuuint64_t)4 * n, (cuuint64_t)lines, (cuuint64_t)nv};
+    cuuint64_t st[2] = {(cuuint64_t)4 * n * 4, (cuuint64_t)16 * lines * n};
+    cuuint32_t box[3] = {(cuuint32_t)(4 * n), 1, (cuuint32_t)gw::zd_valence_per_tile(sp.K2)};
+    cuuint32_t es[3] = {1, 1, 1};
+    CUresult r = h->encode(&z.tmV[side], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(psiv), d, st, box, es,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(h, GW_ERR_CUDA, "cuTensorMapEncodeTiled (last-axis output) failed (%d)", (int)r);
-    // the scratch slots as [nslots n rows][K12] entries: phase 2 loads batches of 2 K2 cells of
-    // all n rows of its slot with one TMA box
-    CUtensorMap tmS;
-    cuuint64_t sd[2] = {(cuuint64_t)pp.K12 * 4, (cuuint64_t)pp.nslots * n};
-    cuuint64_t sst[1] = {(cuuint64_t)pp.K12 * 16};
-    cuuint32_t sbox[2] = {(cuuint32_t)(8 * sp.K2), (cuuint32_t)n};
-    r = h->encode(&tmS, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, pp.scr, sd, sst, sbox, fes, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(h, GW_ERR_CUDA, "cuTensorMapEncodeTiled (pair scratch) failed (%d)", (int)r);
-    Scope sc(h, "pair_from_f");
-    CK(h, gw::launch_pair_tf_from_f(tmF, tmS, R, pp, M, h->st), "pair elements from F");
+    if (r != CUDA_SUCCESS) return fail(h, GW_ERR_CUDA, "cuTensorMapEncodeTiled (valence grids) failed (%d)", (int)r);
+    z.nv[side] = nv;
+    return GW_OK;
+}
+
+gw_status zd_conduction(gw_chi0 *h, const ZdPlan &z, const void *psic, int c0, int cb, int side)
+{
+    Scope sc(h, "zd_slices");
+    CK(h, gw::launch_zd_rows((const float4 *)psic + (int64_t)c0 * h->nr, cb, z.n, h->zdA[side], h->st),
+       "conduction slices");
+    return GW_OK;
+}
+
+gw_status zd_block(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::PairPlan &pp, int vside, int cside, int v0,
+                   int vb, int cb, double2 *M, int64_t sv, int64_t sc)
+{
+    const int n = z.n;
+    for (int b0 = 0; b0 < vb; b0 += z.vs) {
+        const int nb = std::min(z.vs, vb - b0);
+        {
+            Scope t(h, "zdft");
+            CK(h, gw::launch_zd_gemm(z.tmV[vside], h->zdA[cside], h->zdE[vside], sp.kz, pp.ax[2].twf, n, z.nv[vside],
+                                     v0 + b0, nb, cb, sp.K2, h->zdF, h->status, h->st),
+               "last-axis transform");
+        }
+        // F as [n^2 lines][R rows of K2P entries]: the middle/first-axis kernel loads a slab pair's
+        // 2n lines of one row (K2 entries each) with one TMA box
+        const int64_t R = (int64_t)nb * cb;
+        CUtensorMap tmF;
+        const int k2p = gw::zd_row_entries(sp.K2);
+        cuuint64_t fd[2] = {(cuuint64_t)R * k2p * 4, (cuuint64_t)n * n};
+        cuuint64_t fst[1] = {(cuuint64_t)R * k2p * 16};
+        cuuint32_t fbox[2] = {(cuuint32_t)(sp.K2 * 4), (cuuint32_t)(2 * n)};
+        cuuint32_t fes[2] = {1, 1};
+        CUresult r = h->encode(&tmF, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->zdF, fd, fst, fbox, fes,
+                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return fail(h, GW_ERR_CUDA, "cuTensorMapEncodeTiled (last-axis output) failed (%d)", (int)r);
+        // the scratch slots as [nslots n rows][K12] entries: phase 2 loads batches of 2 K2 cells of
+        // all n rows of its slot with one TMA box
+        CUtensorMap tmS;
+        cuuint64_t sd[2] = {(cuuint64_t)pp.K12 * 4, (cuuint64_t)pp.nslots * n};
+        cuuint64_t sst[1] = {(cuuint64_t)pp.K12 * 16};
+        cuuint32_t sbox[2] = {(cuuint32_t)(8 * sp.K2), (cuuint32_t)n};
+        r = h->encode(&tmS, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, pp.scr, sd, sst, sbox, fes, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return fail(h, GW_ERR_CUDA, "cuTensorMapEncodeTiled (pair scratch) failed (%d)", (int)r);
+        Scope t(h, "pair_from_f");
+        CK(h, gw::launch_pair_tf_from_f(tmF, tmS, R, cb, sv, sc, pp, M + (int64_t)b0 * sv * sp.ng, h->st),
+           "pair elements from F");
+    }
+    return GW_OK;
+}
+
+// Pairs [p0, p0 + cnt) of slot pairs (psiv, psic), whole valence rows when the plan is on.
+gw_status pair_rows(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::PairPlan &pp, const void *psiv,
+                    const void *psic, int nc, int64_t p0, int64_t cnt, double2 *M, int vside, int cside)
+{
+    if (z.on) return zd_block(h, z, sp, pp, vside, cside, (int)(p0 / nc), (int)(cnt / nc), nc, M, nc, 1);
+    Scope sc(h, "pair_mtxel");
+    CK(h, run_pair(h, psiv, psic, nc, p0, cnt, pp, M), "pair kernel");
     return GW_OK;
 }
 
@@ -860,7 +948,7 @@ int gw_chi0_streams(gw_chi0 *h, int iq)
     if (!h) return -(int)GW_ERR_ARG;
     gw_status s = check_slot(h, iq);
     if (s) return -(int)s;
-    if (zd_route(h, iq, h->keep_m)) return 1; // the tensor-core stage (a) leaves no room beside it
+    if (zd_grid(h, h->sph[iq])) return 1; // stage (a) on the tensor cores runs on one stream
     return overlap_enabled(h, pair_plan(h, h->sph[iq])) ? 2 : 1;
 }
 
@@ -884,7 +972,10 @@ void gw_chi0_destroy(gw_chi0 *h)
     dfree(h, h->EBbuf, h->EBcap);
     dfree(h, h->ZBbuf, h->ZBcap);
     dfree(h, h->MBbuf, h->MBcap);
-    dfree(h, h->zdA, h->zdAcap);
+    for (int i = 0; i < 2; ++i) {
+        dfree(h, h->zdA[i], h->zdAcap[i]);
+        dfree(h, h->zdE[i], h->zdEcap[i]);
+    }
     dfree(h, h->zdF, h->zdFcap);
     for (int b = 0; b < 2; ++b) {
         dfree(h, h->ovZ[b], h->ovZcap[b]);
@@ -1122,16 +1213,21 @@ gw_status gw_chi0_pair_elements_block(gw_chi0 *h, int iq, int c0, int cb, double
     if (c0 < 0 || cb < 0 || c0 + cb > h->cond.nb)
         return fail(h, GW_ERR_ARG, "conduction block [%d, %d) outside [0, %d)", c0, c0 + cb, h->cond.nb);
     if (cb && !M) return fail(h, GW_ERR_ARG, "null M");
-    if (!zd_route(h, iq, h->keep_m)) return fail(h, GW_ERR_UNSUPPORTED, "slot %d does not take the tensor-core route", iq);
+    const BandSet &v = h->val[iq];
+    const Sphere &sp = h->sph[iq];
+    const int nv = v.nb;
+    if (h->d.n[0] != 48 || h->keep_m || h->d.pair_chunk < nv || !zd_grid(h, sp))
+        return fail(h, GW_ERR_UNSUPPORTED, "slot %d does not take the tensor-core route", iq);
     if (cb == 0) return GW_OK;
-    const int nv = h->val[iq].nb, cbmax = zd_chunk_bands(h, iq);
-    CUtensorMap tmA, tmC;
-    if ((s = zd_prepare(h, iq, &tmA, &tmC))) return s;
-    const gw::PairPlan pp = pair_plan(h, h->sph[iq]);
-    const int ng = h->sph[iq].ng;
-    for (int b0 = 0; b0 < cb; b0 += cbmax) {
-        const int n = std::min(cbmax, cb - b0);
-        if ((s = zd_stage_a(h, iq, tmA, tmC, c0 + b0, n, pp, (double2 *)M + (int64_t)b0 * nv * ng))) return s;
+    ZdPlan z;
+    if ((s = zd_plan(h, sp, nv, cb, false, true, 1, 1, z))) return s;
+    const gw::PairPlan pp = pair_plan(h, sp);
+    if ((s = zd_valence(h, z, sp, v.psi, nv))) return s;
+    for (int b0 = 0; b0 < cb; b0 += z.cb) {
+        const int n = std::min(z.cb, cb - b0);
+        if ((s = zd_conduction(h, z, h->cond.psi, c0 + b0, n)) ||
+            (s = zd_block(h, z, sp, pp, 0, 0, 0, nv, n, (double2 *)M + (int64_t)b0 * nv * sp.ng, 1, nv)))
+            return s;
     }
     return GW_OK;
 }
@@ -1185,10 +1281,8 @@ gw_status gw_chi0_compute(gw_chi0 *h, int nq, const int *iq, int nw, const doubl
         gw_status s = resident_begin(h, P, ng, &keep);
         if (s) return s;
         double2 *Mres = keep ? h->Mres : nullptr;
-        // one frequency: a chunk's contraction is about as long as the next chunk's pair elements
-        // and hides behind them; with more, the contractions (the shallow-ring variant) queue up
-        // behind the two slice buffers and the single stream is faster
-        if (nw == 1 && overlap_enabled(h, pp) && fault_chunk() < 0 && !zd_route(h, iq[i], keep)) {
+        // with several frequencies the contractions queue up behind the two slice buffers: one stream
+        if (nw == 1 && overlap_enabled(h, pp) && fault_chunk() < 0 && !zd_grid(h, sp)) {
             s = compute_overlap(h, iq[i], om, cq, dq, Mres);
             if (s) return s;
             Scope sc(h, "symmetrize");
@@ -1198,30 +1292,38 @@ gw_status gw_chi0_compute(gw_chi0 *h, int nq, const int *iq, int nw, const doubl
             if (keep) h->Mres_iq = iq[i];
             continue;
         }
-        if (zd_route(h, iq[i], keep) && fault_chunk() < 0) {
-            const int nv = v.nb, cb = zd_chunk_bands(h, iq[i]);
-            s = ensure_work(h, (size_t)nv * cb * ng, (size_t)nv * cb * nw);
-            if (s) return s;
-            CUtensorMap tmA, tmC;
-            if ((s = zd_prepare(h, iq[i], &tmA, &tmC))) return s;
-            for (int c0 = 0; c0 < h->cond.nb; c0 += cb) {
-                const int cbc = std::min(cb, h->cond.nb - c0);
-                const int64_t cnt = (int64_t)nv * cbc;
-                if ((s = zd_stage_a(h, iq[i], tmA, tmC, c0, cbc, pp, h->Mbuf))) return s;
-                {
-                    Scope sc(h, "delta");
-                    CK(h, gw::launch_delta_block(v.energy, h->cond.energy, nv, c0, cbc, om, h->dbuf, h->st), "delta");
-                }
-                if ((s = contract_chunk(h, h->Mbuf, cnt, ng, h->dbuf, cnt, nw, cq))) return s;
-                if (dq) {
-                    Scope sc(h, "diag");
-                    CK(h, gw::launch_diag(h->Mbuf, cnt, ng, h->dbuf, cnt, nw, dq, ng, h->st), "diag");
+        ZdPlan z;
+        if (fault_chunk() < 0 && (s = zd_plan(h, sp, v.nb, h->cond.nb, keep, false, 1, nw, z))) return s;
+        if (z.on) {
+            const int nc = h->cond.nb;
+            if ((s = ensure_work(h, keep ? 0 : (size_t)z.vb * z.cb * ng, (size_t)z.vb * z.cb * nw)) ||
+                (s = zd_valence(h, z, sp, v.psi, v.nb)))
+                return s;
+            for (int c0 = 0; c0 < nc; c0 += z.cb) {
+                const int cb = std::min(z.cb, nc - c0);
+                if ((s = zd_conduction(h, z, h->cond.psi, c0, cb))) return s;
+                for (int v0 = 0; v0 < v.nb; v0 += z.vb) {
+                    const int vb = std::min(z.vb, v.nb - v0);
+                    const int64_t cnt = (int64_t)vb * cb; // rows vl cb + cl
+                    double2 *Mc = keep ? Mres + (int64_t)v0 * nc * ng : h->Mbuf;
+                    if ((s = zd_block(h, z, sp, pp, 0, 0, v0, vb, cb, Mc, cb, 1))) return s;
+                    {
+                        Scope sc(h, "delta");
+                        CK(h, gw::launch_delta(v.energy + v0, h->cond.energy + c0, cb, 0, cnt, om, h->dbuf, h->st),
+                           "delta");
+                    }
+                    if ((s = contract_chunk(h, Mc, cnt, ng, h->dbuf, cnt, nw, cq))) return s;
+                    if (dq) {
+                        Scope sc(h, "diag");
+                        CK(h, gw::launch_diag(Mc, cnt, ng, h->dbuf, cnt, nw, dq, ng, h->st), "diag");
+                    }
                 }
             }
             Scope sc(h, "symmetrize");
             CK(h, gw::launch_symmetrize(cq, ng, nw, h->st), "symmetrize");
             off += (size_t)nw * ng * ng;
             doff += (size_t)nw * ng;
+            if (keep) h->Mres_iq = iq[i];
             continue;
         }
         s = ensure_work(h, (size_t)chunk * ng, (size_t)chunk * nw);

@@ -81,15 +81,22 @@ std::string tune_key(gw_chi0 *h, const BatchLayout &L, int nw)
 
 // Enqueue the producer stages: pair elements of every slot, Delta, and (split precision)
 // the square roots.  The slices depend on the frequency and are enqueued per frequency.
-gw_status batch_stage_a(gw_chi0 *h, int nq, const int *iq, const gw::OmegaList &om, const BatchLayout &L)
+gw_status batch_stage_a(gw_chi0 *h, int nq, const int *iq, const gw::OmegaList &om, const BatchLayout &L,
+                        std::vector<ZdPlan> &zd)
 {
+    bool rows = false; // the conduction slices are the same for every slot
     for (int i = 0; i < nq; ++i) {
         const BandSet &v = h->val[iq[i]];
-        gw::PairPlan pp = pair_plan(h, h->sph[iq[i]]);
-        {
-            Scope sc(h, "pair_mtxel");
-            CK(h, run_pair(h, v.psi, h->cond.psi, h->cond.nb, 0, L.P[i], pp, h->Mall + L.moff[i]), "pair kernel");
+        const Sphere &sp = h->sph[iq[i]];
+        gw::PairPlan pp = pair_plan(h, sp);
+        gw_status s;
+        if (zd[i].on) {
+            if ((s = zd_valence(h, zd[i], sp, v.psi, v.nb)) ||
+                (!rows && (s = zd_conduction(h, zd[i], h->cond.psi, 0, h->cond.nb))))
+                return s;
+            rows = true;
         }
+        if ((s = pair_rows(h, zd[i], sp, pp, v.psi, h->cond.psi, h->cond.nb, 0, L.P[i], h->Mall + L.moff[i]))) return s;
         Scope sc(h, "delta");
         CK(h, gw::launch_delta(v.energy, h->cond.energy, h->cond.nb, 0, L.P[i], om, h->Dall + L.doff[i], h->st),
            "delta");
@@ -149,7 +156,7 @@ gw_status batch_oz_jobs(gw_chi0 *h, int nq, int w, const BatchLayout &L, double2
 // cleared afterwards by the real run) and keep the fastest.  The split contraction has one tile
 // shape: nothing to time.
 gw_status batch_autotune(gw_chi0 *h, int nq, const int *iq, int nw, const gw::OmegaList &om, const BatchLayout &L,
-                         double2 *chi)
+                         double2 *chi, std::vector<ZdPlan> &zd)
 {
     const std::string key = tune_key(h, L, nw);
     auto it = h->tune_cache.find(key);
@@ -160,7 +167,7 @@ gw_status batch_autotune(gw_chi0 *h, int nq, const int *iq, int nw, const gw::Om
     }
     std::array<int, 2> pick = {h->tuned_bt, h->tuned_waves};
     if (h->d.prec == GW_PREC_FP64) {
-        gw_status s = batch_stage_a(h, nq, iq, om, L);
+        gw_status s = batch_stage_a(h, nq, iq, om, L, zd);
         if (s) return s;
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
@@ -208,7 +215,12 @@ gw_status compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const double 
          (s = grow(h, (void **)&h->Eall, &h->Eall_cap, sizeof(int) * L.Etot, "resident exponents"))))
         return s;
     if (!h->cap_st) CK(h, cudaStreamCreateWithFlags(&h->cap_st, cudaStreamNonBlocking), "capture stream");
-    if ((s = batch_autotune(h, nq, iq, nw, om, L, (double2 *)chi))) return s;
+    // stage (a)'s route per slot, and the buffers the slots share, before the capture
+    std::vector<ZdPlan> zd(nq);
+    for (int i = 0; i < nq; ++i)
+        if ((s = zd_plan(h, h->sph[iq[i]], h->val[iq[i]].nb, h->cond.nb, true, false, 1, 1, zd[i]))) return s;
+    for (auto &z : zd) z.on = z.on && zd_holds(h, z);
+    if ((s = batch_autotune(h, nq, iq, nw, om, L, (double2 *)chi, zd))) return s;
 
     const std::string key = batch_key(h, nq, iq, nw, omega, chi, diag) + "|" + std::to_string(h->tuned_bt) + "," +
                             std::to_string(h->tuned_waves);
@@ -261,7 +273,7 @@ gw_status compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const double 
                                  cudaSuccess))
                     body = fail(h, GW_ERR_CUDA, "capture: memset");
             }
-            if (!body) body = batch_stage_a(h, nq, iq, om, L);
+            if (!body) body = batch_stage_a(h, nq, iq, om, L, zd);
             if (!body && h->d.prec == GW_PREC_FP64) {
                 int nitems = 0;
                 for (auto &j : fj) nitems = std::max(nitems, j.item_start + (int)((int64_t)j.ksplit * j.ntile *

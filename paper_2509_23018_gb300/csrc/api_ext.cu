@@ -72,6 +72,12 @@ gw_status gw_chi0_adjoint(gw_chi0 *h, int iq, double omega, const double *W, dou
     ACK(cudaMemsetAsync(pbv, 0, szV, h->st), "zero");
     ACK(cudaMemsetAsync(pbc, 0, szC, h->st), "zero");
     gw::PairPlan pp = pair_plan(h, sp);
+    ZdPlan z;
+    if ((s = zd_plan(h, sp, nv, nc, true, false, 1, 1, z)) ||
+        (z.on && ((s = zd_valence(h, z, sp, v.psi, nv)) || (s = zd_conduction(h, z, c.psi, 0, nc))))) {
+        cleanup();
+        return s;
+    }
     // split precision: Y = M W as a split product, W's slices once per call
     const bool split = h->d.prec == GW_PREC_OZAKI_BF16;
     if (split && (s = oz_prepare_b(h, Wh, ng, ng))) {
@@ -81,9 +87,9 @@ gw_status gw_chi0_adjoint(gw_chi0 *h, int iq, double omega, const double *W, dou
     for (int v0 = 0; v0 < nv; v0 += (int)vch) {
         const int nvc = (int)std::min<int64_t>(vch, nv - v0);
         const int64_t p0 = (int64_t)v0 * nc, cnt = (int64_t)nvc * nc;
-        {
-            Scope sc(h, "pair_mtxel");
-            ACK(run_pair(h, v.psi, c.psi, nc, p0, cnt, pp, Mb), "pair kernel");
+        if ((s = pair_rows(h, z, sp, pp, v.psi, c.psi, nc, p0, cnt, Mb))) {
+            cleanup();
+            return s;
         }
         {
             Scope sc(h, "adj_zgemm");
@@ -213,7 +219,12 @@ gw_status gw_chi0_compute_subspace(gw_chi0 *h, int iq, int neig, const double *b
     const int ng = sp.ng;
     if (neig < 1 || neig > ng) return fail(h, GW_ERR_ARG, "need 1 <= neig <= ng");
     const int64_t P = (int64_t)v.nb * h->cond.nb;
-    const int64_t chunk = std::min<int64_t>(h->d.pair_chunk, P);
+    const double2 *Mres = resident_for(h, iq); // kept by the last gw_chi0_compute of this slot
+    ZdPlan z;
+    if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, nw, z)) ||
+                  (z.on && ((s = zd_valence(h, z, sp, v.psi, v.nb)) || (s = zd_conduction(h, z, h->cond.psi, 0, h->cond.nb))))))
+        return s;
+    const int64_t chunk = z.on ? (int64_t)z.vb * z.cb : std::min<int64_t>(h->d.pair_chunk, P);
     CK(h, cudaMemsetAsync(chi_sub, 0, sizeof(double2) * (size_t)nw * neig * neig, h->st), "zero chi");
     if ((s = ensure_work(h, (size_t)chunk * ng, (size_t)chunk * nw)) ||
         (s = grow(h, (void **)&h->MBbuf, &h->MBcap, sizeof(double2) * (size_t)chunk * neig, "projected M")))
@@ -221,14 +232,10 @@ gw_status gw_chi0_compute_subspace(gw_chi0 *h, int iq, int neig, const double *b
     const bool split = h->d.prec == GW_PREC_OZAKI_BF16;
     if (split && (s = oz_prepare_b(h, (const double2 *)basis, ng, neig))) return s;
     gw::PairPlan pp = pair_plan(h, sp);
-    const double2 *Mres = resident_for(h, iq); // kept by the last gw_chi0_compute of this slot
     for (int64_t p0 = 0; p0 < P; p0 += chunk) {
         const int64_t cnt = std::min(chunk, P - p0);
         const double2 *Mc = Mres ? Mres + p0 * ng : h->Mbuf;
-        if (!Mres) {
-            Scope sc(h, "pair_mtxel");
-            CK(h, run_pair(h, v.psi, h->cond.psi, h->cond.nb, p0, cnt, pp, h->Mbuf), "pair kernel");
-        }
+        if (!Mres && (s = pair_rows(h, z, sp, pp, v.psi, h->cond.psi, h->cond.nb, p0, cnt, h->Mbuf))) return s;
         {
             Scope sc(h, "subspace_projection");
             if (split) {
@@ -332,20 +339,21 @@ gw_status gw_chi0_compute_real(gw_chi0 *h, int iq, int nw, const double *omega, 
     const int ng = sp.ng;
     const int64_t nn = (int64_t)ng * ng;
     const int64_t P = (int64_t)v.nb * h->cond.nb;
-    const int64_t chunk = std::min<int64_t>(h->d.pair_chunk, P);
+    const double2 *Mres = resident_for(h, iq); // kept by the last gw_chi0_compute of this slot
+    ZdPlan z;
+    if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, 3 * nw, z)) ||
+                  (z.on && ((s = zd_valence(h, z, sp, v.psi, v.nb)) || (s = zd_conduction(h, z, h->cond.psi, 0, h->cond.nb))))))
+        return s;
+    const int64_t chunk = z.on ? (int64_t)z.vb * z.cb : std::min<int64_t>(h->d.pair_chunk, P);
     if ((s = grow(h, (void **)&h->realbuf, &h->realcap, sizeof(double2) * 3 * nw * nn, "real-axis parts")) ||
         (s = ensure_work(h, (size_t)chunk * ng, (size_t)chunk * 3 * nw)))
         return s;
     CK(h, cudaMemsetAsync(h->realbuf, 0, sizeof(double2) * 3 * nw * nn, h->st), "zero parts");
     gw::PairPlan pp = pair_plan(h, sp);
-    const double2 *Mres = resident_for(h, iq); // kept by the last gw_chi0_compute of this slot
     for (int64_t p0 = 0; p0 < P; p0 += chunk) {
         const int64_t cnt = std::min(chunk, P - p0);
         const double2 *Mc = Mres ? Mres + p0 * ng : h->Mbuf;
-        if (!Mres) {
-            Scope sc(h, "pair_mtxel");
-            CK(h, run_pair(h, v.psi, h->cond.psi, h->cond.nb, p0, cnt, pp, h->Mbuf), "pair kernel");
-        }
+        if (!Mres && (s = pair_rows(h, z, sp, pp, v.psi, h->cond.psi, h->cond.nb, p0, cnt, h->Mbuf))) return s;
         {
             Scope sc(h, "delta");
             CK(h, gw::launch_delta_real(v.energy, h->cond.energy, h->cond.nb, p0, cnt, om, eta, h->dbuf, h->st),
@@ -398,7 +406,9 @@ gw_status gw_chi0_jvp(gw_chi0 *h, int iq, int nw, const double *omega, const dou
     const int ng = sp.ng, nc = c.nb;
     const int64_t nn = (int64_t)ng * ng;
     const int64_t P = (int64_t)v.nb * nc;
-    const int64_t chunk = std::min<int64_t>(h->d.pair_chunk, P);
+    ZdPlan z; // side 0: the stored bands, side 1: the tangents
+    if ((s = zd_plan(h, sp, v.nb, nc, true, false, 2, 2 * nw, z))) return s;
+    const int64_t chunk = z.on ? (int64_t)z.vb * z.cb : std::min<int64_t>(h->d.pair_chunk, P);
     // work held only for this call
     void *gv = nullptr, *gc = nullptr;
     double2 *X1 = nullptr, *X2 = nullptr, *T = nullptr;
@@ -419,7 +429,9 @@ gw_status gw_chi0_jvp(gw_chi0 *h, int iq, int nw, const double *omega, const dou
         (s = dalloc(h, (void **)&X1, szx, "tangent pairs")) || (s = dalloc(h, (void **)&X2, szx, "tangent pairs")) ||
         (s = dalloc(h, (void **)&T, szt, "tangent parts")) || (s = dalloc(h, (void **)&wb, szw, "tangent weights")) ||
         (s = ensure_work(h, (size_t)chunk * ng, (size_t)chunk * 2 * nw)) || (s = band_grids(h, v, dcoeff_v, gv)) ||
-        (s = band_grids(h, c, dcoeff_c, gc))) {
+        (s = band_grids(h, c, dcoeff_c, gc)) ||
+        (z.on && ((s = zd_valence(h, z, sp, v.psi, v.nb, 0)) || (s = zd_valence(h, z, sp, gv, v.nb, 1)) ||
+                  (s = zd_conduction(h, z, c.psi, 0, nc, 0)) || (s = zd_conduction(h, z, gc, 0, nc, 1))))) {
         cleanup();
         return s;
     }
@@ -439,11 +451,14 @@ gw_status gw_chi0_jvp(gw_chi0 *h, int iq, int nw, const double *omega, const dou
     for (int64_t p0 = 0; p0 < P; p0 += chunk) {
         const int64_t cnt = std::min(chunk, P - p0);
         const double2 *Mc = Mres ? Mres + p0 * ng : h->Mbuf;
+        if ((!Mres && (s = pair_rows(h, z, sp, pp, v.psi, c.psi, nc, p0, cnt, h->Mbuf))) ||
+            (s = pair_rows(h, z, sp, pp, gv, c.psi, nc, p0, cnt, X1, 1, 0)) ||
+            (s = pair_rows(h, z, sp, pp, v.psi, gc, nc, p0, cnt, X2, 0, 1))) {
+            cleanup();
+            return s;
+        }
         {
-            Scope sc(h, "pair_mtxel");
-            if (!Mres) JCK(run_pair(h, v.psi, c.psi, nc, p0, cnt, pp, h->Mbuf), "pair kernel");
-            JCK(run_pair(h, gv, c.psi, nc, p0, cnt, pp, X1), "pair kernel (tangent valence)");
-            JCK(run_pair(h, v.psi, gc, nc, p0, cnt, pp, X2), "pair kernel (tangent conduction)");
+            Scope sc(h, "jvp_mix");
             JCK(gw::launch_jvp_mix(Mc, X1, X2, cnt * ng, h->st), "M +- dM");
         }
         {

@@ -158,12 +158,15 @@ struct gw_chi0 {
         void *p = nullptr;
         size_t cap = 0;
     } gpp[9];
-    // stage (a) with the last-axis transform on the tensor cores (zdft.cu): valence slices of the
-    // slot being computed and the transform output F of one chunk
-    void *zdA = nullptr;
-    size_t zdAcap = 0;  // bytes
+    // stage (a) with the last-axis transform on the tensor cores (zdft.cu): row slices of a conduction
+    // block and column exponents of the valence bands (two of each: the forward derivative has
+    // tangent grids too), and the transform output F of a sub-block
+    void *zdA[2] = {nullptr, nullptr};
+    size_t zdAcap[2] = {0, 0}; // bytes
+    int *zdE[2] = {nullptr, nullptr};
+    size_t zdEcap[2] = {0, 0}; // bytes
     float4 *zdF = nullptr;
-    size_t zdFcap = 0;  // bytes
+    size_t zdFcap = 0;         // bytes
     // scratch slots of the two-float pair kernel (sized in set_gsphere, outside any capture)
     float4 *pscr = nullptr;
     size_t pscr_cap = 0; // bytes
@@ -261,12 +264,26 @@ gw_status compute_overlap(gw_chi0 *h, int iq, const gw::OmegaList &om, double2 *
 // Stage (a) with the last-axis transform on the tensor cores: whether slot iq takes it, the
 // conduction bands per chunk, the valence slices (once per call), and one chunk's pair
 // elements M[cl nv + v] for the conduction bands c0 .. c0 + cb - 1.
-bool zd_route(gw_chi0 *h, int iq, bool resident);
-gw_status ensure_overlap_stream(gw_chi0 *h);
-int zd_chunk_bands(gw_chi0 *h, int iq);
-gw_status zd_prepare(gw_chi0 *h, int iq, CUtensorMap *tmA, CUtensorMap *tmC);
-gw_status zd_stage_a(gw_chi0 *h, int iq, const CUtensorMap &tmA, const CUtensorMap &tmC, int c0, int cb,
-                     const gw::PairPlan &pp, double2 *M);
+// Stage (a) on the tensor cores for one call.  zd_plan: blocks of vb x cb pairs (rows: cb = nc, whole
+// valence rows in pair order) and the buffers for `sides` sets of bands; on = false when the route
+// does not take the sphere, would be slower (unless forced) or lacks memory.  zd_valence /
+// zd_conduction prepare a side's bands; zd_block forms M[(v - v0) sv + c sc] of a block.
+struct ZdPlan {
+    bool on = false;
+    int n = 0, vb = 0, cb = 0, vs = 0;          // vs: valence bands per sub-block
+    size_t abytes = 0, ebytes = 0, fper = 0;    // row slices, exponents, F of one valence band
+    int nv[2] = {0, 0};
+    CUtensorMap tmV[2];
+};
+gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw,
+                  ZdPlan &z);
+bool zd_holds(const gw_chi0 *h, const ZdPlan &z); // side 0 and F as planned (a later plan may have lost them)
+gw_status zd_valence(gw_chi0 *h, ZdPlan &z, const Sphere &sp, const void *psiv, int nv, int side = 0);
+gw_status zd_conduction(gw_chi0 *h, const ZdPlan &z, const void *psic, int c0, int cb, int side = 0);
+gw_status zd_block(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::PairPlan &pp, int vside, int cside, int v0,
+                   int vb, int cb, double2 *M, int64_t sv, int64_t sc);
+gw_status pair_rows(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::PairPlan &pp, const void *psiv,
+                    const void *psic, int nc, int64_t p0, int64_t cnt, double2 *M, int vside = 0, int cside = 0);
 bool overlap_enabled(gw_chi0 *h, const gw::PairPlan &pp);
 
 // batched path (api_batch.cu)

@@ -58,26 +58,27 @@ cudaError_t launch_band_setup_tf(const double2 *coeff, const int32_t *gofs, int 
 // ---- stage (a) last-axis transform on the tensor cores (zdft.cu) and the rest of the pair
 // transform from its output (pair_tf_ct.cuh)
 constexpr int kZdSlices = 6; // BF16 slices per operand (balanced base-256 digits)
-// valence slices A[kZdSlices][n^2 lines][nv][2n] (BF16) of two-float band grids psiv [nv][n^3]
-cudaError_t launch_zd_aslices(const void *psiv, int nv, int n, uint16_t *A, cudaStream_t st);
-bool zd_supported(int n, int K2, int nv);
-int zd_conduction_per_tile(int K2);
+// row slices of nr two-float band grids psi [nr][n^3], zd_row_bytes(nr, n) bytes: images of the
+// product's shared-memory tiles, [n^2 lines][row tiles of 128][2 n / 16 stages][kZdSlices]
+cudaError_t launch_zd_rows(const void *psi, int nr, int n, void *A, cudaStream_t st);
+size_t zd_row_bytes(int nr, int n);
+// column exponents E[nb][n^2 lines] of two-float band grids psi [nb][n^3]
+cudaError_t launch_zd_colexp(const void *psi, int nb, int n, int *E, cudaStream_t st);
+bool zd_supported(int n, int K2);
+int zd_valence_per_tile(int K2);
+int zd_row_entries(int K2); // entries of F per (line, row): K2 rounded up to even
 size_t zd_smem_bytes(int n, int K2);
-// F[l][cl nv + v][q] (two-float) = sum_i2 conj(psi_v[l][i2]) W^{kz[q] i2} psi_c[l][i2] for the
-// conduction bands c = c0 + cl, cl < cb; tmA maps the valence slices (box {32, 128, 1, 6},
-// 64-byte swizzle)
-// tmC maps the conduction grids as FP32 [nc][n^2 lines][4n], box {4n, 1, zd_conduction_per_tile(K2)}
-cudaError_t launch_zd_gemm(const CUtensorMap &tmA, const CUtensorMap &tmC, const void *psic, const int *kz,
-                           const float4 *twf, int n, int nv, int c0, int cb, int K2, float4 *F, int *status,
-                           cudaStream_t st);
-// M[r][g] of the chunk's R pairs from F (middle and first axis of the pair transform)
-// (tmF: F as [N^2 lines][R K2] two-float entries, FP32 elements, box {4 K2, 2 N}; tmS: the plan's
+// F[l][vl cb + cl][q] (two-float, zd_row_entries(K2) entries a row) = sum_i2 conj(psi_v[l][i2]) W^{kz[q] i2} psi_c[l][i2] for the
+// valence bands v = v0 + vl, vl < vb, and the cb conduction bands whose row slices A holds; tmV
+// maps the valence grids as FP32 [nv][n^2 lines][4n], box {4n, 1, zd_valence_per_tile(K2)}
+cudaError_t launch_zd_gemm(const CUtensorMap &tmV, const void *A, const int *E, const int *kz, const float4 *twf, int n,
+                           int nv, int v0, int vb, int cb, int K2, float4 *F, int *status, cudaStream_t st);
+// M[(vl sv + cl sc) ng + g] of the block's R pairs, row vl cb + cl, from F (middle and first axis of
+// the pair transform)
+// (tmF: F as [N^2 lines][R rows of zd_row_entries(K2)] two-float entries, FP32 elements, box {4 K2, 2 N}; tmS: the plan's
 // scratch slots as [nslots N rows][K12] two-float entries, box {8 K2, N}; no swizzle)
-cudaError_t launch_pair_tf_from_f(const CUtensorMap &tmF, const CUtensorMap &tmS, int64_t R, const PairPlan &pp,
-                                  double2 *M, cudaStream_t st);
-// delta[w][cl nv + v] = 4x/(x^2 + w^2), x = ev[v] - ec[c0 + cl], the row order of the chunks above
-cudaError_t launch_delta_block(const double *ev, const double *ec, int nv, int c0, int cb, const OmegaList &om,
-                               double *delta, cudaStream_t st);
+cudaError_t launch_pair_tf_from_f(const CUtensorMap &tmF, const CUtensorMap &tmS, int64_t R, int cb, int64_t sv,
+                                  int64_t sc, const PairPlan &pp, double2 *M, cudaStream_t st);
 
 // ---- energy factor, diagonal, symmetrisation (reduce.cu)
 // delta[w][p - p0] = 4x/(x^2 + w^2), x = ev[v] - ec[c]

@@ -392,16 +392,20 @@ size_t pair_tf_ct_smem_bytes(const PairPlan &pp)
     }
 }
 
-cudaError_t launch_pair_tf_from_f(const CUtensorMap &tmF, const CUtensorMap &tmS, int64_t R, const PairPlan &pp,
-                                  double2 *M, cudaStream_t st)
+cudaError_t launch_pair_tf_from_f(const CUtensorMap &tmF, const CUtensorMap &tmS, int64_t R, int cb, int64_t sv,
+                                  int64_t sc, const PairPlan &pp, double2 *M, cudaStream_t st)
 {
     if (R == 0) return cudaSuccess;
-    if (pp.n[0] != 48 || pp.n[1] != 48 || pp.n[2] != 48 || !pp.scr || !pp.slot_flags || pp.nslots <= 0)
-        return cudaErrorInvalidValue;
-    const double invd = 1.0 / ((double)pp.n[0] * pp.n[1] * pp.n[2]);
+    const int n = pp.n[0];
+    if (pp.n[1] != n || pp.n[2] != n || !pp.scr || !pp.slot_flags || pp.nslots <= 0) return cudaErrorInvalidValue;
+    const double invd = 1.0 / ((double)n * n * n);
     const float invh = (float)invd;
     const tf inv{invh, (float)(invd - (double)invh)};
-    return launch_pair_tf_from_f_g48(tmF, tmS, R, pp, tf_consts(), inv, M, st);
+    switch (n) {
+    case 40: return launch_pair_tf_from_f_g40(tmF, tmS, R, cb, sv, sc, pp, tf_consts(), inv, M, st);
+    case 48: return launch_pair_tf_from_f_g48(tmF, tmS, R, cb, sv, sc, pp, tf_consts(), inv, M, st);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t pair_tf_scratch(const PairPlan &pp, int *nslots, size_t *slot_elems)

@@ -359,17 +359,16 @@ __device__ __forceinline__ void tma2_hint(void *dst, const CUtensorMap *m, uint6
                  : "memory");
 }
 
-// First stage (lazy radix 4, no twiddles: make_prune_plan(N)'s stage 0) of nlines lines stored
+// First stage (lazy, no twiddles: make_prune_plan(N)'s stage 0) of nlines lines stored
 // row-major as a TMA box leaves them: line l = sl half + q (sl = 0 or 1) has its point k at
 // x[(sl N + k) es + q].  The slab pair's F rows: half = K2, es = K2; a phase-2 batch of cells:
 // half = nlines, es = the box width.  Output in the column layout y[l CS + k]; lines fastest
 // over the threads (lm).
 template <int N>
 __device__ __forceinline__ void tstage0_rows(const float4 *__restrict__ x, float4 *__restrict__ y, int half, int es,
-                                             int nlines, int CS, LMap lm)
+                                             int nlines, int CS, LMap lm, const TfConsts &k)
 {
     constexpr int R = make_prune_plan(N).r[0], nb = N / R;
-    static_assert(R == 4, "the first stage is radix 4");
     int l = lm.l0, j = lm.j0;
     while (j < nb) {
         const int sl = l >= half ? 1 : 0;
@@ -377,7 +376,7 @@ __device__ __forceinline__ void tstage0_rows(const float4 *__restrict__ x, float
         tcx v[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = tc_load(xl + (j + r * nb) * es);
-        tdft4<false>(v);
+        tdft_lazy<R>(v, k);
         float4 *yl = y + l * CS + j * R;
 #pragma unroll
         for (int r = 0; r < R; ++r) tc_store(yl + r, v[r]);
@@ -395,8 +394,8 @@ __host__ __device__ constexpr int from_f_buf(int ncols, int cs) { return (ncols 
 
 template <int N>
 __global__ void __launch_bounds__(pair_threads<N>(), pair_min_blocks<N>())
-    pair_kernel_tf_from_f(const __grid_constant__ CUtensorMap tmF, const __grid_constant__ CUtensorMap tmS, int64_t R,
-                          PairPlan pp, TfConsts kc, tf inv_nr, double2 *__restrict__ M)
+    pair_kernel_tf_from_f(const __grid_constant__ CUtensorMap tmF, const __grid_constant__ CUtensorMap tmS, int cb,
+                          int64_t sv, int64_t sc, PairPlan pp, TfConsts kc, tf inv_nr, double2 *__restrict__ M)
 {
     static_assert(N % 2 == 0, "slabs go in pairs");
     static_assert(make_prune_plan(N).nst == 3, "two full i1 stages: the result returns to the input buffer");
@@ -443,7 +442,7 @@ __global__ void __launch_bounds__(pair_threads<N>(), pair_min_blocks<N>())
         if (threadIdx.x == 0) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             bar_expect(&fbar, fbytes);
-            tma2_hint(C, &tmF, &fbar, (int)(row * K2 * 4), i0 * N, stream);
+            tma2_hint(C, &tmF, &fbar, (int)(row * ((K2 + 1) / 2 * 2) * 4), i0 * N, stream);
         }
     };
     const LMap lm = lmap_lines_fastest(ncols);
@@ -456,7 +455,7 @@ __global__ void __launch_bounds__(pair_threads<N>(), pair_min_blocks<N>())
             if (threadIdx.x == 0) atomicOr(pp.status, kStatusTimeout);
             return;
         }
-        tstage0_rows<N>(X, Y, K2, K2, ncols, CS, lm);
+        tstage0_rows<N>(X, Y, K2, K2, ncols, CS, lm, kc);
         __syncthreads();
         const float4 *y1 = tstages_ct<N, 1, make_prune_plan(N).r[0], true, true>(Y, X, ncols, CS, tw, kc, 1, -1, lm);
         // y1 = X, after a barrier: Y is free
@@ -487,7 +486,8 @@ __global__ void __launch_bounds__(pair_threads<N>(), pair_min_blocks<N>())
             tma2_hint(C, &tmS, &fbar, d0 * 4, slot * N, stream);
         }
     };
-    double2 *out = M + row * pp.ng;
+    const int64_t vl = row / cb;
+    double2 *out = M + (vl * sv + (row - vl * cb) * sc) * pp.ng;
     fetch_cells(0, Xb);
     for (int d0 = 0, b = 0; d0 < K12; d0 += NB, b ^= 1, ++nf) {
         float4 *X = Xb + b * BUF, *Y = Xb + (b ^ 1) * BUF;
@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(pair_threads<N>(), pair_min_blocks<N>())
             return;
         }
         const LMap lm2 = lmap_lines_fastest(nbat);
-        tstage0_rows<N>(X, Y, nbat, NB, nbat, CS, lm2);
+        tstage0_rows<N>(X, Y, nbat, NB, nbat, CS, lm2, kc);
         __syncthreads();
         const float4 *y0 = tstages_ct<N, 1, make_prune_plan(N).r[0], true, true>(Y, X, nbat, CS, tw, kc, 1, -1, lm2);
         // y0 = X, after a barrier: Y is free
@@ -526,8 +526,8 @@ inline size_t pair_tf_from_f_smem(const PairPlan &pp)
 }
 
 template <int N>
-inline cudaError_t launch_pair_tf_from_f_cube(const CUtensorMap &tmF, const CUtensorMap &tmS, int64_t R,
-                                              const PairPlan &pp, const TfConsts &kc, tf inv_nr, double2 *M,
+inline cudaError_t launch_pair_tf_from_f_cube(const CUtensorMap &tmF, const CUtensorMap &tmS, int64_t R, int cb,
+                                              int64_t sv, int64_t sc, const PairPlan &pp, const TfConsts &kc, tf inv_nr, double2 *M,
                                               cudaStream_t st)
 {
     const size_t sm = pair_tf_from_f_smem<N>(pp);
@@ -535,7 +535,7 @@ inline cudaError_t launch_pair_tf_from_f_cube(const CUtensorMap &tmF, const CUte
         cudaFuncSetAttribute(pair_kernel_tf_from_f<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(pp.slot_flags, 0, sizeof(int) * pp.nslots, st)) != cudaSuccess) return e;
-    pair_kernel_tf_from_f<N><<<(unsigned)R, pair_threads<N>(), sm, st>>>(tmF, tmS, R, pp, kc, inv_nr, M);
+    pair_kernel_tf_from_f<N><<<(unsigned)R, pair_threads<N>(), sm, st>>>(tmF, tmS, cb, sv, sc, pp, kc, inv_nr, M);
     return cudaGetLastError();
 }
 
@@ -552,7 +552,7 @@ inline cudaError_t pair_tf_cube_slots(const PairPlan &pp, int *nslots)
         (e = cudaGetDevice(&dev)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return e;
-    if constexpr (N == 48) { // the pool also serves the kernel that starts from the tensor-core output
+    if constexpr (N == 40 || N == 48) { // the pool also serves the kernel that starts from the tensor-core output
         const size_t sm2 = pair_tf_from_f_smem<N>(pp);
         int occ2 = 0;
         if ((e = cudaFuncSetAttribute(pair_kernel_tf_from_f<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -646,7 +646,9 @@ cudaError_t pair_tf_slots_g48(const PairPlan &, int *);
 cudaError_t launch_pair_tf_g72(const float4 *, const float4 *, int, int64_t, int64_t, const PairPlan &,
                                const TfConsts &, tf, double2 *, cudaStream_t);
 cudaError_t pair_tf_slots_g72(const PairPlan &, int *);
-cudaError_t launch_pair_tf_from_f_g48(const CUtensorMap &, const CUtensorMap &, int64_t, const PairPlan &,
-                                      const TfConsts &, tf, double2 *, cudaStream_t);
+cudaError_t launch_pair_tf_from_f_g40(const CUtensorMap &, const CUtensorMap &, int64_t, int, int64_t, int64_t,
+                                      const PairPlan &, const TfConsts &, tf, double2 *, cudaStream_t);
+cudaError_t launch_pair_tf_from_f_g48(const CUtensorMap &, const CUtensorMap &, int64_t, int, int64_t, int64_t,
+                                      const PairPlan &, const TfConsts &, tf, double2 *, cudaStream_t);
 
 } // namespace gw

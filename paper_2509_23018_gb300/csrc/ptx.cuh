@@ -153,4 +153,23 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t base, uint32_t ncols)
                    "=r"(v[29]), "=r"(v[30]), "=r"(v[31])                                                           \
                  : "r"(taddr))
 
+// 16 lanes x 64 (x8) or 32 (x4) columns: lane l holds, per 8 columns j, columns 8 j + 2 (l % 4) + {0, 1} of
+// TMEM lane l / 4 in registers 4 j, 4 j + 1 and of TMEM lane l / 4 + 8 in 4 j + 2, 4 j + 3
+#define GW_TMEM_LD_16X256_X8(taddr, v) \
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15," \
+                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];" \
+                 : "=r"((v)[0]), "=r"((v)[1]), "=r"((v)[2]), "=r"((v)[3]), "=r"((v)[4]), "=r"((v)[5]), \
+                   "=r"((v)[6]), "=r"((v)[7]), "=r"((v)[8]), "=r"((v)[9]), "=r"((v)[10]), "=r"((v)[11]), \
+                   "=r"((v)[12]), "=r"((v)[13]), "=r"((v)[14]), "=r"((v)[15]), "=r"((v)[16]), \
+                   "=r"((v)[17]), "=r"((v)[18]), "=r"((v)[19]), "=r"((v)[20]), "=r"((v)[21]), \
+                   "=r"((v)[22]), "=r"((v)[23]), "=r"((v)[24]), "=r"((v)[25]), "=r"((v)[26]), \
+                   "=r"((v)[27]), "=r"((v)[28]), "=r"((v)[29]), "=r"((v)[30]), "=r"((v)[31]) \
+                 : "r"(taddr))
+#define GW_TMEM_LD_16X256_X4(taddr, v) \
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];" \
+                 : "=r"((v)[0]), "=r"((v)[1]), "=r"((v)[2]), "=r"((v)[3]), "=r"((v)[4]), "=r"((v)[5]), \
+                   "=r"((v)[6]), "=r"((v)[7]), "=r"((v)[8]), "=r"((v)[9]), "=r"((v)[10]), "=r"((v)[11]), \
+                   "=r"((v)[12]), "=r"((v)[13]), "=r"((v)[14]), "=r"((v)[15]) \
+                 : "r"(taddr))
+
 } // namespace gw

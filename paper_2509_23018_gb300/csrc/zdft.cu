@@ -4,8 +4,8 @@
 // product along the last axis at the kept frequencies kz[q] is
 //     F[v][c][l][q] = sum_{i2} conj(psi_v[l][i2]) W_q[i2] psi_c[l][i2],   W_q[i2] = e^{+2 pi i kz[q] i2 / N},
 // the first stage of the forward transform of the product (the definition after Eq. ff-ch).
-// Over the pairs of a chunk it is, line by line, a complex matrix product whose operands
-// belong to one band each: rows conj(psi_v[l]) (valence), columns W_q psi_c[l] (conduction).
+// Over the pairs of a block it is, line by line, a complex matrix product whose operands
+// belong to one band each: rows psi_c[l] (conduction), columns W_q conj(psi_v[l]) (valence).
 // Written in real form (K = 2 N: Re and Im of each point interleaved), it runs as an
 // Ozaki-style split product (the scheme of stage (b)):
 //   * each operand row / column is scaled by its own power of two 2^E (|x| < 2^E) and cut into
@@ -19,8 +19,9 @@
 //     lies 2^-48 below the leading group);
 //   * the four accumulators are summed in two-float arithmetic (two-sums for the exact groups)
 //     into F, which the pair kernel's remaining stages (middle and first axis) take from there.
-// The valence slices are formed once per call (band setup); the conduction columns are formed
-// per tile on the chip, from psi_c and the twiddles, by producer warps.
+// The row slices of a block of conduction bands are formed once (zd_rows_kernel), as the images
+// of the shared-memory tiles that the product copies; the valence columns are formed on the chip,
+// from psi_v and the twiddles, by producer warps, once for all the row tiles of a line.
 #include "internal.h"
 #include "ptx.cuh"
 #include "fft_tf.cuh"
@@ -65,14 +66,14 @@ __device__ __forceinline__ void zd_digits(float h, float l, int E, uint16_t out[
     }
 }
 
-// The same digits with the line's scale sc = 2^(47 - E) and the slice weights w[i] = 2^(E - 7 - 8i)
-// precomputed (-70 <= E <= 60, so that both stay normal FP32 numbers).
-__device__ __forceinline__ void zd_digits_w(float h, float l, float sc, const float w[kZdSlices],
-                                            uint16_t out[kZdSlices])
+// The same digits where the line's scale 2^(47 - E) and every weight are normal FP32 numbers
+// (-70 <= E <= 120).
+__device__ __forceinline__ void zd_digits_n(float h, float l, int E, uint16_t out[kZdSlices])
 {
-    const float Y = __fmul_rn(h, sc), L = __fmul_rn(l, sc);
+    const float sc = __int_as_float((127 + 47 - E) << 23);
+    const float Y = __fmul_rn(h, sc);
     const float T = rintf(__fmul_rn(Y, 0x1p-24f));
-    float U = __fadd_rn(rintf(__fmaf_rn(-0x1p24f, T, Y)), rintf(L));
+    float U = __fadd_rn(rintf(__fmaf_rn(-0x1p24f, T, Y)), rintf(__fmul_rn(l, sc)));
     float d[kZdSlices];
 #pragma unroll
     for (int i = kZdSlices - 1; i >= 3; --i) {
@@ -88,8 +89,10 @@ __device__ __forceinline__ void zd_digits_w(float h, float l, float sc, const fl
         V = q;
     }
     d[0] = V;
+    const int w0 = (127 + E - 7) << 23;
 #pragma unroll
-    for (int i = 0; i < kZdSlices; ++i) out[i] = (uint16_t)(__float_as_uint(__fmul_rn(d[i], w[i])) >> 16);
+    for (int i = 0; i < kZdSlices; ++i)
+        out[i] = (uint16_t)(__float_as_uint(__fmul_rn(d[i], __int_as_float(w0 - i * (8 << 23)))) >> 16);
 }
 
 // exponent E with |x| < 2^E for a line's largest component magnitude m (E = -126 for m = 0)
@@ -100,88 +103,19 @@ __device__ __forceinline__ int zd_expo(float m)
     return (be == 0 ? -126 : be - 127) + 1;
 }
 
-// ------------------------------------------------------------------ valence slices
-// A[i][l][v][k] (BF16, k = 2 i2 + {Re, Im}) of the rows psi_v[l][.]: one warp per (v, l).
-__global__ void __launch_bounds__(256) zd_aslices_kernel(const float4 *__restrict__ psi, int nv, int n, int nlines,
-                                                         uint16_t *__restrict__ A)
-{
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= nv * nlines) return;
-    const int v = warp % nv, l = warp / nv;
-    const float4 *row = psi + ((int64_t)v * nlines + l) * n;
-    float m = 0.0f;
-    for (int i = lane; i < n; i += 32) {
-        const float4 x = row[i];
-        m = fmaxf(m, fmaxf(fabsf(x.x), fabsf(x.z)) * (1.0f + 0x1p-20f));
-    }
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    const int E = zd_expo(m);
-    const int64_t plane = (int64_t)nlines * nv * 2 * n;
-    uint16_t *dst = A + ((int64_t)l * nv + v) * 2 * n;
-    for (int i = lane; i < n; i += 32) {
-        const float4 x = row[i];
-        uint16_t dr[kZdSlices], di[kZdSlices];
-        zd_digits(x.x, x.y, E, dr);
-        zd_digits(x.z, x.w, E, di);
-#pragma unroll
-        for (int s = 0; s < kZdSlices; ++s)
-            *(uint32_t *)(dst + s * plane + 2 * i) = (uint32_t)dr[s] | ((uint32_t)di[s] << 16);
-    }
-}
-
-cudaError_t launch_zd_aslices(const void *psiv, int nv, int n, uint16_t *A, cudaStream_t st)
-{
-    const int nlines = n * n;
-    const int64_t warps = (int64_t)nv * nlines;
-    zd_aslices_kernel<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>((const float4 *)psiv, nv, n, nlines, A);
-    return cudaGetLastError();
-}
-
-__host__ __device__ __forceinline__ int zd_conduction_per_tile_d(int K2)
-{
-    const int ct = 128 / (2 * K2);
-    return ct < 4 ? ct : 4;
-}
-
-// ------------------------------------------------------------------ the product
-// One block per SM, persistent over units u = (line l, row tile mt); per unit the block keeps
-// the valence slices of its 128 rows resident (three K-chunks of 32 real entries, TMA) and
-// runs over the conduction tiles ct of the chunk (CT bands, 2 K2 real columns each, padded to
-// 128 columns): producer warps form the tile's column slices in stages of 16 real entries into a
-// 2-deep ring, one thread issues the tcgen05 products into four accumulators of 128 TMEM columns
-// each, and the epilogue warps sum the accumulators into F.  A 128 x N x 16 product costs about
-// the same time at N = 64 as at N = 128 (the probe's 128 x 64 rate is 2/3 of its 128 x 128 rate:
-// feeding the 128 x 16 A operand sets the pace, whether A is read from shared memory or from TMEM),
-// so the tile is 128 columns wide; its four accumulators then fill the 512 TMEM columns and are
-// not double-buffered.  The epilogue hands them back as soon as its last TMEM loads have landed,
-// before that chunk's arithmetic and stores.  (64-column tiles with two accumulator buffers took
-// 2.40 against 2.30 ms per 48^3 chunk; eight epilogue warps of 16-column chunks 2.36 ms; a Re/Im
-// column order without the producers' shared-memory store conflicts 2.34 ms.)
-//  warp 0: TMA; warp 1: MMA (and TMEM); warps 2..5: epilogue (TMEM lane quadrant warp % 4);
-//  warps 6..11: producers.
+// ------------------------------------------------------------------ operand tiles in shared memory
 constexpr int kZdN = 128;                              // columns per tile
-constexpr int kZdKC = 32;                              // real K entries per valence K-chunk
-constexpr int kZdKB = 16;                              // real K entries per column stage
-constexpr int kZdStages = 6;                           // column stages per tile (K = 96)
-constexpr int kZdThreads = 384;
-constexpr int kZdProducers = 6;                        // producer warps
-constexpr unsigned kZdASlice = 128 * kZdKC * 2;        // one slice of one K-chunk: 8 KB
-constexpr unsigned kZdAChunk = kZdSlices * kZdASlice;  // 48 KB
-constexpr unsigned kZdBSlice = kZdN * kZdKB * 2;       // 4 KB
-constexpr unsigned kZdBStage = kZdSlices * kZdBSlice;  // 24 KB
+constexpr int kZdM = 128;                              // rows per tile
+constexpr int kZdKB = 16;                              // real K entries per stage (8 points)
+constexpr int kZdMaxStages = 6;                        // stages per tile, 2 N / 16: N <= 48
+constexpr unsigned kZdSlice = kZdN * kZdKB * 2;        // one slice of one stage: 4 KB
+constexpr unsigned kZdStage = kZdSlices * kZdSlice;    // 24 KB
 // idesc: D = F32, A = B = BF16, both K-major, N = 128, M = 128
 constexpr uint32_t kZdIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kZdN >> 3) << 17) |
-                              ((uint32_t)(128 >> 4) << 24);
+                              ((uint32_t)(kZdM >> 4) << 24);
 
-// K-major operand tiles.  Valence slices (written by TMA), 64-byte swizzling: row r of 64 bytes
-// (32 BF16), 8-row atoms of 512 bytes, 16-byte chunk j of row r stored at chunk j ^ ((r % 8) >> 1).
-// Column stages (written by the producers), 32-byte swizzling: row r of 32 bytes (16 BF16), 8-row
-// atoms of 256 bytes, chunk j of row r stored at chunk j ^ ((r % 8) >> 2).
-__device__ __forceinline__ uint64_t sdesc_sw64(uint32_t addr)
-{
-    return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
-}
+// K-major operand tiles of both operands, 32-byte swizzling: row r of 32 bytes (16 BF16), 8-row
+// atoms of 256 bytes, 16-byte chunk j of row r stored at chunk j ^ ((r % 8) >> 2).
 __device__ __forceinline__ uint64_t sdesc_sw32(uint32_t addr)
 {
     return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(256 >> 4) << 32) |
@@ -192,11 +126,119 @@ __device__ __forceinline__ uint32_t sw32_off(int r, int k) // byte offset of ele
     return (uint32_t)((r >> 3) * 256 + (r & 7) * 32 + ((((k >> 3) ^ ((r & 7) >> 2)) & 1) << 4) + (k & 7) * 2);
 }
 
-__device__ __forceinline__ void tma4(void *dst, const CUtensorMap *m, uint64_t *b, int x, int y, int z, int w)
+// ------------------------------------------------------------------ row slices
+// A[l][mt][ks][slice] (4 KB images of the swizzled tile of 128 rows x 16 real entries, so that one
+// bulk copy of 24 KB brings a stage) of the rows psi[r][l][.], r < nr, zero above: one warp per row
+// of a line, 8 warps per block.
+__global__ void __launch_bounds__(256) zd_rows_kernel(const float4 *__restrict__ psi, int nr, int n, int nlines,
+                                                      int nmt, unsigned char *__restrict__ A)
 {
-    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-                 "%5}], [%6];" ::"r"(su32(dst)),
-                 "l"(m), "r"(x), "r"(y), "r"(z), "r"(w), "r"(su32(b))
+    const int lane = threadIdx.x & 31, l = blockIdx.y, r = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int nst = n / 8;
+    unsigned char *dst = A + ((int64_t)l * nmt + r / kZdM) * nst * kZdStage;
+    const int rt = r % kZdM;
+    const float4 *row = psi + ((int64_t)min(r, nr - 1) * nlines + l) * n;
+    float m = 0.0f;
+    float4 x[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int i = lane + 32 * u;
+        x[u] = i < n && r < nr ? row[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        m = fmaxf(m, fmaxf(fabsf(x[u].x), fabsf(x[u].z)) * (1.0f + 0x1p-20f));
+    }
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const int E = zd_expo(m);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int i = lane + 32 * u;
+        if (i >= n) break;
+        uint16_t dr[kZdSlices], di[kZdSlices];
+        zd_digits(x[u].x, x[u].y, E, dr);
+        zd_digits(x[u].z, x[u].w, E, di);
+        unsigned char *p = dst + (i >> 3) * kZdStage + sw32_off(rt, 2 * (i & 7));
+#pragma unroll
+        for (int s = 0; s < kZdSlices; ++s) *(uint32_t *)(p + s * kZdSlice) = (uint32_t)dr[s] | ((uint32_t)di[s] << 16);
+    }
+}
+
+// E[band][l]: exponent of a line's columns W_q conj(psi): |W_q psi| <= |Re psi| + |Im psi|
+// (-70 <= E, so that the digits' scale and every weight stay normal FP32 numbers)
+__global__ void __launch_bounds__(256) zd_colexp_kernel(const float4 *__restrict__ psi, int nb, int n, int nlines,
+                                                        int *__restrict__ E)
+{
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (w >= (int64_t)nb * nlines) return;
+    float m = 0.0f;
+    for (int i = lane; i < n; i += 32) {
+        const float4 x = psi[w * n + i];
+        m = fmaxf(m, (fabsf(x.x) + fabsf(x.z)) * (1.0f + 0x1p-20f));
+    }
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) E[w] = min(120, max(-70, zd_expo(m)));
+}
+
+size_t zd_row_bytes(int nr, int n)
+{
+    return (size_t)n * n * ((nr + kZdM - 1) / kZdM) * (n / 8) * kZdStage;
+}
+
+cudaError_t launch_zd_rows(const void *psi, int nr, int n, void *A, cudaStream_t st)
+{
+    const int nmt = (nr + kZdM - 1) / kZdM;
+    zd_rows_kernel<<<dim3(nmt * (kZdM / 8), n * n), 256, 0, st>>>((const float4 *)psi, nr, n, n * n, nmt,
+                                                                  (unsigned char *)A);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_zd_colexp(const void *psi, int nb, int n, int *E, cudaStream_t st)
+{
+    const int64_t warps = (int64_t)nb * n * n;
+    zd_colexp_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>((const float4 *)psi, nb, n, n * n, E);
+    return cudaGetLastError();
+}
+
+// Entries of F per (row, line): the kept frequencies, padded to whole 32-byte sectors.
+int zd_row_entries(int K2) { return (K2 + 1) / 2 * 2; }
+
+int zd_valence_per_tile(int K2) { return std::max(1, std::min(6, kZdN / (2 * zd_row_entries(K2)))); }
+
+// ------------------------------------------------------------------ the product
+// One block per SM, persistent over units u = (line l, valence tile of CT bands); per unit the
+// producer warps form the tile's column slices (CT bands, 2 K2P real columns each, K2 rounded up to
+// even; the others of 128 are zero), all 2 N / 16 stages of 16 real entries resident, and the block
+// runs over the row tiles of 128 conduction bands, whose slices the TMA warp copies stage by stage
+// into a ring.  One
+// thread issues the tcgen05 products into four accumulators of 128 TMEM columns each, and the
+// epilogue warps sum the accumulators into F.  A 128 x N x 16 product costs about the same time at
+// N = 64 as at N = 128 (feeding the 128 x 16 A operand sets the pace, whether A is read from shared
+// memory or from TMEM), so the tile is 128 columns wide; its four accumulators then fill the 512 TMEM
+// columns and are not double-buffered.  Each is handed back on its own as soon as its TMEM
+// loads have landed, least significant first, and a tile's first two stages issue their products in
+// that order: 15 of the 21 belong to the first accumulator handed back.
+// A stage's columns are released by the last row tile's products, so the producers refill them while
+// that tile finishes; the line tiles of the next unit are loaded a unit ahead.
+//
+// What bounds it: shared memory.  A 128 x 128 x 16 product reads 8 KB of operands in its 64 clocks, all
+// that shared memory delivers, so whatever else passes through it (the row stages' copies, the
+// producers' stores, the epilogue's TMEM loads and F's stores) adds to the products' time: 0.95 ms of
+// products in 1.97 ms for a 48^3 block of 8192 pairs (16 x 512 bands, K2 = 15), tensor pipe 46 %.  With
+// the valence bands in the rows (resident) and each tile of conduction columns formed for one row
+// tile it took 2.30 ms; F stored entry by entry, 32 half sectors an instruction, 2.9 ms; exchanged in
+// quads by shuffles 2.25 ms; row stages in a ring of two instead of three 2.4 ms.
+//  warps 0..3: TMA, MMA (and TMEM), two producers; warps 4..11: epilogue (TMEM lane quadrant
+//  warp % 4, half of the columns each); warps 12..15: producers.
+constexpr int kZdThreads = 512;
+constexpr int kZdProducers = 6; // producer warps
+constexpr int kZdPsiSlots = 2;  // ring of valence-band line tiles
+constexpr int kZdMaxRing = 4;   // ring of row stages (2 to 4, what shared memory holds)
+constexpr int kZdRounds = 3;    // (band, frequency) pairs per producer lane: 64 pairs, 6 warps x 4
+
+__device__ __forceinline__ void bulk_copy(void *dst, const void *src, unsigned bytes, uint64_t *b)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     su32(dst)),
+                 "l"(src), "r"(bytes), "r"(su32(b))
                  : "memory");
 }
 __device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -209,86 +251,62 @@ __device__ __forceinline__ float zd_2sum(float a, float b, float &e)
     return s;
 }
 
-constexpr int kZdPsiSlots = 4; // ring of conduction-band line tiles
-
 struct ZdArgs {
-    CUtensorMap tmA;        // A slices [6][lines][nv][2N] bf16, box {32, 128, 1, 6}, 64-byte swizzle
-    CUtensorMap tmC;        // conduction grids as FP32 [nc][lines][4N], box {4N, 1, CT}
+    CUtensorMap tmV;        // valence grids as FP32 [nv][lines][4N], box {4N, 1, CT}
+    const unsigned char *A; // row slices (zd_rows_kernel) of the block's cb conduction bands
+    const int *E;           // [nv][lines] column exponents
     const int *kz;          // [K2] kept last-axis frequencies
-    float4 *F;              // [lines][R][K2] two-float, R = rows of the chunk = nv * cb, r = cl * nv + v
+    float4 *F;              // [lines][vb cb][K2P] two-float, row vl cb + cl
     int *status;
-    int n, nv, c0, cb, K2, CT, nunits, nmt;
-    // work items: units (line, row tile) 0 .. nfull - 1 whole, then each remaining unit split
-    // into nsplit parts by conduction tiles (the last wave of the persistent blocks)
-    int nct, nfull, nsplit, nitems;
+    int n, nv, v0, vb, cb, K2, K2P, CT, nvt, nmt, nunits, ast; // ast: stages of the row ring
 };
-
-// work item -> line l, row tile mt and conduction tiles [ct0, ct1)
-__device__ __forceinline__ void zd_item(const ZdArgs &a, int item, int &l, int &mt, int &ct0, int &ct1)
-{
-    int unit = item, part = 0, np = 1;
-    if (item >= a.nfull) {
-        const int k = item - a.nfull;
-        unit = a.nfull + k / a.nsplit;
-        part = k - (k / a.nsplit) * a.nsplit;
-        np = a.nsplit;
-    }
-    l = unit / a.nmt;
-    mt = unit - l * a.nmt;
-    ct0 = part * a.nct / np;
-    ct1 = (part + 1) * a.nct / np;
-}
 
 __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_constant__ ZdArgs a,
                                                                 const float4 *__restrict__ twf)
 {
     extern __shared__ __align__(1024) unsigned char smraw[];
     unsigned char *sm = (unsigned char *)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
-    unsigned char *sA = sm;                               // 3 K-chunks x 48 KB
-    unsigned char *sB = sA + 3 * kZdAChunk;               // 2 stages x 24 KB
-    float4 *ring = (float4 *)(sB + 2 * kZdBStage);        // [slots][CT][N] conduction line tiles
-    float4 *wt = ring + kZdPsiSlots * a.CT * a.n;         // [K2][N] twiddles W^{kz[q] i2}
-    int2 *ctab = (int2 *)(wt + a.K2 * a.n);               // [64] column pair -> (band, F offset)
+    const int nst = a.n / 8, ncol = 2 * a.K2P;            // stages; real columns per valence band
+    const uint32_t ast = a.ast;
+    unsigned char *sA = sm;                               // ast x 24 KB
+    unsigned char *sB = sA + ast * kZdStage;              // nst x 24 KB
+    float4 *ring = (float4 *)(sB + nst * kZdStage);       // [slots][CT][N] valence line tiles
+    float4 *wt = ring + kZdPsiSlots * a.CT * a.n;         // [N] twiddles W^t
+    int2 *ctab = (int2 *)(wt + a.n);                      // [64] column pair -> (band, F offset)
     uint64_t *bar = (uint64_t *)(ctab + kZdN / 2);
-    uint64_t *aFull = bar, *aEmpty = bar + 1, *bFull = bar + 2, *bEmpty = bar + 4, *tFull = bar + 6,
-             *tEmpty = bar + 8, *fin = bar + 10, *pFull = bar + 11, *pEmpty = pFull + kZdPsiSlots;
-    uint32_t *tslot = (uint32_t *)(pEmpty + kZdPsiSlots);
+    uint64_t *aFull = bar, *aEmpty = aFull + kZdMaxRing, *bFull = aEmpty + kZdMaxRing, *bEmpty = bFull + kZdMaxStages,
+             *tFull = bEmpty + kZdMaxStages, *tEmpty = tFull + 1, *pFull = tEmpty + 4, *pEmpty = pFull + kZdPsiSlots,
+             *fin = pEmpty + kZdPsiSlots;
+    uint32_t *tslot = (uint32_t *)(fin + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = threadIdx.x; i < a.K2 * a.n; i += blockDim.x) {
-        const int q = i / a.n, i2 = i - q * a.n;
-        wt[i] = twf[(a.kz[q] * i2) % a.n];
-    }
-    // the epilogue's column pairs (Re, Im of kept frequency q of band cl of the tile): cl and the
-    // offset cl nv K2 + q of its F entry from the row's first (padding pairs: cl >= CT)
+    for (int i = threadIdx.x; i < a.n; i += blockDim.x) wt[i] = twf[i];
+    // the epilogue's column pairs (Re, Im of entry q of band vl of the tile): vl and the offset
+    // vl cb K2P + q of its F entry from the row's first (padding pairs: vl >= CT)
     for (int pi = threadIdx.x; pi < kZdN / 2; pi += blockDim.x) {
-        const int cl = pi / a.K2, q = pi - cl * a.K2;
-        ctab[pi] = make_int2(cl, cl * a.nv * a.K2 + q);
+        const int vl = pi / a.K2P, q = pi - vl * a.K2P;
+        ctab[pi] = make_int2(vl, vl * a.cb * a.K2P + q);
     }
-    {
-        // the padding columns of both stages stay zero (their products never reach F)
-        const int ncol = 2 * a.K2, npad = kZdN - zd_conduction_per_tile_d(a.K2) * ncol;
-        for (int e = threadIdx.x; e < 2 * kZdSlices * npad * (kZdKB / 2); e += blockDim.x) {
-            const int st = e / (kZdSlices * npad * (kZdKB / 2)), r1 = e % (kZdSlices * npad * (kZdKB / 2));
-            const int sl = r1 / (npad * (kZdKB / 2)), r2 = r1 % (npad * (kZdKB / 2));
-            const int col = kZdN - npad + r2 / (kZdKB / 2), k = 2 * (r2 % (kZdKB / 2));
-            *(uint32_t *)(sB + st * kZdBStage + sl * kZdBSlice + sw32_off(col, k)) = 0u;
-        }
-    }
+    // columns that no frequency fills stay zero in every stage
+    for (int i = threadIdx.x; i < nst * (int)kZdStage / 16; i += blockDim.x)
+        ((uint4 *)sB)[i] = make_uint4(0u, 0u, 0u, 0u);
+    fence_async_shared();
     if (threadIdx.x == 0) {
-        bar_init(aFull, 1);
-        bar_init(aEmpty, 1);
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < kZdMaxRing; ++i) {
+            bar_init(&aFull[i], 1);
+            bar_init(&aEmpty[i], 1);
+        }
+        for (int i = 0; i < kZdMaxStages; ++i) {
             bar_init(&bFull[i], kZdProducers);
             bar_init(&bEmpty[i], 1);
-            bar_init(&tFull[i], 1);
-            bar_init(&tEmpty[i], 128);
         }
-        bar_init(fin, 1);
+        bar_init(tFull, 1);
+        for (int i = 0; i < 4; ++i) bar_init(&tEmpty[i], 8);
         for (int i = 0; i < kZdPsiSlots; ++i) {
             bar_init(&pFull[i], 1);
             bar_init(&pEmpty[i], kZdProducers);
         }
+        bar_init(fin, 1);
         bar_fence_init();
     }
     if (warp == 1) tmem_alloc(tslot, 512);
@@ -296,125 +314,87 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = *tslot;
-    const int ncol = 2 * a.K2;                // real columns per conduction band
     bool ok = true;
 
-    if (warp == 0) {
-        // ---- TMA: the unit's valence slices, once the previous unit's products are done
-        if (lane == 0) {
-            uint32_t u = 0, tile = 0;
-            const unsigned pbytes = (unsigned)a.CT * a.n * 16; // CT lines of N two-float points
-            for (int item = blockIdx.x; item < a.nitems && ok; item += gridDim.x, ++u) {
-                int l, mt, ct0, ct1;
-                zd_item(a, item, l, mt, ct0, ct1);
-                if (!bar_wait(aEmpty, (u & 1) ^ 1)) { ok = false; break; }
-                bar_expect(aFull, 3 * kZdAChunk);
-                for (int kc = 0; kc < 3; ++kc) tma4(sA + kc * kZdAChunk, &a.tmA, aFull, kc * kZdKC, mt * 128, l, 0);
-                for (int ct = ct0; ct < ct1 && ok; ++ct, ++tile) {
-                    const uint32_t ps = tile % kZdPsiSlots, pn = tile / kZdPsiSlots;
-                    if (!bar_wait(&pEmpty[ps], (pn & 1) ^ 1)) { ok = false; break; }
-                    bar_expect(&pFull[ps], pbytes);
-                    tma3(ring + ps * a.CT * a.n, &a.tmC, &pFull[ps], 0, l, a.c0 + ct * a.CT);
-                }
-            }
-            // every load has landed before the block may leave
-            if (u > 0 && ok && !bar_wait(aFull, (u - 1) & 1)) ok = false;
-            for (uint32_t t = tile > kZdPsiSlots ? tile - kZdPsiSlots : 0; t < tile && ok; ++t)
-                if (!bar_wait(&pFull[t % kZdPsiSlots], (t / kZdPsiSlots) & 1)) ok = false;
-            if (!ok) atomicOr(a.status, kStatusTimeout);
-        }
-    } else if (warp == 1) {
-        // ---- MMA issue
-        if (lane == 0) {
-            // descriptor address fields count 16-byte units: offsets below 256 KB add in place
-            const uint64_t ad0 = sdesc_sw64(su32(sA)), bd0 = sdesc_sw32(su32(sB));
-            uint32_t u = 0, it = 0, tile = 0;
-            for (int item = blockIdx.x; item < a.nitems && ok; item += gridDim.x, ++u) {
-                int l, mt, ct0, ct1;
-                zd_item(a, item, l, mt, ct0, ct1);
-                if (!bar_wait(aFull, u & 1)) { ok = false; break; }
-                for (int ct = ct0; ct < ct1 && ok; ++ct, ++tile) {
-                    if (!bar_wait(&tEmpty[0], (tile & 1) ^ 1)) { ok = false; break; }
-                    tc_fence_after();
-                    for (int ks = 0; ks < kZdStages && ok; ++ks, ++it) {
-                        const uint32_t st = it & 1;
-                        if (!bar_wait(&bFull[st], (it >> 1) & 1)) { ok = false; break; }
-                        tc_fence_after();
-                        // the 21 products of the stage, unrolled: A is K-chunk ks / 2 from its
-                        // 32-byte half ks % 2, descriptors advance by constant offsets, and a
-                        // group's first product of the tile (stage 0, i = 0, j = group) starts its
-                        // accumulator
-                        const uint64_t ad = ad0 + (uint64_t)(((ks >> 1) * kZdAChunk + (ks & 1) * 32) >> 4);
-                        const uint64_t bd = bd0 + (uint64_t)((st * kZdBStage) >> 4);
-                        const uint32_t acc0 = ks > 0 ? 1u : 0u;
-#pragma unroll
-                        for (int i = 0; i < kZdSlices; ++i)
-#pragma unroll
-                            for (int j = 0; j < kZdSlices - i; ++j) {
-                                const int g = i + j < 3 ? i + j : 3;
-                                const bool first = i == 0 && j <= 3;
-                                umma_f16(tbase + g * kZdN, ad + (uint64_t)((i * kZdASlice) >> 4),
-                                         bd + (uint64_t)((j * kZdBSlice) >> 4), kZdIdesc, first ? acc0 : 1u);
-                            }
-                        umma_commit(&bEmpty[st]);
-                    }
-                    umma_commit(&tFull[0]);
-                }
-                umma_commit(aEmpty);
-            }
-            umma_commit(fin);
-            bar_wait(fin, 0);
-            if (!ok) atomicOr(a.status, kStatusTimeout);
-        }
-    } else if (warp < 6) {
-        // ---- epilogue: one tile row (valence band) per thread
-        const int q4 = warp & 3, r = q4 * 32 + lane;
+    // registers: 512 x 128 at launch; the epilogue warps hold 64 columns of two accumulators and
+    // take 176 a thread, the other two warpgroups keep 80
+    if (warp >= 4 && warp < 12) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
+        // ---- epilogue: a quadrant's 32 rows (conduction bands) x 64 of the 128 columns per warp.  The
+        // 16 x 256-bit load shape gives the four lanes of a quad four consecutive entries (Re, Im) of
+        // one row, so that a store instruction writes 64 contiguous bytes (whole sectors) of 8 rows.
+        const int q4 = warp & 3, half = (warp - 4) >> 2;
+        const uint32_t ta = tbase + ((uint32_t)(q4 * 32) << 16) + half * 64;
         uint32_t tile = 0;
-        for (int item = blockIdx.x; item < a.nitems && ok; item += gridDim.x) {
-            int l, mt, ct0, ct1;
-            zd_item(a, item, l, mt, ct0, ct1);
-            const int v = mt * 128 + r;
-            for (int ct = ct0; ct < ct1; ++ct, ++tile) {
-                // F index of the row's first entry in this tile, and the bands the tile holds
-                const int64_t rowbase = ((int64_t)l * a.cb * a.nv + (int64_t)ct * a.CT * a.nv + v) * a.K2;
-                const int clmax = min(a.CT, a.cb - ct * a.CT);
-                const bool got = bar_wait(&tFull[0], tile & 1);
+        for (int u = blockIdx.x; u < a.nunits && ok; u += gridDim.x) {
+            const int l = u / a.nvt, vt = u - l * a.nvt;
+            const int vmax = min(a.CT, a.vb - vt * a.CT);
+            for (int mt = 0; mt < a.nmt; ++mt, ++tile) {
+                const bool got = bar_wait(tFull, tile & 1);
                 if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t ta = tbase + ((uint32_t)(q4 * 32) << 16);
-                const int cend = a.CT * ncol; // columns holding bands
-#pragma unroll 1
-                for (int c0 = 0; c0 < cend; c0 += 32) {
-                    uint32_t g0[32], g1[32], g2[32], g3[32];
-                    GW_TMEM_LD32(ta + 0 * kZdN + c0, g0);
-                    GW_TMEM_LD32(ta + 1 * kZdN + c0, g1);
-                    GW_TMEM_LD32(ta + 2 * kZdN + c0, g2);
-                    GW_TMEM_LD32(ta + 3 * kZdN + c0, g3);
+                auto release = [&](int g) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) bar_arrive(&tEmpty[g]);
+                };
+                // s + e: the sum of the groups so far and its error, from the least significant up.
+                // Registers 32 h + 4 j + 2 i + {0, 1}: row 16 h + 8 i + lane / 4, entry 4 j + lane % 4
+                uint32_t s[64], e[64];
+                GW_TMEM_LD_16X256_X8(ta + 3 * kZdN, e);
+                GW_TMEM_LD_16X256_X8(ta + 3 * kZdN + (16u << 16), e + 32);
+                tmem_wait_ld();
+                release(3);
+                GW_TMEM_LD_16X256_X8(ta + 2 * kZdN, s);
+                GW_TMEM_LD_16X256_X8(ta + 2 * kZdN + (16u << 16), s + 32);
+                tmem_wait_ld();
+                release(2);
+#pragma unroll
+                for (int c = 0; c < 64; ++c) {
+                    float er;
+                    s[c] = __float_as_uint(zd_2sum(__uint_as_float(s[c]), __uint_as_float(e[c]), er));
+                    e[c] = __float_as_uint(er);
+                }
+#pragma unroll
+                for (int c0 = 0; c0 < 64; c0 += 16) {
+                    const uint32_t tc = ta + ((uint32_t)(c0 >> 5) << 20) + (c0 & 16) * 2;
+                    uint32_t v[32];
+                    GW_TMEM_LD_16X256_X4(tc + kZdN, v);
+                    GW_TMEM_LD_16X256_X4(tc, v + 16);
                     tmem_wait_ld();
-                    if (c0 + 32 >= cend) {
-                        // the accumulators are in registers: the next tile's products may start
-                        tc_fence_before();
-                        bar_arrive(&tEmpty[0]);
+                    if (c0 == 48) {
+                        release(1);
+                        if (lane == 0) bar_arrive(&tEmpty[0]);
                     }
-                    if (v < a.nv) {
 #pragma unroll
-                        for (int cc = 0; cc < 32; cc += 2) {
-                            const int2 cp = ctab[(c0 + cc) >> 1]; // Re column c0 + cc, Im column + 1
-                            if (cp.x < clmax) {
-                                float x[2], y[2];
+                    for (int g = 0; g < 2; ++g)
 #pragma unroll
-                                for (int p = 0; p < 2; ++p) {
-                                    float e1, e2;
-                                    const float s1 = zd_2sum(__uint_as_float(g0[cc + p]), __uint_as_float(g1[cc + p]), e1);
-                                    const float s2 = zd_2sum(s1, __uint_as_float(g2[cc + p]), e2);
-                                    const float t = __fadd_rn(__fadd_rn(e1, e2), __uint_as_float(g3[cc + p]));
-                                    x[p] = __fadd_rn(s2, t);
-                                    y[p] = __fsub_rn(t, __fsub_rn(x[p], s2));
-                                }
-                                const int64_t fi = rowbase + cp.y;
-                                if (!GW_IN(fi, (int64_t)a.n * a.n * a.cb * a.nv * a.K2, a.status)) continue;
-                                a.F[fi] = make_float4(x[0], y[0], x[1], y[1]);
-                            }
+                        for (int c = 0; c < 16; ++c) {
+                            float er;
+                            s[c0 + c] =
+                                __float_as_uint(zd_2sum(__uint_as_float(v[16 * g + c]), __uint_as_float(s[c0 + c]), er));
+                            e[c0 + c] = __float_as_uint(__fadd_rn(__uint_as_float(e[c0 + c]), er));
+                        }
+                }
+                const int64_t unit0 = ((int64_t)l * a.vb + (int64_t)vt * a.CT) * a.cb;
+                const int r0 = mt * kZdM + q4 * 32 + (lane >> 2);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int2 cp = ctab[half * 32 + 4 * j + (lane & 3)];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) { // rows r0 + 8 i
+                        const int c = 32 * (i >> 1) + 4 * j + 2 * (i & 1), cl = r0 + 8 * i;
+                        float h[2], y[2];
+#pragma unroll
+                        for (int m = 0; m < 2; ++m) {
+                            const float t = __uint_as_float(e[c + m]), b = __uint_as_float(s[c + m]);
+                            h[m] = __fadd_rn(b, t);
+                            y[m] = __fsub_rn(t, __fsub_rn(h[m], b));
+                        }
+                        if (cp.x < vmax && cl < a.cb) {
+                            const int64_t fi = (unit0 + cl) * a.K2P + cp.y;
+                            if (!GW_IN(fi, (int64_t)a.n * a.n * a.cb * a.vb * a.K2P, a.status)) continue;
+                            a.F[fi] = make_float4(h[0], y[0], h[1], y[1]);
                         }
                     }
                 }
@@ -422,73 +402,198 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
         }
         if (!ok && lane == 0) atomicOr(a.status, kStatusTimeout);
     } else {
-        // ---- producers: column slices of the conduction tile, stage by stage.  Lane (cl, k2) =
-        // (lane / 8, lane % 8) owns the points i2 = 8 ks + k2 of band cl, loaded once per tile for
-        // the six stages; producer warp pw forms the frequencies q = pw, pw + 6, ...
-        const int pw = warp - 6;
-        const int ncomb = a.CT * 8; // lanes holding a band (CT <= 4)
-        const int cl = lane >> 3, k2 = lane & 7;
-        uint32_t it = 0, tile = 0;
-        for (int item = blockIdx.x; item < a.nitems && ok; item += gridDim.x) {
-            int l, mt, ct0, ct1;
-            zd_item(a, item, l, mt, ct0, ct1);
-            for (int ct = ct0; ct < ct1 && ok; ++ct, ++tile) {
-                // the tile's conduction lines, staged by the TMA warp
-                const uint32_t ps = tile % kZdPsiSlots, pn = tile / kZdPsiSlots;
-                const bool pgot = bar_wait(&pFull[ps], pn & 1);
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        if (warp == 0) {
+            // ---- TMA: line tiles one unit ahead, row slices stage by stage
+            if (lane == 0) {
+                uint32_t it = 0, nu = 0, np = 0;
+                const unsigned pbytes = (unsigned)a.CT * a.n * 16; // CT lines of N two-float points
+                auto lines = [&](int u) {
+                    if (u >= a.nunits) return;
+                    const uint32_t ps = np % kZdPsiSlots;
+                    if (!bar_wait(&pEmpty[ps], ((np / kZdPsiSlots) & 1) ^ 1)) {
+                        ok = false;
+                        return;
+                    }
+                    const int l = u / a.nvt, vt = u - l * a.nvt;
+                    bar_expect(&pFull[ps], pbytes);
+                    tma3(ring + ps * a.CT * a.n, &a.tmV, &pFull[ps], 0, l, a.v0 + vt * a.CT);
+                    ++np;
+                };
+                lines(blockIdx.x);
+                for (int u = blockIdx.x; u < a.nunits && ok; u += gridDim.x, ++nu) {
+                    lines(u + gridDim.x);
+                    const unsigned char *src = a.A + (int64_t)(u / a.nvt) * a.nmt * nst * kZdStage;
+                    for (int j = 0; j < a.nmt * nst && ok; ++j, ++it) {
+                        const uint32_t as = it % ast;
+                        if (!bar_wait(&aEmpty[as], ((it / ast) & 1) ^ 1)) { ok = false; break; }
+                        bar_expect(&aFull[as], kZdStage);
+                        bulk_copy(sA + as * kZdStage, src + (int64_t)j * kZdStage, kZdStage, &aFull[as]);
+                    }
+                }
+                // every copy has landed before the block may leave
+                for (uint32_t j = it > ast ? it - ast : 0; j < it; ++j) bar_wait(&aFull[j % ast], (j / ast) & 1);
+                for (uint32_t j = np > kZdPsiSlots ? np - kZdPsiSlots : 0; j < np; ++j)
+                    bar_wait(&pFull[j % kZdPsiSlots], (j / kZdPsiSlots) & 1);
+                if (!ok) atomicOr(a.status, kStatusTimeout);
+            }
+        } else if (warp == 1) {
+            // ---- MMA issue
+            if (lane == 0) {
+                // The pipe holds few products, so what this thread does between two stages shows: a
+                // stage's barriers are awaited between the products of the stage before.
+                // descriptor address fields count 16-byte units: offsets below 256 KB add in place
+                const uint64_t ad0 = sdesc_sw32(su32(sA)), bd0 = sdesc_sw32(su32(sB));
+                uint32_t as = 0, ph = 0, tph = 1, nu = 0;
+                if (blockIdx.x < a.nunits && (!bar_wait(&bFull[0], 0) || !bar_wait(&aFull[0], 0))) ok = false;
+                tc_fence_after();
+                for (int u = blockIdx.x; u < a.nunits && ok; u += gridDim.x, ++nu) {
+                    const bool more = u + (int)gridDim.x < a.nunits;
+                    for (int mt = 0; mt < a.nmt && ok; ++mt, tph ^= 1) {
+                        const bool last = mt == a.nmt - 1;
+                        // The 21 products of a stage, unrolled, descriptors advanced by constant offsets.
+                        // A tile's first two stages go together, accumulator by accumulator as the
+                        // epilogue hands them back (the least significant, with 15 products, first);
+                        // a group's first product of the tile starts its accumulator.
+                        auto issue = [&](int g, uint64_t ad, uint64_t bd, uint32_t acc0) {
+#pragma unroll
+                            for (int i = 0; i < kZdSlices; ++i)
+#pragma unroll
+                                for (int j = 0; j < kZdSlices - i; ++j)
+                                    if ((i + j < 3 ? i + j : 3) == g)
+                                        umma_f16(tbase + g * kZdN, ad + (uint64_t)((i * kZdSlice) >> 4),
+                                                 bd + (uint64_t)((j * kZdSlice) >> 4), kZdIdesc,
+                                                 i == 0 && j == g ? acc0 : 1u);
+                        };
+                        auto advance = [&] {
+                            if (++as == ast) {
+                                as = 0;
+                                ph ^= 1;
+                            }
+                        };
+                        auto await = [&](bool newb, int ks, uint32_t unit) { // stage ks of this unit or the next
+                            if (newb && !bar_wait(&bFull[ks], unit & 1)) ok = false;
+                            if (!bar_wait(&aFull[as], ph)) ok = false;
+                            tc_fence_after();
+                        };
+                        {
+                            const uint32_t s0 = as;
+                            const uint64_t a0 = ad0 + (uint64_t)((s0 * kZdStage) >> 4);
+                            advance();
+                            const uint32_t s1 = as;
+                            const uint64_t a1 = ad0 + (uint64_t)((s1 * kZdStage) >> 4), b1 = bd0 + (kZdStage >> 4);
+                            if (!bar_wait(&tEmpty[3], tph)) ok = false;
+                            tc_fence_after();
+                            issue(3, a0, bd0, 0u);
+                            await(mt == 0, 1, nu);
+                            if (!bar_wait(&tEmpty[2], tph)) ok = false;
+                            tc_fence_after();
+                            issue(2, a0, bd0, 0u);
+                            issue(3, a1, b1, 1u);
+                            issue(2, a1, b1, 1u);
+                            if (!bar_wait(&tEmpty[1], tph) || !bar_wait(&tEmpty[0], tph)) ok = false;
+                            tc_fence_after();
+                            issue(1, a0, bd0, 0u);
+                            issue(0, a0, bd0, 0u);
+                            umma_commit(&aEmpty[s0]);
+                            if (last) umma_commit(&bEmpty[0]);
+                            issue(1, a1, b1, 1u);
+                            advance();
+                            await(mt == 0, 2, nu);
+                            issue(0, a1, b1, 1u);
+                            umma_commit(&aEmpty[s1]);
+                            if (last) umma_commit(&bEmpty[1]);
+                        }
+                        for (int ks = 2; ks < nst && ok; ++ks) {
+                            const uint64_t ad = ad0 + (uint64_t)((as * kZdStage) >> 4);
+                            const uint64_t bd = bd0 + (uint64_t)((ks * kZdStage) >> 4);
+                            const uint32_t cur = as;
+                            advance();
+                            issue(2, ad, bd, 1u);
+                            issue(1, ad, bd, 1u);
+                            issue(0, ad, bd, 1u);
+                            // the next stage: of this tile, of the next tile or of the next unit
+                            if (ks + 1 < nst) await(mt == 0, ks + 1, nu);
+                            else if (!last || more) await(last, 0, nu + 1);
+                            issue(3, ad, bd, 1u);
+                            umma_commit(&aEmpty[cur]);
+                            if (last) umma_commit(&bEmpty[ks]);
+                        }
+                        umma_commit(tFull);
+                    }
+                }
+                umma_commit(fin);
+                bar_wait(fin, 0);
+                if (!ok) atomicOr(a.status, kStatusTimeout);
+            }
+        } else {
+            // ---- producers: column slices of the valence tile, stage by stage.  A lane owns point
+            // i2 = 8 ks + k2 (k2 = lane % 8) of up to three (band, frequency) pairs, the same in every
+            // stage and unit.
+            const int pw = warp < 4 ? warp - 2 : warp - 10, k2 = lane & 7, npair = a.CT * a.K2;
+            int vl[kZdRounds], col[kZdRounds], w0[kZdRounds], dw[kZdRounds]; // twiddle index, its step per stage
+#pragma unroll
+            for (int j = 0; j < kZdRounds; ++j) {
+                const int p = (j * kZdProducers + pw) * 4 + (lane >> 3);
+                vl[j] = p < npair ? p / a.K2 : -1;
+                const int q = p < npair ? p - vl[j] * a.K2 : 0, kz = a.kz[q];
+                col[j] = vl[j] * ncol + 2 * q;
+                w0[j] = (kz * k2) % a.n;
+                dw[j] = (kz * 8) % a.n;
+            }
+            uint32_t nu = 0;
+            for (int u = blockIdx.x; u < a.nunits && ok; u += gridDim.x, ++nu) {
+                const int l = u / a.nvt, vt = u - l * a.nvt;
+                const uint32_t ps = nu % kZdPsiSlots;
+                const bool pgot = bar_wait(&pFull[ps], (nu / kZdPsiSlots) & 1);
                 if (!__all_sync(0xffffffffu, pgot)) { ok = false; break; }
                 const float4 *pl = ring + ps * a.CT * a.n;
-                const int c = ct * a.CT + cl;
-                float4 x[kZdStages];
-                float m = 0.0f;
+                int E[kZdRounds], w[kZdRounds];
 #pragma unroll
-                for (int ks = 0; ks < kZdStages; ++ks) {
-                    x[ks] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (lane < ncomb && c < a.cb) x[ks] = pl[cl * a.n + ks * 8 + k2];
-                    m = fmaxf(m, (fabsf(x[ks].x) + fabsf(x[ks].z)) * (1.0f + 0x1p-20f));
+                for (int j = 0; j < kZdRounds; ++j) {
+                    const int v = vt * a.CT + vl[j];
+                    w[j] = w0[j];
+                    E[j] = vl[j] >= 0 && v < a.vb ? __ldg(a.E + (int64_t)(a.v0 + v) * a.n * a.n + l) : -70;
                 }
-                // the 8 lanes of one band hold its whole line: the band's maximum
-                for (int o = 4; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                const int E = max(-70, zd_expo(m)); // keeps the scale and every weight normal
-                const float sc = __int_as_float((127 + 47 - E) << 23);
-                float w[kZdSlices];
+                for (int ks = 0; ks < nst; ++ks) {
+                    const bool got = bar_wait(&bEmpty[ks], (nu & 1) ^ 1);
+                    if (!__all_sync(0xffffffffu, got)) { ok = false; break; } // warp-uniform exit
+                    unsigned char *B = sB + ks * kZdStage;
 #pragma unroll
-                for (int i = 0; i < kZdSlices; ++i) w[i] = __int_as_float((127 + E - 7 - 8 * i) << 23);
-                __syncwarp();
-                if (lane == 0) bar_arrive(&pEmpty[ps]); // the slot's values are in registers
+                    for (int j = 0; j < kZdRounds; ++j) {
+                        if (vl[j] < 0) continue;
+                        const int i2 = ks * 8 + k2;
+                        float4 x = pl[vl[j] * a.n + i2];
+                        if (vt * a.CT + vl[j] >= a.vb) x = make_float4(0.f, 0.f, 0.f, 0.f);
+                        const tcx b = tc_mulc(tcx{{x.x, x.y}, {x.z, x.w}}, tc_load(wt + w[j])); // conj(x) W
+                        w[j] += dw[j];
+                        if (w[j] >= a.n) w[j] -= a.n;
+                        uint16_t dr[kZdSlices], di[kZdSlices];
+                        zd_digits_n(b.re.hi, b.re.lo, E[j], dr);
+                        zd_digits_n(b.im.hi, b.im.lo, E[j], di);
+                        const int colr = col[j];
+                        if (!GW_IN(colr + 1, kZdN, a.status)) continue;
+                        // rows (Re c, Im c): Re column (Re b, -Im b); Im column (Im b, Re b).  The lanes of
+                        // pairs 2 and 3 store their Im column first: the four pairs' columns, 64 bytes
+                        // apart, would share banks two by two
+                        const bool im = (lane & 16) != 0;
+                        unsigned char *p0 = B + sw32_off(colr + im, 2 * k2), *p1 = B + sw32_off(colr + !im, 2 * k2);
 #pragma unroll
-                for (int ks = 0; ks < kZdStages; ++ks, ++it) {
-                    if (!ok) continue;
-                    const uint32_t st = it & 1;
-                    const bool got = bar_wait(&bEmpty[st], ((it >> 1) & 1) ^ 1);
-                    if (!__all_sync(0xffffffffu, got)) { ok = false; continue; } // warp-uniform exit
-                    unsigned char *B = sB + st * kZdBStage;
-                    if (lane < ncomb) {
-                        const tcx xv = {{x[ks].x, x[ks].y}, {x[ks].z, x[ks].w}};
-                        const float4 *wrow = wt + ks * 8 + k2;
-                        for (int q = pw; q < a.K2; q += kZdProducers) {
-                            const tcx b = tc_mul(xv, tc_load(wrow + q * a.n));
-                            uint16_t dr[kZdSlices], di[kZdSlices];
-                            zd_digits_w(b.re.hi, b.re.lo, sc, w, dr);
-                            zd_digits_w(b.im.hi, b.im.lo, sc, w, di);
-                            const int colr = cl * ncol + 2 * q;
-                            if (!GW_IN(colr + 1, kZdN, a.status)) continue;
-                            unsigned char *pr = B + sw32_off(colr, 2 * k2), *pi = B + sw32_off(colr + 1, 2 * k2);
-#pragma unroll
-                            for (int sl = 0; sl < kZdSlices; ++sl) {
-                                // Re column: (Re b, Im b); Im column: (Im b, -Re b)
-                                *(uint32_t *)(pr + sl * kZdBSlice) = (uint32_t)dr[sl] | ((uint32_t)di[sl] << 16);
-                                *(uint32_t *)(pi + sl * kZdBSlice) = (uint32_t)di[sl] | ((uint32_t)(dr[sl] ^ 0x8000u) << 16);
-                            }
+                        for (int sl = 0; sl < kZdSlices; ++sl) {
+                            const uint32_t vr = (uint32_t)dr[sl] | ((uint32_t)(di[sl] ^ 0x8000u) << 16);
+                            const uint32_t vi = (uint32_t)di[sl] | ((uint32_t)dr[sl] << 16);
+                            *(uint32_t *)(p0 + sl * kZdSlice) = im ? vi : vr;
+                            *(uint32_t *)(p1 + sl * kZdSlice) = im ? vr : vi;
                         }
                     }
                     fence_async_shared();
                     __syncwarp();
-                    if (lane == 0) bar_arrive(&bFull[st]);
+                    if (lane == 0) bar_arrive(&bFull[ks]);
                 }
+                if (lane == 0) bar_arrive(&pEmpty[ps]);
             }
+            if (!ok && lane == 0) atomicOr(a.status, kStatusTimeout);
         }
-        if (!ok && lane == 0) atomicOr(a.status, kStatusTimeout);
     }
     tc_fence_before();
     __syncthreads();
@@ -496,42 +601,52 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
     if (warp == 1) tmem_dealloc(tbase, 512);
 }
 
-size_t zd_smem_bytes(int n, int K2)
+static size_t zd_smem(int n, int K2, int ast)
 {
-    return 1024 + 3 * kZdAChunk + 2 * kZdBStage + 16 * (size_t)kZdPsiSlots * zd_conduction_per_tile_d(K2) * n +
-           16 * (size_t)K2 * n +
-           8 * (kZdN / 2) + 8 * 24 + 64;
+    return 1024 + (ast + n / 8) * (size_t)kZdStage + 16 * (size_t)kZdPsiSlots * zd_valence_per_tile(K2) * n +
+           16 * (size_t)n + 8 * (kZdN / 2) + 8 * 40 + 64;
 }
 
-// The route's shapes: 48-point lines (three valence K-chunks of 32 real entries, six column
-// stages of 16), at most 32 kept frequencies, and the block's shared memory (valence slices,
-// column stages, ring, twiddle table) within the 227 KB a block may opt into.
-bool zd_supported(int n, int K2, int nv)
+// stages of the row ring: what shared memory holds (three for 48-point lines, four for 40)
+static int zd_ring(int n, int K2)
 {
-    return n == 48 && K2 >= 1 && K2 <= 32 && nv >= 1 && 2 * n == 3 * kZdKC && 2 * n == kZdStages * kZdKB &&
-           zd_smem_bytes(n, K2) <= (size_t)227 * 1024;
+    int ast = kZdMaxRing;
+    while (ast > 2 && zd_smem(n, K2, ast) > (size_t)227 * 1024) --ast;
+    return ast;
 }
 
-int zd_conduction_per_tile(int K2) { return zd_conduction_per_tile_d(K2); }
+size_t zd_smem_bytes(int n, int K2) { return zd_smem(n, K2, zd_ring(n, K2)); }
 
-cudaError_t launch_zd_gemm(const CUtensorMap &tmA, const CUtensorMap &tmC, const void *, const int *kz,
-                           const float4 *twf, int n, int nv, int c0, int cb, int K2, float4 *F, int *status,
-                           cudaStream_t st)
+// The route's shapes: lines of 40 or 48 points (the grids whose remaining axes are built from F), at
+// most 32 kept frequencies, and the block's shared memory (column stages, ring of row stages, line
+// tiles) within the 227 KB a block may opt into.
+bool zd_supported(int n, int K2)
+{
+    return (n == 40 || n == 48) && K2 >= 1 && K2 <= 32 && zd_smem_bytes(n, K2) <= (size_t)227 * 1024;
+}
+
+cudaError_t launch_zd_gemm(const CUtensorMap &tmV, const void *A, const int *E, const int *kz, const float4 *twf, int n,
+                           int nv, int v0, int vb, int cb, int K2, float4 *F, int *status, cudaStream_t st)
 {
     ZdArgs a;
-    a.tmA = tmA;
-    a.tmC = tmC;
+    a.tmV = tmV;
+    a.A = (const unsigned char *)A;
+    a.E = E;
     a.kz = kz;
     a.F = F;
     a.status = status;
     a.n = n;
     a.nv = nv;
-    a.c0 = c0;
+    a.v0 = v0;
+    a.vb = vb;
     a.cb = cb;
     a.K2 = K2;
-    a.CT = zd_conduction_per_tile(K2);
-    a.nmt = (nv + 127) / 128;
-    a.nunits = n * n * a.nmt;
+    a.K2P = zd_row_entries(K2);
+    a.ast = zd_ring(n, K2);
+    a.CT = zd_valence_per_tile(K2);
+    a.nvt = (vb + a.CT - 1) / a.CT;
+    a.nmt = (cb + kZdM - 1) / kZdM;
+    a.nunits = n * n * a.nvt;
     const size_t sm = zd_smem_bytes(n, K2);
     cudaError_t e = cudaFuncSetAttribute(zd_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
@@ -539,15 +654,7 @@ cudaError_t launch_zd_gemm(const CUtensorMap &tmA, const CUtensorMap &tmC, const
     if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return e;
-    const int grid = std::min(a.nunits, sms);
-    // the persistent blocks take items b, b + grid, ...: whole units while every block gets one,
-    // then the rem remaining units in parts, so that the last wave ends evenly
-    a.nct = (cb + a.CT - 1) / a.CT;
-    a.nfull = a.nunits / grid * grid;
-    const int rem = a.nunits - a.nfull;
-    a.nsplit = rem > 0 ? std::max(1, std::min(a.nct, grid / rem)) : 1;
-    a.nitems = a.nfull + rem * a.nsplit;
-    zd_gemm_kernel<<<grid, kZdThreads, sm, st>>>(a, twf);
+    zd_gemm_kernel<<<std::min(a.nunits, sms), kZdThreads, sm, st>>>(a, twf);
     return cudaGetLastError();
 }
 

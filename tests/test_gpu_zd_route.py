@@ -1,0 +1,84 @@
+"""Stage (a) on the tensor cores, all callers, on the two grids it is built for: row tiles of 128
+conduction bands (one short, one exact, one over), partial valence tiles, odd and even numbers of kept
+z-frequencies, chunks that hold less than a row of pairs, and a conduction set of several blocks.
+Against the library's FP64 mode (an independent path, 1e-15).  Two-float stage (a) keeps 2e-13 and the
+contraction at seven-slice accuracy, a five-slice expansion, 32 * 5 * 2^-45 = 5e-12 of the product of two
+columns' largest magnitudes per pair: relative to the columns' norms below 2e-11 for these bands."""
+import numpy as np
+import pytest
+
+import gwgen
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+TOL = 2e-11
+
+
+@pytest.fixture(scope="module")
+def gw():
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    import paper_2509_23018_gb300 as gw
+    return gw
+
+
+def dev(x):
+    return torch.as_tensor(np.ascontiguousarray(x), device="cuda")
+
+
+def rel(a, b):
+    return float(torch.linalg.vector_norm(a - b) / torch.linalg.vector_norm(b))
+
+
+SHAPES = [(40, 9, 127, 1500, 333, 8192), (40, 33, 256, 3000, 900, 4096), (40, 4, 129, 1500, 401, 8192),
+          (48, 20, 300, 2500, 700, 2100), (48, 7, 500, 2000, 500, 400), (48, 3, 1100, 3000, 300, 8192)]
+
+
+@pytest.mark.parametrize("n,nv,nc,ngpsi,ng,chunk", SHAPES)
+def test_route_matches_fp64(gw, n, nv, nc, ngpsi, ng, chunk):
+    p = gwgen.make_problem((n, n, n), nv, nc, ngpsi, ng, seed=n + nv)
+    rng = np.random.default_rng(nc)
+    W = dev(gwgen.hermitian(rng, ng))
+    tan = [dev(rng.standard_normal(c.shape) + 1j * rng.standard_normal(c.shape)) * 1e-2 for c in (p.cv, p.cc)]
+    tan += [dev(rng.standard_normal(len(e))) for e in (p.ev, p.ec)]
+    basis = dev(np.linalg.qr(rng.standard_normal((ng, 24)) + 1j * rng.standard_normal((ng, 24)))[0])
+    out = {}
+    for mode, kw in (("fp64", dict(prec="fp64")), ("split", dict(prec="ozaki", nslices=7, mtxel="twofloat"))):
+        h = gw.from_problem(p, pair_chunk=chunk, **kw)
+        if mode == "split":
+            assert h.streams(0) == 1
+        r = {"chi": h.compute(0, [0.0, 3.0])[0], "batch": h.compute_batch([0], [0.0, 3.0])[0],
+             "sub": h.compute_subspace(0, basis, [1.0]), "real": h.compute_real(0, [4.0], 0.2),
+             "jvp": h.jvp(0, [2.0], *tan)}
+        r.update(zip(("dev", "dec", "dcv", "dcc"), h.adjoint(0, W)[1:]))
+        h.keep_pair_elements(True)
+        r["kept"] = h.compute(0, [0.0])[0]
+        r["kept_sub"] = h.compute_subspace(0, basis, [1.0])
+        h.sync()
+        out[mode] = {k: v.clone() for k, v in r.items()}
+        h.destroy()
+    # the forward derivative and the real axis subtract contractions of larger magnitude
+    loose = {"jvp": 5, "real": 5, "dev": 5, "dec": 5}
+    bad = {k: rel(v, out["fp64"][k]) for k, v in out["split"].items() if rel(v, out["fp64"][k]) > TOL * loose.get(k, 1)}
+    assert not bad
+
+
+def test_route_yields_to_the_memory_budget(gw):
+    """A budget without room for the route's buffers: the FFT pair kernel serves the call as before."""
+    p = gwgen.make_problem((40, 40, 40), 8, 200, 1500, 300, seed=9)
+    ref = gw.from_problem(p, prec="fp64").compute(0, [0.0])[0]
+    # grids, pair elements and slices need about 0.25 GB; the route's slices and F 0.6 GB more
+    h = gw.from_problem(p, prec="ozaki", nslices=7, mtxel="twofloat", mem_budget_bytes=500 << 20)
+    assert rel(h.compute(0, [0.0])[0], ref) < TOL
+    h.sync()
+    assert h.device_bytes() <= 500 << 20
+
+
+def test_eight_slices_keep_the_fft_kernel_elsewhere(gw):
+    """At eight slices the pair elements' own error would show: other calls than chi on 48^3 keep the FFT
+    kernel and stay within its error (bound of the six-slice expansion: 32 * 6 * 2^-54 = 1e-14 a pair)."""
+    p = gwgen.make_problem((40, 40, 40), 8, 200, 1500, 300, seed=9)
+    ref = gw.from_problem(p, prec="fp64").compute(0, [0.0])[0]
+    h = gw.from_problem(p, prec="ozaki", nslices=8, mtxel="twofloat")
+    assert rel(h.compute(0, [0.0])[0], ref) < 4e-14
+    h.sync()
