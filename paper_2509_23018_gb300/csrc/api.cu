@@ -572,31 +572,50 @@ gw_status ensure_overlap_stream(gw_chi0 *h)
 
 // ------------------------------------------------------------------ stage (a) on the tensor cores
 // The last-axis transform of the pair products as a split product per grid line (zdft.cu), the
-// middle and first axes from its output, for two-float stage (a) on the 40^3 and 48^3 grids.  A block
-// is vb valence x cb conduction bands; the row slices of the conduction block are formed once, and the
-// valence bands run over it in sub-blocks whose transform output F fits the work buffer.  On one
-// stream: the last-axis product and the split contraction each need whole SMs.
+// middle and first axes from its output, for two-float stage (a): on the 40^3 and 48^3 grids in one
+// kernel, on others of the lengths of pair_split_supported with the cells in global memory between
+// two.  A block is vb valence x cb conduction bands; the row slices of the conduction block are formed
+// once, and the valence bands run over it in sub-blocks whose transform output F fits the work buffer.
+// On one stream: the last-axis product and the split contraction each need whole SMs.
 // GW_CHI0_STAGE_A=fft selects the FFT pair kernel instead.
+
+// grids whose middle and first axes run in one kernel, with the pair kernel's scratch slots
+static bool zd_fused(const gw_chi0 *h)
+{
+    const int *n = h->d.n;
+    return n[0] == n[1] && n[1] == n[2] && (n[0] == 40 || n[0] == 48);
+}
+
 static bool zd_grid(const gw_chi0 *h, const Sphere &sp)
 {
     static const bool fft_only = [] {
         const char *e = getenv("GW_CHI0_STAGE_A");
         return e && strcmp(e, "fft") == 0;
     }();
-    const int n = h->d.n[0];
-    return !fft_only && h->d.mtxel_prec == GW_MTXEL_TWOFLOAT && h->d.n[1] == n && h->d.n[2] == n && sp.nslots > 0 &&
-           h->pscr && gw::zd_supported(n, sp.K2);
+    const int *n = h->d.n;
+    if (fft_only || h->d.mtxel_prec != GW_MTXEL_TWOFLOAT || !gw::zd_supported(n[2], sp.K2)) return false;
+    if (zd_fused(h)) return sp.nslots > 0 && h->pscr;
+    // 24^3 keeps its grid-specialised FFT kernel, which runs beside the contraction on a second stream
+    const bool small_cube = n[0] == n[1] && n[1] == n[2] && n[0] <= 24;
+    return !small_cube && gw::pair_split_supported(n[0]) && gw::pair_split_supported(n[1]);
 }
 
-// Whether a block of vb x cb pairs takes less time this way.  In units of one pair of the FFT kernel
-// (1.04 us on 48^3, 0.84 on 40^3; below about 600 pairs its blocks do not fill the GPU): a tile of 128
-// conduction bands x CT valence bands over all lines costs 70 (48^3) or 50 (40^3), however few of
-// its rows and columns hold bands, and the other two axes 0.25 a pair.
+// Whether a block of vb x cb pairs takes less time this way, from microseconds measured on one GB300:
+// the FFT kernel 1.04 a pair on 48^3, 0.84 on 40^3, 5.1 on 72^3, 28e-6 a grid point where it is not
+// grid-specialised, and no less than for the 600 pairs that fill the GPU; here 5.2e-3 per line, stage
+// of 8 points and tile of 128 conduction bands x CT valence bands, however few of its rows and columns
+// hold bands, and for the other two axes 7.2e-6 per line and kept frequency of a pair.
 static bool zd_faster(const gw_chi0 *h, const Sphere &sp, int vb, int cb)
 {
-    const int ct = gw::zd_valence_per_tile(sp.K2);
-    const double tiles = (double)((cb + 127) / 128) * ((vb + ct - 1) / ct), pairs = (double)vb * cb;
-    return tiles * (h->d.n[0] == 48 ? 70.0 : 50.0) + 0.25 * pairs < std::max(pairs, 600.0);
+    const int *n = h->d.n, ct = gw::zd_valence_per_tile(n[2], sp.K2);
+    const bool cube = n[0] == n[1] && n[1] == n[2];
+    const double lines = (double)n[0] * n[1], pairs = (double)vb * cb;
+    const double tiles = (double)((cb + 127) / 128) * ((vb + ct - 1) / ct);
+    const double fft = cube && n[0] == 48   ? 1.04
+                       : cube && n[0] == 40 ? 0.84
+                       : cube && n[0] == 72 ? 5.1
+                                            : 28e-6 * lines * n[2];
+    return tiles * lines * ((n[2] + 7) / 8) * 5.2e-3 + 7.2e-6 * lines * sp.K2 * pairs < fft * std::max(pairs, 600.0);
 }
 
 // Room for the route's buffers beside what the call will still take: with a memory budget, the
@@ -622,12 +641,13 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
 {
     z = ZdPlan();
     if (!zd_grid(h, sp)) return GW_OK;
-    const int n = h->d.n[0], ct = gw::zd_valence_per_tile(sp.K2);
+    const int *n = h->d.n, ct = gw::zd_valence_per_tile(n[2], sp.K2), lines = n[0] * n[1];
+    const bool chi48 = zd_fused(h) && n[0] == 48 && !rows;
     // The route's pair elements carry 2e-13 (its fourth accumulator rounds in FP32), the FFT kernel's
     // 8e-15.  At up to seven slices the contraction's own error is ten times that and more.  At eight,
     // and with the FP64 contraction, the route serves chi on 48^3 alone (8.7e-14 at eight slices); on
     // the other calls it would raise the error, by up to three times for the gradients.
-    if ((h->d.prec == GW_PREC_FP64 || h->d.nslices > 7) && (rows || n != 48)) return GW_OK;
+    if ((h->d.prec == GW_PREC_FP64 || h->d.nslices > 7) && !chi48) return GW_OK;
     if (rows) {
         z.cb = nc;
     } else { // conduction blocks of about 512: four row tiles share a valence tile's columns
@@ -641,10 +661,11 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
     if (vb >= ct && vb < nv) vb -= vb % ct;
     z.vb = (int)vb;
     if (!force && !zd_faster(h, sp, z.vb, z.cb)) return GW_OK;
-    z.n = n;
-    z.abytes = gw::zd_row_bytes(z.cb, n);
-    z.ebytes = sizeof(int) * (size_t)n * n * nv;
-    z.fper = sizeof(float4) * (size_t)n * n * z.cb * gw::zd_row_entries(sp.K2); // F of one valence band
+    z.abytes = gw::zd_row_bytes(z.cb, n[2], lines);
+    z.ebytes = sizeof(int) * (size_t)lines * nv;
+    // per valence band: F, and the cells between the two kernels of the other axes
+    z.fper = sizeof(float4) * (size_t)lines * z.cb * gw::zd_row_entries(sp.K2);
+    z.sper = zd_fused(h) ? 0 : sizeof(float4) * (size_t)n[0] * z.cb * sp.K12;
     // F of as many valence bands as 5 GB hold (whole tiles), fewer where memory is short
     int vs = (int)std::min<size_t>(z.vb, std::max<size_t>(1, (size_t)5000000000 / z.fper));
     for (;; vs = vs > ct ? std::max(ct, vs / 2) : vs / 2) {
@@ -654,6 +675,7 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
         for (int i = 0; i < sides; ++i)
             by += (z.abytes > h->zdAcap[i] ? z.abytes - h->zdAcap[i] : 0) + (z.ebytes > h->zdEcap[i] ? z.ebytes - h->zdEcap[i] : 0);
         by += z.fper * vs > h->zdFcap ? z.fper * vs - h->zdFcap : 0;
+        by += z.sper * vs > h->zdScap ? z.sper * vs - h->zdScap : 0;
         if (force || zd_room(h, by, (int64_t)z.vb * z.cb, sp.ng, nw)) break;
     }
     z.vs = vs;
@@ -663,6 +685,7 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
         if (!(s = grow(h, &h->zdA[i], &h->zdAcap[i], z.abytes, "conduction slices")))
             s = grow(h, (void **)&h->zdE[i], &h->zdEcap[i], z.ebytes, "column exponents");
     if (!s) s = grow(h, (void **)&h->zdF, &h->zdFcap, z.fper * vs, "last-axis transform");
+    if (!s && z.sper) s = grow(h, (void **)&h->zdS, &h->zdScap, z.sper * vs, "transform cells");
     if (s == GW_ERR_OOM && !force) { // the FFT route needs none of these
         h->err = err;
         return GW_OK;
@@ -674,21 +697,35 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
 
 bool zd_holds(const gw_chi0 *h, const ZdPlan &z)
 {
-    return h->zdAcap[0] >= z.abytes && h->zdEcap[0] >= z.ebytes && h->zdFcap >= z.fper * z.vs;
+    return h->zdAcap[0] >= z.abytes && h->zdEcap[0] >= z.ebytes && h->zdFcap >= z.fper * z.vs &&
+           h->zdScap >= z.sper * z.vs;
+}
+
+// A tensor map of two-float entries as FP32: rows of `row` entries, boxes of `w` entries x `hgt` rows.
+static gw_status zd_map(gw_chi0 *h, CUtensorMap *tm, void *p, uint64_t row, uint64_t rows, int w, int hgt, const char *what)
+{
+    cuuint64_t d[2] = {(cuuint64_t)row * 4, (cuuint64_t)rows};
+    cuuint64_t st[1] = {(cuuint64_t)row * 16};
+    cuuint32_t box[2] = {(cuuint32_t)(4 * w), (cuuint32_t)hgt};
+    cuuint32_t es[2] = {1, 1};
+    CUresult r = h->encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, p, d, st, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? GW_OK : fail(h, GW_ERR_CUDA, "cuTensorMapEncodeTiled (%s) failed (%d)", what, (int)r);
 }
 
 gw_status zd_valence(gw_chi0 *h, ZdPlan &z, const Sphere &sp, const void *psiv, int nv, int side)
 {
-    const int n = z.n;
-    const int64_t lines = (int64_t)n * n;
+    const int n = h->d.n[2];
+    const int64_t lines = (int64_t)h->d.n[0] * h->d.n[1];
     {
         Scope sc(h, "zd_slices");
-        CK(h, gw::launch_zd_colexp(psiv, nv, n, h->zdE[side], h->st), "column exponents");
+        CK(h, gw::launch_zd_colexp(psiv, nv, n, (int)lines, h->zdE[side], h->st), "column exponents");
     }
     // the valence grids, line by line: box of one line of CT bands
-    cuuint64_t d[3] = {(cuuint64_t)4 * n, (cuuint64_t)lines, (cuuint64_t)nv};
-    cuuint64_t st[2] = {(cuuint64_t)4 * n * 4, (cuuint64_t)16 * lines * n};
-    cuuint32_t box[3] = {(cuuint32_t)(4 * n), 1, (cuuint32_t)gw::zd_valence_per_tile(sp.K2)};
+    const int part = gw::zd_line_split(n);
+    cuuint64_t d[3] = {(cuuint64_t)4 * n / part, (cuuint64_t)lines * part, (cuuint64_t)nv};
+    cuuint64_t st[2] = {(cuuint64_t)16 * n / part, (cuuint64_t)16 * lines * n};
+    cuuint32_t box[3] = {(cuuint32_t)(4 * n / part), (cuuint32_t)part, (cuuint32_t)gw::zd_valence_per_tile(n, sp.K2)};
     cuuint32_t es[3] = {1, 1, 1};
     CUresult r = h->encode(&z.tmV[side], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(psiv), d, st, box, es,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -701,7 +738,8 @@ gw_status zd_valence(gw_chi0 *h, ZdPlan &z, const Sphere &sp, const void *psiv, 
 gw_status zd_conduction(gw_chi0 *h, const ZdPlan &z, const void *psic, int c0, int cb, int side)
 {
     Scope sc(h, "zd_slices");
-    CK(h, gw::launch_zd_rows((const float4 *)psic + (int64_t)c0 * h->nr, cb, z.n, h->zdA[side], h->st),
+    CK(h, gw::launch_zd_rows((const float4 *)psic + (int64_t)c0 * h->nr, cb, h->d.n[2], h->d.n[0] * h->d.n[1],
+                             h->zdA[side], h->st),
        "conduction slices");
     return GW_OK;
 }
@@ -709,40 +747,35 @@ gw_status zd_conduction(gw_chi0 *h, const ZdPlan &z, const void *psic, int c0, i
 gw_status zd_block(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::PairPlan &pp, int vside, int cside, int v0,
                    int vb, int cb, double2 *M, int64_t sv, int64_t sc)
 {
-    const int n = z.n;
+    const int *n = h->d.n;
+    const int lines = n[0] * n[1];
+    gw_status s;
     for (int b0 = 0; b0 < vb; b0 += z.vs) {
         const int nb = std::min(z.vs, vb - b0);
         {
             Scope t(h, "zdft");
-            CK(h, gw::launch_zd_gemm(z.tmV[vside], h->zdA[cside], h->zdE[vside], sp.kz, pp.ax[2].twf, n, z.nv[vside],
-                                     v0 + b0, nb, cb, sp.K2, h->zdF, h->status, h->st),
+            CK(h, gw::launch_zd_gemm(z.tmV[vside], h->zdA[cside], h->zdE[vside], sp.kz, pp.ax[2].twf, n[2], lines,
+                                     z.nv[vside], v0 + b0, nb, cb, sp.K2, h->zdF, h->status, h->st),
                "last-axis transform");
         }
-        // F as [n^2 lines][R rows of K2P entries]: the middle/first-axis kernel loads a slab pair's
-        // 2n lines of one row (K2 entries each) with one TMA box
+        // F as [lines][R rows of K2P entries]: the middle-axis kernel loads the 2 n1 lines of a slab pair
+        // of one row (K2 entries each) with one TMA box
         const int64_t R = (int64_t)nb * cb;
-        CUtensorMap tmF;
-        const int k2p = gw::zd_row_entries(sp.K2);
-        cuuint64_t fd[2] = {(cuuint64_t)R * k2p * 4, (cuuint64_t)n * n};
-        cuuint64_t fst[1] = {(cuuint64_t)R * k2p * 16};
-        cuuint32_t fbox[2] = {(cuuint32_t)(sp.K2 * 4), (cuuint32_t)(2 * n)};
-        cuuint32_t fes[2] = {1, 1};
-        CUresult r = h->encode(&tmF, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->zdF, fd, fst, fbox, fes,
-                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return fail(h, GW_ERR_CUDA, "cuTensorMapEncodeTiled (last-axis output) failed (%d)", (int)r);
-        // the scratch slots as [nslots n rows][K12] entries: phase 2 loads batches of 2 K2 cells of
-        // all n rows of its slot with one TMA box
-        CUtensorMap tmS;
-        cuuint64_t sd[2] = {(cuuint64_t)pp.K12 * 4, (cuuint64_t)pp.nslots * n};
-        cuuint64_t sst[1] = {(cuuint64_t)pp.K12 * 16};
-        cuuint32_t sbox[2] = {(cuuint32_t)(8 * sp.K2), (cuuint32_t)n};
-        r = h->encode(&tmS, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, pp.scr, sd, sst, sbox, fes, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return fail(h, GW_ERR_CUDA, "cuTensorMapEncodeTiled (pair scratch) failed (%d)", (int)r);
+        CUtensorMap tmF, tmS;
+        if ((s = zd_map(h, &tmF, h->zdF, R * gw::zd_row_entries(sp.K2), lines, sp.K2, 2 * n[1], "last-axis output")))
+            return s;
+        double2 *Mb = M + (int64_t)b0 * sv * sp.ng;
         Scope t(h, "pair_from_f");
-        CK(h, gw::launch_pair_tf_from_f(tmF, tmS, R, cb, sv, sc, pp, M + (int64_t)b0 * sv * sp.ng, h->st),
-           "pair elements from F");
+        if (z.sper == 0) {
+            // the scratch slots as [nslots n rows][K12] entries: phase 2 loads batches of 2 K2 cells of
+            // all n rows of its slot with one TMA box
+            if ((s = zd_map(h, &tmS, pp.scr, pp.K12, (uint64_t)pp.nslots * n[0], 2 * sp.K2, n[0], "pair scratch"))) return s;
+            CK(h, gw::launch_pair_tf_from_f(tmF, tmS, R, cb, sv, sc, pp, Mb, h->st), "pair elements from F");
+        } else {
+            if ((s = zd_map(h, &tmS, h->zdS, pp.K12, (uint64_t)R * n[0], 2 * sp.K2, n[0], "transform cells"))) return s;
+            CK(h, gw::launch_pair_split1(tmF, R, pp, h->zdS, h->st), "middle axis from F");
+            CK(h, gw::launch_pair_split2(tmS, R, cb, sv, sc, pp, Mb, h->st), "pair elements from cells");
+        }
     }
     return GW_OK;
 }
@@ -977,6 +1010,7 @@ void gw_chi0_destroy(gw_chi0 *h)
         dfree(h, h->zdE[i], h->zdEcap[i]);
     }
     dfree(h, h->zdF, h->zdFcap);
+    dfree(h, h->zdS, h->zdScap);
     for (int b = 0; b < 2; ++b) {
         dfree(h, h->ovZ[b], h->ovZcap[b]);
         dfree(h, h->ovE[b], h->ovEcap[b]);
@@ -1216,7 +1250,7 @@ gw_status gw_chi0_pair_elements_block(gw_chi0 *h, int iq, int c0, int cb, double
     const BandSet &v = h->val[iq];
     const Sphere &sp = h->sph[iq];
     const int nv = v.nb;
-    if (h->d.n[0] != 48 || h->keep_m || h->d.pair_chunk < nv || !zd_grid(h, sp))
+    if (!zd_fused(h) || h->d.n[0] != 48 || h->keep_m || h->d.pair_chunk < nv || !zd_grid(h, sp))
         return fail(h, GW_ERR_UNSUPPORTED, "slot %d does not take the tensor-core route", iq);
     if (cb == 0) return GW_OK;
     ZdPlan z;

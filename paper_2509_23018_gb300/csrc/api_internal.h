@@ -167,6 +167,8 @@ struct gw_chi0 {
     size_t zdEcap[2] = {0, 0}; // bytes
     float4 *zdF = nullptr;
     size_t zdFcap = 0;         // bytes
+    float4 *zdS = nullptr;     // cells between the middle- and first-axis kernels, where they are two
+    size_t zdScap = 0;         // bytes
     // scratch slots of the two-float pair kernel (sized in set_gsphere, outside any capture)
     float4 *pscr = nullptr;
     size_t pscr_cap = 0; // bytes
@@ -270,8 +272,8 @@ gw_status compute_overlap(gw_chi0 *h, int iq, const gw::OmegaList &om, double2 *
 // zd_conduction prepare a side's bands; zd_block forms M[(v - v0) sv + c sc] of a block.
 struct ZdPlan {
     bool on = false;
-    int n = 0, vb = 0, cb = 0, vs = 0;          // vs: valence bands per sub-block
-    size_t abytes = 0, ebytes = 0, fper = 0;    // row slices, exponents, F of one valence band
+    int vb = 0, cb = 0, vs = 0;                        // vs: valence bands per sub-block
+    size_t abytes = 0, ebytes = 0, fper = 0, sper = 0; // row slices, exponents; F and cells of one valence band
     int nv[2] = {0, 0};
     CUtensorMap tmV[2];
 };

@@ -58,21 +58,31 @@ cudaError_t launch_band_setup_tf(const double2 *coeff, const int32_t *gofs, int 
 // ---- stage (a) last-axis transform on the tensor cores (zdft.cu) and the rest of the pair
 // transform from its output (pair_tf_ct.cuh)
 constexpr int kZdSlices = 6; // BF16 slices per operand (balanced base-256 digits)
-// row slices of nr two-float band grids psi [nr][n^3], zd_row_bytes(nr, n) bytes: images of the
-// product's shared-memory tiles, [n^2 lines][row tiles of 128][2 n / 16 stages][kZdSlices]
-cudaError_t launch_zd_rows(const void *psi, int nr, int n, void *A, cudaStream_t st);
-size_t zd_row_bytes(int nr, int n);
-// column exponents E[nb][n^2 lines] of two-float band grids psi [nb][n^3]
-cudaError_t launch_zd_colexp(const void *psi, int nb, int n, int *E, cudaStream_t st);
+// n: points of a line (the last axis), lines: n0 n1
+// row slices of nr two-float band grids psi [nr][lines][n], zd_row_bytes(nr, n, lines) bytes: images of
+// the product's shared-memory tiles, [lines][row tiles of 128][stages of 8 points][kZdSlices]
+cudaError_t launch_zd_rows(const void *psi, int nr, int n, int lines, void *A, cudaStream_t st);
+size_t zd_row_bytes(int nr, int n, int lines);
+// column exponents E[nb][lines] of two-float band grids psi [nb][lines][n]
+cudaError_t launch_zd_colexp(const void *psi, int nb, int n, int lines, int *E, cudaStream_t st);
 bool zd_supported(int n, int K2);
-int zd_valence_per_tile(int K2);
+int zd_valence_per_tile(int n, int K2);
 int zd_row_entries(int K2); // entries of F per (line, row): K2 rounded up to even
-size_t zd_smem_bytes(int n, int K2);
-// F[l][vl cb + cl][q] (two-float, zd_row_entries(K2) entries a row) = sum_i2 conj(psi_v[l][i2]) W^{kz[q] i2} psi_c[l][i2] for the
-// valence bands v = v0 + vl, vl < vb, and the cb conduction bands whose row slices A holds; tmV
-// maps the valence grids as FP32 [nv][n^2 lines][4n], box {4n, 1, zd_valence_per_tile(K2)}
+// F[l][vl cb + cl][q] (two-float, zd_row_entries(K2) entries a row) = sum_i2
+// conj(psi_v[l][i2]) W^{kz[q] i2} psi_c[l][i2] for the valence bands v = v0 + vl, vl < vb, and the cb
+// conduction bands whose row slices A holds; tmV maps the valence grids as FP32 [nv][lines][4n], box
+// {4n, 1, zd_valence_per_tile(n, K2)}, or with s = zd_line_split(n) as [nv][s lines][4n / s], box
+// {4n / s, s, zd_valence_per_tile(n, K2)}
+int zd_line_split(int n);
 cudaError_t launch_zd_gemm(const CUtensorMap &tmV, const void *A, const int *E, const int *kz, const float4 *twf, int n,
-                           int nv, int v0, int vb, int cb, int K2, float4 *F, int *status, cudaStream_t st);
+                           int lines, int nv, int v0, int vb, int cb, int K2, float4 *F, int *status, cudaStream_t st);
+// The middle and first axes from F for any n0, n1 of pair_split_supported, in two kernels with the
+// cells S [R][n0][K12] (two-float) between them: pair_split1 (tmF as below), pair_split2 (tmS: S as
+// [R n0 rows][K12] entries, FP32 elements, box {8 K2, n0}).
+bool pair_split_supported(int n);
+cudaError_t launch_pair_split1(const CUtensorMap &tmF, int64_t R, const PairPlan &pp, float4 *S, cudaStream_t st);
+cudaError_t launch_pair_split2(const CUtensorMap &tmS, int64_t R, int cb, int64_t sv, int64_t sc, const PairPlan &pp,
+                               double2 *M, cudaStream_t st);
 // M[(vl sv + cl sc) ng + g] of the block's R pairs, row vl cb + cl, from F (middle and first axis of
 // the pair transform)
 // (tmF: F as [N^2 lines][R rows of zd_row_entries(K2)] two-float entries, FP32 elements, box {4 K2, 2 N}; tmS: the plan's

@@ -10,7 +10,7 @@
 #include "internal.h"
 #include "fft.cuh"
 #include "fft_tf.cuh"
-#include "pair_tf_ct.cuh"
+#include "pair_split_ct.cuh"
 
 namespace gw {
 
@@ -390,6 +390,45 @@ size_t pair_tf_ct_smem_bytes(const PairPlan &pp)
     case 72: return pair_tf_ct_smem<72>(pp);
     default: return 0;
     }
+}
+
+bool pair_split_supported(int n)
+{
+#define GW_CASE(N) case N:
+    switch (n) {
+        GW_PAIR_SPLIT_LENGTHS(GW_CASE)
+        return true;
+    default: return false;
+    }
+#undef GW_CASE
+}
+
+cudaError_t launch_pair_split1(const CUtensorMap &tmF, int64_t R, const PairPlan &pp, float4 *S, cudaStream_t st)
+{
+    if (R == 0) return cudaSuccess;
+#define GW_CASE(N) \
+    case N: return pair_split1_n##N(tmF, R, pp, tf_consts(), S, st);
+    switch (pp.n[1]) {
+        GW_PAIR_SPLIT_LENGTHS(GW_CASE)
+    default: return cudaErrorInvalidValue;
+    }
+#undef GW_CASE
+}
+
+cudaError_t launch_pair_split2(const CUtensorMap &tmS, int64_t R, int cb, int64_t sv, int64_t sc, const PairPlan &pp,
+                               double2 *M, cudaStream_t st)
+{
+    if (R == 0) return cudaSuccess;
+    const double invd = 1.0 / ((double)pp.n[0] * pp.n[1] * pp.n[2]);
+    const float invh = (float)invd;
+    const tf inv{invh, (float)(invd - (double)invh)};
+#define GW_CASE(N) \
+    case N: return pair_split2_n##N(tmS, R, cb, sv, sc, pp, tf_consts(), inv, M, st);
+    switch (pp.n[0]) {
+        GW_PAIR_SPLIT_LENGTHS(GW_CASE)
+    default: return cudaErrorInvalidValue;
+    }
+#undef GW_CASE
 }
 
 cudaError_t launch_pair_tf_from_f(const CUtensorMap &tmF, const CUtensorMap &tmS, int64_t R, int cb, int64_t sv,

@@ -1,0 +1,12 @@
+// Middle- and first-axis kernels of the tensor-core route, axis lengths 20, 24, 25, 27, 30.
+#include "pair_split_ct.cuh"
+
+namespace gw {
+
+GW_PAIR_SPLIT_DEF(20)
+GW_PAIR_SPLIT_DEF(24)
+GW_PAIR_SPLIT_DEF(25)
+GW_PAIR_SPLIT_DEF(27)
+GW_PAIR_SPLIT_DEF(30)
+
+} // namespace gw

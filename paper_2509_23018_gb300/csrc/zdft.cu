@@ -14,7 +14,7 @@
 //     scales and the tensor cores accumulate true values;
 //   * the slice products i + j <= 5 are kept (the rest lies below 2^-48 of the operands'
 //     scales); the products with i + j = 0, 1, 2 go to three FP32 accumulators of their own:
-//     each of their terms is a multiple of one unit of that group with |sum| <= 3 * 96 * 2^14
+//     each of their terms is a multiple of one unit of that group with |sum| <= 3 * 144 * 2^14
 //     < 2^24, so those sums are exact; i + j = 3..5 share a fourth accumulator (its rounding
 //     lies 2^-48 below the leading group);
 //   * the four accumulators are summed in two-float arithmetic (two-sums for the exact groups)
@@ -104,15 +104,13 @@ __device__ __forceinline__ int zd_expo(float m)
 }
 
 // ------------------------------------------------------------------ operand tiles in shared memory
-constexpr int kZdN = 128;                              // columns per tile
 constexpr int kZdM = 128;                              // rows per tile
+constexpr int kZdAcc = 128;                            // TMEM columns per accumulator
 constexpr int kZdKB = 16;                              // real K entries per stage (8 points)
-constexpr int kZdMaxStages = 6;                        // stages per tile, 2 N / 16: N <= 48
-constexpr unsigned kZdSlice = kZdN * kZdKB * 2;        // one slice of one stage: 4 KB
+constexpr int kZdMaxStages = 9;                        // stages per tile: lines of up to 72 points
+constexpr unsigned kZdSlice = kZdM * kZdKB * 2;        // one row slice of one stage: 4 KB
 constexpr unsigned kZdStage = kZdSlices * kZdSlice;    // 24 KB
-// idesc: D = F32, A = B = BF16, both K-major, N = 128, M = 128
-constexpr uint32_t kZdIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kZdN >> 3) << 17) |
-                              ((uint32_t)(kZdM >> 4) << 24);
+static __host__ __device__ constexpr int zd_stages(int n) { return (n + 7) / 8; }
 
 // K-major operand tiles of both operands, 32-byte swizzling: row r of 32 bytes (16 BF16), 8-row
 // atoms of 256 bytes, 16-byte chunk j of row r stored at chunk j ^ ((r % 8) >> 2).
@@ -128,20 +126,20 @@ __device__ __forceinline__ uint32_t sw32_off(int r, int k) // byte offset of ele
 
 // ------------------------------------------------------------------ row slices
 // A[l][mt][ks][slice] (4 KB images of the swizzled tile of 128 rows x 16 real entries, so that one
-// bulk copy of 24 KB brings a stage) of the rows psi[r][l][.], r < nr, zero above: one warp per row
-// of a line, 8 warps per block.
+// bulk copy of 24 KB brings a stage) of the rows psi[r][l][.], r < nr, zero above and past the line's
+// n points: one warp per row of a line, 8 warps per block.
 __global__ void __launch_bounds__(256) zd_rows_kernel(const float4 *__restrict__ psi, int nr, int n, int nlines,
                                                       int nmt, unsigned char *__restrict__ A)
 {
     const int lane = threadIdx.x & 31, l = blockIdx.y, r = blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int nst = n / 8;
+    const int nst = zd_stages(n);
     unsigned char *dst = A + ((int64_t)l * nmt + r / kZdM) * nst * kZdStage;
     const int rt = r % kZdM;
     const float4 *row = psi + ((int64_t)min(r, nr - 1) * nlines + l) * n;
     float m = 0.0f;
-    float4 x[2];
+    float4 x[3];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
+    for (int u = 0; u < 3; ++u) {
         const int i = lane + 32 * u;
         x[u] = i < n && r < nr ? row[i] : make_float4(0.f, 0.f, 0.f, 0.f);
         m = fmaxf(m, fmaxf(fabsf(x[u].x), fabsf(x[u].z)) * (1.0f + 0x1p-20f));
@@ -149,9 +147,9 @@ __global__ void __launch_bounds__(256) zd_rows_kernel(const float4 *__restrict__
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     const int E = zd_expo(m);
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
+    for (int u = 0; u < 3; ++u) {
         const int i = lane + 32 * u;
-        if (i >= n) break;
+        if (i >= 8 * nst) break;
         uint16_t dr[kZdSlices], di[kZdSlices];
         zd_digits(x[u].x, x[u].y, E, dr);
         zd_digits(x[u].z, x[u].w, E, di);
@@ -178,38 +176,34 @@ __global__ void __launch_bounds__(256) zd_colexp_kernel(const float4 *__restrict
     if (lane == 0) E[w] = min(120, max(-70, zd_expo(m)));
 }
 
-size_t zd_row_bytes(int nr, int n)
+size_t zd_row_bytes(int nr, int n, int lines)
 {
-    return (size_t)n * n * ((nr + kZdM - 1) / kZdM) * (n / 8) * kZdStage;
+    return (size_t)lines * ((nr + kZdM - 1) / kZdM) * zd_stages(n) * kZdStage;
 }
 
-cudaError_t launch_zd_rows(const void *psi, int nr, int n, void *A, cudaStream_t st)
+cudaError_t launch_zd_rows(const void *psi, int nr, int n, int lines, void *A, cudaStream_t st)
 {
     const int nmt = (nr + kZdM - 1) / kZdM;
-    zd_rows_kernel<<<dim3(nmt * (kZdM / 8), n * n), 256, 0, st>>>((const float4 *)psi, nr, n, n * n, nmt,
+    zd_rows_kernel<<<dim3(nmt * (kZdM / 8), lines), 256, 0, st>>>((const float4 *)psi, nr, n, lines, nmt,
                                                                   (unsigned char *)A);
     return cudaGetLastError();
 }
 
-cudaError_t launch_zd_colexp(const void *psi, int nb, int n, int *E, cudaStream_t st)
+cudaError_t launch_zd_colexp(const void *psi, int nb, int n, int lines, int *E, cudaStream_t st)
 {
-    const int64_t warps = (int64_t)nb * n * n;
-    zd_colexp_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>((const float4 *)psi, nb, n, n * n, E);
+    const int64_t warps = (int64_t)nb * lines;
+    zd_colexp_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>((const float4 *)psi, nb, n, lines, E);
     return cudaGetLastError();
 }
-
-// Entries of F per (row, line): the kept frequencies, padded to whole 32-byte sectors.
-int zd_row_entries(int K2) { return (K2 + 1) / 2 * 2; }
-
-int zd_valence_per_tile(int K2) { return std::max(1, std::min(6, kZdN / (2 * zd_row_entries(K2)))); }
 
 // ------------------------------------------------------------------ the product
 // One block per SM, persistent over units u = (line l, valence tile of CT bands); per unit the
 // producer warps form the tile's column slices (CT bands, 2 K2P real columns each, K2 rounded up to
-// even; the others of 128 are zero), all 2 N / 16 stages of 16 real entries resident, and the block
-// runs over the row tiles of 128 conduction bands, whose slices the TMA warp copies stage by stage
-// into a ring.  One
-// thread issues the tcgen05 products into four accumulators of 128 TMEM columns each, and the
+// even; the others of 128 are zero), all stages of 16 real entries resident (points past the line's
+// end are zero), and the block runs over the row tiles of 128 conduction bands, whose slices the TMA
+// warp copies stage by stage into a ring.  Lines whose column stages leave no room for the ring (57 to
+// 72 points) take tiles of 96 columns.  One thread issues the tcgen05 products into four accumulators
+// of 128 TMEM columns each, and the
 // epilogue warps sum the accumulators into F.  A 128 x N x 16 product costs about the same time at
 // N = 64 as at N = 128 (feeding the 128 x 16 A operand sets the pace, whether A is read from shared
 // memory or from TMEM), so the tile is 128 columns wide; its four accumulators then fill the 512 TMEM
@@ -251,29 +245,38 @@ __device__ __forceinline__ float zd_2sum(float a, float b, float &e)
     return s;
 }
 
+// one slot of the line-tile ring, in float4: CT lines, to 128 bytes (TMA destinations)
+static __host__ __device__ int zd_ring_stride(int CT, int n) { return (CT * n + 7) / 8 * 8; }
+
 struct ZdArgs {
-    CUtensorMap tmV;        // valence grids as FP32 [nv][lines][4N], box {4N, 1, CT}
+    CUtensorMap tmV;        // valence grids as FP32 [nv][lines][4N], box {4N, 1, CT} (zd_line_split)
     const unsigned char *A; // row slices (zd_rows_kernel) of the block's cb conduction bands
     const int *E;           // [nv][lines] column exponents
     const int *kz;          // [K2] kept last-axis frequencies
     float4 *F;              // [lines][vb cb][K2P] two-float, row vl cb + cl
     int *status;
-    int n, nv, v0, vb, cb, K2, K2P, CT, nvt, nmt, nunits, ast; // ast: stages of the row ring
+    int n, lines, lsplit, nv, v0, vb, cb, K2, K2P, CT, nvt, nmt, nunits, ast; // ast: stages of the row ring
 };
 
+template <int NT>
 __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_constant__ ZdArgs a,
                                                                 const float4 *__restrict__ twf)
 {
+    constexpr unsigned kBSlice = NT * kZdKB * 2, kBStage = kZdSlices * kBSlice;
+    // idesc: D = F32, A = B = BF16, both K-major, N = NT, M = 128
+    constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) |
+                                ((uint32_t)(kZdM >> 4) << 24);
     extern __shared__ __align__(1024) unsigned char smraw[];
     unsigned char *sm = (unsigned char *)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
-    const int nst = a.n / 8, ncol = 2 * a.K2P;            // stages; real columns per valence band
+    const int nst = zd_stages(a.n), ncol = 2 * a.K2P;     // stages; real columns per valence band
     const uint32_t ast = a.ast;
     unsigned char *sA = sm;                               // ast x 24 KB
-    unsigned char *sB = sA + ast * kZdStage;              // nst x 24 KB
-    float4 *ring = (float4 *)(sB + nst * kZdStage);       // [slots][CT][N] valence line tiles
-    float4 *wt = ring + kZdPsiSlots * a.CT * a.n;         // [N] twiddles W^t
+    unsigned char *sB = sA + ast * kZdStage;              // nst x 24 KB (18 KB at 96 columns)
+    float4 *ring = (float4 *)(sB + nst * kBStage);        // [slots][CT][N] valence line tiles
+    const int rst = zd_ring_stride(a.CT, a.n);
+    float4 *wt = ring + kZdPsiSlots * rst;                // [N] twiddles W^t
     int2 *ctab = (int2 *)(wt + a.n);                      // [64] column pair -> (band, F offset)
-    uint64_t *bar = (uint64_t *)(ctab + kZdN / 2);
+    uint64_t *bar = (uint64_t *)(ctab + 64);
     uint64_t *aFull = bar, *aEmpty = aFull + kZdMaxRing, *bFull = aEmpty + kZdMaxRing, *bEmpty = bFull + kZdMaxStages,
              *tFull = bEmpty + kZdMaxStages, *tEmpty = tFull + 1, *pFull = tEmpty + 4, *pEmpty = pFull + kZdPsiSlots,
              *fin = pEmpty + kZdPsiSlots;
@@ -283,12 +286,12 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
     for (int i = threadIdx.x; i < a.n; i += blockDim.x) wt[i] = twf[i];
     // the epilogue's column pairs (Re, Im of entry q of band vl of the tile): vl and the offset
     // vl cb K2P + q of its F entry from the row's first (padding pairs: vl >= CT)
-    for (int pi = threadIdx.x; pi < kZdN / 2; pi += blockDim.x) {
+    for (int pi = threadIdx.x; pi < 64; pi += blockDim.x) {
         const int vl = pi / a.K2P, q = pi - vl * a.K2P;
         ctab[pi] = make_int2(vl, vl * a.cb * a.K2P + q);
     }
     // columns that no frequency fills stay zero in every stage
-    for (int i = threadIdx.x; i < nst * (int)kZdStage / 16; i += blockDim.x)
+    for (int i = threadIdx.x; i < nst * (int)kBStage / 16; i += blockDim.x)
         ((uint4 *)sB)[i] = make_uint4(0u, 0u, 0u, 0u);
     fence_async_shared();
     if (threadIdx.x == 0) {
@@ -341,12 +344,12 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                 // s + e: the sum of the groups so far and its error, from the least significant up.
                 // Registers 32 h + 4 j + 2 i + {0, 1}: row 16 h + 8 i + lane / 4, entry 4 j + lane % 4
                 uint32_t s[64], e[64];
-                GW_TMEM_LD_16X256_X8(ta + 3 * kZdN, e);
-                GW_TMEM_LD_16X256_X8(ta + 3 * kZdN + (16u << 16), e + 32);
+                GW_TMEM_LD_16X256_X8(ta + 3 * kZdAcc, e);
+                GW_TMEM_LD_16X256_X8(ta + 3 * kZdAcc + (16u << 16), e + 32);
                 tmem_wait_ld();
                 release(3);
-                GW_TMEM_LD_16X256_X8(ta + 2 * kZdN, s);
-                GW_TMEM_LD_16X256_X8(ta + 2 * kZdN + (16u << 16), s + 32);
+                GW_TMEM_LD_16X256_X8(ta + 2 * kZdAcc, s);
+                GW_TMEM_LD_16X256_X8(ta + 2 * kZdAcc + (16u << 16), s + 32);
                 tmem_wait_ld();
                 release(2);
 #pragma unroll
@@ -359,7 +362,7 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                 for (int c0 = 0; c0 < 64; c0 += 16) {
                     const uint32_t tc = ta + ((uint32_t)(c0 >> 5) << 20) + (c0 & 16) * 2;
                     uint32_t v[32];
-                    GW_TMEM_LD_16X256_X4(tc + kZdN, v);
+                    GW_TMEM_LD_16X256_X4(tc + kZdAcc, v);
                     GW_TMEM_LD_16X256_X4(tc, v + 16);
                     tmem_wait_ld();
                     if (c0 == 48) {
@@ -393,7 +396,7 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                         }
                         if (cp.x < vmax && cl < a.cb) {
                             const int64_t fi = (unit0 + cl) * a.K2P + cp.y;
-                            if (!GW_IN(fi, (int64_t)a.n * a.n * a.cb * a.vb * a.K2P, a.status)) continue;
+                            if (!GW_IN(fi, (int64_t)a.lines * a.cb * a.vb * a.K2P, a.status)) continue;
                             a.F[fi] = make_float4(h[0], y[0], h[1], y[1]);
                         }
                     }
@@ -417,7 +420,7 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                     }
                     const int l = u / a.nvt, vt = u - l * a.nvt;
                     bar_expect(&pFull[ps], pbytes);
-                    tma3(ring + ps * a.CT * a.n, &a.tmV, &pFull[ps], 0, l, a.v0 + vt * a.CT);
+                    tma3(ring + ps * rst, &a.tmV, &pFull[ps], 0, l * a.lsplit, a.v0 + vt * a.CT);
                     ++np;
                 };
                 lines(blockIdx.x);
@@ -461,8 +464,8 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
 #pragma unroll
                                 for (int j = 0; j < kZdSlices - i; ++j)
                                     if ((i + j < 3 ? i + j : 3) == g)
-                                        umma_f16(tbase + g * kZdN, ad + (uint64_t)((i * kZdSlice) >> 4),
-                                                 bd + (uint64_t)((j * kZdSlice) >> 4), kZdIdesc,
+                                        umma_f16(tbase + g * kZdAcc, ad + (uint64_t)((i * kZdSlice) >> 4),
+                                                 bd + (uint64_t)((j * kBSlice) >> 4), kIdesc,
                                                  i == 0 && j == g ? acc0 : 1u);
                         };
                         auto advance = [&] {
@@ -481,7 +484,7 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                             const uint64_t a0 = ad0 + (uint64_t)((s0 * kZdStage) >> 4);
                             advance();
                             const uint32_t s1 = as;
-                            const uint64_t a1 = ad0 + (uint64_t)((s1 * kZdStage) >> 4), b1 = bd0 + (kZdStage >> 4);
+                            const uint64_t a1 = ad0 + (uint64_t)((s1 * kZdStage) >> 4), b1 = bd0 + (kBStage >> 4);
                             if (!bar_wait(&tEmpty[3], tph)) ok = false;
                             tc_fence_after();
                             issue(3, a0, bd0, 0u);
@@ -506,7 +509,7 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                         }
                         for (int ks = 2; ks < nst && ok; ++ks) {
                             const uint64_t ad = ad0 + (uint64_t)((as * kZdStage) >> 4);
-                            const uint64_t bd = bd0 + (uint64_t)((ks * kZdStage) >> 4);
+                            const uint64_t bd = bd0 + (uint64_t)((ks * kBStage) >> 4);
                             const uint32_t cur = as;
                             advance();
                             issue(2, ad, bd, 1u);
@@ -547,24 +550,24 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                 const uint32_t ps = nu % kZdPsiSlots;
                 const bool pgot = bar_wait(&pFull[ps], (nu / kZdPsiSlots) & 1);
                 if (!__all_sync(0xffffffffu, pgot)) { ok = false; break; }
-                const float4 *pl = ring + ps * a.CT * a.n;
+                const float4 *pl = ring + ps * rst;
                 int E[kZdRounds], w[kZdRounds];
 #pragma unroll
                 for (int j = 0; j < kZdRounds; ++j) {
                     const int v = vt * a.CT + vl[j];
                     w[j] = w0[j];
-                    E[j] = vl[j] >= 0 && v < a.vb ? __ldg(a.E + (int64_t)(a.v0 + v) * a.n * a.n + l) : -70;
+                    E[j] = vl[j] >= 0 && v < a.vb ? __ldg(a.E + (int64_t)(a.v0 + v) * a.lines + l) : -70;
                 }
                 for (int ks = 0; ks < nst; ++ks) {
                     const bool got = bar_wait(&bEmpty[ks], (nu & 1) ^ 1);
                     if (!__all_sync(0xffffffffu, got)) { ok = false; break; } // warp-uniform exit
-                    unsigned char *B = sB + ks * kZdStage;
+                    unsigned char *B = sB + ks * kBStage;
 #pragma unroll
                     for (int j = 0; j < kZdRounds; ++j) {
                         if (vl[j] < 0) continue;
                         const int i2 = ks * 8 + k2;
-                        float4 x = pl[vl[j] * a.n + i2];
-                        if (vt * a.CT + vl[j] >= a.vb) x = make_float4(0.f, 0.f, 0.f, 0.f);
+                        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (i2 < a.n && vt * a.CT + vl[j] < a.vb) x = pl[vl[j] * a.n + i2];
                         const tcx b = tc_mulc(tcx{{x.x, x.y}, {x.z, x.w}}, tc_load(wt + w[j])); // conj(x) W
                         w[j] += dw[j];
                         if (w[j] >= a.n) w[j] -= a.n;
@@ -572,7 +575,7 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                         zd_digits_n(b.re.hi, b.re.lo, E[j], dr);
                         zd_digits_n(b.im.hi, b.im.lo, E[j], di);
                         const int colr = col[j];
-                        if (!GW_IN(colr + 1, kZdN, a.status)) continue;
+                        if (!GW_IN(colr + 1, NT, a.status)) continue;
                         // rows (Re c, Im c): Re column (Re b, -Im b); Im column (Im b, Re b).  The lanes of
                         // pairs 2 and 3 store their Im column first: the four pairs' columns, 64 bytes
                         // apart, would share banks two by two
@@ -582,8 +585,8 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                         for (int sl = 0; sl < kZdSlices; ++sl) {
                             const uint32_t vr = (uint32_t)dr[sl] | ((uint32_t)(di[sl] ^ 0x8000u) << 16);
                             const uint32_t vi = (uint32_t)di[sl] | ((uint32_t)dr[sl] << 16);
-                            *(uint32_t *)(p0 + sl * kZdSlice) = im ? vi : vr;
-                            *(uint32_t *)(p1 + sl * kZdSlice) = im ? vr : vi;
+                            *(uint32_t *)(p0 + sl * kBSlice) = im ? vi : vr;
+                            *(uint32_t *)(p1 + sl * kBSlice) = im ? vr : vi;
                         }
                     }
                     fence_async_shared();
@@ -601,34 +604,55 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
     if (warp == 1) tmem_dealloc(tbase, 512);
 }
 
-static size_t zd_smem(int n, int K2, int ast)
+// Entries of F per (row, line): the kept frequencies, padded to whole 32-byte sectors.
+int zd_row_entries(int K2) { return (K2 + 1) / 2 * 2; }
+
+static int zd_bands(int nt, int K2) { return std::max(1, std::min(6, nt / (2 * zd_row_entries(K2)))); }
+
+static size_t zd_smem(int n, int K2, int nt, int ast)
 {
-    return 1024 + (ast + n / 8) * (size_t)kZdStage + 16 * (size_t)kZdPsiSlots * zd_valence_per_tile(K2) * n +
-           16 * (size_t)n + 8 * (kZdN / 2) + 8 * 40 + 64;
+    return 1024 + ast * (size_t)kZdStage + zd_stages(n) * (size_t)(kZdSlices * nt * kZdKB * 2) +
+           16 * (size_t)kZdPsiSlots * zd_ring_stride(zd_bands(nt, K2), n) + 16 * (size_t)n + 8 * 64 + 8 * 48 + 64;
 }
 
-// stages of the row ring: what shared memory holds (three for 48-point lines, four for 40)
-static int zd_ring(int n, int K2)
+// The tile's columns (128, or 96 for long lines) and the stages of the row ring: what shared memory
+// holds (48-point lines: 128 columns, three stages; 72: 96 columns, two).  False: neither fits.
+static bool zd_shape(int n, int K2, int &nt, int &ast)
 {
-    int ast = kZdMaxRing;
-    while (ast > 2 && zd_smem(n, K2, ast) > (size_t)227 * 1024) --ast;
-    return ast;
+    const size_t room = (size_t)227 * 1024;
+    for (nt = 128; nt >= 96; nt -= 32)
+        if (2 * zd_row_entries(K2) <= nt && zd_smem(n, K2, nt, 2) <= room) {
+            for (ast = kZdMaxRing; zd_smem(n, K2, nt, ast) > room; --ast) {}
+            return true;
+        }
+    return false;
 }
 
-size_t zd_smem_bytes(int n, int K2) { return zd_smem(n, K2, zd_ring(n, K2)); }
-
-// The route's shapes: lines of 40 or 48 points (the grids whose remaining axes are built from F), at
-// most 32 kept frequencies, and the block's shared memory (column stages, ring of row stages, line
-// tiles) within the 227 KB a block may opt into.
+// The route's shapes: lines of 24 to 72 points (at least three stages; 3 * 144 * 2^14 < 2^24), at most
+// 32 kept frequencies.
 bool zd_supported(int n, int K2)
 {
-    return (n == 40 || n == 48) && K2 >= 1 && K2 <= 32 && zd_smem_bytes(n, K2) <= (size_t)227 * 1024;
+    int nt, ast;
+    return n >= 24 && n <= 8 * kZdMaxStages && n % zd_line_split(n) == 0 && K2 >= 1 && K2 <= 32 &&
+           zd_shape(n, K2, nt, ast);
+}
+
+// A tensor map's box takes 256 entries: longer lines (4 n FP32) are mapped as two.
+int zd_line_split(int n) { return n > 64 ? 2 : 1; }
+
+int zd_valence_per_tile(int n, int K2)
+{
+    int nt = 128, ast = 2;
+    zd_shape(n, K2, nt, ast);
+    return zd_bands(nt, K2);
 }
 
 cudaError_t launch_zd_gemm(const CUtensorMap &tmV, const void *A, const int *E, const int *kz, const float4 *twf, int n,
-                           int nv, int v0, int vb, int cb, int K2, float4 *F, int *status, cudaStream_t st)
+                           int lines, int nv, int v0, int vb, int cb, int K2, float4 *F, int *status, cudaStream_t st)
 {
     ZdArgs a;
+    int nt;
+    if (!zd_shape(n, K2, nt, a.ast)) return cudaErrorInvalidValue;
     a.tmV = tmV;
     a.A = (const unsigned char *)A;
     a.E = E;
@@ -636,25 +660,27 @@ cudaError_t launch_zd_gemm(const CUtensorMap &tmV, const void *A, const int *E, 
     a.F = F;
     a.status = status;
     a.n = n;
+    a.lines = lines;
+    a.lsplit = zd_line_split(n);
     a.nv = nv;
     a.v0 = v0;
     a.vb = vb;
     a.cb = cb;
     a.K2 = K2;
     a.K2P = zd_row_entries(K2);
-    a.ast = zd_ring(n, K2);
-    a.CT = zd_valence_per_tile(K2);
+    a.CT = zd_bands(nt, K2);
     a.nvt = (vb + a.CT - 1) / a.CT;
     a.nmt = (cb + kZdM - 1) / kZdM;
-    a.nunits = n * n * a.nvt;
-    const size_t sm = zd_smem_bytes(n, K2);
-    cudaError_t e = cudaFuncSetAttribute(zd_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    a.nunits = lines * a.nvt;
+    const size_t sm = zd_smem(n, K2, nt, a.ast);
+    auto kernel = nt == 96 ? zd_gemm_kernel<96> : zd_gemm_kernel<128>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return e;
-    zd_gemm_kernel<<<std::min(a.nunits, sms), kZdThreads, sm, st>>>(a, twf);
+    kernel<<<std::min(a.nunits, sms), kZdThreads, sm, st>>>(a, twf);
     return cudaGetLastError();
 }
 
