@@ -73,7 +73,10 @@ typedef enum {
  * carry more work per useful bit on a slower pipe.  gw_chi0_create rejects it with GW_ERR_ARG.
  */
 typedef enum {
-    GW_PREC_FP64 = 0,      /* FP64 FFT + FP64 tensor-core (DMMA) contraction */
+    GW_PREC_FP64 = 0,      /* FP64 FFT + contraction to FP64 accuracy: of computed pair elements by seven
+                              nine-bit slices on the BF16 tensor cores (62 bits of a column's largest
+                              entry, whole-number sums), otherwise on the FP64 tensor cores (DMMA);
+                              a budget without room for the slices leaves all of it to DMMA */
     GW_PREC_OZAKI_BF16 = 1 /* FP64 FFT + split-precision contraction on BF16 tensor cores */
 } gw_prec;
 

@@ -116,9 +116,9 @@ gw_status batch_oz_split(gw_chi0 *h, int nq, int w, const BatchLayout &L)
         const int ng = L.ng[sg.q];
         const double *sp = h->SPall + L.doff[sg.q] + (int64_t)w * L.P[sg.q] + sg.p0;
         const double2 *M = h->Mall + L.moff[sg.q] + sg.p0 * ng;
-        CK(h, gw::launch_oz_colexp(M, sg.cnt, ng, sp, h->Eall + sg.eoff, h->st), "oz exponents");
+        CK(h, gw::launch_oz_colexp(M, sg.cnt, ng, sp, h->Eall + sg.eoff, nullptr, h->st), "oz exponents");
         CK(h, gw::launch_oz_slice(M, sg.cnt, ng, sp, h->Eall + sg.eoff, gw::oz_slices(h->d.nslices), sg.kpad,
-                                  (uint16_t *)h->Zall + sg.zoff, h->st),
+                                  (uint16_t *)h->Zall + sg.zoff, nullptr, h->st),
            "oz slices");
     }
     return GW_OK;
@@ -280,7 +280,7 @@ gw_status compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const double 
                                                                                    (j.ntile + 1) / 2));
                 const int grid = std::max(1, std::min(nitems, 2 * num_sms()));
                 if (gw::launch_contract_f64_jobs(h->tuned_bt, (const gw::F64Job *)ng.jobs, (int)fj.size(), nitems,
-                                                 grid, h->status, h->st) != cudaSuccess)
+                                                 grid, h->status, nullptr, h->st) != cudaSuccess)
                     body = fail(h, GW_ERR_CUDA, "capture: contraction");
             } else if (!body) {
                 for (int w = 0; w < nw && !body; ++w) {
@@ -288,7 +288,8 @@ gw_status compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const double 
                     if (body) break;
                     if (gw::launch_oz_gemm_jobs((const gw::OzJob *)((char *)ng.jobs + offs[w]),
                                                 (const gw::OzItem *)((char *)ng.jobs + offs[nw]), (int)items.size(),
-                                                oz_clusters(items.size()), oz_scratch(h), h->status, h->st) != cudaSuccess)
+                                                oz_clusters(items.size()), oz_scratch(h), h->status, nullptr,
+                                                h->st) != cudaSuccess)
                         body = fail(h, GW_ERR_CUDA, "capture: split contraction");
                 }
             }

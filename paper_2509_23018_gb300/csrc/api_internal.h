@@ -81,6 +81,9 @@ struct gw_chi0 {
     size_t dcap = 0;
     // split-precision work buffers
     void *Zbuf = nullptr;      // bf16 slices [s][2 ng][kpad]
+    int *f64guard = nullptr;   // set by the slicing kernels where the sliced FP64 contraction does not hold
+    size_t f64guard_cap = 0;
+    bool zbusy = false;        // Zbuf is in use by the call that allocates (see dalloc)
     size_t Zcap = 0;           // bytes
     double *spbuf = nullptr;   // sqrt(-Delta) [nw][chunk]
     size_t spcap = 0;
@@ -232,18 +235,20 @@ gw_status upload_jobs(gw_chi0 *h, const void *src, size_t bytes, const void **de
 gw_status f64_jobs(gw_chi0 *h, std::vector<gw::F64Job> &jobs, const double2 *M, int64_t P, int ng,
                    const double *delta, int64_t dstride, int nw, double2 *chi, int bt);
 int f64_schedule(std::vector<gw::F64Job> &jobs, int waves);
-gw_status launch_f64_jobs(gw_chi0 *h, std::vector<gw::F64Job> &jobs, int bt, int waves);
+gw_status launch_f64_jobs(gw_chi0 *h, std::vector<gw::F64Job> &jobs, int bt, int waves, const int *guard = nullptr);
 gw_status make_tmap_z(gw_chi0 *h, CUtensorMap *map, void *Z, int64_t kpad, int nrows, int s, int box_rows);
-gw_status oz_job(gw_chi0 *h, gw::OzJob &j, void *Z, int64_t kpad, int ng, const int *E, double2 *chi);
+// nslices: 9-bit slices, 0 for the handle's
+gw_status oz_job(gw_chi0 *h, gw::OzJob &j, void *Z, int64_t kpad, int ng, const int *E, double2 *chi, int nslices = 0);
 int oz_clusters(size_t nitems);
 gw_status oz_items(gw_chi0 *h, std::vector<gw::OzJob> &jobs, std::vector<gw::OzItem> &items);
 inline gw::OzScratch oz_scratch(const gw_chi0 *h) { return {h->ozpart, h->ozflags}; }
 gw_status launch_oz_general(gw_chi0 *h, const std::vector<gw::OzJob> &jobs);
-gw_status launch_oz_jobs(gw_chi0 *h, std::vector<gw::OzJob> &jobs);
+gw_status launch_oz_jobs(gw_chi0 *h, std::vector<gw::OzJob> &jobs, const int *guard = nullptr);
 gw_status contract_chunk_ozaki(gw_chi0 *h, const double2 *M, int64_t P, int ng, const double *delta, int64_t dstride,
                                int nw, double2 *chi);
+// given: M comes from the caller of the API rather than from the bands
 gw_status contract_chunk(gw_chi0 *h, const double2 *M, int64_t P, int ng, const double *delta, int64_t dstride,
-                         int nw, double2 *chi);
+                         int nw, double2 *chi, bool given = false);
 int64_t oz_kpad(int ka);
 // nslices > 0 overrides the handle's slice count (both calls of one product must agree)
 gw_status oz_prepare_b(gw_chi0 *h, const double2 *B, int ka, int nout, int nslices = 0);

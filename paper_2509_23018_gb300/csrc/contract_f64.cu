@@ -13,6 +13,9 @@
 // list of work items (job, upper tile, pair split), ordered largest job first; block b
 // takes items b, b + gridDim.x, ...  Partial tiles are added into chi with FP64 atomics.
 // The tile edge is a template parameter chosen by the autotuner (32 or 64 complex).
+//
+// It serves pair elements that the caller passes in, batches, calls of few pairs, and the chunks that the
+// contraction by slices (ozaki.cu) gives back.
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -27,8 +30,9 @@ constexpr size_t f64_smem() { return 2 * (size_t)kF64Stages * kF64BK * 2 * BT * 
 
 template <int BT>
 __global__ void __launch_bounds__(kF64Threads) contract_f64_kernel(const F64Job *__restrict__ jobs, int njobs,
-                                                                   int nitems, int *status)
+                                                                   int nitems, int *status, const int *guard)
 {
+    if (guard && *guard == 0) return; // the sliced contraction took the chunk
     constexpr int WR = BT / 2, WC = BT / 4, MT = WR / 8, NT = WC / 8;
     constexpr unsigned kTileBytes = kF64BK * BT * 2 * sizeof(double);
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -165,19 +169,19 @@ int contract_f64_bk() { return kF64BK; }
 size_t contract_f64_smem(int bt) { return bt == 32 ? f64_smem<32>() : f64_smem<64>(); }
 
 cudaError_t launch_contract_f64_jobs(int bt, const F64Job *jobs, int njobs, int nitems, int grid, int *status,
-                                     cudaStream_t st)
+                                     const int *guard, cudaStream_t st)
 {
     if (nitems == 0) return cudaSuccess;
     if (bt == 32) {
         cudaError_t e = cudaFuncSetAttribute(contract_f64_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)f64_smem<32>());
         if (e != cudaSuccess) return e;
-        contract_f64_kernel<32><<<grid, kF64Threads, f64_smem<32>(), st>>>(jobs, njobs, nitems, status);
+        contract_f64_kernel<32><<<grid, kF64Threads, f64_smem<32>(), st>>>(jobs, njobs, nitems, status, guard);
     } else {
         cudaError_t e = cudaFuncSetAttribute(contract_f64_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)f64_smem<64>());
         if (e != cudaSuccess) return e;
-        contract_f64_kernel<64><<<grid, kF64Threads, f64_smem<64>(), st>>>(jobs, njobs, nitems, status);
+        contract_f64_kernel<64><<<grid, kF64Threads, f64_smem<64>(), st>>>(jobs, njobs, nitems, status, guard);
     }
     return cudaGetLastError();
 }

@@ -137,7 +137,8 @@ struct __align__(128) F64Job {
     int64_t P;
     int ng, ntile, ksplit, item_start;
 };
-cudaError_t launch_contract_f64_jobs(int bt, const F64Job *jobs, int njobs, int nitems, int grid, int *status,
+// guard (or null): runs only where *guard is set
+cudaError_t launch_contract_f64_jobs(int bt, const F64Job *jobs, int njobs, int nitems, int grid, int *status, const int *guard,
                                      cudaStream_t st);
 int contract_f64_bk();
 size_t contract_f64_smem(int bt);
@@ -145,8 +146,10 @@ size_t contract_f64_smem(int bt);
 // ---- stage (b), split precision on BF16 tensor cores (ozaki.cu)
 // sp[i] = sqrt(-delta[i])
 cudaError_t launch_oz_sqrt(const double *delta, int64_t n, double *sp, cudaStream_t st);
-// E[g] = column exponent of s_p M[p][g] over the chunk
-cudaError_t launch_oz_colexp(const double2 *M, int64_t P, int ng, const double *sp, int *E, cudaStream_t st);
+// E[g] = column exponent of s_p M[p][g] over the chunk; guard (or null): set to 1 where the FP64
+// contraction by slices does not hold (entries not finite, columns scaled by more than 2^+-390)
+cudaError_t launch_oz_colexp(const double2 *M, int64_t P, int ng, const double *sp, int *E, int *guard,
+                             cudaStream_t st);
 // A group of nw <= oz_group_w() frequencies at once (scales sp + w dstride): exponents E[w][ng],
 // slices of frequency w at Z + w zstride (bf16 elements); M read once per pass for the group.
 int oz_group_w();
@@ -154,7 +157,8 @@ cudaError_t launch_oz_split_multi(const double2 *M, int64_t P, int ng, const dou
                                   int *E, int s, int64_t kpad, void *Z, int64_t zstride, cudaStream_t st);
 // Z[i][j][p] bf16 slices, rows p in [P, kpad) zero
 cudaError_t launch_oz_slice(const double2 *M, int64_t P, int ng, const double *sp, const int *E, int s,
-                            int64_t kpad, void *Z, cudaStream_t st);
+                            int64_t kpad, void *Z, int *guard, cudaStream_t st);
+int oz_f64_slices(); // slices of the FP64 contraction
 // One job = the split contraction of one chunk into one chi block (upper tiles).
 struct __align__(128) OzJob {
     CUtensorMap tmA, tmB; // slices [s][2 ng][kpad] bf16, boxes {64, 128}
@@ -183,9 +187,10 @@ struct OzScratch {
 };
 size_t oz_part_bytes();
 int oz_slot_flags();
-// clusters: pairs of CTAs
+// clusters: pairs of CTAs; guard (or null): the FP64 contraction (oz_f64_slices() slices), which leaves
+// the chunk alone where *guard is set
 cudaError_t launch_oz_gemm_jobs(const OzJob *jobs, const OzItem *items, int nitems, int clusters, OzScratch scr,
-                                int *status, cudaStream_t st);
+                                int *status, const int *guard, cudaStream_t st);
 int oz_slices(int nslices); // 9-bit slices for the accuracy of nslices six-bit ones
 // Slices of the general split product Y = A B: the rows of A or the columns of B, `rows` of them
 // with ka complex entries each, entry g of row p at A[p sr + g sk], into s nine-bit BF16 slices

@@ -146,7 +146,7 @@ extern "C" gw_status gw_chi0_contract_noalloc(int nv, int nc, const double *ev, 
         return GW_ERR_CUDA;
     }
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(items, 2LL * sms));
-    if (gw::launch_contract_f64_jobs(kNoAllocTile, djobs, nw, items, grid, status, st) != cudaSuccess ||
+    if (gw::launch_contract_f64_jobs(kNoAllocTile, djobs, nw, items, grid, status, nullptr, st) != cudaSuccess ||
         gw::launch_symmetrize((double2 *)chi, ng, nw, st) != cudaSuccess) {
         cudaGetLastError();
         return GW_ERR_CUDA;

@@ -19,8 +19,13 @@
 // epilogue adds the segments, times 2^(-9 (t - 2)), in two-float arithmetic in registers and adds
 //     chi += -2^(E_G + E_G' - 16) (hi + lo)
 // once per tile in FP64, with atomic adds so that the chunks (pair segments) of one chi block may
-// run concurrently in one launch (one chunk's sums are the same bits in every run).  FP64 is kept for Delta, the scaling, the accumulation across
-// chunks and the symmetrisation.
+// run concurrently in one launch (one chunk's sums are the same bits in every run).  FP64 is kept for
+// Delta, the scaling, the accumulation across chunks and the symmetrisation.
+//
+// The FP64 contraction of computed pair elements takes the same route with seven slices (62 bits of
+// each column's largest entry, where a double keeps 53 of each entry) and without any FP32 sum beyond
+// a segment: the segments' sums, whole numbers, are added as 64-bit integers over a K block of 1024
+// pairs, and the blocks in FP64 (OzProd::F64 below).
 #include "internal.h"
 #include "ptx.cuh"
 #include "fft_tf.cuh"
@@ -39,6 +44,8 @@ int oz_slices(int nslices) { return nslices <= 4 ? 3 : nslices == 5 ? 4 : nslice
 constexpr int kOzBM = 128, kOzBK = 64; // rows of A (and of B) per CTA of a pair; K entries per ring stage
 constexpr int kOzThreads = 384;        // a warpgroup with the TMA and MMA warps, two of epilogue warps
 constexpr int kOzNoColumn = -400;      // exponent of an all-zero column
+constexpr int kOzMaxExpo = 390;        // exponents that the FP64 contraction's scaling takes, +-
+constexpr int kOzF64Slices = 7;
 
 // K runs in blocks of kOzKBlock K-steps (of 64 entries), every slice group over one block before
 // the next, so that a slice comes from DRAM once per block and from L2 for its other products.
@@ -47,7 +54,13 @@ constexpr int kOzNoColumn = -400;      // exponent of an all-zero column
 constexpr int kOzKBlock = 16;
 // K-steps that slice group t sums in FP32 before the epilogue takes the sum (bounds at the top of
 // this file)
-__device__ __forceinline__ int oz_segment(int t) { return t == 2 ? 8 : t <= 4 ? 4 : kOzKBlock; }
+// (F64: four K-steps for every group: below 2^24 unless 256 pairs' digits are all near their largest
+// with one sign)
+template <bool F64>
+__device__ __forceinline__ int oz_segment(int t)
+{
+    return t == 2 ? 8 : t <= 4 || F64 ? 4 : kOzKBlock;
+}
 
 // ------------------------------------------------------------------ split, step 1: column exponents
 // E[g] = max_p ilogb(max(|Re A|, |Im A|)) + 2 over the chunk, A = s_p M[p][g].
@@ -57,8 +70,11 @@ __global__ void oz_sqrt_kernel(const double *__restrict__ delta, int64_t n, doub
     if (i < n) sp[i] = sqrt(-delta[i]);
 }
 
+// GUARD: sets *guard where an entry is not finite or a column's scale is out of range (FP64
+// contraction: the DMMA kernel then takes the chunk).
+template <bool GUARD>
 __global__ void oz_colexp_kernel(const double2 *__restrict__ M, int64_t P, int ng, const double *__restrict__ sp,
-                                 int *__restrict__ E)
+                                 int *__restrict__ E, int *guard)
 {
     __shared__ int red[8][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -69,6 +85,8 @@ __global__ void oz_colexp_kernel(const double2 *__restrict__ M, int64_t P, int n
             const double2 m = M[p * ng + g];
             const double a = oz_bits_d(oz_absmax_bits(m.x, m.y)) * sp[p];
             e = max(e, oz_expo_pos(a, kOzNoColumn));
+            if constexpr (GUARD)
+                if ((oz_dbits(a) & 0x7fffffffffffffffull) >= 0x7ff0000000000000ull || e > kOzMaxExpo) *guard = 1;
         }
     }
     red[wid][lane] = e;
@@ -132,9 +150,11 @@ __device__ __forceinline__ void oz_store_row_digits(const long long nb[16], int 
 // Five blocks per SM (48 registers, a 24-byte spill) keep more of the 16 loads per thread in flight
 // than the four the unconstrained build allows: the split preparation of a 48^3 q-point (16 chunks)
 // takes 5.04 against 5.32 ms (six blocks, 40 registers and a 60-byte spill: 5.17 ms).
+// GUARD: as in oz_colexp_kernel, for a column that is not zero but below the exponent range.
+template <bool GUARD>
 __global__ void __launch_bounds__(256, 5) oz_slice_kernel(const double2 *__restrict__ M, int64_t P, int ng,
                                                        const double *__restrict__ spv, const int *__restrict__ E,
-                                                       int s, int64_t kpad, __nv_bfloat16 *__restrict__ Z)
+                                                       int s, int64_t kpad, __nv_bfloat16 *__restrict__ Z, int *guard)
 {
     const int64_t p0 = (int64_t)blockIdx.y * 64;
     const OzTileThread tt = oz_tile_thread();
@@ -149,6 +169,8 @@ __global__ void __launch_bounds__(256, 5) oz_slice_kernel(const double2 *__restr
     for (int t = 0; t < 16; ++t) {
         const int64_t p = p0 + tt.pl0 + t;
         const double a = p < P ? Md[2 * (p * ng + g) + tt.c] * spv[p] : 0.0;
+        if constexpr (GUARD)
+            if (E[g] < -kOzMaxExpo && a != 0.0) *guard = 1;
         nb[t] = oz_round_scaled(a, sh) + bias;
     }
     const int64_t j = 2 * (int64_t)g + tt.c;
@@ -491,10 +513,14 @@ struct OzCfg {
 
 // The segments of an item of nk K-steps with s slices, in the order every role walks them: K block
 // by K block, from the least significant group up, the group's segments of the block.
+template <bool F64>
 struct OzSegments {
     int nk, s, kc, t, k0, len;
     __device__ __forceinline__ OzSegments(int nk_, int s_) : nk(nk_), s(s_), kc(0), t(s_ + 1), k0(0) { cut(); }
-    __device__ __forceinline__ void cut() { len = min(min(nk, kc + kOzKBlock) - k0, oz_segment(t)); }
+    __device__ __forceinline__ void cut() { len = min(min(nk, kc + kOzKBlock) - k0, oz_segment<F64>(t)); }
+    // of a K block: first segment of its group, last segment of all
+    __device__ __forceinline__ bool opens() const { return k0 == kc; }
+    __device__ __forceinline__ bool closes() const { return t == 2 && k0 + len >= min(nk, kc + kOzKBlock); }
     __device__ __forceinline__ bool more() const { return kc < nk; }
     __device__ __forceinline__ void next()
     {
@@ -532,15 +558,32 @@ __device__ __forceinline__ double oz_scaled_double(float x, int ex)
                             (int)(u << 29));
 }
 
-// GEN = false: the Hermitian contraction above (upper tiles, chi epilogue).  GEN = true: the
-// general product out += A B (all tiles, each owned by one pair of CTAs, plain FP64 adds).
-template <bool GEN>
+// where an epilogue thread's sums belong: complex row g of nr, columns g0 .. of nc
+struct OzPlace {
+    int g, g0, nr, nc, eg;
+    const int *ecol;
+    double *row, *part;
+};
+
+// Split: the Hermitian contraction above (upper tiles, chi epilogue), two-float sums.  General: the
+// product out += A B (all tiles, each owned by one pair of CTAs, plain FP64 adds).  F64: the Hermitian
+// contraction with seven slices, sums exact up to the last unit of a 64-bit integer per K block of 1024
+// pairs: groups t = 8..5 in units of 2^-54 (|sum| < 2^57), rounded to units of 2^-37 before t = 4..2
+// (|sum| <= 2 1024 2^14 2^37 = 2^62), 2^-51 of a pair's largest product.  A block's sum goes to chi (or
+// to the part's place in scratch) in FP64, so a chunk of 8192 pairs is rounded eight times where a chain
+// of DMMAs is rounded 2048 times.  Measured on a chunk of 8192 pairs, N_G = 2000: 2.55 ms
+// (28 products, 1.4 PFLOP/s) and 0.33 ms for the slices where the DMMA kernel, at 0.86 of its pipe's rate,
+// takes 138; error of chi against 64 bits 1.1e-15 where it leaves 1.9e-15.
+enum class OzProd { Split, General, F64 };
+template <OzProd MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
     oz_gemm_kernel(const OzJob *__restrict__ jobs, const OzItem *__restrict__ items, int nitems, OzScratch scr,
-                   int *status)
+                   int *status, const int *guard)
 {
     using C = OzCfg;
     constexpr int ST = C::Stages, NB = C::Bufs;
+    constexpr bool GEN = MODE == OzProd::General, F64 = MODE == OzProd::F64;
+    if (F64 && *guard) return; // the DMMA kernel takes the chunk
     extern __shared__ __align__(1024) unsigned char smraw[];
     unsigned char *sm = (unsigned char *)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
     unsigned char *sA = sm;                 // [stages][Bytes]
@@ -586,7 +629,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
                 const OzItem w = items[item];
                 const OzJob &jb = jobs[w.job];
                 const int ra = (2 * w.I + (int)rank) * kOzBM, rb = (2 * w.J + (int)rank) * kOzBM;
-                for (OzSegments g(w.nk, jb.s); g.more() && ok; g.next())
+                for (OzSegments<F64> g(w.nk, jb.s); g.more() && ok; g.next())
                     for (int i = 1; i < g.t && ok; ++i)
                         for (int kb = 0; kb < g.len; ++kb, ++it) {
                             const uint32_t st = it % ST;
@@ -606,7 +649,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
             uint32_t it = 0, seg = 0;
             for (int item = cl0; item < nitems && ok; item += ncl) {
                 const OzItem w = items[item];
-                for (OzSegments g(w.nk, jobs[w.job].s); g.more() && ok; g.next(), ++seg) {
+                for (OzSegments<F64> g(w.nk, jobs[w.job].s); g.more() && ok; g.next(), ++seg) {
                     const uint32_t b = seg % NB;
                     if (!pair_wait(&tempty[b], ((seg / NB) & 1) ^ 1)) { ok = false; break; }
                     tc_fence_after();
@@ -646,19 +689,50 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
         // from the neighbouring lane.
         const uint32_t flip = !GEN && odd ? 0x80000000u : 0u, rflip = GEN && !odd ? 0x80000000u : 0u;
         const uint32_t tempty0 = cluster_map(tempty, 0);
-        float hi[NO], lo[NO];
+        constexpr int64_t kPart = 2 * 8 * 32 * NO; // doubles of one part
+        auto place = [&](const OzItem &w, const OzJob &jb) {
+            OzPlace p;
+            p.g = (2 * w.I + (int)rank) * (kOzBM / 2) + (r >> 1);
+            p.g0 = w.J * kOzBM + half * NO;
+            p.nr = GEN ? jb.rows_a : jb.ng;
+            p.nc = GEN ? jb.cols_b : jb.ng;
+            p.ecol = GEN ? jb.E2 : jb.E;
+            p.eg = p.g < p.nr ? __ldg(jb.E + p.g) - 16 : 0;
+            p.row = (GEN ? jb.out + (int64_t)p.g * jb.ldo : jb.chi + 2 * (int64_t)p.g * jb.ng) + 2 * p.g0 + odd;
+            // a part of a split tile: this warp's sums go to its place in scratch, lane by lane
+            p.part = !GEN && w.parts > 1 ? scr.sums + ((int64_t)w.slot * w.parts + w.part) * kPart +
+                                               ((int)rank * 8 + warp - 4) * (32 * NO) + lane
+                                         : nullptr;
+            return p;
+        };
+        float hi[F64 ? 1 : NO], lo[F64 ? 1 : NO];
+        long long acc[F64 ? NO : 1];
         uint32_t seg = 0;
         for (int item = cl0; item < nitems && ok; item += ncl) {
             const OzItem w = items[item];
             const OzJob &jb = jobs[w.job];
+            if constexpr (!F64) {
 #pragma unroll
-            for (int j = 0; j < NO; ++j) hi[j] = lo[j] = 0.0f;
-            for (OzSegments g(w.nk, jb.s); g.more(); g.next(), ++seg) {
+                for (int j = 0; j < NO; ++j) hi[j] = lo[j] = 0.0f;
+            }
+            for (OzSegments<F64> sg(w.nk, jb.s); sg.more(); sg.next(), ++seg) {
                 const uint32_t b = seg % NB;
                 const bool got = pair_wait(&tfull[b], (seg / NB) & 1);
                 if (!__all_sync(0xffffffffu, got)) { ok = false; break; } // warp-uniform exit
                 tc_fence_after();
-                const float wt = __int_as_float((127 - kOzBeta * (g.t - 2)) << 23); // the group's weight
+                const float wt = __int_as_float((127 - kOzBeta * (sg.t - 2)) << 23); // the group's weight
+                if constexpr (F64) {
+                    if (sg.opens() && sg.t == jb.s + 1) {
+#pragma unroll
+                        for (int j = 0; j < NO; ++j) acc[j] = 0;
+                    } else if (sg.opens() && sg.t == 4) {
+#pragma unroll
+                        for (int j = 0; j < NO; ++j) acc[j] = (acc[j] + (1 << 16)) >> 17;
+                    }
+                }
+                // F64: the group's unit is 2^ush of the sum's (t = 2: 2^37, into the high word)
+                const int ush = sg.t >= 5 ? kOzBeta * (8 - sg.t) : 37 - kOzBeta * (sg.t - 2);
+                const int umul = sg.t == 2 ? 0 : 1 << ush, hmul = sg.t == 2 ? 1 << (ush - 32) : 0;
                 const uint32_t ta = tbase + ((uint32_t)(q * 32) << 16) + b * C::Cols + half * COLS;
 #pragma unroll
                 for (int c0 = 0; c0 < COLS; c0 += 32) {
@@ -669,31 +743,42 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
                     for (int cc = 0; cc < 16; ++cc) {
                         const uint32_t rv = __shfl_xor_sync(0xffffffffu, v[2 * cc + 1], 1) ^ rflip;
                         const float x = __fadd_rn(__uint_as_float(v[2 * cc] ^ flip), __uint_as_float(rv));
-                        oz_add(hi[(c0 >> 1) + cc], lo[(c0 >> 1) + cc], __fmul_rn(wt, x));
+                        if constexpr (F64) {
+                            const int xi = __float2int_rn(x);
+                            acc[(c0 >> 1) + cc] += (long long)xi * umul + ((long long)(xi * hmul) << 32);
+                        } else {
+                            oz_add(hi[(c0 >> 1) + cc], lo[(c0 >> 1) + cc], __fmul_rn(wt, x));
+                        }
                     }
                 }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) bar_arrive_cluster(tempty0 + 8 * b);
+                if constexpr (F64) {
+                    if (sg.closes()) { // the K block's sums, |E| <= 400: the scale is a normal number
+                        const OzPlace p = place(w, jb);
+#pragma unroll
+                        for (int j = 0; j < NO; ++j)
+                            if (p.g < p.nr && p.g0 + j < p.nc && p.g <= p.g0 + j) {
+                                const int ex = p.eg + __ldg(p.ecol + p.g0 + j) - 37;
+                                const double y = (double)acc[j] * __hiloint2double((1023 + ex) << 20, 0);
+                                if (p.part) __stcg(p.part + 32 * j, sg.kc == 0 ? y : __ldcg(p.part + 32 * j) + y);
+                                else if (y != 0.0) atomicAdd(p.row + 2 * j, -y);
+                            }
+                    }
+                }
             }
             if (!ok) break;
-            const int g = (2 * w.I + (int)rank) * (kOzBM / 2) + (r >> 1); // complex row
-            const int g0 = w.J * kOzBM + half * NO;                       // first complex column
-            const int nr = GEN ? jb.rows_a : jb.ng, nc = GEN ? jb.cols_b : jb.ng;
-            const int *ecol = GEN ? jb.E2 : jb.E;
-            const int eg = g < nr ? __ldg(jb.E + g) - 16 : 0;
-            double *row = (GEN ? jb.out + (int64_t)g * jb.ldo : jb.chi + 2 * (int64_t)g * jb.ng) + 2 * g0 + odd;
-            // a part of a split tile: this warp's sums go to its place in scratch, lane by lane
-            double *part = nullptr;
-            constexpr int64_t kPart = 2 * 8 * 32 * NO; // doubles of one part
-            if (!GEN && w.parts > 1)
-                part = scr.sums + ((int64_t)w.slot * w.parts + w.part) * kPart +
-                       ((int)rank * 8 + warp - 4) * (32 * NO) + lane;
+            const OzPlace p = place(w, jb);
+            const int g = p.g, g0 = p.g0, nr = p.nr, nc = p.nc, eg = p.eg;
+            const int *ecol = p.ecol;
+            double *row = p.row, *part = p.part;
 #pragma unroll
             for (int j = 0; j < NO; ++j)
-                if (g < nr && g0 + j < nc && (GEN || g <= g0 + j)) {
+                if (!F64 && g < nr && g0 + j < nc && (GEN || g <= g0 + j)) {
                     const int ex = eg + __ldg(ecol + g0 + j);
-                    const double y = oz_scaled_double(hi[j], ex) + oz_scaled_double(lo[j], ex);
+                    const int q = F64 ? 0 : j;
+                    const double y = oz_scaled_double(hi[q], ex) + oz_scaled_double(lo[q], ex);
                     if constexpr (GEN) row[2 * j] += y; // the tile belongs to this pair of CTAs alone
                     else if (part) __stcg(part + 32 * j, y);
                     else if (y != 0.0) atomicAdd(row + 2 * j, -y); // other pair segments may add here too
@@ -747,13 +832,16 @@ cudaError_t launch_oz_sqrt(const double *delta, int64_t n, double *sp, cudaStrea
     return cudaGetLastError();
 }
 
-cudaError_t launch_oz_colexp(const double2 *M, int64_t P, int ng, const double *sp, int *E, cudaStream_t st)
+cudaError_t launch_oz_colexp(const double2 *M, int64_t P, int ng, const double *sp, int *E, int *guard,
+                             cudaStream_t st)
 {
     oz_fill_kernel<<<(ng + 255) / 256, 256, 0, st>>>(E, ng, kOzNoColumn);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || P == 0) return e;
     int gy = (int)std::min<int64_t>((P + 63) / 64, 256);
-    oz_colexp_kernel<<<dim3((ng + 31) / 32, gy), 256, 0, st>>>(M, P, ng, sp, E);
+    const dim3 grid((ng + 31) / 32, gy);
+    if (guard) oz_colexp_kernel<true><<<grid, 256, 0, st>>>(M, P, ng, sp, E, guard);
+    else oz_colexp_kernel<false><<<grid, 256, 0, st>>>(M, P, ng, sp, E, guard);
     return cudaGetLastError();
 }
 
@@ -777,38 +865,42 @@ cudaError_t launch_oz_split_multi(const double2 *M, int64_t P, int ng, const dou
 }
 
 cudaError_t launch_oz_slice(const double2 *M, int64_t P, int ng, const double *sp, const int *E, int s,
-                            int64_t kpad, void *Z, cudaStream_t st)
+                            int64_t kpad, void *Z, int *guard, cudaStream_t st)
 {
-    oz_slice_kernel<<<dim3((ng + 31) / 32, (unsigned)(kpad / 64)), 256, 0, st>>>(M, P, ng, sp, E, s, kpad,
-                                                                                  (__nv_bfloat16 *)Z);
+    const dim3 grid((ng + 31) / 32, (unsigned)(kpad / 64));
+    if (guard) oz_slice_kernel<true><<<grid, 256, 0, st>>>(M, P, ng, sp, E, s, kpad, (__nv_bfloat16 *)Z, guard);
+    else oz_slice_kernel<false><<<grid, 256, 0, st>>>(M, P, ng, sp, E, s, kpad, (__nv_bfloat16 *)Z, guard);
     return cudaGetLastError();
 }
 
-template <bool GEN>
+template <OzProd MODE>
 static cudaError_t launch_gemm(const OzJob *jobs, const OzItem *items, int nitems, int clusters, OzScratch scr,
-                               int *status, cudaStream_t st)
+                               int *status, const int *guard, cudaStream_t st)
 {
     if (nitems == 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)OzCfg::Smem);
     if (e != cudaSuccess) return e;
-    oz_gemm_kernel<GEN><<<2 * clusters, kOzThreads, OzCfg::Smem, st>>>(jobs, items, nitems, scr, status);
+    oz_gemm_kernel<MODE><<<2 * clusters, kOzThreads, OzCfg::Smem, st>>>(jobs, items, nitems, scr, status, guard);
     return cudaGetLastError();
 }
+
+int oz_f64_slices() { return kOzF64Slices; }
 
 size_t oz_part_bytes() { return sizeof(double) * 2 * 8 * 32 * (OzCfg::Cols / 4); }
 int oz_slot_flags() { return 16; }
 
 cudaError_t launch_oz_gemm_jobs(const OzJob *jobs, const OzItem *items, int nitems, int clusters, OzScratch scr,
-                                int *status, cudaStream_t st)
+                                int *status, const int *guard, cudaStream_t st)
 {
-    return launch_gemm<false>(jobs, items, nitems, clusters, scr, status, st);
+    return guard ? launch_gemm<OzProd::F64>(jobs, items, nitems, clusters, scr, status, guard, st)
+                 : launch_gemm<OzProd::Split>(jobs, items, nitems, clusters, scr, status, guard, st);
 }
 
 cudaError_t launch_oz_gemm_general(const OzJob *jobs, const OzItem *items, int nitems, int clusters, int *status,
                                    cudaStream_t st)
 {
-    return launch_gemm<true>(jobs, items, nitems, clusters, OzScratch{}, status, st);
+    return launch_gemm<OzProd::General>(jobs, items, nitems, clusters, OzScratch{}, status, nullptr, st);
 }
 
 cudaError_t launch_oz_split(const double2 *A, int64_t rows, int ka, int64_t sr, int64_t sk, bool conj, int s,
