@@ -143,7 +143,8 @@ GW_API gw_status gw_chi0_set_gsphere(gw_chi0 *h, int iq, int ng, const int32_t *
  * Forward chi0 for nq slots and nw imaginary frequencies (steps a1-a7 after setup).  With
  * two-float stage (a), on grids whose first two axes have 20 to 72 points and whose last has 24 to 72
  * (not 24^3), the last axis of the pair transform runs on the BF16 tensor cores where that is faster
- * (see gw_chi0_pair_elements_block); elsewhere stage (a) is the pruned FFT pair kernel.  The other
+ * (see gw_chi0_pair_elements_block); FP64 stage (a) likewise, to FP64 accuracy, for last axes of 24 to
+ * 56 points and any such first two; elsewhere stage (a) is the pruned FFT pair kernel.  The other
  * calls that form pair elements for whole valence rows choose alike.
  *   iq     host int [nq]      slots to compute.
  *   omega  host double [nw]   imaginary-axis frequencies w >= 0 (eV).

@@ -24,13 +24,27 @@ gw_status cuda_fail(gw_chi0 *h, cudaError_t e, const char *what)
 gw_status dalloc(gw_chi0 *h, void **p, size_t n, const char *what)
 {
     if (n == 0) n = 16;
-    // FP64 mode can do without its slices: they make room for what a call needs
+    // the buffers of stage (a) on the tensor cores and FP64 mode's slices are an optimisation: between
+    // the calls that use them they make room for what another needs
     auto reclaim = [&] {
-        if (h->d.prec != GW_PREC_FP64 || !h->Zbuf || h->zbusy) return false;
-        dfree(h, h->Zbuf, h->Zcap);
-        h->Zbuf = nullptr;
-        h->Zcap = 0;
-        return true;
+        const size_t held = h->bytes;
+        auto give = [&](auto *&b, size_t &cap) {
+            if (!b) return;
+            drop_graphs(h);
+            dfree(h, b, cap);
+            b = nullptr;
+            cap = 0;
+        };
+        if (h->d.prec == GW_PREC_FP64 && !h->zbusy) give(h->Zbuf, h->Zcap);
+        if (!h->zdbusy) {
+            for (int i = 0; i < 2; ++i) {
+                give(h->zdA[i], h->zdAcap[i]);
+                give(h->zdE[i], h->zdEcap[i]);
+            }
+            give(h->zdF, h->zdFcap);
+            give(h->zdS, h->zdScap);
+        }
+        return h->bytes < held;
     };
     if (h->d.mem_budget_bytes && h->bytes + n > h->d.mem_budget_bytes) reclaim();
     if (h->d.mem_budget_bytes && h->bytes + n > h->d.mem_budget_bytes)
@@ -670,13 +684,14 @@ gw_status ensure_overlap_stream(gw_chi0 *h)
 // two.  A block is vb valence x cb conduction bands; the row slices of the conduction block are formed
 // once, and the valence bands run over it in sub-blocks whose transform output F fits the work buffer.
 // On one stream: the last-axis product and the split contraction each need whole SMs.
-// GW_CHI0_STAGE_A=fft selects the FFT pair kernel instead.
+// GW_CHI0_STAGE_A=fft selects the FFT pair kernel instead.  FP64 stage (a) takes the same steps with
+// zdft64.cu and FP64 middle- and first-axis kernels.
 
 // grids whose middle and first axes run in one kernel, with the pair kernel's scratch slots
 static bool zd_fused(const gw_chi0 *h)
 {
     const int *n = h->d.n;
-    return n[0] == n[1] && n[1] == n[2] && (n[0] == 40 || n[0] == 48);
+    return h->d.mtxel_prec == GW_MTXEL_TWOFLOAT && n[0] == n[1] && n[1] == n[2] && (n[0] == 40 || n[0] == 48);
 }
 
 static bool zd_grid(const gw_chi0 *h, const Sphere &sp)
@@ -686,7 +701,10 @@ static bool zd_grid(const gw_chi0 *h, const Sphere &sp)
         return e && strcmp(e, "fft") == 0;
     }();
     const int *n = h->d.n;
-    if (fft_only || h->d.mtxel_prec != GW_MTXEL_TWOFLOAT || !gw::zd_supported(n[2], sp.K2)) return false;
+    if (fft_only) return false;
+    if (h->d.mtxel_prec == GW_MTXEL_FP64)
+        return gw::zd64_supported(n[2], sp.K2) && gw::pair_split_supported(n[0]) && gw::pair_split_supported(n[1]);
+    if (!gw::zd_supported(n[2], sp.K2)) return false;
     if (zd_fused(h)) return sp.nslots > 0 && h->pscr;
     // 24^3 keeps its grid-specialised FFT kernel, which runs beside the contraction on a second stream
     const bool small_cube = n[0] == n[1] && n[1] == n[2] && n[0] <= 24;
@@ -698,12 +716,18 @@ static bool zd_grid(const gw_chi0 *h, const Sphere &sp)
 // grid-specialised, and no less than for the 600 pairs that fill the GPU; here 5.2e-3 per line, stage
 // of 8 points and tile of 128 conduction bands x CT valence bands, however few of its rows and columns
 // hold bands, and for the other two axes 7.2e-6 per line and kept frequency of a pair.
+// FP64: the FFT kernel 61e-6 a grid point (48^3; 79e-6 on 24^3) and no less than for one pair an SM; here
+// 14e-3 and 34e-6.
 static bool zd_faster(const gw_chi0 *h, const Sphere &sp, int vb, int cb)
 {
-    const int *n = h->d.n, ct = gw::zd_valence_per_tile(n[2], sp.K2);
+    const bool f64 = h->d.mtxel_prec == GW_MTXEL_FP64;
+    const int *n = h->d.n, ct = f64 ? gw::zd64_valence_per_tile(sp.K2) : gw::zd_valence_per_tile(n[2], sp.K2);
     const bool cube = n[0] == n[1] && n[1] == n[2];
     const double lines = (double)n[0] * n[1], pairs = (double)vb * cb;
     const double tiles = (double)((cb + 127) / 128) * ((vb + ct - 1) / ct);
+    if (f64)
+        return tiles * lines * ((n[2] + 7) / 8) * 14e-3 + 34e-6 * lines * sp.K2 * pairs <
+               61e-6 * lines * n[2] * std::max(pairs, 152.0);
     const double fft = cube && n[0] == 48   ? 1.04
                        : cube && n[0] == 40 ? 0.84
                        : cube && n[0] == 72 ? 5.1
@@ -734,13 +758,15 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
 {
     z = ZdPlan();
     if (!zd_grid(h, sp)) return GW_OK;
-    const int *n = h->d.n, ct = gw::zd_valence_per_tile(n[2], sp.K2), lines = n[0] * n[1];
+    z.f64 = h->d.mtxel_prec == GW_MTXEL_FP64;
+    const int *n = h->d.n, lines = n[0] * n[1];
+    const int ct = z.f64 ? gw::zd64_valence_per_tile(sp.K2) : gw::zd_valence_per_tile(n[2], sp.K2);
     const bool chi48 = zd_fused(h) && n[0] == 48 && !rows;
     // The route's pair elements carry 2e-13 (its fourth accumulator rounds in FP32), the FFT kernel's
     // 8e-15.  At up to seven slices the contraction's own error is ten times that and more.  At eight,
     // and with the FP64 contraction, the route serves chi on 48^3 alone (8.7e-14 at eight slices); on
     // the other calls it would raise the error, by up to three times for the gradients.
-    if ((h->d.prec == GW_PREC_FP64 || h->d.nslices > 7) && !chi48) return GW_OK;
+    if (!z.f64 && (h->d.prec == GW_PREC_FP64 || h->d.nslices > 7) && !chi48) return GW_OK;
     if (rows) {
         z.cb = nc;
     } else { // conduction blocks of about 512: four row tiles share a valence tile's columns
@@ -754,7 +780,7 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
     if (vb >= ct && vb < nv) vb -= vb % ct;
     z.vb = (int)vb;
     if (!force && !zd_faster(h, sp, z.vb, z.cb)) return GW_OK;
-    z.abytes = gw::zd_row_bytes(z.cb, n[2], lines);
+    z.abytes = z.f64 ? gw::zd64_row_bytes(z.cb, n[2], lines) : gw::zd_row_bytes(z.cb, n[2], lines);
     z.ebytes = sizeof(int) * (size_t)lines * nv;
     // per valence band: F, and the cells between the two kernels of the other axes
     z.fper = sizeof(float4) * (size_t)lines * z.cb * gw::zd_row_entries(sp.K2);
@@ -774,13 +800,18 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
     z.vs = vs;
     const std::string err = h->err;
     gw_status s = GW_OK;
+    const bool before = h->zdbusy; // an earlier plan of this call
+    h->zdbusy = true;
     for (int i = 0; i < sides && !s; ++i)
         if (!(s = grow(h, &h->zdA[i], &h->zdAcap[i], z.abytes, "conduction slices")))
             s = grow(h, (void **)&h->zdE[i], &h->zdEcap[i], z.ebytes, "column exponents");
     if (!s) s = grow(h, (void **)&h->zdF, &h->zdFcap, z.fper * vs, "last-axis transform");
     if (!s && z.sper) s = grow(h, (void **)&h->zdS, &h->zdScap, z.sper * vs, "transform cells");
+    if (!s && z.f64 && !(s = grow(h, (void **)&h->zdguard, &h->zdguard_cap, sizeof(int), "slice check")))
+        CK(h, cudaMemsetAsync(h->zdguard, 0, sizeof(int), h->st), "slice check");
     if (s == GW_ERR_OOM && !force) { // the FFT route needs none of these
         h->err = err;
+        h->zdbusy = before;
         return GW_OK;
     }
     if (s) return s;
@@ -812,28 +843,34 @@ gw_status zd_valence(gw_chi0 *h, ZdPlan &z, const Sphere &sp, const void *psiv, 
     const int64_t lines = (int64_t)h->d.n[0] * h->d.n[1];
     {
         Scope sc(h, "zd_slices");
-        CK(h, gw::launch_zd_colexp(psiv, nv, n, (int)lines, h->zdE[side], h->st), "column exponents");
+        if (z.f64)
+            CK(h, gw::launch_zd64_colexp(psiv, nv, n, (int)lines, h->zdE[side], h->zdguard, h->st), "column exponents");
+        else CK(h, gw::launch_zd_colexp(psiv, nv, n, (int)lines, h->zdE[side], h->st), "column exponents");
     }
     // the valence grids, line by line: box of one line of CT bands
     const int part = gw::zd_line_split(n);
     cuuint64_t d[3] = {(cuuint64_t)4 * n / part, (cuuint64_t)lines * part, (cuuint64_t)nv};
     cuuint64_t st[2] = {(cuuint64_t)16 * n / part, (cuuint64_t)16 * lines * n};
-    cuuint32_t box[3] = {(cuuint32_t)(4 * n / part), (cuuint32_t)part, (cuuint32_t)gw::zd_valence_per_tile(n, sp.K2)};
+    const int ct = z.f64 ? gw::zd64_valence_per_tile(sp.K2) : gw::zd_valence_per_tile(n, sp.K2);
+    cuuint32_t box[3] = {(cuuint32_t)(4 * n / part), (cuuint32_t)part, (cuuint32_t)ct};
     cuuint32_t es[3] = {1, 1, 1};
     CUresult r = h->encode(&z.tmV[side], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(psiv), d, st, box, es,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(h, GW_ERR_CUDA, "cuTensorMapEncodeTiled (valence grids) failed (%d)", (int)r);
     z.nv[side] = nv;
+    z.psiv[side] = psiv;
     return GW_OK;
 }
 
-gw_status zd_conduction(gw_chi0 *h, const ZdPlan &z, const void *psic, int c0, int cb, int side)
+gw_status zd_conduction(gw_chi0 *h, ZdPlan &z, const void *psic, int c0, int cb, int side)
 {
     Scope sc(h, "zd_slices");
-    CK(h, gw::launch_zd_rows((const float4 *)psic + (int64_t)c0 * h->nr, cb, h->d.n[2], h->d.n[0] * h->d.n[1],
-                             h->zdA[side], h->st),
-       "conduction slices");
+    const int n = h->d.n[2], lines = h->d.n[0] * h->d.n[1];
+    z.psic[side] = (const double2 *)psic + (int64_t)c0 * h->nr; // 16 bytes an entry in either form
+    if (z.f64)
+        CK(h, gw::launch_zd64_rows(z.psic[side], cb, n, lines, h->zdA[side], h->zdguard, h->st), "conduction slices");
+    else CK(h, gw::launch_zd_rows(z.psic[side], cb, n, lines, h->zdA[side], h->st), "conduction slices");
     return GW_OK;
 }
 
@@ -847,7 +884,12 @@ gw_status zd_block(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::Pair
         const int nb = std::min(z.vs, vb - b0);
         {
             Scope t(h, "zdft");
-            CK(h, gw::launch_zd_gemm(z.tmV[vside], h->zdA[cside], h->zdE[vside], sp.kz, pp.ax[2].twf, n[2], lines,
+            if (z.f64)
+                CK(h, gw::launch_zd64_gemm(z.tmV[vside], h->zdA[cside], h->zdE[vside], sp.kz, pp.ax[2].tw, n[2], lines,
+                                           z.nv[vside], v0 + b0, nb, cb, sp.K2, (double2 *)h->zdF, h->zdguard,
+                                           h->status, h->st),
+                   "last-axis transform");
+            else CK(h, gw::launch_zd_gemm(z.tmV[vside], h->zdA[cside], h->zdE[vside], sp.kz, pp.ax[2].twf, n[2], lines,
                                      z.nv[vside], v0 + b0, nb, cb, sp.K2, h->zdF, h->status, h->st),
                "last-axis transform");
         }
@@ -866,6 +908,16 @@ gw_status zd_block(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::Pair
             CK(h, gw::launch_pair_tf_from_f(tmF, tmS, R, cb, sv, sc, pp, Mb, h->st), "pair elements from F");
         } else {
             if ((s = zd_map(h, &tmS, h->zdS, pp.K12, (uint64_t)R * n[0], 2 * sp.K2, n[0], "transform cells"))) return s;
+            if (z.f64) { // and the FFT pair kernel, which returns at once unless the slices do not hold
+                gw::PairPlan pg = pp;
+                pg.guard = h->zdguard;
+                CK(h, gw::launch_pair_split64_1(tmF, R, pg, (double2 *)h->zdS, h->st), "middle axis from F");
+                CK(h, gw::launch_pair_split64_2(tmS, R, cb, sv, sc, pg, Mb, h->st), "pair elements from cells");
+                CK(h, gw::launch_pair((const double2 *)z.psiv[vside] + (int64_t)(v0 + b0) * h->nr,
+                                      (const double2 *)z.psic[cside], cb, 0, R, pg, Mb, h->st),
+                   "pair kernel");
+                continue;
+            }
             CK(h, gw::launch_pair_split1(tmF, R, pp, h->zdS, h->st), "middle axis from F");
             CK(h, gw::launch_pair_split2(tmS, R, cb, sv, sc, pp, Mb, h->st), "pair elements from cells");
         }
@@ -1105,6 +1157,7 @@ void gw_chi0_destroy(gw_chi0 *h)
     }
     dfree(h, h->zdF, h->zdFcap);
     dfree(h, h->zdS, h->zdScap);
+    dfree(h, h->zdguard, h->zdguard_cap);
     for (int b = 0; b < 2; ++b) {
         dfree(h, h->ovZ[b], h->ovZcap[b]);
         dfree(h, h->ovE[b], h->ovEcap[b]);
@@ -1349,6 +1402,7 @@ gw_status gw_chi0_pair_elements_block(gw_chi0 *h, int iq, int c0, int cb, double
         return fail(h, GW_ERR_UNSUPPORTED, "slot %d does not take the tensor-core route", iq);
     if (cb == 0) return GW_OK;
     ZdPlan z;
+    ZdUse use{h};
     if ((s = zd_plan(h, sp, nv, cb, false, true, 1, 1, z))) return s;
     const gw::PairPlan pp = pair_plan(h, sp);
     if ((s = zd_valence(h, z, sp, v.psi, nv))) return s;
@@ -1422,6 +1476,7 @@ gw_status gw_chi0_compute(gw_chi0 *h, int nq, const int *iq, int nw, const doubl
             continue;
         }
         ZdPlan z;
+        ZdUse use{h};
         if (fault_chunk() < 0 && (s = zd_plan(h, sp, v.nb, h->cond.nb, keep, false, 1, nw, z))) return s;
         if (z.on) {
             const int nc = h->cond.nb;

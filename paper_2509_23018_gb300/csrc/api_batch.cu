@@ -94,6 +94,7 @@ gw_status batch_stage_a(gw_chi0 *h, int nq, const int *iq, const gw::OmegaList &
             if ((s = zd_valence(h, zd[i], sp, v.psi, v.nb)) ||
                 (!rows && (s = zd_conduction(h, zd[i], h->cond.psi, 0, h->cond.nb))))
                 return s;
+            zd[i].psic[0] = h->cond.psi;
             rows = true;
         }
         if ((s = pair_rows(h, zd[i], sp, pp, v.psi, h->cond.psi, h->cond.nb, 0, L.P[i], h->Mall + L.moff[i]))) return s;
@@ -217,6 +218,7 @@ gw_status compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const double 
     if (!h->cap_st) CK(h, cudaStreamCreateWithFlags(&h->cap_st, cudaStreamNonBlocking), "capture stream");
     // stage (a)'s route per slot, and the buffers the slots share, before the capture
     std::vector<ZdPlan> zd(nq);
+    ZdUse use{h};
     for (int i = 0; i < nq; ++i)
         if ((s = zd_plan(h, h->sph[iq[i]], h->val[iq[i]].nb, h->cond.nb, true, false, 1, 1, zd[i]))) return s;
     for (auto &z : zd) z.on = z.on && zd_holds(h, z);

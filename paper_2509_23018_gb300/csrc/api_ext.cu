@@ -73,6 +73,7 @@ gw_status gw_chi0_adjoint(gw_chi0 *h, int iq, double omega, const double *W, dou
     ACK(cudaMemsetAsync(pbc, 0, szC, h->st), "zero");
     gw::PairPlan pp = pair_plan(h, sp);
     ZdPlan z;
+    ZdUse use{h};
     if ((s = zd_plan(h, sp, nv, nc, true, false, 1, 1, z)) ||
         (z.on && ((s = zd_valence(h, z, sp, v.psi, nv)) || (s = zd_conduction(h, z, c.psi, 0, nc))))) {
         cleanup();
@@ -221,6 +222,7 @@ gw_status gw_chi0_compute_subspace(gw_chi0 *h, int iq, int neig, const double *b
     const int64_t P = (int64_t)v.nb * h->cond.nb;
     const double2 *Mres = resident_for(h, iq); // kept by the last gw_chi0_compute of this slot
     ZdPlan z;
+    ZdUse use{h};
     if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, nw, z)) ||
                   (z.on && ((s = zd_valence(h, z, sp, v.psi, v.nb)) || (s = zd_conduction(h, z, h->cond.psi, 0, h->cond.nb))))))
         return s;
@@ -341,6 +343,7 @@ gw_status gw_chi0_compute_real(gw_chi0 *h, int iq, int nw, const double *omega, 
     const int64_t P = (int64_t)v.nb * h->cond.nb;
     const double2 *Mres = resident_for(h, iq); // kept by the last gw_chi0_compute of this slot
     ZdPlan z;
+    ZdUse use{h};
     if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, 3 * nw, z)) ||
                   (z.on && ((s = zd_valence(h, z, sp, v.psi, v.nb)) || (s = zd_conduction(h, z, h->cond.psi, 0, h->cond.nb))))))
         return s;
@@ -407,6 +410,7 @@ gw_status gw_chi0_jvp(gw_chi0 *h, int iq, int nw, const double *omega, const dou
     const int64_t nn = (int64_t)ng * ng;
     const int64_t P = (int64_t)v.nb * nc;
     ZdPlan z; // side 0: the stored bands, side 1: the tangents
+    ZdUse use{h};
     if ((s = zd_plan(h, sp, v.nb, nc, true, false, 2, 2 * nw, z))) return s;
     const int64_t chunk = z.on ? (int64_t)z.vb * z.cb : std::min<int64_t>(h->d.pair_chunk, P);
     // work held only for this call

@@ -172,6 +172,9 @@ struct gw_chi0 {
     size_t zdFcap = 0;         // bytes
     float4 *zdS = nullptr;     // cells between the middle- and first-axis kernels, where they are two
     size_t zdScap = 0;         // bytes
+    bool zdbusy = false;       // a call has planned with these buffers (ZdUse)
+    int *zdguard = nullptr;    // FP64: set where the slices do not hold and the FFT kernel takes over
+    size_t zdguard_cap = 0;
     // scratch slots of the two-float pair kernel (sized in set_gsphere, outside any capture)
     float4 *pscr = nullptr;
     size_t pscr_cap = 0; // bytes
@@ -277,16 +280,24 @@ gw_status compute_overlap(gw_chi0 *h, int iq, const gw::OmegaList &om, double2 *
 // zd_conduction prepare a side's bands; zd_block forms M[(v - v0) sv + c sc] of a block.
 struct ZdPlan {
     bool on = false;
+    bool f64 = false;                                  // FP64 (zdft64.cu), two-float otherwise
     int vb = 0, cb = 0, vs = 0;                        // vs: valence bands per sub-block
     size_t abytes = 0, ebytes = 0, fper = 0, sper = 0; // row slices, exponents; F and cells of one valence band
     int nv[2] = {0, 0};
     CUtensorMap tmV[2];
+    const void *psiv[2] = {nullptr, nullptr}, *psic[2] = {nullptr, nullptr}; // each side's bands, as last prepared
+};
+// The route's buffers stay until the call that planned with them returns; between calls they make room
+// for what others need (dalloc).
+struct ZdUse {
+    gw_chi0 *h;
+    ~ZdUse() { h->zdbusy = false; }
 };
 gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw,
                   ZdPlan &z);
 bool zd_holds(const gw_chi0 *h, const ZdPlan &z); // side 0 and F as planned (a later plan may have lost them)
 gw_status zd_valence(gw_chi0 *h, ZdPlan &z, const Sphere &sp, const void *psiv, int nv, int side = 0);
-gw_status zd_conduction(gw_chi0 *h, const ZdPlan &z, const void *psic, int c0, int cb, int side = 0);
+gw_status zd_conduction(gw_chi0 *h, ZdPlan &z, const void *psic, int c0, int cb, int side = 0);
 gw_status zd_block(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::PairPlan &pp, int vside, int cside, int v0,
                    int vb, int cb, double2 *M, int64_t sv, int64_t sc);
 gw_status pair_rows(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::PairPlan &pp, const void *psiv,

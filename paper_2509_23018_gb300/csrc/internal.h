@@ -35,6 +35,8 @@ struct PairPlan {
     int *slot_flags;
     int nslots;
     int *status;          // device status word (kStatusNoSlot)
+    // the FP64 pair kernel runs only where *guard is set, pair_split64_* only where it is not (null: both run)
+    const int *guard = nullptr;
 };
 // Scratch the two-float pair kernel needs for a plan: *nslots slots of *slot_elems float4
 // (0 slots: the plan runs on the runtime-shape kernel, which needs none).
@@ -89,6 +91,21 @@ cudaError_t launch_pair_split2(const CUtensorMap &tmS, int64_t R, int cb, int64_
 // scratch slots as [nslots N rows][K12] two-float entries, box {8 K2, N}; no swizzle)
 cudaError_t launch_pair_tf_from_f(const CUtensorMap &tmF, const CUtensorMap &tmS, int64_t R, int cb, int64_t sv,
                                   int64_t sc, const PairPlan &pp, double2 *M, cudaStream_t st);
+
+// ---- the same in FP64 (zdft64.cu, pair_split64.cu): seven nine-bit slices per operand, double2 grids, F
+// and cells.  Lines of 24 to 56 points.  guard: set by the slicing kernels where an entry is not finite
+// or a line is scaled by more than 2^+-400; the product returns at once where it is set.
+size_t zd64_row_bytes(int nr, int n, int lines); // row slices and exponents
+cudaError_t launch_zd64_rows(const void *psi, int nr, int n, int lines, void *A, int *guard, cudaStream_t st);
+cudaError_t launch_zd64_colexp(const void *psi, int nb, int n, int lines, int *E, int *guard, cudaStream_t st);
+bool zd64_supported(int n, int K2);
+int zd64_valence_per_tile(int K2);
+cudaError_t launch_zd64_gemm(const CUtensorMap &tmV, const void *A, const int *E, const int *kz, const double2 *tw, int n,
+                             int lines, int nv, int v0, int vb, int cb, int K2, double2 *F, const int *guard,
+                             int *status, cudaStream_t st);
+cudaError_t launch_pair_split64_1(const CUtensorMap &tmF, int64_t R, const PairPlan &pp, double2 *S, cudaStream_t st);
+cudaError_t launch_pair_split64_2(const CUtensorMap &tmS, int64_t R, int cb, int64_t sv, int64_t sc, const PairPlan &pp,
+                                  double2 *M, cudaStream_t st);
 
 // ---- energy factor, diagonal, symmetrisation (reduce.cu)
 // delta[w][p - p0] = 4x/(x^2 + w^2), x = ev[v] - ec[c]

@@ -10,7 +10,7 @@
 #include "internal.h"
 #include "fft.cuh"
 #include "fft_tf.cuh"
-#include "pair_split_ct.cuh"
+#include "pair_split64_ct.cuh"
 
 namespace gw {
 
@@ -209,6 +209,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_kernel(const double2 *__res
                                                              const double2 *__restrict__ psic, int nc, int64_t p0,
                                                              PairPlan pp, double2 *__restrict__ M)
 {
+    if (pp.guard && *pp.guard == 0) return;
     extern __shared__ __align__(16) unsigned char smem[];
     const int n0 = pp.n[0], n1 = pp.n[1], n2 = pp.n[2];
     const int ns = n1 * n2;
@@ -409,6 +410,31 @@ cudaError_t launch_pair_split1(const CUtensorMap &tmF, int64_t R, const PairPlan
 #define GW_CASE(N) \
     case N: return pair_split1_n##N(tmF, R, pp, tf_consts(), S, st);
     switch (pp.n[1]) {
+        GW_PAIR_SPLIT_LENGTHS(GW_CASE)
+    default: return cudaErrorInvalidValue;
+    }
+#undef GW_CASE
+}
+
+cudaError_t launch_pair_split64_1(const CUtensorMap &tmF, int64_t R, const PairPlan &pp, double2 *S, cudaStream_t st)
+{
+    if (R == 0) return cudaSuccess;
+#define GW_CASE(N) \
+    case N: return pair_split64_1_n##N(tmF, R, pp, S, st);
+    switch (pp.n[1]) {
+        GW_PAIR_SPLIT_LENGTHS(GW_CASE)
+    default: return cudaErrorInvalidValue;
+    }
+#undef GW_CASE
+}
+
+cudaError_t launch_pair_split64_2(const CUtensorMap &tmS, int64_t R, int cb, int64_t sv, int64_t sc, const PairPlan &pp,
+                                  double2 *M, cudaStream_t st)
+{
+    if (R == 0) return cudaSuccess;
+#define GW_CASE(N) \
+    case N: return pair_split64_2_n##N(tmS, R, cb, sv, sc, pp, M, st);
+    switch (pp.n[0]) {
         GW_PAIR_SPLIT_LENGTHS(GW_CASE)
     default: return cudaErrorInvalidValue;
     }

@@ -171,5 +171,10 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t base, uint32_t ncols)
                    "=r"((v)[6]), "=r"((v)[7]), "=r"((v)[8]), "=r"((v)[9]), "=r"((v)[10]), "=r"((v)[11]), \
                    "=r"((v)[12]), "=r"((v)[13]), "=r"((v)[14]), "=r"((v)[15]) \
                  : "r"(taddr))
+#define GW_TMEM_LD_16X256_X2(taddr, v) \
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];" \
+                 : "=r"((v)[0]), "=r"((v)[1]), "=r"((v)[2]), "=r"((v)[3]), "=r"((v)[4]), "=r"((v)[5]), \
+                   "=r"((v)[6]), "=r"((v)[7]) \
+                 : "r"(taddr))
 
 } // namespace gw

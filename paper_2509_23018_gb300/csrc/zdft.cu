@@ -25,6 +25,7 @@
 #include "internal.h"
 #include "ptx.cuh"
 #include "fft_tf.cuh"
+#include "zd_tiles.cuh"
 
 #include <algorithm>
 
@@ -104,25 +105,9 @@ __device__ __forceinline__ int zd_expo(float m)
 }
 
 // ------------------------------------------------------------------ operand tiles in shared memory
-constexpr int kZdM = 128;                              // rows per tile
-constexpr int kZdAcc = 128;                            // TMEM columns per accumulator
-constexpr int kZdKB = 16;                              // real K entries per stage (8 points)
 constexpr int kZdMaxStages = 9;                        // stages per tile: lines of up to 72 points
 constexpr unsigned kZdSlice = kZdM * kZdKB * 2;        // one row slice of one stage: 4 KB
 constexpr unsigned kZdStage = kZdSlices * kZdSlice;    // 24 KB
-static __host__ __device__ constexpr int zd_stages(int n) { return (n + 7) / 8; }
-
-// K-major operand tiles of both operands, 32-byte swizzling: row r of 32 bytes (16 BF16), 8-row
-// atoms of 256 bytes, 16-byte chunk j of row r stored at chunk j ^ ((r % 8) >> 2).
-__device__ __forceinline__ uint64_t sdesc_sw32(uint32_t addr)
-{
-    return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(256 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
-}
-__device__ __forceinline__ uint32_t sw32_off(int r, int k) // byte offset of element k (< 16) of row r
-{
-    return (uint32_t)((r >> 3) * 256 + (r & 7) * 32 + ((((k >> 3) ^ ((r & 7) >> 2)) & 1) << 4) + (k & 7) * 2);
-}
 
 // ------------------------------------------------------------------ row slices
 // A[l][mt][ks][slice] (4 KB images of the swizzled tile of 128 rows x 16 real entries, so that one
@@ -228,15 +213,6 @@ constexpr int kZdPsiSlots = 2;  // ring of valence-band line tiles
 constexpr int kZdMaxRing = 4;   // ring of row stages (2 to 4, what shared memory holds)
 constexpr int kZdRounds = 3;    // (band, frequency) pairs per producer lane: 64 pairs, 6 warps x 4
 
-__device__ __forceinline__ void bulk_copy(void *dst, const void *src, unsigned bytes, uint64_t *b)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     su32(dst)),
-                 "l"(src), "r"(bytes), "r"(su32(b))
-                 : "memory");
-}
-__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
 // two-sum with the sum's rounding error
 __device__ __forceinline__ float zd_2sum(float a, float b, float &e)
 {
@@ -244,9 +220,6 @@ __device__ __forceinline__ float zd_2sum(float a, float b, float &e)
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
     return s;
 }
-
-// one slot of the line-tile ring, in float4: CT lines, to 128 bytes (TMA destinations)
-static __host__ __device__ int zd_ring_stride(int CT, int n) { return (CT * n + 7) / 8 * 8; }
 
 struct ZdArgs {
     CUtensorMap tmV;        // valence grids as FP32 [nv][lines][4N], box {4N, 1, CT} (zd_line_split)
