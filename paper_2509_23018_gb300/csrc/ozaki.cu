@@ -493,14 +493,13 @@ __global__ void __launch_bounds__(256, NE > 4 ? 3 : 4) gpp_prep_split_kernel(con
 // over all its slice groups and K-segments (64 per epilogue thread: Re or Im parts, two of the real
 // products each), so a segment costs TMEM loads and FP32 adds, and FP64 work and atomics come once
 // per item.  Two accumulators in TMEM alternate between segments, so a segment's epilogue overlaps
-// the next one's MMAs; without any epilogue work the 16 launches of
-// a 48^3 q-point take 16.5 ms instead of 19.0.
+// the next one's MMAs.  The issuing warp runs converged (umma_f16_run): issued by a lone thread the 16
+// launches of a 48^3 q-point take 19.2 ms instead of 17.5.
 //
-// Measured (split contraction of one 8192-pair chunk, N_G = 2000, 7-slice accuracy): 1.21 ms, 15
-// products of nine-bit slices, 1.63 PFLOP/s on them; one CTA per tile with 28 products of six-bit
-// slices and an FP64 atomic epilogue per slice group took 2.44 ms (1.50 PFLOP/s).  N_G = 6000: 9.6
-// against 24.0 ms.  General product of the self-energy (N_G = 6000, 384 bands, 24 products): 20.8
-// against 54.3 ms.
+// Measured (split contraction of one 8192-pair chunk, N_G = 2000, 7-slice accuracy): 1.09 ms, 15
+// products of nine-bit slices, 1.80 PFLOP/s on them; one CTA per tile with 28 products of six-bit
+// slices and an FP64 atomic epilogue per slice group took 2.44 ms (1.50 PFLOP/s).  General product of the
+// self-energy (N_G = 6000, 384 bands): 19.1 against 54.3 ms.
 struct OzCfg {
     static constexpr unsigned Bytes = kOzBM * kOzBK * 2;     // of A, and of B, per stage and CTA
     static constexpr int Stages = 6;                         // TMA ring depth
@@ -571,8 +570,8 @@ struct OzPlace {
 // pairs: groups t = 8..5 in units of 2^-54 (|sum| < 2^57), rounded to units of 2^-37 before t = 4..2
 // (|sum| <= 2 1024 2^14 2^37 = 2^62), 2^-51 of a pair's largest product.  A block's sum goes to chi (or
 // to the part's place in scratch) in FP64, so a chunk of 8192 pairs is rounded eight times where a chain
-// of DMMAs is rounded 2048 times.  Measured on a chunk of 8192 pairs, N_G = 2000: 2.55 ms
-// (28 products, 1.4 PFLOP/s) and 0.33 ms for the slices where the DMMA kernel, at 0.86 of its pipe's rate,
+// of DMMAs is rounded 2048 times.  Measured on a chunk of 8192 pairs, N_G = 2000: 2.44 ms
+// (28 products, 1.5 PFLOP/s) and 0.33 ms for the slices where the DMMA kernel, at 0.86 of its pipe's rate,
 // takes 138; error of chi against 64 bits 1.1e-15 where it leaves 1.9e-15.
 enum class OzProd { Split, General, F64 };
 template <OzProd MODE>
@@ -645,33 +644,41 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
                 for (uint32_t j = it > ST ? it - ST : 0; j < it; ++j) pair_wait(&full[j % ST], (j / ST) & 1);
             if (!ok) atomicOr(status, kStatusTimeout);
         }
-        if (warp == 1 && lane == 0 && rank == 0) {
-            uint32_t it = 0, seg = 0;
+        if (warp == 1 && rank == 0) { // the warp converged (umma_f16_run)
+            const uint32_t lead = elect_lane(), tb = __shfl_sync(0xffffffffu, tbase, 0);
+            const uint32_t ad = sdesc_sw128_low(su32(sA)), bd = sdesc_sw128_low(su32(sB));
+            auto wait = [&](uint64_t *b, uint32_t parity) {
+                if (!__all_sync(0xffffffffu, pair_wait(b, parity))) ok = false;
+            };
+            uint32_t st = 0, ph = 0, seg = 0;
             for (int item = cl0; item < nitems && ok; item += ncl) {
                 const OzItem w = items[item];
                 for (OzSegments<F64> g(w.nk, jobs[w.job].s); g.more() && ok; g.next(), ++seg) {
                     const uint32_t b = seg % NB;
-                    if (!pair_wait(&tempty[b], ((seg / NB) & 1) ^ 1)) { ok = false; break; }
+                    wait(&tempty[b], ((seg / NB) & 1) ^ 1);
                     tc_fence_after();
                     const int n = (g.t - 1) * g.len; // ring stages of the segment
-                    for (int j = 0; j < n; ++j, ++it) {
-                        const uint32_t st = it % ST;
-                        if (!pair_wait(&full[st], (it / ST) & 1)) { ok = false; break; }
+                    for (int j = 0; j < n && ok; ++j) {
+                        wait(&full[st], ph);
                         tc_fence_after();
-                        const uint32_t a0 = su32(sA + st * C::Bytes), b0 = su32(sB + st * C::Bytes);
+                        const uint32_t o = st * (C::Bytes >> 4);
 #pragma unroll
                         for (int kk = 0; kk < kOzBK / 16; ++kk)
-                            umma_f16_pair(tbase + b * C::Cols, sdesc_sw128(a0 + kk * 32), sdesc_sw128(b0 + kk * 32),
+                            umma_f16_pair(lead, tb + b * C::Cols, ad + o + kk * 2, bd + o + kk * 2, kSdescSw128High,
                                           C::Idesc, (j == 0 && kk == 0) ? 0u : 1u);
-                        umma_commit_pair(&empty[st]);
+                        umma_commit_pair(lead, &empty[st]);
+                        if (++st == ST) {
+                            st = 0;
+                            ph ^= 1;
+                        }
                     }
-                    umma_commit_pair(&tfull[b]);
+                    umma_commit_pair(lead, &tfull[b]);
                 }
             }
             // every issued MMA has completed before the pair tears down
-            umma_commit_pair(fin);
-            pair_wait(fin, 0);
-            if (!ok) atomicOr(status, kStatusTimeout);
+            umma_commit_pair(lead, fin);
+            wait(fin, 0);
+            if (!ok && lead) atomicOr(status, kStatusTimeout);
         } else if (warp == 1 && lane == 0) {
             pair_wait(fin, 0); // the pair's last commit has reached this CTA too
         }

@@ -3,7 +3,7 @@
 //
 // What bounds them: the FP64 pipe (two FMAs a clock and SM).  Hence the pruned last stages, and stages
 // that skip the products with W^0: 1.18 us a pair on 48^3 (K2 = 15, N_G = 2000; 0.53 million FP64
-// instructions, 0.9 us at the pipe's rate), 0.20 on 24^3.  With the last axis and the slices 1.87 and 0.41
+// instructions, 0.9 us at the pipe's rate), 0.20 on 24^3.  With the last axis and the slices 1.83 and 0.40
 // where the FFT pair kernel takes 6.7 and 1.09.
 #pragma once
 #include "pair_split_ct.cuh"

@@ -65,10 +65,45 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr)
     return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
            ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
+// its low and high word
+__device__ __forceinline__ uint32_t sdesc_sw128_low(uint32_t addr) { return ((addr & 0x3FFFF) >> 4) | (1u << 16); }
+constexpr uint32_t kSdescSw128High = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ void umma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
 {
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
                  ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc)
+                 : "memory");
+}
+// The same for a warp that runs its issue loop converged, so that addresses stay in uniform registers (a
+// lone thread moves every descriptor there first, 95 clocks a product): the elected lane issues, and
+// the descriptors come as their low words and a common high word.  Product k of a run of len products
+// that share A: the first fills the A collector, the others take A from there.
+__device__ __forceinline__ uint32_t elect_lane()
+{
+    uint32_t e;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+    return e;
+}
+__device__ __forceinline__ void umma_f16_run(uint32_t lead, uint32_t d, uint32_t a, uint32_t b, uint32_t high,
+                                             uint32_t idesc, uint32_t acc, int k, int len)
+{
+#define GW_UMMA_COLLECT(op)                                                                                        \
+    asm volatile("{\n .reg .pred p, q;\n .reg .b64 da, db;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"        \
+                 " mov.b64 da, {%1, %6};\n mov.b64 db, {%2, %6};\n"                                                \
+                 " @q tcgen05.mma.cta_group::1.kind::f16" op " [%0], da, db, %3, p;\n}" ::"r"(d),                   \
+                 "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(lead), "r"(high)                                        \
+                 : "memory")
+    if (len == 1) GW_UMMA_COLLECT("");
+    else if (k == 0) GW_UMMA_COLLECT(".collector::a::fill");
+    else if (k == len - 1) GW_UMMA_COLLECT(".collector::a::lastuse");
+    else GW_UMMA_COLLECT(".collector::a::use");
+#undef GW_UMMA_COLLECT
+}
+__device__ __forceinline__ void umma_commit_lead(uint32_t lead, uint64_t *b)
+{
+    asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+                 " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(su32(b)),
+                 "r"(lead)
                  : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint64_t *b)
@@ -120,17 +155,22 @@ __device__ __forceinline__ void tma3_pair(void *dst, const CUtensorMap *m, uint3
                  "l"(m), "r"(x), "r"(y), "r"(z), "r"(a)
                  : "memory");
 }
-__device__ __forceinline__ void umma_f16_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
+// by the elected lane of a converged warp (umma_f16_run)
+__device__ __forceinline__ void umma_f16_pair(uint32_t lead, uint32_t d, uint32_t a, uint32_t b, uint32_t high,
+                                              uint32_t idesc, uint32_t acc)
 {
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc)
+    asm volatile("{\n .reg .pred p, q;\n .reg .b64 da, db;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+                 " mov.b64 da, {%1, %6};\n mov.b64 db, {%2, %6};\n"
+                 " @q tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, p;\n}" ::"r"(d),
+                 "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(lead), "r"(high)
                  : "memory");
 }
 // arrive at the barrier at this offset in both CTAs when the MMAs issued so far have completed
-__device__ __forceinline__ void umma_commit_pair(uint64_t *b)
+__device__ __forceinline__ void umma_commit_pair(uint32_t lead, uint64_t *b)
 {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(su32(b)), "h"((uint16_t)3)
+    asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n"
+                 " @q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}"
+                 ::"r"(su32(b)), "h"((uint16_t)3), "r"(lead)
                  : "memory");
 }
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t *slot, uint32_t ncols)

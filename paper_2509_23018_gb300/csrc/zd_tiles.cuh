@@ -11,11 +11,9 @@ static __host__ __device__ constexpr int zd_stages(int n) { return (n + 7) / 8; 
 
 // K-major operand tiles of both operands, 32-byte swizzling: row r of 32 bytes (16 BF16), 8-row
 // atoms of 256 bytes, 16-byte chunk j of row r stored at chunk j ^ ((r % 8) >> 2).
-__device__ __forceinline__ uint64_t sdesc_sw32(uint32_t addr)
-{
-    return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(256 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
-}
+// Low and high word of their descriptors.
+__device__ __forceinline__ uint32_t sdesc_sw32_low(uint32_t addr) { return ((addr & 0x3FFFF) >> 4) | (1u << 16); }
+constexpr uint32_t kSdescSw32High = (256u >> 4) | (1u << 14) | (6u << 29);
 __device__ __forceinline__ uint32_t sw32_off(int r, int k) // byte offset of element k (< 16) of row r
 {
     return (uint32_t)((r >> 3) * 256 + (r & 7) * 32 + ((((k >> 3) ^ ((r & 7) >> 2)) & 1) << 4) + (k & 7) * 2);

@@ -198,13 +198,15 @@ cudaError_t launch_zd_colexp(const void *psi, int nb, int n, int lines, int *E, 
 // A stage's columns are released by the last row tile's products, so the producers refill them while
 // that tile finishes; the line tiles of the next unit are loaded a unit ahead.
 //
-// What bounds it: shared memory.  A 128 x 128 x 16 product reads 8 KB of operands in its 64 clocks, all
-// that shared memory delivers, so whatever else passes through it (the row stages' copies, the
-// producers' stores, the epilogue's TMEM loads and F's stores) adds to the products' time: 0.95 ms of
-// products in 1.97 ms for a 48^3 block of 8192 pairs (16 x 512 bands, K2 = 15), tensor pipe 46 %.  With
-// the valence bands in the rows (resident) and each tile of conduction columns formed for one row
-// tile it took 2.30 ms; F stored entry by entry, 32 half sectors an instruction, 2.9 ms; exchanged in
-// quads by shuffles 2.25 ms; row stages in a ring of two instead of three 2.4 ms.
+// What bounds it: the tensor pipe and, behind it, F's stores.  A 128 x 128 x 16 product reads 8 KB of
+// operands in its 64 clocks, all that shared memory delivers, so whatever else passes through it (the row
+// stages' copies, the producers' stores) adds to the products' time.  1.80 ms for a 48^3 block of 8192
+// pairs (16 x 512 bands, K2 = 15), 1.13 ms of it with nothing but the products; 1.45 without F's stores,
+// 4.9 GB.  Issued by a lone thread, which moves every descriptor from its own registers to uniform ones, a
+// product took 95 clocks whatever its size, 1.97 ms in all.  With the valence bands in the rows
+// (resident) and each tile of conduction columns formed for one row tile it took 2.30 ms; F stored entry
+// by entry, 32 half sectors an instruction, 2.9 ms; exchanged in quads by shuffles 2.25 ms; row stages in
+// a ring of two instead of three 2.4 ms.
 //  warps 0..3: TMA, MMA (and TMEM), two producers; warps 4..11: epilogue (TMEM lane quadrant
 //  warp % 4, half of the columns each); warps 12..15: producers.
 constexpr int kZdThreads = 512;
@@ -414,14 +416,21 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                 if (!ok) atomicOr(a.status, kStatusTimeout);
             }
         } else if (warp == 1) {
-            // ---- MMA issue
-            if (lane == 0) {
-                // The pipe holds few products, so what this thread does between two stages shows: a
+            // ---- MMA issue, the warp converged (umma_f16_run)
+            {
+                const uint32_t lead = elect_lane(), tb = __shfl_sync(0xffffffffu, tbase, 0);
+                auto wait = [&](uint64_t *b, uint32_t parity) {
+                    if (!__all_sync(0xffffffffu, bar_wait(b, parity))) ok = false;
+                };
+                // The pipe holds few products, so what this warp does between two stages shows: a
                 // stage's barriers are awaited between the products of the stage before.
                 // descriptor address fields count 16-byte units: offsets below 256 KB add in place
-                const uint64_t ad0 = sdesc_sw32(su32(sA)), bd0 = sdesc_sw32(su32(sB));
+                const uint32_t ad0 = sdesc_sw32_low(su32(sA)), bd0 = sdesc_sw32_low(su32(sB));
                 uint32_t as = 0, ph = 0, tph = 1, nu = 0;
-                if (blockIdx.x < a.nunits && (!bar_wait(&bFull[0], 0) || !bar_wait(&aFull[0], 0))) ok = false;
+                if (blockIdx.x < a.nunits) {
+                    wait(&bFull[0], 0);
+                    wait(&aFull[0], 0);
+                }
                 tc_fence_after();
                 for (int u = blockIdx.x; u < a.nunits && ok; u += gridDim.x, ++nu) {
                     const bool more = u + (int)gridDim.x < a.nunits;
@@ -431,15 +440,22 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                         // A tile's first two stages go together, accumulator by accumulator as the
                         // epilogue hands them back (the least significant, with 15 products, first);
                         // a group's first product of the tile starts its accumulator.
-                        auto issue = [&](int g, uint64_t ad, uint64_t bd, uint32_t acc0) {
+                        // products of A slice i with the B slices j0 .. j1, one after the other: A is read once
+                        auto run = [&](int i, int j0, int j1, uint32_t ad, uint32_t bd, uint32_t acc0) {
+#pragma unroll
+                            for (int j = 0; j < kZdSlices; ++j)
+                                if (j >= j0 && j <= j1) {
+                                    const int g = i + j < 3 ? i + j : 3;
+                                    umma_f16_run(lead, tb + g * kZdAcc, ad + (uint32_t)((i * kZdSlice) >> 4),
+                                                 bd + (uint32_t)((j * kBSlice) >> 4), kSdescSw32High, kIdesc,
+                                                 i == 0 && j == g ? acc0 : 1u, j - j0, j1 - j0 + 1);
+                                }
+                        };
+                        auto issue = [&](int g, uint32_t ad, uint32_t bd, uint32_t acc0) {
 #pragma unroll
                             for (int i = 0; i < kZdSlices; ++i)
-#pragma unroll
-                                for (int j = 0; j < kZdSlices - i; ++j)
-                                    if ((i + j < 3 ? i + j : 3) == g)
-                                        umma_f16(tbase + g * kZdAcc, ad + (uint64_t)((i * kZdSlice) >> 4),
-                                                 bd + (uint64_t)((j * kBSlice) >> 4), kIdesc,
-                                                 i == 0 && j == g ? acc0 : 1u);
+                                if (g == 3) run(i, i < 3 ? 3 - i : 0, kZdSlices - 1 - i, ad, bd, acc0);
+                                else if (i <= g) run(i, g - i, g - i, ad, bd, acc0);
                         };
                         auto advance = [&] {
                             if (++as == ast) {
@@ -448,59 +464,62 @@ __global__ void __launch_bounds__(kZdThreads, 1) zd_gemm_kernel(const __grid_con
                             }
                         };
                         auto await = [&](bool newb, int ks, uint32_t unit) { // stage ks of this unit or the next
-                            if (newb && !bar_wait(&bFull[ks], unit & 1)) ok = false;
-                            if (!bar_wait(&aFull[as], ph)) ok = false;
+                            if (newb) wait(&bFull[ks], unit & 1);
+                            wait(&aFull[as], ph);
                             tc_fence_after();
                         };
                         {
                             const uint32_t s0 = as;
-                            const uint64_t a0 = ad0 + (uint64_t)((s0 * kZdStage) >> 4);
+                            const uint32_t a0 = ad0 + (uint32_t)((s0 * kZdStage) >> 4);
                             advance();
                             const uint32_t s1 = as;
-                            const uint64_t a1 = ad0 + (uint64_t)((s1 * kZdStage) >> 4), b1 = bd0 + (kBStage >> 4);
-                            if (!bar_wait(&tEmpty[3], tph)) ok = false;
+                            const uint32_t a1 = ad0 + (uint32_t)((s1 * kZdStage) >> 4), b1 = bd0 + (kBStage >> 4);
+                            wait(&tEmpty[3], tph);
                             tc_fence_after();
                             issue(3, a0, bd0, 0u);
                             await(mt == 0, 1, nu);
-                            if (!bar_wait(&tEmpty[2], tph)) ok = false;
+                            wait(&tEmpty[2], tph);
                             tc_fence_after();
                             issue(2, a0, bd0, 0u);
                             issue(3, a1, b1, 1u);
                             issue(2, a1, b1, 1u);
-                            if (!bar_wait(&tEmpty[1], tph) || !bar_wait(&tEmpty[0], tph)) ok = false;
+                            wait(&tEmpty[1], tph);
+                            wait(&tEmpty[0], tph);
                             tc_fence_after();
                             issue(1, a0, bd0, 0u);
                             issue(0, a0, bd0, 0u);
-                            umma_commit(&aEmpty[s0]);
-                            if (last) umma_commit(&bEmpty[0]);
+                            umma_commit_lead(lead, &aEmpty[s0]);
+                            if (last) umma_commit_lead(lead, &bEmpty[0]);
                             issue(1, a1, b1, 1u);
                             advance();
                             await(mt == 0, 2, nu);
                             issue(0, a1, b1, 1u);
-                            umma_commit(&aEmpty[s1]);
-                            if (last) umma_commit(&bEmpty[1]);
+                            umma_commit_lead(lead, &aEmpty[s1]);
+                            if (last) umma_commit_lead(lead, &bEmpty[1]);
                         }
                         for (int ks = 2; ks < nst && ok; ++ks) {
-                            const uint64_t ad = ad0 + (uint64_t)((as * kZdStage) >> 4);
-                            const uint64_t bd = bd0 + (uint64_t)((ks * kBStage) >> 4);
+                            const uint32_t ad = ad0 + (uint32_t)((as * kZdStage) >> 4);
+                            const uint32_t bd = bd0 + (uint32_t)((ks * kBStage) >> 4);
                             const uint32_t cur = as;
                             advance();
-                            issue(2, ad, bd, 1u);
-                            issue(1, ad, bd, 1u);
-                            issue(0, ad, bd, 1u);
+                            run(0, 0, 5, ad, bd, 1u);
+                            run(1, 0, 4, ad, bd, 1u);
                             // the next stage: of this tile, of the next tile or of the next unit
                             if (ks + 1 < nst) await(mt == 0, ks + 1, nu);
                             else if (!last || more) await(last, 0, nu + 1);
-                            issue(3, ad, bd, 1u);
-                            umma_commit(&aEmpty[cur]);
-                            if (last) umma_commit(&bEmpty[ks]);
+                            run(2, 0, 3, ad, bd, 1u);
+                            run(3, 0, 2, ad, bd, 1u);
+                            run(4, 0, 1, ad, bd, 1u);
+                            run(5, 0, 0, ad, bd, 1u);
+                            umma_commit_lead(lead, &aEmpty[cur]);
+                            if (last) umma_commit_lead(lead, &bEmpty[ks]);
                         }
-                        umma_commit(tFull);
+                        umma_commit_lead(lead, tFull);
                     }
                 }
-                umma_commit(fin);
-                bar_wait(fin, 0);
-                if (!ok) atomicOr(a.status, kStatusTimeout);
+                umma_commit_lead(lead, fin);
+                wait(fin, 0);
+                if (!ok && lead) atomicOr(a.status, kStatusTimeout);
             }
         } else {
             // ---- producers: column slices of the valence tile, stage by stage.  A lane owns point

@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256) zd64_colexp_kernel(const double2 *__restr
 //  warps 0..3: TMA, MMA (and TMEM), two producers; warps 4..11: epilogue (TMEM lane quadrant
 //  warp % 4, half of the columns each); warps 12..15: producers.
 //
-// 4.75 ms for 8192 pairs on 48^3 (8 x 1024 bands, K2 = 15), of which the products take 1.8; the FFT pair
+// 4.31 ms for 8192 pairs on 48^3 (8 x 1024 bands, K2 = 15), of which the products take 1.8; the FFT pair
 // kernel spends most of its 55 ms on this axis, on the FP64 pipe.  The epilogue uses no FP64 instruction:
 // converting and scaling 96 x 128 sums there would take longer than the tile's products.
 constexpr int kQdThreads = 512;
@@ -334,22 +334,40 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
                 if (!ok) atomicOr(a.status, kStatusTimeout);
             }
         } else if (warp == 1) {
-            // ---- MMA issue
-            if (lane == 0) {
-                const uint64_t ad0 = sdesc_sw32(su32(sA)), bd0 = sdesc_sw32(su32(sB));
+            // ---- MMA issue, the warp converged (umma_f16_run)
+            {
+                const uint32_t lead = elect_lane(), tb = __shfl_sync(0xffffffffu, tbase, 0);
+                auto wait = [&](uint64_t *b, uint32_t parity) {
+                    if (!__all_sync(0xffffffffu, bar_wait(b, parity))) ok = false;
+                };
+                const uint32_t ad0 = sdesc_sw32_low(su32(sA)), bd0 = sdesc_sw32_low(su32(sB));
                 uint32_t as = 0, ph = 0, nu = 0;
                 uint32_t e012 = 1, e3 = 1; // parities of the accumulators' next release
-                if (blockIdx.x < a.nunits && (!bar_wait(&bFull[0], 0) || !bar_wait(&aFull[0], 0))) ok = false;
+                if (blockIdx.x < a.nunits) {
+                    wait(&bFull[0], 0);
+                    wait(&aFull[0], 0);
+                }
                 tc_fence_after();
-                auto issue = [&](auto G, uint64_t ad, uint64_t bd, uint32_t acc0) {
+                // group g, at a pass's first stage
+                auto issue = [&](auto G, uint32_t ad, uint32_t bd) {
                     constexpr int g = decltype(G)::value;
 #pragma unroll
                     for (int i = 0; i <= g; ++i)
-                        umma_f16(tbase + qd_slot(g) * kZdAcc, ad + (uint64_t)((i * kQdASlice) >> 4),
-                                 bd + (uint64_t)(((g - i) * kQdBSlice) >> 4), kQdIdesc, i == 0 ? acc0 : 1u);
+                        umma_f16_run(lead, tb + qd_slot(g) * kZdAcc, ad + (uint32_t)((i * kQdASlice) >> 4),
+                                 bd + (uint32_t)(((g - i) * kQdBSlice) >> 4), kSdescSw32High, kQdIdesc,
+                                     i == 0 ? 0u : 1u, 0, 1);
+                };
+                // A slice i with its B slices of the pass's groups g0 .. g1, one after the other: A is read once
+                auto run = [&](int i, int g0, int g1, uint32_t ad, uint32_t bd) {
+#pragma unroll
+                    for (int j = 0; j < kQdSlices; ++j)
+                        if (i + j >= g0 && i + j <= g1)
+                            umma_f16_run(lead, tb + qd_slot(i + j) * kZdAcc, ad + (uint32_t)((i * kQdASlice) >> 4),
+                                         bd + (uint32_t)((j * kQdBSlice) >> 4), kSdescSw32High, kQdIdesc, 1u,
+                                         j - (g0 > i ? g0 - i : 0), g1 - i + 1 - (g0 > i ? g0 - i : 0));
                 };
                 auto room = [&](int slot, uint32_t par) {
-                    if (!bar_wait(&tEmpty[slot], par)) ok = false;
+                    wait(&tEmpty[slot], par);
                     tc_fence_after();
                 };
                 for (int u = blockIdx.x; u < a.nunits && ok; u += gridDim.x, ++nu) {
@@ -358,9 +376,9 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
                         const bool last = mt == a.nmt - 1;
                         for (int ps = 0; ps < 2 && ok; ++ps) {
                             for (int ks = 0; ks < nst && ok; ++ks) {
-                                const uint64_t ad = ad0 + (uint64_t)((as * kQdAStage) >> 4);
-                                const uint64_t bd = bd0 + (uint64_t)((ks * kQdBStage) >> 4);
-                                const uint32_t cur = as, acc0 = ks == 0 ? 0u : 1u;
+                                const uint32_t ad = ad0 + (uint32_t)((as * kQdAStage) >> 4);
+                                const uint32_t bd = bd0 + (uint32_t)((ks * kQdBStage) >> 4);
+                                const uint32_t cur = as;
                                 if (++as == ast) {
                                     as = 0;
                                     ph ^= 1;
@@ -370,41 +388,53 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
                                     const bool wrap = ks + 1 == nst;
                                     if (wrap && ps == 1 && last && !more) return;
                                     const bool newb = wrap ? ps == 1 && last : ps == 0 && mt == 0;
-                                    if (newb && !bar_wait(&bFull[wrap ? 0 : ks + 1], (wrap ? nu + 1 : nu) & 1)) ok = false;
-                                    if (!bar_wait(&aFull[as], ph)) ok = false;
+                                    if (newb) wait(&bFull[wrap ? 0 : ks + 1], (wrap ? nu + 1 : nu) & 1);
+                                    wait(&aFull[as], ph);
                                     tc_fence_after();
                                 };
-                                if (ps == 0) {
-                                    if (ks == 0) room(0, e012);
-                                    issue(QdInt<6>{}, ad, bd, acc0);
-                                    if (ks == 0) room(1, e012);
-                                    issue(QdInt<5>{}, ad, bd, acc0);
+                                if (ks == 0 && ps == 0) {
+                                    room(0, e012);
+                                    issue(QdInt<6>{}, ad, bd);
+                                    room(1, e012);
+                                    issue(QdInt<5>{}, ad, bd);
                                     next();
-                                    if (ks == 0) room(2, e012);
-                                    issue(QdInt<4>{}, ad, bd, acc0);
+                                    room(2, e012);
+                                    issue(QdInt<4>{}, ad, bd);
+                                } else if (ks == 0) {
+                                    room(3, e3);
+                                    issue(QdInt<3>{}, ad, bd);
+                                    room(0, e012);
+                                    issue(QdInt<2>{}, ad, bd);
+                                    next();
+                                    room(1, e012);
+                                    issue(QdInt<1>{}, ad, bd);
+                                    room(2, e012);
+                                    issue(QdInt<0>{}, ad, bd);
+                                } else if (ps == 0) {
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i) run(i, 4, 6, ad, bd);
+                                    next();
+#pragma unroll
+                                    for (int i = 4; i < 7; ++i) run(i, 4, 6, ad, bd);
                                 } else {
-                                    if (ks == 0) room(3, e3);
-                                    issue(QdInt<3>{}, ad, bd, acc0);
-                                    if (ks == 0) room(0, e012);
-                                    issue(QdInt<2>{}, ad, bd, acc0);
+                                    run(0, 0, 3, ad, bd);
+                                    run(1, 0, 3, ad, bd);
                                     next();
-                                    if (ks == 0) room(1, e012);
-                                    issue(QdInt<1>{}, ad, bd, acc0);
-                                    if (ks == 0) room(2, e012);
-                                    issue(QdInt<0>{}, ad, bd, acc0);
-                                    if (last) umma_commit(&bEmpty[ks]);
+                                    run(2, 0, 3, ad, bd);
+                                    run(3, 0, 3, ad, bd);
                                 }
-                                umma_commit(&aEmpty[cur]);
+                                if (ps == 1 && last) umma_commit_lead(lead, &bEmpty[ks]);
+                                umma_commit_lead(lead, &aEmpty[cur]);
                             }
                             e012 ^= 1;
-                            umma_commit(tFull);
+                            umma_commit_lead(lead, tFull);
                         }
                         e3 ^= 1;
                     }
                 }
-                umma_commit(fin);
-                bar_wait(fin, 0);
-                if (!ok) atomicOr(a.status, kStatusTimeout);
+                umma_commit_lead(lead, fin);
+                wait(fin, 0);
+                if (!ok && lead) atomicOr(a.status, kStatusTimeout);
             }
         } else {
             // ---- producers: column slices of the valence tile, stage by stage.  A lane owns point
