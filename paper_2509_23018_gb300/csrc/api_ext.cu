@@ -273,6 +273,27 @@ static gw_status square_product(gw_chi0 *h, const double2 *A, const double2 *B, 
 // Slices of the split products of the last Newton-Schulz steps (the most the digit step takes).
 constexpr int kEpsFinalSlices = 8;
 
+// Accuracy (the ABI's nslices) of a step that starts at ||I - A X|| <= rho, which it squares: the least
+// whose products change the residual by no more than a quarter of that, or than 2e-5, which the last two
+// steps bring to 1e-19.  With n 9-bit slices an entry of a product of two N x N matrices carries about
+// N^(1/2) 2^(-9n) of its row's and column's largest entries, the matrix N^(1/2) times that, and the
+// residual ||A|| <= b times it; the factor 8 covers the step's two products.  N_G = 2000, b = 52: six
+// of eleven steps with three slices (6 products each), three with four (10), two with six (21), where
+// nine had five (15): 30.2 -> 23.4 ms for two frequencies.
+static int eps_step_slices(const gw_chi0 *h, int ng, double b, double *rho)
+{
+    const double next = *rho * *rho;
+    for (int nslices : {4, 5}) { // three and four slices
+        const double f = 8.0 * ng * b * std::ldexp(1.0, -9 * gw::oz_slices(nslices));
+        if (nslices < h->d.nslices && f <= std::max(0.25 * next, 2e-5)) {
+            *rho = next + f;
+            return nslices;
+        }
+    }
+    *rho = next;
+    return 0;
+}
+
 gw_status gw_chi0_epsilon_inverse(gw_chi0 *h, int ng, int nw, const double *chi, const double *vcoul,
                                   double *epsinv)
 {
@@ -309,10 +330,13 @@ gw_status gw_chi0_epsilon_inverse(gw_chi0 *h, int ng, int nw, const double *chi,
         steps = std::max(steps, 1);
         CK(h, gw::launch_eps_init(X, ng, bmax, h->st), "X0");
         // The error of the converged iterate is the rounding of the last steps' products (earlier
-        // errors are squared away), so in split precision the last two steps take the most slices.
+        // errors are squared away), so in split precision the last two steps take the most slices, and
+        // the earlier ones no more than their own error asks for (eps_step_slices).
+        double rho = r;
         for (int k = 0; k < steps; ++k) {
             Scope sp(h, "eps_products"); // two N_G^3 products per step: the launch count gives the steps
-            const int s = (h->d.prec == GW_PREC_OZAKI_BF16 && k >= steps - 2) ? kEpsFinalSlices : 0;
+            int s = 0;
+            if (h->d.prec == GW_PREC_OZAKI_BF16) s = k >= steps - 2 ? kEpsFinalSlices : eps_step_slices(h, ng, b, &rho);
             if ((st = square_product(h, A, X, ng, T, s)) || (st = square_product(h, X, T, ng, Pm, s))) return st;
             CK(h, gw::launch_eps_step(X, Pm, (int64_t)nn, h->st), "Newton-Schulz step");
         }
