@@ -250,16 +250,14 @@ __global__ void __launch_bounds__(256) adj_pair_kernel(const double2 *__restrict
 // an entry either way; Gb is not read again), the i0 sums per cell reading it from L2, both line
 // transforms in hi + lo pairs; H is written in two-float form.  Keeping conj(g_p) out of shared
 // memory lets four blocks run per SM on 40^3 instead of two.
-// N > 0: a cubic N^3 grid, the line transforms and index arithmetic specialised at compile time;
-// N = 0: any grid, runtime plans.
-template <int N>
+// Any grid, runtime plans; the cubic grids below take adj_cells_tf_kernel and adj_slab_tf_kernel.
 __global__ void __launch_bounds__(256) adj_pair_tf_kernel(double2 *__restrict__ Gb, PairPlan pp,
                                                           const int *__restrict__ cell_start,
                                                           const int *__restrict__ cell_g, int ncell, TfConsts kc,
                                                           tf sc, float4 *__restrict__ H)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int n0 = N ? N : pp.n[0], n1 = N ? N : pp.n[1], n2 = N ? N : pp.n[2];
+    const int n0 = pp.n[0], n1 = pp.n[1], n2 = pp.n[2];
     const int ns = n1 * n2;
     float4 *a = (float4 *)smem, *b = a + ns;
     float4 *tw0 = b + ns, *tw1 = tw0 + n0, *tw2 = tw1 + n1;
@@ -293,9 +291,7 @@ __global__ void __launch_bounds__(256) adj_pair_tf_kernel(double2 *__restrict__ 
             tc_store(a + cell_pos, acc);
         }
         __syncthreads();
-        float4 *r;
-        if constexpr (N > 0) r = tfft_lines_ct<N>(a, b, pp.K2, n1, tw1, kc); // along i1, K2 lines
-        else r = tfft_lines(a, b, pp.K2, n1, 1, pp.ax[1], tw1, kc);
+        float4 *r = tfft_lines(a, b, pp.K2, n1, 1, pp.ax[1], tw1, kc); // along i1, K2 lines
         float4 *o = (r == a) ? b : a;
         for (int i = threadIdx.x; i < ns; i += blockDim.x) o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncthreads();
@@ -304,15 +300,186 @@ __global__ void __launch_bounds__(256) adj_pair_tf_kernel(double2 *__restrict__ 
             o[i1 * n2 + kz[q]] = r[i];
         }
         __syncthreads();
-        const float4 *t;
-        if constexpr (N > 0) t = tfft_lines_ct<N>(o, r, n1, n2, tw2, kc); // along i2
-        else t = tfft_lines(o, r, n1, n2, 1, pp.ax[2], tw2, kc);
+        const float4 *t = tfft_lines(o, r, n1, n2, 1, pp.ax[2], tw2, kc); // along i2
         for (int i = threadIdx.x; i < ns; i += blockDim.x) {
             const tcx z = tc_load(t + i);
             tc_store(out + (int64_t)i0 * ns + i, tcx{tf_mul(z.re, sc), tf_neg(tf_mul(z.im, sc))});
         }
         __syncthreads();
     }
+}
+
+// The back-projection on a cubic N^3 grid in two kernels, the transforms of the pair elements from F
+// (pair_split_ct.cuh) turned around: the sphere's points along i0, (k1, k2) cell by cell, then slab by
+// slab the K2 columns along i1 and all N lines along i2.
+//
+// What bounds them: issue on the FP32 pipes, about 10 million two-float operations a pair on 40^3, most
+// of them along i2.  The cells' i0 transform is an FFT (a direct sum over the sphere for every slab costs as
+// much as the lines along i2), lines run fastest over the threads at an odd stride, and the first stage
+// of i1 and of i2 reads its inputs where they are, zeros never stored.  The cells pass through the
+// end of the pair's own H: S row i0 lies behind every slab up to i0 - 1.
+// ADJ_FIGURES
+constexpr int kAdjBatch = 32; // cells per batch
+template <int N>
+__global__ void __launch_bounds__(192, N <= 48 ? 4 : 2)
+    adj_cells_tf_kernel(const double2 *__restrict__ Gb, PairPlan pp, TfConsts kc, tf sc, float4 *__restrict__ H)
+{
+    constexpr int CS = N + 1;
+    extern __shared__ __align__(16) unsigned char smem[];
+    float4 *X = (float4 *)smem, *Y = X + kAdjBatch * CS, *tw = Y + kAdjBatch * CS;
+    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = pp.ax[0].twf[i];
+    const int64_t p = blockIdx.x, nr = (int64_t)N * N * N;
+    const int K12 = pp.K12;
+    float4 *S = H + (p + 1) * nr - (int64_t)N * K12;
+    const double2 *g = Gb + p * pp.ng;
+    for (int d0 = 0; d0 < K12; d0 += kAdjBatch) {
+        const int nbat = min(kAdjBatch, K12 - d0);
+        for (int i = threadIdx.x; i < nbat * CS; i += blockDim.x) X[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        __syncthreads();
+        const int m1 = pp.cstart[d0 + nbat];
+        for (int m = pp.cstart[d0] + threadIdx.x; m < m1; m += blockDim.x) {
+            const int2 pt = pp.cpts[m];
+            if (!GW_IN(pt.x, pp.ng, pp.status) || !GW_IN((pt.y >> 8) - d0, nbat, pp.status)) continue;
+            const double2 x = g[pt.x]; // conj(g_p) / N_r
+            tc_store(X + ((pt.y >> 8) - d0) * CS + (pt.y & 255), tcx{tf_mul(tf_from(x.x), sc), tf_mul(tf_from(-x.y), sc)});
+        }
+        __syncthreads();
+        const float4 *r = tfft_lines_ct<N, true>(X, Y, nbat, CS, tw, kc);
+        for (int e = threadIdx.x; e < nbat * N; e += blockDim.x) {
+            const int i0 = e / nbat, d = e - i0 * nbat;
+            S[(int64_t)i0 * K12 + d0 + d] = r[d * CS + i0];
+        }
+        __syncthreads();
+    }
+}
+
+// 5-point transform of inputs 0 and 4 alone (v[1..3] zero)
+__device__ __forceinline__ void adj_dft5_ends(tcx *v, const TfConsts &k)
+{
+    const tcx a = v[0], b = v[4];
+    const tcx t1 = tc_addl(a, tc_rmul(b, k.c1)), u1 = tc_muli(tc_rmul(b, k.s1));
+    const tcx t2 = tc_addl(a, tc_rmul(b, k.c2)), u2 = tc_muli(tc_rmul(b, k.s2));
+    v[0] = tc_norm(tc_addl(a, b));
+    v[1] = tc_norm(tc_subl(t1, u1)); // W_5^{4 k} = conj(W_5^k)
+    v[4] = tc_norm(tc_addl(t1, u1));
+    v[2] = tc_norm(tc_subl(t2, u2));
+    v[3] = tc_norm(tc_addl(t2, u2));
+}
+
+// First stage of make_rad_plan(N) with inputs ld(line, point, present); lines fastest over the threads.
+// The kept frequencies lie around 0, so that a 5-point transform mostly has its first and last input.
+template <int N, class LD>
+__device__ __forceinline__ void adj_stage0(LD ld, float4 *__restrict__ y, int nlines, int CS, LMap lm, const TfConsts &kc)
+{
+    constexpr int R = make_rad_plan(N).r[0], nb = N / R;
+    int l = lm.l0, j = lm.j0;
+    while (j < nb) {
+        tcx v[R];
+        bool in[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = ld(l, j + r * nb, in[r]);
+        bool inner = R != 5;
+#pragma unroll
+        for (int r = 1; r + 1 < R; ++r) inner = inner || in[r];
+        if (inner) tdftR<R>(v, kc);
+        else if constexpr (R == 5) adj_dft5_ends(v, kc);
+        float4 *yl = y + l * CS + j * R;
+#pragma unroll
+        for (int r = 0; r < R; ++r) tc_store(yl + r, v[r]);
+        l += lm.dl;
+        j += lm.dj;
+        if (l >= nlines) {
+            l -= nlines;
+            ++j;
+        }
+    }
+}
+
+template <int N>
+constexpr int adj_slab_threads()
+{
+    return N <= 24 ? 192 : N <= 48 ? 256 : 512;
+}
+template <int N>
+__global__ void __launch_bounds__(adj_slab_threads<N>(), N <= 40 ? 3 : N <= 48 ? 2 : 1)
+    adj_slab_tf_kernel(PairPlan pp, TfConsts kc, float4 *__restrict__ H)
+{
+    constexpr int CS = N + 1, ns = N * N, R0 = make_rad_plan(N).r[0];
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int K2 = pp.K2, K12 = pp.K12;
+    float4 *Z1 = (float4 *)smem, *Z2 = Z1 + N * CS, *tw = Z2 + N * CS, *srow = tw + N; // [2][K12]
+    short *cm = (short *)(srow + 2 * K12), *qinv = cm + K2 * N; // cell at (k1, q), column of i2 (or -1)
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+        tw[i] = pp.ax[0].twf[i];
+        qinv[i] = -1;
+    }
+    for (int i = threadIdx.x; i < K2 * N; i += blockDim.x) cm[i] = -1;
+    __syncthreads();
+    for (int q = threadIdx.x; q < K2; q += blockDim.x) qinv[pp.kz[q]] = (short)q;
+    for (int d = threadIdx.x; d < K12; d += blockDim.x) {
+        const int cl = pp.cell[d];
+        if (GW_IN(cl >> 8, K2, pp.status)) cm[(cl & 255) * K2 + (cl >> 8)] = (short)d;
+    }
+    const int64_t p = blockIdx.x, nr = (int64_t)N * ns;
+    float4 *out = H + p * nr;
+    const float4 *S = out + nr - (int64_t)N * K12;
+    auto fetch = [&](int i0) {
+        for (int d = threadIdx.x; d < K12; d += blockDim.x)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(srow + (i0 & 1) * K12 + d)),
+                         "l"(S + (int64_t)i0 * K12 + d)
+                         : "memory");
+    };
+    fetch(0);
+    const LMap lm1 = lmap_lines_fastest(K2), lm2 = lmap_lines_fastest(N);
+    const tcx zero{{0.f, 0.f}, {0.f, 0.f}};
+    for (int i0 = 0; i0 < N; ++i0) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads(); // row i0 is here, and the slab before is written
+        if (i0 + 1 < N) fetch(i0 + 1);
+        const float4 *sr = srow + (i0 & 1) * K12;
+        float4 *Y1 = Z2, *Y2 = Z2 + K2 * CS; // the K2 columns, K2 <= N / 2
+        adj_stage0<N>(
+            [&](int q, int k1, bool &in) {
+                const int d = cm[k1 * K2 + q];
+                in = d >= 0;
+                return in ? tc_load(sr + d) : zero;
+            },
+            Y1, K2, CS, lm1, kc);
+        __syncthreads();
+        const float4 *r = tstages_ct<N, 1, R0, false, true>(Y1, Y2, K2, CS, tw, kc, 1, -1, lm1);
+        adj_stage0<N>(
+            [&](int i1, int i2, bool &in) {
+                const int q = qinv[i2];
+                in = q >= 0;
+                return in ? tc_load(r + q * CS + i1) : zero;
+            },
+            Z1, N, CS, lm2, kc);
+        __syncthreads();
+        const float4 *t = tstages_ct<N, 1, R0, false, true>(Z1, Z2, N, CS, tw, kc, 1, -1, lm2);
+        for (int i = threadIdx.x; i < ns; i += blockDim.x) {
+            const float4 z = t[i / N * CS + i % N];
+            out[(int64_t)i0 * ns + i] = make_float4(z.x, z.y, -z.z, -z.w);
+        }
+    }
+}
+
+template <int N>
+static cudaError_t launch_adj_cube(const double2 *Gb, int64_t P, const PairPlan &pp, tf sc, float4 *H, cudaStream_t st)
+{
+    const size_t sm1 = sizeof(float4) * (2 * (size_t)kAdjBatch * (N + 1) + N);
+    const size_t sm2 = sizeof(float4) * (2 * (size_t)N * (N + 1) + N + 2 * (size_t)pp.K12) +
+                       sizeof(short) * ((size_t)pp.K2 * N + N);
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(adj_cells_tf_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1)) !=
+            cudaSuccess ||
+        (e = cudaFuncSetAttribute(adj_slab_tf_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2)) !=
+            cudaSuccess)
+        return e;
+    adj_cells_tf_kernel<N><<<(unsigned)P, 192, sm1, st>>>(Gb, pp, tf_consts(), sc, H);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    adj_slab_tf_kernel<N><<<(unsigned)P, adj_slab_threads<N>(), sm2, st>>>(pp, tf_consts(), H);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_adj_pair(double2 *Gb, int64_t P, const PairPlan &pp, const int *cell_start,
@@ -326,17 +493,18 @@ cudaError_t launch_adj_pair(double2 *Gb, int64_t P, const PairPlan &pp, const in
         const float hi = (float)inv;
         const tf sc{hi, (float)(inv - (double)hi)};
         const bool cubic = pp.n[0] == pp.n[1] && pp.n[1] == pp.n[2];
-        auto run = [&](auto kern) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess) return e;
-            kern<<<(unsigned)P, 256, sm, st>>>(Gb, pp, cell_start, cell_g, ncell, tf_consts(), sc, (float4 *)H);
-            return cudaGetLastError();
-        };
-        if (cubic && pp.n[0] == 24) return run(adj_pair_tf_kernel<24>);
-        if (cubic && pp.n[0] == 40) return run(adj_pair_tf_kernel<40>);
-        if (cubic && pp.n[0] == 48) return run(adj_pair_tf_kernel<48>);
-        if (cubic && pp.n[0] == 72) return run(adj_pair_tf_kernel<72>);
-        return run(adj_pair_tf_kernel<0>);
+        // the columns of i1 lie in one of the two buffers of i2
+        if (cubic && 2 * pp.K2 <= pp.n[0]) {
+            if (pp.n[0] == 24) return launch_adj_cube<24>(Gb, P, pp, sc, (float4 *)H, st);
+            if (pp.n[0] == 40) return launch_adj_cube<40>(Gb, P, pp, sc, (float4 *)H, st);
+            if (pp.n[0] == 48) return launch_adj_cube<48>(Gb, P, pp, sc, (float4 *)H, st);
+            if (pp.n[0] == 72) return launch_adj_cube<72>(Gb, P, pp, sc, (float4 *)H, st);
+        }
+        cudaError_t e =
+            cudaFuncSetAttribute(adj_pair_tf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+        adj_pair_tf_kernel<<<(unsigned)P, 256, sm, st>>>(Gb, pp, cell_start, cell_g, ncell, tf_consts(), sc, (float4 *)H);
+        return cudaGetLastError();
     }
     size_t sm = sizeof(double2) * (2 * (size_t)pp.n[1] * pp.n[2] + pp.n[0] + pp.n[1] + pp.n[2] + pp.ng) +
                 sizeof(int) * pp.K2;
