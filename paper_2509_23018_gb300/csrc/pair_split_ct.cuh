@@ -2,8 +2,8 @@
 // axis lengths: one kernel per middle-axis length N1 (a pair's slabs to the sphere's (k1, k2) cells)
 // and one per first-axis length N0 (cells to sphere points), the cells [pair][n0][K12] in global
 // memory between them.  Bound by issue like pair_kernel_tf_from_f, which runs both phases of the cubic
-// 40^3 and 48^3 grids in one kernel with the cells in L2: 0.253 us a pair on 48^3 (K2 = 15) where these
-// two take 0.258.  72^3 (K2 = 23): 1.18 us a pair, and 3.1 with the last axis and its slices, where the
+// 40^3 and 48^3 grids in one kernel with the cells in L2: 0.248 us a pair on 48^3 (K2 = 15) where these
+// two take 2 % more.  72^3 (K2 = 23): 1.18 us a pair, and 3.1 with the last axis and its slices, where the
 // FFT pair kernel takes 5.1; 30 x 36 x 40: 0.15, and 0.41, where the runtime-shape kernel takes 1.26.
 #pragma once
 #include "pair_tf_ct.cuh"
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kSplitThreads, split_min_blocks<N>())
             tma2_hint(C, &tmF, &fbar, (int)(row * k2p * 4), i0 * N, stream);
         }
     };
-    const LMap lm = lmap_lines_fastest(ncols);
+    const LMap lm = lmap_lines(ncols);
     fetch(0, X);
     uint32_t nf = 0;
     for (int i0 = 0; i0 < n0; i0 += 2, ++nf) {
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kSplitThreads, split_min_blocks<N>())
             if (threadIdx.x == 0) atomicOr(pp.status, kStatusTimeout);
             return;
         }
-        const LMap lm = lmap_lines_fastest(nbat);
+        const LMap lm = lmap_lines(nbat);
         tstage0_rows<N>(X, Y, nbat, NB, nbat, CS, lm, kc);
         __syncthreads();
         float4 *y = tstages_ct<N, 1, make_prune_plan(N).r[0], true, true>(Y, X, nbat, CS, tw, kc, 1, -1, lm);

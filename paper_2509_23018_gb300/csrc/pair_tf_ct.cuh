@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(pair_threads<N>(), pair_min_blocks<N>())
             tma2_hint(C, &tmF, &fbar, (int)(row * ((K2 + 1) / 2 * 2) * 4), i0 * N, stream);
         }
     };
-    const LMap lm = lmap_lines_fastest(ncols);
+    const LMap lm = lmap_lines(ncols);
     fetch(0, Xb);
     uint32_t nf = 0;
     for (int i0 = 0, b = 0; i0 < N; i0 += 2, b ^= 1, ++nf) {
@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(pair_threads<N>(), pair_min_blocks<N>())
             if (threadIdx.x == 0) atomicOr(pp.status, kStatusTimeout);
             return;
         }
-        const LMap lm2 = lmap_lines_fastest(nbat);
+        const LMap lm2 = lmap_lines(nbat);
         tstage0_rows<N>(X, Y, nbat, NB, nbat, CS, lm2, kc);
         __syncthreads();
         const float4 *y0 = tstages_ct<N, 1, make_prune_plan(N).r[0], true, true>(Y, X, nbat, CS, tw, kc, 1, -1, lm2);
