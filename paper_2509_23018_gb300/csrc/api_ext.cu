@@ -279,7 +279,8 @@ constexpr int kEpsFinalSlices = 8;
 // N^(1/2) 2^(-9n) of its row's and column's largest entries, the matrix N^(1/2) times that, and the
 // residual ||A|| <= b times it; the factor 8 covers the step's two products.  N_G = 2000, b = 52: six
 // of eleven steps with three slices (6 products each), three with four (10), two with six (21), where
-// nine had five (15): 30.2 -> 23.4 ms for two frequencies.
+// nine had five (15): 30.2 -> 23.4 ms for two frequencies (21.7 with the
+// column slices and the stores of the products as they are now).
 static int eps_step_slices(const gw_chi0 *h, int ng, double b, double *rho)
 {
     const double next = *rho * *rho;

@@ -253,6 +253,8 @@ gw_status contract_chunk_ozaki(gw_chi0 *h, const double2 *M, int64_t P, int ng, 
 gw_status contract_chunk(gw_chi0 *h, const double2 *M, int64_t P, int ng, const double *delta, int64_t dstride,
                          int nw, double2 *chi, bool given = false);
 int64_t oz_kpad(int ka);
+cudaError_t launch_oz_columns(const double2 *B, int ka, int nout, int64_t ldb, int s, int64_t kpad, void *Z, int *E,
+                              cudaStream_t st);
 // nslices > 0 overrides the handle's slice count (both calls of one product must agree)
 gw_status oz_prepare_b(gw_chi0 *h, const double2 *B, int ka, int nout, int nslices = 0);
 gw_status oz_product(gw_chi0 *h, const double2 *A, int64_t rows, int ka, int nout, double2 *Y, int nslices = 0);

@@ -47,7 +47,7 @@ int p_batch(const gw_chi0 *h, int ebx, int ng, int s, int64_t kpad)
 }
 
 gw_status gen_job(gw_chi0 *h, gw::OzJob &j, void *ZA, int rows_a, void *ZB, int nout, int64_t kpad, const int *EA,
-                  const int *EB, double2 *out, int64_t ldo)
+                  const int *EB, double2 *out, int64_t ldo, bool add)
 {
     std::memset(&j, 0, sizeof j);
     const int s = gw::oz_slices(h->d.nslices);
@@ -61,6 +61,7 @@ gw_status gen_job(gw_chi0 *h, gw::OzJob &j, void *ZA, int rows_a, void *ZB, int 
     j.ldo = 2 * ldo;
     j.rows_a = rows_a;
     j.cols_b = nout;
+    j.add = add;
     j.nk = (int)(kpad / gw::oz_box_k());
     j.s = s;
     return GW_OK;
@@ -116,7 +117,6 @@ gw_status sigma_split(gw_chi0 *h, int nb, int nocc, int nsig, int ng, const doub
             CK(h, gw::launch_oz_split(Mn, nsig, ng, ng, 1, false, s, kpad, ZA, EA, h->st), "M_n slices");
             CK(h, gw::launch_oz_split(Mn, nsig, ng, ng, 1, true, s, kpad, ZB, EB, h->st), "conj(M_n)^T slices");
         }
-        if (it.p0 == 0) CK(h, cudaMemsetAsync(XT, 0, sizeof(double2) * (size_t)ng * ldx, h->st), "zero X^T");
         {
             double d[gw::kGppMaxE];
             for (int j = 0; j < it.cp; ++j) d[j] = E[it.e0 + it.p0 + j] - En[it.n];
@@ -129,7 +129,7 @@ gw_status sigma_split(gw_chi0 *h, int nb, int nocc, int nsig, int ng, const doub
         jobs.assign(it.cp, gw::OzJob{});
         for (int j = 0; j < it.cp; ++j)
             if ((st = gen_job(h, jobs[j], ZP + 2 * zp1 * j, ng, ZB, nsig, kpad, EP + (size_t)j * ng, EB,
-                              XT + (size_t)(it.p0 + j) * nsig, ldx)))
+                              XT + (size_t)(it.p0 + j) * nsig, ldx, false)))
                 return st;
         {
             Scope sc(h, "gpp_gemm_x");
@@ -138,13 +138,12 @@ gw_status sigma_split(gw_chi0 *h, int nb, int nocc, int nsig, int ng, const doub
         if (it.p0 + it.cp == it.cx) {
             {
                 Scope sc(h, "oz_split_x");
-                CK(h, gw::launch_oz_split(XT, it.cx * nsig, ng, 1, ldx, false, s, kpad, ZX, EX, h->st),
-                   "X^T slices");
+                CK(h, launch_oz_columns(XT, ng, it.cx * nsig, ldx, s, kpad, ZX, EX, h->st), "X^T slices");
             }
             // Sigma^T[m][(e, l)] += sum_c M_n[m][c] X^T[c][(e, l)]
             jobs.assign(1, gw::OzJob{});
             if ((st = gen_job(h, jobs[0], ZA, nsig, ZX, it.cx * nsig, kpad, EA, EX, ST + (size_t)it.e0 * nsig,
-                              (int64_t)ne * nsig)))
+                              (int64_t)ne * nsig, true)))
                 return st;
             Scope sc(h, "gpp_gemm_sigma");
             if ((st = launch_oz_general(h, jobs))) return st;

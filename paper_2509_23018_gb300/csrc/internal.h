@@ -163,7 +163,7 @@ size_t contract_f64_smem(int bt);
 // ---- stage (b), split precision on BF16 tensor cores (ozaki.cu)
 // sp[i] = sqrt(-delta[i])
 cudaError_t launch_oz_sqrt(const double *delta, int64_t n, double *sp, cudaStream_t st);
-// E[g] = column exponent of s_p M[p][g] over the chunk; guard (or null): set to 1 where the FP64
+// E[g] = column exponent of s_p M[p][g] (sp null: of M[p][g]) over the chunk; guard (or null): set to 1 where the FP64
 // contraction by slices does not hold (entries not finite, columns scaled by more than 2^+-390)
 cudaError_t launch_oz_colexp(const double2 *M, int64_t P, int ng, const double *sp, int *E, int *guard,
                              cudaStream_t st);
@@ -188,7 +188,7 @@ struct __align__(128) OzJob {
     const int *E2;
     double *out;
     int64_t ldo;
-    int rows_a, cols_b;
+    int rows_a, cols_b, add; // add = 0: out = A B
 };
 // One unit of work of a launch: a tile of a job (oz_box_rows() complex rows and columns) over the
 // K-steps [kb0, kb0 + nk).  parts > 1: part `part` of the K range of tile `slot` of the launch's split

@@ -72,7 +72,8 @@ __global__ void oz_sqrt_kernel(const double *__restrict__ delta, int64_t n, doub
 
 // GUARD: sets *guard where an entry is not finite or a column's scale is out of range (FP64
 // contraction: the DMMA kernel then takes the chunk).
-template <bool GUARD>
+// SCALE = false: of M itself (the column operand of a general product).
+template <bool GUARD, bool SCALE>
 __global__ void oz_colexp_kernel(const double2 *__restrict__ M, int64_t P, int ng, const double *__restrict__ sp,
                                  int *__restrict__ E, int *guard)
 {
@@ -83,7 +84,7 @@ __global__ void oz_colexp_kernel(const double2 *__restrict__ M, int64_t P, int n
     if (g < ng) {
         for (int64_t p = (int64_t)blockIdx.y * 8 + wid; p < P; p += (int64_t)gridDim.y * 8) {
             const double2 m = M[p * ng + g];
-            const double a = oz_bits_d(oz_absmax_bits(m.x, m.y)) * sp[p];
+            const double b = oz_bits_d(oz_absmax_bits(m.x, m.y)), a = SCALE ? b * sp[p] : b;
             e = max(e, oz_expo_pos(a, kOzNoColumn));
             if constexpr (GUARD)
                 if ((oz_dbits(a) & 0x7fffffffffffffffull) >= 0x7ff0000000000000ull || e > kOzMaxExpo) *guard = 1;
@@ -151,7 +152,7 @@ __device__ __forceinline__ void oz_store_row_digits(const long long nb[16], int 
 // than the four the unconstrained build allows: the split preparation of a 48^3 q-point (16 chunks)
 // takes 5.04 against 5.32 ms (six blocks, 40 registers and a 60-byte spill: 5.17 ms).
 // GUARD: as in oz_colexp_kernel, for a column that is not zero but below the exponent range.
-template <bool GUARD>
+template <bool GUARD, bool SCALE>
 __global__ void __launch_bounds__(256, 5) oz_slice_kernel(const double2 *__restrict__ M, int64_t P, int ng,
                                                        const double *__restrict__ spv, const int *__restrict__ E,
                                                        int s, int64_t kpad, __nv_bfloat16 *__restrict__ Z, int *guard)
@@ -168,7 +169,7 @@ __global__ void __launch_bounds__(256, 5) oz_slice_kernel(const double2 *__restr
 #pragma unroll
     for (int t = 0; t < 16; ++t) {
         const int64_t p = p0 + tt.pl0 + t;
-        const double a = p < P ? Md[2 * (p * ng + g) + tt.c] * spv[p] : 0.0;
+        const double b = p < P ? Md[2 * (p * ng + g) + tt.c] : 0.0, a = SCALE ? (p < P ? b * spv[p] : 0.0) : b;
         if constexpr (GUARD)
             if (E[g] < -kOzMaxExpo && a != 0.0) *guard = 1;
         nb[t] = oz_round_scaled(a, sh) + bias;
@@ -786,7 +787,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
                     const int ex = eg + __ldg(ecol + g0 + j);
                     const int q = F64 ? 0 : j;
                     const double y = oz_scaled_double(hi[q], ex) + oz_scaled_double(lo[q], ex);
-                    if constexpr (GEN) row[2 * j] += y; // the tile belongs to this pair of CTAs alone
+                    if constexpr (GEN) row[2 * j] = jb.add ? row[2 * j] + y : y; // the pair of CTAs owns the tile
                     else if (part) __stcg(part + 32 * j, y);
                     else if (y != 0.0) atomicAdd(row + 2 * j, -y); // other pair segments may add here too
                 }
@@ -847,8 +848,9 @@ cudaError_t launch_oz_colexp(const double2 *M, int64_t P, int ng, const double *
     if (e != cudaSuccess || P == 0) return e;
     int gy = (int)std::min<int64_t>((P + 63) / 64, 256);
     const dim3 grid((ng + 31) / 32, gy);
-    if (guard) oz_colexp_kernel<true><<<grid, 256, 0, st>>>(M, P, ng, sp, E, guard);
-    else oz_colexp_kernel<false><<<grid, 256, 0, st>>>(M, P, ng, sp, E, guard);
+    if (!sp) oz_colexp_kernel<false, false><<<grid, 256, 0, st>>>(M, P, ng, sp, E, guard);
+    else if (guard) oz_colexp_kernel<true, true><<<grid, 256, 0, st>>>(M, P, ng, sp, E, guard);
+    else oz_colexp_kernel<false, true><<<grid, 256, 0, st>>>(M, P, ng, sp, E, guard);
     return cudaGetLastError();
 }
 
@@ -875,8 +877,10 @@ cudaError_t launch_oz_slice(const double2 *M, int64_t P, int ng, const double *s
                             int64_t kpad, void *Z, int *guard, cudaStream_t st)
 {
     const dim3 grid((ng + 31) / 32, (unsigned)(kpad / 64));
-    if (guard) oz_slice_kernel<true><<<grid, 256, 0, st>>>(M, P, ng, sp, E, s, kpad, (__nv_bfloat16 *)Z, guard);
-    else oz_slice_kernel<false><<<grid, 256, 0, st>>>(M, P, ng, sp, E, s, kpad, (__nv_bfloat16 *)Z, guard);
+    __nv_bfloat16 *z = (__nv_bfloat16 *)Z;
+    if (!sp) oz_slice_kernel<false, false><<<grid, 256, 0, st>>>(M, P, ng, sp, E, s, kpad, z, guard);
+    else if (guard) oz_slice_kernel<true, true><<<grid, 256, 0, st>>>(M, P, ng, sp, E, s, kpad, z, guard);
+    else oz_slice_kernel<false, true><<<grid, 256, 0, st>>>(M, P, ng, sp, E, s, kpad, z, guard);
     return cudaGetLastError();
 }
 
