@@ -579,6 +579,49 @@ __global__ void adj_val_tf_kernel(const float4 *__restrict__ psic, int v0, const
     tc_store(o, tc_add(tc_load(o), tcx{acc.re, tf_neg(acc.im)}));
 }
 
+// Both products of NV valence rows from one pass over H, a grid point per thread: psibar_c[c] +=
+// sum_v psi_v H[v][c] as it goes, psibar_v[v] += psi_c conj(H[v][c]) = conj(conj(psi_c) H[v][c]) in
+// registers over all c.  The sums are lazy two-float (tc_acc), renormalised every fourth term.  H is the
+// traffic: 384 conduction bands and 48 valence bands in rows of five on 40^3 (18.9 GB) take 7.1 ms where the
+// two kernels above, which read it twice, take 9.2.  Segments of c in blocks of their own take 9.6.
+template <int NV>
+__global__ void __launch_bounds__(64) adj_products_tf_kernel(const float4 *__restrict__ psiv,
+                                                             const float4 *__restrict__ psic,
+                                                             const float4 *__restrict__ H, int nc, int64_t nr,
+                                                             float4 *__restrict__ pbv, float4 *__restrict__ pbc)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nr) return;
+    tcx pv[NV], av[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        pv[v] = tc_load(psiv + v * nr + i);
+        av[v] = tcx{{0.f, 0.f}, {0.f, 0.f}};
+    }
+#pragma unroll 2
+    for (int c = 0; c < nc; ++c) {
+        const tcx pc = tc_load(psic + c * nr + i), pcc{pc.re, tf_neg(pc.im)};
+        const tcx old = tc_load(pbc + c * nr + i);
+        tcx h[NV], ac{{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll
+        for (int v = 0; v < NV; ++v) h[v] = tc_load(H + ((int64_t)v * nc + c) * nr + i);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            tc_acc(ac, pv[v], h[v]);
+            if (v == 3) ac = tc_norm(ac);
+            tc_acc(av[v], pcc, h[v]);
+            if ((c & 3) == 3) av[v] = tc_norm(av[v]);
+        }
+        tc_store(pbc + c * nr + i, tc_add(old, tc_norm(ac)));
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        const tcx a = tc_norm(av[v]);
+        float4 *o = pbv + v * nr + i;
+        tc_store(o, tc_add(tc_load(o), tcx{a.re, tf_neg(a.im)}));
+    }
+}
+
 // Two-float accumulators to FP64, in place (same 16 bytes per point).
 __global__ void tf_to_f64_kernel(void *__restrict__ x, int64_t n)
 {
@@ -600,6 +643,25 @@ cudaError_t launch_adj_products(const void *psiv, const void *psic, int v0, int 
                                 int64_t nr, bool tf, double2 *pbv, double2 *pbc, cudaStream_t st)
 {
     if (tf) {
+        // One pass where the grid's points alone fill the GPU and the rows fit the registers.  27000 points:
+        // 0.60 against 0.47 ms (12 x 200 bands, two groups of rows); 110592 points, 8 rows as two groups of
+        // four: 0.80 against 0.79; 64000 points, five rows: 7.1 against 9.2.
+        if (nr >= 60000 && nvc <= 6) {
+            const float4 *pv = (const float4 *)psiv + v0 * nr;
+            auto run = [&](auto kern) {
+                kern<<<(unsigned)((nr + 63) / 64), 64, 0, st>>>(pv, (const float4 *)psic, (const float4 *)H, nc, nr,
+                                                                (float4 *)pbv + v0 * nr, (float4 *)pbc);
+                return cudaGetLastError();
+            };
+            switch (nvc) {
+            case 1: return run(adj_products_tf_kernel<1>);
+            case 2: return run(adj_products_tf_kernel<2>);
+            case 3: return run(adj_products_tf_kernel<3>);
+            case 4: return run(adj_products_tf_kernel<4>);
+            case 5: return run(adj_products_tf_kernel<5>);
+            default: return run(adj_products_tf_kernel<6>);
+            }
+        }
         dim3 gc((unsigned)((nr + 255) / 256), nc);
         adj_cond_tf_kernel<<<gc, 256, 0, st>>>((const float4 *)psiv, v0, nvc, (const float4 *)H, nc, nr,
                                                (float4 *)pbc);
