@@ -289,18 +289,19 @@ def reference_arm(args):
 # DRAM bytes per launch of the dominant kernel, from one ncu capture of an identical launch
 # (8192 pairs, N_G = 2000); set to None whenever that kernel changes.
 TRAFFIC = {
-    "contract_f64": {"bytes_per_launch": 1.941011e9 + 0.034306e9,
-                     "source": "ncu dram__bytes_read+write, contract_f64_kernel, p1_48cube_onechunk"},
+    "contract_f64": None,
     # the FFT route of stage (a) (fp64 and pre-tensor-core paths): taken before the tensor-core
     # route existed; the kernel is unchanged since
     "pair_mtxel": {"bytes_per_launch": 3.112e9 + 1.486e9,
                    "source": "ncu dram__bytes_read+write, pair_kernel_tf_ct<48>, p1_48cube_onechunk"},
     # the tensor-core route of the 48^3 workload: one 8192-pair block (16 valence x 512 conduction
     # bands), the launch shape the bench's step repeats 16 times
-    "zdft": None,
-    "pair_from_f": None,
-    "ozaki_gemm": None,
-    "ozaki_gemm_single_stream": None,
+    "zdft": {"bytes_per_launch": 1.390811e9 + 4.830885e9, "source": "ncu dram__bytes_read+write, zd_gemm_kernel"},
+    "pair_from_f": {"bytes_per_launch": 4.880909e9 + 1.243656e9,
+                    "source": "ncu dram__bytes_read+write, pair_kernel_tf_from_f<48>"},
+    "ozaki_gemm": {"bytes_per_launch": 0.995768e9 + 0.079937e9, "source": "ncu dram__bytes_read+write, oz_gemm_kernel"},
+    "ozaki_gemm_single_stream": {"bytes_per_launch": 0.995768e9 + 0.079937e9,
+                                 "source": "ncu dram__bytes_read+write, oz_gemm_kernel"},
 }
 
 
@@ -583,12 +584,12 @@ def _full_ops(n):
     return ops
 
 
-def backprojection_ops_per_pair(cfg, k2):
-    """FP32 operations of the two-float adjoint back-projection per pair: per i0 slab the sphere's
-    sums per (k1, k2) cell (a complex product and a complex sum per point), K2 lines along i1,
-    N1 lines along i2, the scaled conjugate of the slab."""
+def backprojection_ops_per_pair(cfg, k2, k12):
+    """FP32 operations of the two-float adjoint back-projection per pair on a cubic grid: K12 lines along
+    i0 (the sphere's cells), then per slab K2 lines along i1 and N1 lines along i2, each as a full
+    transform (the first stages skip zeros), the scaled points of the sphere."""
     n0, n1, n2 = cfg.grid
-    return n0 * (cfg.ng * (_CMUL + 22) + k2 * _full_ops(n1) + n1 * _full_ops(n2) + n1 * n2 * 14)
+    return k12 * _full_ops(n0) + n0 * (k2 * _full_ops(n1) + n1 * _full_ops(n2)) + cfg.ng * 14
 
 
 def _hbm_peak():
@@ -602,11 +603,35 @@ def oz_kpad(ka):
     return 2 * ((ka + 63) // 64 * 64)
 
 
+OZ_F64_PRODUCTS = 28  # seven nine-bit slices
+
+
 def oz_products(nslices):
     """Slice products of a split contraction at the accuracy of nslices six-bit slices: the library
     takes n = 3, 3, 4, 5, 5, 6 nine-bit slices for nslices = 3 .. 8 and keeps n (n + 1) / 2 products."""
     n = {3: 3, 4: 3, 5: 4, 6: 5, 7: 5, 8: 6}[nslices]
     return n * (n + 1) // 2
+
+
+def eps_slice_products(n, b, nslices):
+    """Slice products of one Newton-Schulz inverse, per matrix product of a step (the library's rule:
+    the last two steps with six slices, the others with the fewest whose error a step can take)."""
+    r = (b - 1.0) / (b + 1.0)
+    steps = max(1, int(np.ceil(np.log2(np.log(1e-17) / np.log(r)))) + 1) if r > 0 else 1
+    rho, out = r, 0
+    for k in range(steps):
+        if k >= steps - 2:
+            out += oz_products(8)
+            continue
+        nxt = rho * rho
+        take, rho = nslices, nxt
+        for s in (4, 5):
+            f = 8.0 * n * b * 2.0 ** (-9 * {4: 3, 5: 4}[s])
+            if s < nslices and f <= max(0.25 * nxt, 2e-5):
+                take, rho = s, nxt + f
+                break
+        out += oz_products(take)
+    return out
 
 
 def mode_roofline(bound, kernel, work, ms, unit_of_work, prec="ozaki"):
@@ -749,11 +774,18 @@ def roofline_for(cfg, prec, nslices, res, single_stream=False):
     tkey = kname + ("_single_stream" if single_stream and prec != "fp64" else "")
     kms, kn = res["timing"].get(kname, (0.0, 0))
     nchunk = -(-cfg.npairs // cfg.pair_chunk)
-    per_launch_flops = 4.0 * cfg.ng * (cfg.ng + 1) * cfg.npairs / nchunk
-    if prec == "ozaki":
-        # low-precision flops of the kept slice pairs, each 4 N_G^2 P per chunk and frequency
-        per_launch_flops = oz_products(nslices) * 4.0 * cfg.ng ** 2 * cfg.npairs / nchunk
-    peak, peak_src = peak_for(prec)
+    # low-precision flops of the kept slice pairs, each 4 N_G^2 P per chunk and frequency.  FP64 by slices:
+    # 28 products, and each launch has a second behind it that returns at once (the DMMA kernel, for
+    # what the slices do not hold); FP64 on DMMA (batches): the upper triangle's FP64 flops
+    sliced = prec == "fp64" and "oz_split" in res["timing"]
+    if prec == "fp64" and not sliced:
+        per_launch_flops = 4.0 * cfg.ng * (cfg.ng + 1) * cfg.npairs / nchunk
+    else:
+        prods = OZ_F64_PRODUCTS if sliced else oz_products(nslices)
+        per_launch_flops = prods * 4.0 * cfg.ng ** 2 * cfg.npairs / nchunk
+    if sliced:
+        kn //= 2
+    peak, peak_src = peak_for("ozaki" if sliced else prec)
     achieved = per_launch_flops / (kms / kn * 1e-3) * 1e-12 if kn else None
     return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": (achieved / peak) if achieved else None,
@@ -817,8 +849,8 @@ def ours(args):
         if blk is not None:
             other["error"] = block_error(f["chi"], blk)
         if err is not None:
-            # the whole matrix against the library's FP64 mode (FP64 stage (a) and DMMA, no shared
-            # arithmetic with the split path; itself within 1e-15 of the oracle's block)
+            # the whole matrix against the library's FP64 mode (seven slices, whole-number sums; itself
+            # within 1e-15 of the oracle's block)
             d = main["chi"] - f["chi"]
             err["rel_frobenius_full_vs_fp64_mode"] = float(np.linalg.norm(d) / np.linalg.norm(f["chi"]))
     cpu = None
@@ -979,10 +1011,11 @@ def adjoint(args):
     roofs = {}
     if (args.mtxel or "twofloat") == "twofloat":
         roofs["back_projection"] = mode_roofline(
-            "alu", "adj_pair_tf_kernel", backprojection_ops_per_pair(cfg, kept_columns(prob, cfg.grid[2])) * P,
+            "alu", "adj_cells_tf_kernel + adj_slab_tf_kernel",
+            backprojection_ops_per_pair(cfg, kept_columns(prob, cfg.grid[2]), cells(prob, cfg.grid)) * P,
             kms.get("adj_pair"), "FP32 operations of the two-float back-projection (bench.backprojection_ops_per_pair) x pairs")
-        roofs["products"] = mode_roofline("hbm", "adj_cond_tf_kernel + adj_val_tf_kernel", 2 * 16.0 * P * nr,
-                                          kms.get("adj_products"), "H read once by each product kernel, 16 B per point")
+        roofs["products"] = mode_roofline("hbm", "products of the gradients", 16.0 * P * nr, kms.get("adj_products"),
+                                          "H read once, 16 B per point")
     if args.prec == "ozaki":
         roofs["y_mw"] = mode_roofline("tensor", "oz_gemm_kernel (general product Y = M W)",
                                       oz_products(s) * 2.0 * P * (2 * cfg.ng) * oz_kpad(cfg.ng), kms.get("adj_zgemm"),
@@ -1106,9 +1139,14 @@ def epsilon(args):
     s = args.nslices
     n = cfg.ng
     if args.prec == "ozaki":
-        per_step = 2 * oz_products(s) * 2.0 * n * (2 * n) * oz_kpad(n)
+        sv = torch.sqrt(v)
+        prods = 0
+        for i in range(len(om)):
+            a = eye - sv[:, None] * chi[i] * sv[None, :]
+            prods += 2 * eps_slice_products(n, float(a.abs().sum(1).max()), s)
         roof = mode_roofline("tensor", "oz_gemm_kernel (general products of the Newton-Schulz steps)",
-                             per_step * steps, kms.get("eps_products"), "low-precision flops of the kept slice pairs")
+                             prods * 2.0 * n * (2 * n) * oz_kpad(n),
+                             kms.get("eps_products"), "low-precision flops of the kept slice pairs")
     else:
         roof = mode_roofline("tensor", "zgemm_kernel (DMMA)", 2 * 8.0 * n ** 3 * steps, kms.get("eps_products"),
                              "FP64 flops of the two complex products per step", prec="fp64")
