@@ -261,7 +261,7 @@ cudaError_t launch_adj_pair(double2 *Gb, int64_t P, const PairPlan &pp, const in
 cudaError_t launch_tf_to_f64(void *x, int64_t n, cudaStream_t st);
 cudaError_t launch_adj_products(const void *psiv, const void *psic, int v0, int nvc, int nc, const double2 *H,
                                 int64_t nr, bool tf, double2 *pbv, double2 *pbc, cudaStream_t st);
-cudaError_t launch_band_adjoint(double2 *pb, int nb, const int n[3], const FftAxis ax[3], const int32_t *gofs,
-                                int ngpsi, double2 *dc, cudaStream_t st);
+cudaError_t launch_band_adjoint(double2 *pb, int nb, const int n[3], const FftAxis ax[3], const int maxabs[3],
+                                const int32_t *gofs, int ngpsi, double2 *dc, cudaStream_t st);
 
 } // namespace gw
