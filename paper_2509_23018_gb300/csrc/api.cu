@@ -343,7 +343,8 @@ gw_status oz_items(gw_chi0 *h, std::vector<gw::OzJob> &jobs, std::vector<gw::OzI
         if (st) return st;
         if (!h->ozflags) {
             if ((st = grow(h, (void **)&h->ozflags, &h->ozflags_cap, flags, "split tile counters"))) return st;
-            CK(h, cudaMemset(h->ozflags, 0, flags), "split tile counters");
+            // on the handle's stream: the default stream is not ordered with the launches that count here
+            CK(h, cudaMemsetAsync(h->ozflags, 0, flags, h->st), "split tile counters");
         }
     }
     const std::vector<gw::OzItem> tail(items.begin() + full, items.end());
@@ -1644,12 +1645,15 @@ gw_status gw_chi0_contract(gw_chi0 *h, int nv, int nc, const double *ev, const d
 gw_status gw_chi0_sync(gw_chi0 *h)
 {
     if (!h) return GW_ERR_ARG;
-    CK(h, cudaStreamSynchronize(h->st), "sync");
     int st = 0;
-    CK(h, cudaMemcpy(&st, h->status, sizeof(int), cudaMemcpyDeviceToHost), "status");
-    CK(h, cudaMemset(h->status, 0, sizeof(int)), "status reset");
-    if ((st & gw::kStatusTimeout) && h->ozflags) // parts that never met leave their counters behind
-        CK(h, cudaMemset(h->ozflags, 0, h->ozflags_cap), "split tile counters");
+    CK(h, cudaMemcpyAsync(&st, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->st), "status");
+    CK(h, cudaStreamSynchronize(h->st), "sync");
+    if (st != 0) { // on the handle's stream, and done before the caller may go on with another one
+        CK(h, cudaMemsetAsync(h->status, 0, sizeof(int), h->st), "status reset");
+        if ((st & gw::kStatusTimeout) && h->ozflags) // parts that never met leave their counters behind
+            CK(h, cudaMemsetAsync(h->ozflags, 0, h->ozflags_cap, h->st), "split tile counters");
+        CK(h, cudaStreamSynchronize(h->st), "status reset");
+    }
     if (st & gw::kStatusTimeout) return fail(h, GW_ERR_TIMEOUT, "a bounded device-side wait gave up");
     if (st & gw::kStatusNoSlot) return fail(h, GW_ERR_CUDA, "a pair block found no free scratch slot");
     if (st & gw::kStatusBounds) return fail(h, GW_ERR_CUDA, "an index outside its buffer (bounds-checked build)");

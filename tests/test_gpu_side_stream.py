@@ -1,0 +1,63 @@
+"""A handle used on a stream of its own while the default stream is busy: what the library clears or
+uploads for itself has to be ordered with the handle's stream, not with the default one.  The default stream
+copies for several times what the call takes, so that anything left to it comes too late."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gw():
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    import paper_2509_23018_gb300 as gw
+    return gw
+
+
+def dev(x):
+    return torch.as_tensor(np.ascontiguousarray(x), device="cuda")
+
+
+class BusyDefaultStream:
+    """Copies on the default stream (about 80 ms) and a side stream as the current one."""
+
+    def __enter__(self):
+        self.a = torch.zeros(1 << 28, dtype=torch.float32, device="cuda")
+        self.b = torch.empty_like(self.a)
+        torch.cuda.synchronize()
+        for _ in range(256):
+            self.b.copy_(self.a)
+        self.busy = torch.cuda.Event()
+        self.busy.record()
+        self.side = torch.cuda.stream(torch.cuda.Stream())
+        self.side.__enter__()
+        return self
+
+    def __exit__(self, *exc):
+        self.side.__exit__(*exc)
+        torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("ng,P", [(300, 4096), (1100, 1024)])
+def test_first_split_tiles(gw, ng, P):
+    """The first launch whose last tiles meet in parts clears their counters (6 and 45 tiles: all of them
+    in parts).  The same bits as on an idle GPU."""
+    rng = np.random.default_rng(ng)
+    M = dev(rng.standard_normal((P, ng)) + 1j * rng.standard_normal((P, ng)))
+    ev, ec = dev(np.full(1, -2.0)), dev(np.full(P, 2.0))
+    make = lambda: gw.Chi0((8, 8, 8), prec="ozaki", nslices=7)  # noqa: E731
+    want = make().contract(ev, ec, M, [0.0])
+    h = make()
+    out = torch.empty_like(want)
+    torch.cuda.synchronize()
+    with BusyDefaultStream() as busy:
+        h.contract(ev, ec, M, [0.0], out=out)
+        h.sync()
+        assert not busy.busy.query()
+        got = out.clone()
+        h.contract(ev, ec, M, [0.0], out=out)  # the counters are left at zero
+        h.sync()
+    assert torch.equal(got, want) and torch.equal(out, want)
+    h.destroy()
