@@ -1120,9 +1120,11 @@ gw_status gw_chi0_create(gw_chi0 **out, const gw_chi0_desc *d, void *stream)
         gw_chi0_destroy(h);
         return GW_ERR_OOM;
     }
-    if (cudaMemcpy(h->tw, tw.data(), sizeof(double2) * ntot, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(h->twf, twf.data(), sizeof(float4) * ntot, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(h->status, 0, sizeof(int)) != cudaSuccess) {
+    // in place before the caller may go on, with whatever stream
+    if (cudaMemcpyAsync(h->tw, tw.data(), sizeof(double2) * ntot, cudaMemcpyHostToDevice, h->st) != cudaSuccess ||
+        cudaMemcpyAsync(h->twf, twf.data(), sizeof(float4) * ntot, cudaMemcpyHostToDevice, h->st) != cudaSuccess ||
+        cudaMemsetAsync(h->status, 0, sizeof(int), h->st) != cudaSuccess ||
+        cudaStreamSynchronize(h->st) != cudaSuccess) {
         cudaGetLastError();
         gw_chi0_destroy(h);
         return GW_ERR_CUDA;

@@ -258,7 +258,11 @@ gw_status compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const double 
         ng.key = key;
         ng.jobs_bytes = blob.size();
         if ((s = dalloc(h, &ng.jobs, ng.jobs_bytes, "graph job tables"))) return s;
-        CK(h, cudaMemcpy(ng.jobs, blob.data(), blob.size(), cudaMemcpyHostToDevice), "graph job tables");
+        if (cudaMemcpyAsync(ng.jobs, blob.data(), blob.size(), cudaMemcpyHostToDevice, h->st) != cudaSuccess) {
+            cudaGetLastError();
+            dfree(h, ng.jobs, ng.jobs_bytes);
+            return fail(h, GW_ERR_CUDA, "graph job tables");
+        }
 
         cudaStream_t user = h->st;
         const bool saved_timing = h->timing;

@@ -61,3 +61,29 @@ def test_first_split_tiles(gw, ng, P):
         h.sync()
     assert torch.equal(got, want) and torch.equal(out, want)
     h.destroy()
+
+
+def test_first_batch(gw):
+    """A batch's job tables are uploaded when its graph is built: a handle made, loaded and run with the default
+    stream busy."""
+    import gwgen
+    p = gwgen.make_problem((24, 24, 24), 4, 60, 600, 130, seed=3)
+    t = {k: dev(getattr(p, k)) for k in ("gpsi", "cv", "ev", "cc", "ec", "gchi")}
+
+    def load(**kw):
+        h = gw.Chi0(p.grid, **kw)
+        h.set_bands(0, 1, t["gpsi"], t["cc"], t["ec"])
+        h.set_bands(0, 0, t["gpsi"], t["cv"], t["ev"])
+        h.set_gsphere(0, t["gchi"])
+        return h
+
+    for kw in (dict(prec="fp64"), dict(prec="ozaki", nslices=7, mtxel="twofloat")):
+        want = load(**kw).compute_batch([0], [0.0, 2.0])[0].clone()
+        out = torch.empty_like(want).reshape(-1)
+        torch.cuda.synchronize()
+        with BusyDefaultStream():
+            h = load(**kw)
+            got = h.compute_batch([0], [0.0, 2.0], out=out)[0].clone()
+            h.sync()
+        assert float(torch.linalg.vector_norm(got - want) / torch.linalg.vector_norm(want)) < 1e-14
+        h.destroy()
