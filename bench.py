@@ -627,7 +627,7 @@ def eps_slice_products(n, b, nslices):
         take, rho = nslices, nxt
         for s in (4, 5):
             f = 8.0 * n * b * 2.0 ** (-9 * {4: 3, 5: 4}[s])
-            if s < nslices and f <= max(0.25 * nxt, 2e-5):
+            if s < nslices and f <= max(0.25 * min(nxt, 1.0 - nxt), 2e-5):
                 take, rho = s, nxt + f
                 break
         out += oz_products(take)

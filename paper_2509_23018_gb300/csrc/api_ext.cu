@@ -270,29 +270,78 @@ static gw_status square_product(gw_chi0 *h, const double2 *A, const double2 *B, 
     return GW_OK;
 }
 
-// Slices of the split products of the last Newton-Schulz steps (the most the digit step takes).
+// Slices of the split products of the last Newton-Schulz steps (the most the digit step takes), the
+// residual ||I - A X||_F from which one more of them ends at rounding, and the residual from which the
+// early steps count as lost.
 constexpr int kEpsFinalSlices = 8;
+constexpr double kEpsNear = 1e-4, kEpsLost = 0.5;
 
 // Accuracy (the ABI's nslices) of a step that starts at ||I - A X|| <= rho, which it squares: the least
-// whose products change the residual by no more than a quarter of that, or than 2e-5, which the last two
-// steps bring to 1e-19.  With n 9-bit slices an entry of a product of two N x N matrices carries about
-// N^(1/2) 2^(-9n) of its row's and column's largest entries, the matrix N^(1/2) times that, and the
-// residual ||A|| <= b times it; the factor 8 covers the step's two products.  N_G = 2000, b = 52: six
-// of eleven steps with three slices (6 products each), three with four (10), two with six (21), where
-// nine had five (15): 30.2 -> 23.4 ms for two frequencies (21.7 with the
-// column slices and the stores of the products as they are now).
+// whose products change the residual by no more than a quarter of that and a quarter of its distance to 1
+// (the residual has to keep falling), or than 2e-5, which the last two steps bring to 1e-19.  With n 9-bit
+// slices an entry of a product of two N x N matrices carries about N^(1/2) 2^(-9n) of its row's and
+// column's largest entries, the matrix N^(1/2) times that, and the residual ||A|| <= b times it; the
+// factor 8 covers the step's two products.  That is what digits without a pattern leave, not a bound:
+// equal entries can add up their errors.  So the residual that the early steps did reach is measured
+// (epsilon_split).
 static int eps_step_slices(const gw_chi0 *h, int ng, double b, double *rho)
 {
     const double next = *rho * *rho;
     for (int nslices : {4, 5}) { // three and four slices
         const double f = 8.0 * ng * b * std::ldexp(1.0, -9 * gw::oz_slices(nslices));
-        if (nslices < h->d.nslices && f <= std::max(0.25 * next, 2e-5)) {
+        if (nslices < h->d.nslices && f <= std::max(0.25 * std::min(next, 1.0 - next), 2e-5)) {
             *rho = next + f;
             return nslices;
         }
     }
     *rho = next;
     return 0;
+}
+
+// X <- 2 X - X A X (T, Pm: work), products with the accuracy of nslices (0: the handle's).
+// resid: where to leave ||I - A X||_F^2 of the X before the step (device), or null.
+static gw_status eps_newton(gw_chi0 *h, const double2 *A, double2 *X, double2 *T, double2 *Pm, int ng, int nslices,
+                            double *resid)
+{
+    Scope sp(h, "eps_products"); // two N_G^3 products per step: the launch count gives the steps
+    gw_status st;
+    if ((st = square_product(h, A, X, ng, T, nslices))) return st;
+    if (resid) CK(h, gw::launch_eps_resid(T, ng, resid, h->st), "residual");
+    if ((st = square_product(h, X, T, ng, Pm, nslices))) return st;
+    CK(h, gw::launch_eps_step(X, Pm, (int64_t)ng * ng, h->st), "Newton-Schulz step");
+    return GW_OK;
+}
+
+// Split precision: steps - 2 steps with no more slices than their error asks for, then steps with the most,
+// each from a measured residual, until one has started below kEpsNear, and a last one.  The error of the
+// result is the rounding of the last two (earlier errors are squared away).  Where the early steps lost
+// the iterate they are taken again, from X0, with the most slices.  N_G = 2000, b = 52, two frequencies: six of
+// eleven steps with three slices (6 products each), three with four (10), two with six (21), where nine had
+// five (15): 30.2 -> 23.4 ms (21.8 with the column slices and the stores of the products as they are now).
+// b = 374: four of fourteen steps with three slices, seven with four, 16.2 ms a frequency.
+static gw_status epsilon_split(gw_chi0 *h, int ng, double b, int steps, const double2 *A, double2 *X, double2 *T,
+                               double2 *Pm, double *resid, const unsigned long long *bmax)
+{
+    gw_status st;
+    double rho = (b - 1.0) / (b + 1.0);
+    for (int k = 0; k < steps - 2; ++k)
+        if ((st = eps_newton(h, A, X, T, Pm, ng, eps_step_slices(h, ng, b, &rho), nullptr))) return st;
+    bool again = false;
+    for (int k = 0; k < steps; ++k) {
+        double e2 = 0.0;
+        if ((st = eps_newton(h, A, X, T, Pm, ng, kEpsFinalSlices, resid))) return st;
+        CK(h, cudaMemcpyAsync(&e2, resid, sizeof e2, cudaMemcpyDeviceToHost, h->st), "residual");
+        CK(h, cudaStreamSynchronize(h->st), "residual");
+        const double e = std::sqrt(e2);
+        if (e <= kEpsNear || (again && !(e < kEpsLost))) break;
+        if (!(e < kEpsLost)) {
+            again = true;
+            CK(h, gw::launch_eps_init(X, ng, bmax, h->st), "X0");
+            for (int j = 0; j < steps - 2; ++j)
+                if ((st = eps_newton(h, A, X, T, Pm, ng, kEpsFinalSlices, nullptr))) return st;
+        }
+    }
+    return eps_newton(h, A, X, T, Pm, ng, kEpsFinalSlices, nullptr);
 }
 
 gw_status gw_chi0_epsilon_inverse(gw_chi0 *h, int ng, int nw, const double *chi, const double *vcoul,
@@ -330,16 +379,11 @@ gw_status gw_chi0_epsilon_inverse(gw_chi0 *h, int ng, int nw, const double *chi,
         if (r > 0.0) steps = (int)std::ceil(std::log2(std::log(1e-17) / std::log(r))) + 1;
         steps = std::max(steps, 1);
         CK(h, gw::launch_eps_init(X, ng, bmax, h->st), "X0");
-        // The error of the converged iterate is the rounding of the last steps' products (earlier
-        // errors are squared away), so in split precision the last two steps take the most slices, and
-        // the earlier ones no more than their own error asks for (eps_step_slices).
-        double rho = r;
-        for (int k = 0; k < steps; ++k) {
-            Scope sp(h, "eps_products"); // two N_G^3 products per step: the launch count gives the steps
-            int s = 0;
-            if (h->d.prec == GW_PREC_OZAKI_BF16) s = k >= steps - 2 ? kEpsFinalSlices : eps_step_slices(h, ng, b, &rho);
-            if ((st = square_product(h, A, X, ng, T, s)) || (st = square_product(h, X, T, ng, Pm, s))) return st;
-            CK(h, gw::launch_eps_step(X, Pm, (int64_t)nn, h->st), "Newton-Schulz step");
+        if (h->d.prec == GW_PREC_OZAKI_BF16) {
+            if ((st = epsilon_split(h, ng, b, steps, A, X, T, Pm, (double *)(bmax + 1), bmax))) return st;
+        } else {
+            for (int k = 0; k < steps; ++k)
+                if ((st = eps_newton(h, A, X, T, Pm, ng, 0, nullptr))) return st;
         }
         CK(h, gw::launch_eps_unsym(X, sv, ng, (double2 *)epsinv + (int64_t)w * nn, h->st), "s X s^-1");
     }

@@ -52,6 +52,26 @@ __global__ void eps_init_kernel(double2 *__restrict__ X, int ng, const unsigned 
     X[e] = make_double2(i == j ? a : 0.0, 0.0);
 }
 
+// *r += sum_ij |delta_ij - T[i][j]|^2
+__global__ void __launch_bounds__(256) eps_resid_kernel(const double2 *__restrict__ T, int ng, double *__restrict__ r)
+{
+    __shared__ double red[8];
+    const int64_t nn = (int64_t)ng * ng;
+    double acc = 0.0;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nn; e += (int64_t)gridDim.x * blockDim.x) {
+        const double2 t = T[e];
+        const double x = t.x - (e % (ng + 1) == 0 ? 1.0 : 0.0);
+        acc = fma(x, x, fma(t.y, t.y, acc));
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) acc += red[w];
+        atomicAdd(r, acc);
+    }
+}
+
 // X = 2 X - P  (P = X A X)
 __global__ void eps_step_kernel(double2 *__restrict__ X, const double2 *__restrict__ P, int64_t n)
 {
@@ -100,6 +120,15 @@ cudaError_t launch_eps_sym(const double2 *chi, const double *sv, int ng, double2
 cudaError_t launch_eps_init(double2 *X, int ng, const unsigned long long *bmax, cudaStream_t st)
 {
     eps_init_kernel<<<blocks((int64_t)ng * ng), 256, 0, st>>>(X, ng, bmax);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_eps_resid(const double2 *T, int ng, double *r, cudaStream_t st)
+{
+    cudaError_t e = cudaMemsetAsync(r, 0, sizeof(double), st);
+    if (e != cudaSuccess) return e;
+    const int64_t want = ((int64_t)ng * ng + 2047) / 2048; // eight entries a thread
+    eps_resid_kernel<<<(unsigned)(want < 1216 ? want : 1216), 256, 0, st>>>(T, ng, r);
     return cudaGetLastError();
 }
 

@@ -133,6 +133,8 @@ cudaError_t launch_eps_sqrt(const double *v, int ng, double *sv, cudaStream_t st
 cudaError_t launch_eps_sym(const double2 *chi, const double *sv, int ng, double2 *A, unsigned long long *bmax,
                            cudaStream_t st);
 cudaError_t launch_eps_init(double2 *X, int ng, const unsigned long long *bmax, cudaStream_t st);
+// *r = ||I - T||_F^2
+cudaError_t launch_eps_resid(const double2 *T, int ng, double *r, cudaStream_t st);
 cudaError_t launch_eps_step(double2 *X, const double2 *P, int64_t n, cudaStream_t st);
 cudaError_t launch_eps_unsym(const double2 *X, const double *sv, int ng, double2 *out, cudaStream_t st);
 
