@@ -54,12 +54,16 @@ constexpr int kOzF64Slices = 7;
 constexpr int kOzKBlock = 16;
 // K-steps that slice group t sums in FP32 before the epilogue takes the sum (bounds at the top of
 // this file)
-// (F64: four K-steps for every group: below 2^24 unless 256 pairs' digits are all near their largest
-// with one sign)
+// (F64: every sum whose rounding would show is exact whatever the digits.  A pair adds at most 2^14 to t = 2,
+// 2^16 to t = 3, 2^17 to t = 4, 3 2^16 to t = 5 and 2^18 to t = 6, so 512, 256, 128, 64 and 64 pairs stay
+// within 2^24.  t = 7 (5 2^16) over 128 pairs and t = 8 (6 2^16) over 1024 may be rounded by up to 4 and 32 in
+// each of their 48 and 448 MMA steps: 2^-51 and 2^-54 of a pair's largest product 2^14 at most, and only where
+// the digits of those slices have one sign throughout.)
 template <bool F64>
 __device__ __forceinline__ int oz_segment(int t)
 {
-    return t == 2 ? 8 : t <= 4 || F64 ? 4 : kOzKBlock;
+    if (F64) return t == 2 ? 8 : t == 3 ? 4 : t == 4 || t == 7 ? 2 : t == 8 ? kOzKBlock : 1;
+    return t == 2 ? 8 : t <= 4 ? 4 : kOzKBlock;
 }
 
 // ------------------------------------------------------------------ split, step 1: column exponents
@@ -568,12 +572,15 @@ struct OzPlace {
 // Split: the Hermitian contraction above (upper tiles, chi epilogue), two-float sums.  General: the
 // product out += A B (all tiles, each owned by one pair of CTAs, plain FP64 adds).  F64: the Hermitian
 // contraction with seven slices, sums exact up to the last unit of a 64-bit integer per K block of 1024
-// pairs: groups t = 8..5 in units of 2^-54 (|sum| < 2^57), rounded to units of 2^-37 before t = 4..2
-// (|sum| <= 2 1024 2^14 2^37 = 2^62), 2^-51 of a pair's largest product.  A block's sum goes to chi (or
-// to the part's place in scratch) in FP64, so a chunk of 8192 pairs is rounded eight times where a chain
-// of DMMAs is rounded 2048 times.  Measured on a chunk of 8192 pairs, N_G = 2000: 2.44 ms
-// (28 products, 1.5 PFLOP/s) and 0.33 ms for the slices where the DMMA kernel, at 0.86 of its pipe's rate,
-// takes 138; error of chi against 64 bits 1.1e-15 where it leaves 1.9e-15.
+// pairs: segments whose FP32 sums are exact whatever the digits (oz_segment), groups t = 8..5 in units of
+// 2^-54 (|sum| < 2^57), rounded to units of 2^-37 before t = 4..2 (|sum| <= 2 1024 2^14 2^37 = 2^62), 2^-51 of
+// a pair's largest product.  A block's sum goes to chi (or to the part's place in scratch) in FP64, so a
+// chunk of 8192 pairs is rounded eight times where a chain of DMMAs is rounded 2048 times.  Measured on a
+// chunk of 8192 pairs, N_G = 2000: 3.12 ms (28 products, 1.18 PFLOP/s, the epilogue of the 55 segments of
+// a K block its bound; segments of 256 pairs throughout, 26 of them, take 2.45 but leave 1e-11 where the digits of
+// many pairs have one sign) and 0.33 ms for the slices where the DMMA kernel, at 0.86 of its pipe's rate, takes
+// 138; error of chi against 64 bits 1.1e-15 where it leaves 1.9e-15.  One code path for t = 2 and another for
+// the rest spills 872 bytes instead of 232: 4.58 ms.
 enum class OzProd { Split, General, F64 };
 template <OzProd MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
@@ -738,10 +745,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
                         for (int j = 0; j < NO; ++j) acc[j] = (acc[j] + (1 << 16)) >> 17;
                     }
                 }
+                const uint32_t ta = tbase + ((uint32_t)(q * 32) << 16) + b * C::Cols + half * COLS;
                 // F64: the group's unit is 2^ush of the sum's (t = 2: 2^37, into the high word)
                 const int ush = sg.t >= 5 ? kOzBeta * (8 - sg.t) : 37 - kOzBeta * (sg.t - 2);
                 const int umul = sg.t == 2 ? 0 : 1 << ush, hmul = sg.t == 2 ? 1 << (ush - 32) : 0;
-                const uint32_t ta = tbase + ((uint32_t)(q * 32) << 16) + b * C::Cols + half * COLS;
 #pragma unroll
                 for (int c0 = 0; c0 < COLS; c0 += 32) {
                     uint32_t v[32];
@@ -750,12 +757,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kOzThreads, 1)
 #pragma unroll
                     for (int cc = 0; cc < 16; ++cc) {
                         const uint32_t rv = __shfl_xor_sync(0xffffffffu, v[2 * cc + 1], 1) ^ rflip;
-                        const float x = __fadd_rn(__uint_as_float(v[2 * cc] ^ flip), __uint_as_float(rv));
-                        if constexpr (F64) {
-                            const int xi = __float2int_rn(x);
+                        const float x0 = __uint_as_float(v[2 * cc] ^ flip), x1 = __uint_as_float(rv);
+                        if constexpr (F64) { // added as integers: two sums of 2^24 may not fit FP32
+                            const int xi = __float2int_rn(x0) + __float2int_rn(x1);
                             acc[(c0 >> 1) + cc] += (long long)xi * umul + ((long long)(xi * hmul) << 32);
                         } else {
-                            oz_add(hi[(c0 >> 1) + cc], lo[(c0 >> 1) + cc], __fmul_rn(wt, x));
+                            oz_add(hi[(c0 >> 1) + cc], lo[(c0 >> 1) + cc], __fmul_rn(wt, __fadd_rn(x0, x1)));
                         }
                     }
                 }

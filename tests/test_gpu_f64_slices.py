@@ -2,6 +2,8 @@
 and K blocks of 1024 short, several frequencies, split tiles, and the chunks that it leaves to the DMMA
 kernel (entries that are not finite, scales beyond 2^+-390).  Against the same contraction of the library's
 own pair elements in torch's FP64: both round a few times per entry, 2^-53 of the columns' norms each."""
+from fractions import Fraction
+
 import gwgen
 import numpy as np
 import pytest
@@ -53,6 +55,39 @@ def test_chi_matches_fp64(gw, nv, nc, ng, chunk):
     assert torch.equal(chi, again)
     h.sync()
     h.destroy()
+
+
+def digits_value(d):
+    """The value in [1, 2) whose seven balanced base-512 digits, relative to a largest entry in [1, 2), are d."""
+    return float(sum(Fraction(v) * Fraction(512) ** (6 - i) for i, v in enumerate(d)) / Fraction(2) ** 61)
+
+
+COHERENT = [[(127, 127), (255, 255), (200, 255)], [(127, 127), (254, 255)], [(127, 127), (255, 255), (255, 255), (200, 255)],
+            [(127, 127)] + [(255, 255)] * 3 + [(200, 255)] * 2, [(120, 127)] + [(230, 255)] * 6, [(64, 64)] + [(-256, -230)] * 6]
+
+
+@pytest.mark.parametrize("nc", [4096, 700])
+@pytest.mark.parametrize("ranges", COHERENT)
+def test_sums_of_coherent_digits(gw, ranges, nc):
+    """Pair elements that nearly coincide, so that the digits of a slice have one sign over all pairs and the
+    FP32 sums of a slice group come close to their largest: one plane wave per band, M(0) = c, Delta = -1.
+    chi(0, 0) = -sum c^2, summed exactly."""
+    rng = np.random.default_rng(len(ranges) + nc)
+    rows = [ranges[i] if i < len(ranges) else (-255, 255) for i in range(7)]
+    c = np.array([digits_value([int(rng.integers(lo, hi + 1)) for lo, hi in rows]) for _ in range(nc)])
+    g = np.stack(np.meshgrid([0, 1, -1], [0, 1, -1], [0, 1, -1], indexing="ij"), -1).reshape(-1, 3).astype(np.int32)
+    coeff = lambda x: torch.as_tensor(np.outer(x, np.eye(27)[0]).astype(complex), device="cuda")  # noqa: E731
+    vec = lambda x, n: torch.full((n,), x, dtype=torch.float64, device="cuda")  # noqa: E731
+    h = gw.Chi0((32, 32, 32), prec="fp64")
+    gd = torch.as_tensor(g, device="cuda")
+    h.set_bands(0, 1, gd, coeff(c), vec(2.0, nc))
+    h.set_bands(0, 0, gd, coeff(np.ones(1)), vec(-2.0, 1))
+    h.set_gsphere(0, gd)
+    chi = h.compute(0, [0.0])[0][0].cpu().numpy()
+    h.sync()
+    h.destroy()
+    want = -sum(Fraction(x) ** 2 for x in c)
+    assert abs((Fraction(float(chi[0, 0].real)) - want) / want) < TOL
 
 
 @pytest.mark.parametrize("scale", [2.0 ** -200, 2.0 ** 210, float("nan"), float("inf")])
