@@ -4,10 +4,13 @@
 // points), with operands cut into seven balanced base-512 digits relative to the line's largest entry:
 // x = 2^(E - 62) sum_{i<7} 512^(6-i) d_i, 62 bits where a double keeps 53 of each entry.  The slices hold
 // the digits themselves (|d_0| <= 128, |d_i| <= 256, exact in BF16), so every accumulator holds whole
-// numbers; the products with i + j <= 6 are kept, one accumulator per i + j (FP32 sums of at most 112
-// points' products: exact for i + j <= 2, and below 2^24 otherwise unless a line's digits are all near
-// their largest with one sign).  The epilogue adds the seven as 64-bit integers in units of 2^-40 of the
-// leading group (|sum| < 2^62), 2^-54 of the operands' largest product, and rounds once, to the double
+// numbers; the products with i + j <= 6 are kept, summed over at most 112 real entries in FP32: one
+// accumulator per i + j, and for lines of more than 32 points two for i + j = 3 (d_1 d_2 and d_2 d_1, the
+// others) and i + j = 4 (d_1 d_3 and d_3 d_1, the others), so that the sums for i + j <= 4 stay within 2^24
+// (at most 64 2^18 and 112 2^17) and are exact whatever the digits.  i + j = 5 and 6 (112 5 2^16, 112 6 2^16) may be rounded by up to 4 in each of their
+// 42 and 49 MMA steps where a line's digits are all near their largest with one sign: 2^-51 of the operands'
+// largest product at most.  The epilogue adds them as 64-bit integers in units of 2^-40 of the leading
+// group (|sum| < 2^62), 2^-54 of the operands' largest product, and rounds once, to the double
 //     F = acc 2^(E_row + E_col - 56).
 #include "internal.h"
 #include "ptx.cuh"
@@ -107,14 +110,16 @@ __global__ void __launch_bounds__(256) zd64_colexp_kernel(const double2 *__restr
 // ------------------------------------------------------------------ the product
 // As zd_gemm_kernel: one block per SM, persistent over units (line, valence tile of CT bands), the
 // column stages resident, the row stages through a ring.  A tile of 128 conduction bands x 96 columns
-// runs in two passes over K, because its seven accumulators of 96 columns do not fit in TMEM: first the
+// runs in two passes over K, because its seven or nine accumulators of 96 columns do not fit in TMEM, five do: first the
 // groups i + j = 6, 5, 4 (18 products a stage), then 3..0 (10 products, for which four of a row stage's
-// seven slices are loaded).  The epilogue keeps the sums as 64-bit integers in between.
+// seven slices are loaded; the second pass starts in the accumulator that the first leaves free).  The
+// epilogue keeps the sums as 64-bit integers in between.
 //  warps 0..3: TMA, MMA (and TMEM), two producers; warps 4..11: epilogue (TMEM lane quadrant
 //  warp % 4, half of the columns each); warps 12..15: producers.
 //
-// 4.31 ms for 8192 pairs on 48^3 (8 x 1024 bands, K2 = 15), of which the products take 1.8; the FFT pair
-// kernel spends most of its 55 ms on this axis, on the FP64 pipe.  The epilogue uses no FP64 instruction:
+// 4.87 ms for 8192 pairs on 48^3 (8 x 1024 bands, K2 = 15), of which the products take 1.8 (4.32 with one
+// accumulator per i + j, which leaves up to 3e-14 of an element where a line's digits have one sign); the
+// FFT pair kernel spends most of its 55 ms on this axis, on the FP64 pipe.  The epilogue uses no FP64 instruction:
 // converting and scaling 96 x 128 sums there would take longer than the tile's products.
 constexpr int kQdThreads = 512;
 constexpr int kQdProducers = 6;
@@ -139,9 +144,17 @@ struct Qd64Args {
     int n, lines, nv, v0, vb, cb, K2, K2P, CT, nvt, nmt, nunits, ast;
 };
 
-// group i + j = g sits in accumulator slot (6 - g) of the first pass (g = 6, 5, 4), and in slots
-// 3, 0, 1, 2 of the second (g = 3, 2, 1, 0)
-__device__ constexpr int qd_slot(int g) { return g >= 4 ? 6 - g : (g == 3 ? 3 : 2 - g); }
+// accumulator slot of the product d_i d_j.  First pass: i + j = 6, 5 in 0, 1 and 4 in 2; second pass: 3 in 4,
+// then 2, 1, 0 in 0, 1, 2.  TWO: slot 3 takes d_0 d_4, d_2 d_2, d_4 d_0 in the first pass and d_0 d_3, d_3 d_0
+// in the second.
+constexpr int kQdSlots = 5;
+template <bool TWO>
+__device__ constexpr int qd_slot(int i, int j)
+{
+    const int g = i + j;
+    if (TWO && (g == 4 ? i != 1 && i != 3 : g == 3 && i != 1 && i != 2)) return 3;
+    return g == 3 ? 4 : g > 3 ? 6 - g : 2 - g;
+}
 
 // m 2^ex, m a 64-bit integer, rounded to a double from the bits (the FP64 pipe would take 2 clocks of
 // the SM for each)
@@ -155,6 +168,7 @@ __device__ __forceinline__ double qd_double(long long v, int ex)
     return __longlong_as_double((long long)(b | ((unsigned long long)v & 0x8000000000000000ull)));
 }
 
+template <bool TWO>
 __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_constant__ Qd64Args a,
                                                                   const double2 *__restrict__ twg)
 {
@@ -171,7 +185,7 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
     int2 *ctab = (int2 *)(wt + a.n);                    // [48] column pair -> (band, F offset)
     uint64_t *bar = (uint64_t *)(ctab + kQdN / 2);
     uint64_t *aFull = bar, *aEmpty = aFull + kQdMaxRing, *bFull = aEmpty + kQdMaxRing, *bEmpty = bFull + kQdMaxStages,
-             *tFull = bEmpty + kQdMaxStages, *tEmpty = tFull + 1, *pFull = tEmpty + 4, *pEmpty = pFull + kQdPsiSlots,
+             *tFull = bEmpty + kQdMaxStages, *tEmpty = tFull + 1, *pFull = tEmpty + kQdSlots, *pEmpty = pFull + kQdPsiSlots,
              *fin = pEmpty + kQdPsiSlots;
     uint32_t *tslot = (uint32_t *)(fin + 1);
 
@@ -195,7 +209,7 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
             bar_init(&bEmpty[i], 1);
         }
         bar_init(tFull, 1);
-        for (int i = 0; i < 4; ++i) bar_init(&tEmpty[i], 8);
+        for (int i = 0; i < kQdSlots; ++i) bar_init(&tEmpty[i], 8);
         for (int i = 0; i < kQdPsiSlots; ++i) {
             bar_init(&pFull[i], 1);
             bar_init(&pEmpty[i], kQdProducers);
@@ -218,10 +232,10 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
         // 16 h + 8 i + lane / 4, entry 4 j + lane % 4
         const int q4 = warp & 3, half = (warp - 4) >> 2;
         const uint32_t ta = tbase + ((uint32_t)(q4 * 32) << 16) + half * (kQdN / 2);
-                auto load = [&](int slot, uint32_t v[48]) {
+        auto load = [&](int slot, uint32_t v[48]) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const uint32_t t = ta + slot * kZdAcc + ((uint32_t)(16 * h) << 16);
+                const uint32_t t = ta + slot * kQdN + ((uint32_t)(16 * h) << 16);
                 GW_TMEM_LD_16X256_X4(t, v + 24 * h);
                 GW_TMEM_LD_16X256_X2(t + 32, v + 24 * h + 16);
             }
@@ -229,6 +243,30 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
             tc_fence_before();
             __syncwarp();
             if (lane == 0) bar_arrive(&tEmpty[slot]);
+        };
+        // acc += (slot s0 + slot s1) mul, half of the rows at a time
+        auto both = [&](int s0, int s1, uint32_t v[48], long long acc[48], int mul) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t t0 = ta + s0 * kQdN + ((uint32_t)(16 * h) << 16), t1 = t0 + (s1 - s0) * kQdN;
+                GW_TMEM_LD_16X256_X4(t0, v);
+                GW_TMEM_LD_16X256_X2(t0 + 32, v + 16);
+                GW_TMEM_LD_16X256_X4(t1, v + 24);
+                GW_TMEM_LD_16X256_X2(t1 + 32, v + 40);
+                tmem_wait_ld();
+                if (h == 1) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        bar_arrive(&tEmpty[s0]);
+                        bar_arrive(&tEmpty[s1]);
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < 24; ++c)
+                    acc[24 * h + c] += (long long)(__float2int_rn(__uint_as_float(v[c])) +
+                                                   __float2int_rn(__uint_as_float(v[24 + c]))) * mul;
+            }
         };
         for (int u = blockIdx.x; u < a.nunits && ok; u += gridDim.x) {
             const int l = u / a.nvt, vt = u - l * a.nvt;
@@ -248,9 +286,12 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
                     acc[c] += (long long)__float2int_rn(__uint_as_float(v[c])) * 512;
                     acc[c] = (acc[c] + (1 << 13)) >> 14; // units of 2^-40
                 }
-                load(2, v); // 4
+                if constexpr (TWO) both(2, 3, v, acc, 16); // 4
+                else {
+                    load(2, v);
 #pragma unroll
-                for (int c = 0; c < 48; ++c) acc[c] += (long long)__float2int_rn(__uint_as_float(v[c])) * 16;
+                    for (int c = 0; c < 48; ++c) acc[c] += (long long)__float2int_rn(__uint_as_float(v[c])) * 16;
+                }
                 got = bar_wait(tFull, 1);
                 if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
                 tc_fence_after();
@@ -263,9 +304,12 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
                 load(2, v); // 0
 #pragma unroll
                 for (int c = 0; c < 48; ++c) acc[c] += (long long)__float2int_rn(__uint_as_float(v[c]) * 256.0f) << 32;
-                load(3, v); // 3
+                if constexpr (TWO) both(3, 4, v, acc, 1 << 13); // 3
+                else {
+                    load(4, v);
 #pragma unroll
-                for (int c = 0; c < 48; ++c) acc[c] += (long long)__float2int_rn(__uint_as_float(v[c])) * (1 << 13);
+                    for (int c = 0; c < 48; ++c) acc[c] += (long long)__float2int_rn(__uint_as_float(v[c])) * (1 << 13);
+                }
 
                 const int64_t unit0 = ((int64_t)l * a.vb + (int64_t)vt * a.CT) * a.cb;
                 const int r0 = mt * kZdM + q4 * 32 + (lane >> 2);
@@ -342,27 +386,31 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
                 };
                 const uint32_t ad0 = sdesc_sw32_low(su32(sA)), bd0 = sdesc_sw32_low(su32(sB));
                 uint32_t as = 0, ph = 0, nu = 0;
-                uint32_t e012 = 1, e3 = 1; // parities of the accumulators' next release
+                uint32_t e03 = 1, e4 = 1; // parities of the accumulators' next release: 0..2 (TWO: 3) every pass, 4 every tile
                 if (blockIdx.x < a.nunits) {
                     wait(&bFull[0], 0);
                     wait(&aFull[0], 0);
                 }
                 tc_fence_after();
-                // group g, at a pass's first stage
-                auto issue = [&](auto G, uint32_t ad, uint32_t bd) {
-                    constexpr int g = decltype(G)::value;
+                // the products of group g in one slot, at a pass's first stage: the first starts the accumulator
+                auto issue = [&](auto G, auto SLOT, uint32_t ad, uint32_t bd) {
+                    constexpr int g = decltype(G)::value, slot = decltype(SLOT)::value;
+                    uint32_t started = 0;
 #pragma unroll
                     for (int i = 0; i <= g; ++i)
-                        umma_f16_run(lead, tb + qd_slot(g) * kZdAcc, ad + (uint32_t)((i * kQdASlice) >> 4),
-                                 bd + (uint32_t)(((g - i) * kQdBSlice) >> 4), kSdescSw32High, kQdIdesc,
-                                     i == 0 ? 0u : 1u, 0, 1);
+                        if (qd_slot<TWO>(i, g - i) == slot) {
+                            umma_f16_run(lead, tb + slot * kQdN, ad + (uint32_t)((i * kQdASlice) >> 4),
+                                         bd + (uint32_t)(((g - i) * kQdBSlice) >> 4), kSdescSw32High, kQdIdesc,
+                                         started, 0, 1);
+                            started = 1;
+                        }
                 };
                 // A slice i with its B slices of the pass's groups g0 .. g1, one after the other: A is read once
                 auto run = [&](int i, int g0, int g1, uint32_t ad, uint32_t bd) {
 #pragma unroll
                     for (int j = 0; j < kQdSlices; ++j)
                         if (i + j >= g0 && i + j <= g1)
-                            umma_f16_run(lead, tb + qd_slot(i + j) * kZdAcc, ad + (uint32_t)((i * kQdASlice) >> 4),
+                            umma_f16_run(lead, tb + qd_slot<TWO>(i, j) * kQdN, ad + (uint32_t)((i * kQdASlice) >> 4),
                                          bd + (uint32_t)((j * kQdBSlice) >> 4), kSdescSw32High, kQdIdesc, 1u,
                                          j - (g0 > i ? g0 - i : 0), g1 - i + 1 - (g0 > i ? g0 - i : 0));
                 };
@@ -393,23 +441,31 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
                                     tc_fence_after();
                                 };
                                 if (ks == 0 && ps == 0) {
-                                    room(0, e012);
-                                    issue(QdInt<6>{}, ad, bd);
-                                    room(1, e012);
-                                    issue(QdInt<5>{}, ad, bd);
+                                    room(0, e03);
+                                    issue(QdInt<6>{}, QdInt<0>{}, ad, bd);
+                                    room(1, e03);
+                                    issue(QdInt<5>{}, QdInt<1>{}, ad, bd);
                                     next();
-                                    room(2, e012);
-                                    issue(QdInt<4>{}, ad, bd);
+                                    room(2, e03);
+                                    issue(QdInt<4>{}, QdInt<2>{}, ad, bd);
+                                    if constexpr (TWO) {
+                                        room(3, e03);
+                                        issue(QdInt<4>{}, QdInt<3>{}, ad, bd);
+                                    }
                                 } else if (ks == 0) {
-                                    room(3, e3);
-                                    issue(QdInt<3>{}, ad, bd);
-                                    room(0, e012);
-                                    issue(QdInt<2>{}, ad, bd);
+                                    room(4, e4);
+                                    issue(QdInt<3>{}, QdInt<4>{}, ad, bd);
+                                    room(0, e03);
+                                    issue(QdInt<2>{}, QdInt<0>{}, ad, bd);
                                     next();
-                                    room(1, e012);
-                                    issue(QdInt<1>{}, ad, bd);
-                                    room(2, e012);
-                                    issue(QdInt<0>{}, ad, bd);
+                                    room(1, e03);
+                                    issue(QdInt<1>{}, QdInt<1>{}, ad, bd);
+                                    room(2, e03);
+                                    issue(QdInt<0>{}, QdInt<2>{}, ad, bd);
+                                    if constexpr (TWO) {
+                                        room(3, e03);
+                                        issue(QdInt<3>{}, QdInt<3>{}, ad, bd);
+                                    }
                                 } else if (ps == 0) {
 #pragma unroll
                                     for (int i = 0; i < 4; ++i) run(i, 4, 6, ad, bd);
@@ -426,10 +482,10 @@ __global__ void __launch_bounds__(kQdThreads, 1) zd64_gemm_kernel(const __grid_c
                                 if (ps == 1 && last) umma_commit_lead(lead, &bEmpty[ks]);
                                 umma_commit_lead(lead, &aEmpty[cur]);
                             }
-                            e012 ^= 1;
+                            e03 ^= 1;
                             umma_commit_lead(lead, tFull);
                         }
-                        e3 ^= 1;
+                        e4 ^= 1;
                     }
                 }
                 umma_commit_lead(lead, fin);
@@ -579,13 +635,15 @@ cudaError_t launch_zd64_gemm(const CUtensorMap &tmV, const void *A, const int *E
     a.ER = zd64_row_expo(const_cast<void *>(A), a.nmt, n, lines);
     a.ast = zd64_smem(n, K2, kQdMaxRing) <= (size_t)227 * 1024 ? kQdMaxRing : 2;
     const size_t sm = zd64_smem(n, K2, a.ast);
-    cudaError_t e = cudaFuncSetAttribute(zd64_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    // up to 64 real entries a sum for i + j = 4 (2^18 each at most) is exact
+    auto kernel = 16 * zd_stages(n) > 64 ? zd64_gemm_kernel<true> : zd64_gemm_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return e;
-    zd64_gemm_kernel<<<std::min(a.nunits, sms), kQdThreads, sm, st>>>(a, tw);
+    kernel<<<std::min(a.nunits, sms), kQdThreads, sm, st>>>(a, tw);
     return cudaGetLastError();
 }
 
