@@ -465,12 +465,26 @@ __global__ void __launch_bounds__(adj_slab_threads<N>(), N <= 40 ? 3 : N <= 48 ?
     }
 }
 
+static size_t adj_slab_smem(const PairPlan &pp)
+{
+    const size_t n = pp.n[0];
+    return sizeof(float4) * (2 * n * (n + 1) + n + 2 * (size_t)pp.K12) + sizeof(short) * (pp.K2 * n + n);
+}
+
+// The spheres that the two kernels take: the columns of i1 lie in one of the two buffers of i2, and two rows of
+// cells beside them fit a block's shared memory (always on 24^3 to 48^3, up to about 1800 cells on 72^3).
+static bool adj_cube_supported(const PairPlan &pp)
+{
+    const int n = pp.n[0];
+    return n == pp.n[1] && n == pp.n[2] && (n == 24 || n == 40 || n == 48 || n == 72) && 2 * pp.K2 <= n &&
+           adj_slab_smem(pp) <= (size_t)227 * 1024;
+}
+
 template <int N>
 static cudaError_t launch_adj_cube(const double2 *Gb, int64_t P, const PairPlan &pp, tf sc, float4 *H, cudaStream_t st)
 {
     const size_t sm1 = sizeof(float4) * (2 * (size_t)kAdjBatch * (N + 1) + N);
-    const size_t sm2 = sizeof(float4) * (2 * (size_t)N * (N + 1) + N + 2 * (size_t)pp.K12) +
-                       sizeof(short) * ((size_t)pp.K2 * N + N);
+    const size_t sm2 = adj_slab_smem(pp);
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(adj_cells_tf_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1)) !=
             cudaSuccess ||
@@ -493,13 +507,11 @@ cudaError_t launch_adj_pair(double2 *Gb, int64_t P, const PairPlan &pp, const in
         const double inv = 1.0 / ((double)pp.n[0] * pp.n[1] * pp.n[2]);
         const float hi = (float)inv;
         const tf sc{hi, (float)(inv - (double)hi)};
-        const bool cubic = pp.n[0] == pp.n[1] && pp.n[1] == pp.n[2];
-        // the columns of i1 lie in one of the two buffers of i2
-        if (cubic && 2 * pp.K2 <= pp.n[0]) {
+        if (adj_cube_supported(pp)) {
             if (pp.n[0] == 24) return launch_adj_cube<24>(Gb, P, pp, sc, (float4 *)H, st);
             if (pp.n[0] == 40) return launch_adj_cube<40>(Gb, P, pp, sc, (float4 *)H, st);
             if (pp.n[0] == 48) return launch_adj_cube<48>(Gb, P, pp, sc, (float4 *)H, st);
-            if (pp.n[0] == 72) return launch_adj_cube<72>(Gb, P, pp, sc, (float4 *)H, st);
+            return launch_adj_cube<72>(Gb, P, pp, sc, (float4 *)H, st);
         }
         cudaError_t e =
             cudaFuncSetAttribute(adj_pair_tf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);

@@ -33,3 +33,27 @@ def test_gradients_match_fp64(gw, n, nv, nc, ngpsi, ng):
         h.destroy()
     for a, b in zip(out[1], out[0]):
         assert float(torch.linalg.vector_norm(a - b) / torch.linalg.vector_norm(b)) < 1e-10
+
+
+@pytest.mark.parametrize("m", [(0, 34, 17), (1, 25, 17)])
+def test_wide_spheres(gw, m):
+    """Boxes of G on 72^3 whose (k1, k2) cells (2415 and 1785) go beyond and up to what a slab block's shared memory
+    holds: gradients against the oracle's adjoint, as the runtime-shape kernel gives them."""
+    import oracle
+    axes = lambda k: np.stack(np.meshgrid(*[np.arange(-x, x + 1) for x in k], indexing="ij"), -1).reshape(-1, 3)  # noqa: E731
+    gchi, gpsi = axes(m).astype(np.int32), axes((1, 1, 0)).astype(np.int32)
+    rng = np.random.default_rng(m[1])
+    q = np.linalg.qr(rng.standard_normal((9, 9)) + 1j * rng.standard_normal((9, 9)))[0]
+    cv, cc, ev, ec = q[:1], q[1:4], np.array([-1.0]), np.array([1.0, 2.0, 4.0])
+    W = gwgen.hermitian(rng, len(gchi))
+    dev = lambda x: torch.as_tensor(np.ascontiguousarray(x), device="cuda")  # noqa: E731
+    h = gw.Chi0((72, 72, 72), prec="ozaki", nslices=7, mtxel="twofloat")
+    h.set_bands(0, 1, dev(gpsi), dev(cc), dev(ec))
+    h.set_bands(0, 0, dev(gpsi), dev(cv), dev(ev))
+    h.set_gsphere(0, dev(gchi))
+    got = h.adjoint(0, dev(W), omega=1.0)
+    h.sync()
+    h.destroy()
+    want = oracle.adjoint(gpsi, cv, ev, gpsi, cc, ec, gchi, W, 1.0)
+    for a, b in zip(got[1:], want[1:]):
+        assert np.linalg.norm(a.cpu().numpy() - b) < 1e-10 * np.linalg.norm(b)
