@@ -750,15 +750,15 @@ static bool zd_faster(const gw_chi0 *h, const Sphere &sp, int vb, int cb)
     return tiles * lines * ((n[2] + 7) / 8) * 5.2e-3 + 7.2e-6 * lines * sp.K2 * pairs < fft * std::max(pairs, 600.0);
 }
 
-// Room for the route's buffers beside what the call will still take: with a memory budget, the
-// pair elements of a chunk, their slices (for a group of frequencies) and the split tiles' scratch
-// come first; without one, the buffers may grow by a quarter of the free memory.
-static bool zd_room(const gw_chi0 *h, size_t grow_by, int64_t pairs, int ng, int nw)
+// Room for the route's buffers beside what the call will still take: with a memory budget, what the
+// caller names (pending), the pair elements of a chunk, their slices (for a group of frequencies) and
+// the split tiles' scratch come first; without one, the buffers may grow by a quarter of the free memory.
+static bool zd_room(const gw_chi0 *h, size_t grow_by, int64_t pairs, int ng, int nw, size_t pending)
 {
     if (grow_by == 0) return true;
     if (h->d.mem_budget_bytes) {
         const double m = 16.0 * pairs * ng, z = 4.0 * gw::oz_slices(h->d.nslices) * ng * (pairs + 64.0);
-        const double later = 3.0 * m + z * std::min(nw, gw::oz_group_w()) + 16.0 * pairs * nw + 100e6;
+        const double later = pending + 3.0 * m + z * std::min(nw, gw::oz_group_w()) + 16.0 * pairs * nw + 100e6;
         return (double)h->bytes + grow_by + later <= (double)h->d.mem_budget_bytes;
     }
     size_t free_b = 0, total_b = 0;
@@ -769,10 +769,11 @@ static bool zd_room(const gw_chi0 *h, size_t grow_by, int64_t pairs, int ng, int
     return grow_by <= free_b / 4;
 }
 
-gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw, ZdPlan &z)
+gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw,
+                  size_t pending, ZdPlan &z)
 {
     z = ZdPlan();
-    if (!zd_grid(h, sp)) return GW_OK;
+    if (h->zdoff || !zd_grid(h, sp)) return GW_OK;
     z.f64 = h->d.mtxel_prec == GW_MTXEL_FP64;
     const int *n = h->d.n, lines = n[0] * n[1];
     const int ct = z.f64 ? gw::zd64_valence_per_tile(sp.K2) : gw::zd_valence_per_tile(n[2], sp.K2);
@@ -810,7 +811,7 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
             by += (z.abytes > h->zdAcap[i] ? z.abytes - h->zdAcap[i] : 0) + (z.ebytes > h->zdEcap[i] ? z.ebytes - h->zdEcap[i] : 0);
         by += z.fper * vs > h->zdFcap ? z.fper * vs - h->zdFcap : 0;
         by += z.sper * vs > h->zdScap ? z.sper * vs - h->zdScap : 0;
-        if (force || zd_room(h, by, (int64_t)z.vb * z.cb, sp.ng, nw)) break;
+        if (force || zd_room(h, by, (int64_t)z.vb * z.cb, sp.ng, nw, pending)) break;
     }
     z.vs = vs;
     const std::string err = h->err;
@@ -831,6 +832,7 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
     }
     if (s) return s;
     z.on = true;
+    h->zdran = true;
     return GW_OK;
 }
 
@@ -1420,7 +1422,7 @@ gw_status gw_chi0_pair_elements_block(gw_chi0 *h, int iq, int c0, int cb, double
     if (cb == 0) return GW_OK;
     ZdPlan z;
     ZdUse use{h};
-    if ((s = zd_plan(h, sp, nv, cb, false, true, 1, 1, z))) return s;
+    if ((s = zd_plan(h, sp, nv, cb, false, true, 1, 1, 0, z))) return s;
     const gw::PairPlan pp = pair_plan(h, sp);
     if ((s = zd_valence(h, z, sp, v.psi, nv))) return s;
     for (int b0 = 0; b0 < cb; b0 += z.cb) {
@@ -1450,9 +1452,8 @@ gw_status gw_chi0_pair_elements(gw_chi0 *h, int iq, int64_t pair_begin, int64_t 
     return GW_OK;
 }
 
-gw_status gw_chi0_compute(gw_chi0 *h, int nq, const int *iq, int nw, const double *omega, double *chi, double *diag)
+static gw_status compute(gw_chi0 *h, int nq, const int *iq, int nw, const double *omega, double *chi, double *diag)
 {
-    if (!h) return GW_ERR_ARG;
     if (nq < 1 || !iq || nw < 1 || nw > gw::kMaxOmega || !omega || !chi)
         return fail(h, GW_ERR_ARG, "bad arguments (nq >= 1, 1 <= nw <= %d, non-null pointers)", gw::kMaxOmega);
     gw::OmegaList om;
@@ -1494,7 +1495,7 @@ gw_status gw_chi0_compute(gw_chi0 *h, int nq, const int *iq, int nw, const doubl
         }
         ZdPlan z;
         ZdUse use{h};
-        if (fault_chunk() < 0 && (s = zd_plan(h, sp, v.nb, h->cond.nb, keep, false, 1, nw, z))) return s;
+        if (fault_chunk() < 0 && (s = zd_plan(h, sp, v.nb, h->cond.nb, keep, false, 1, nw, 0, z))) return s;
         if (z.on) {
             const int nc = h->cond.nb;
             if ((s = ensure_work(h, keep ? 0 : (size_t)z.vb * z.cb * ng, (size_t)z.vb * z.cb * nw)) ||
@@ -1560,6 +1561,12 @@ gw_status gw_chi0_compute(gw_chi0 *h, int nq, const int *iq, int nw, const doubl
     return GW_OK;
 }
 
+gw_status gw_chi0_compute(gw_chi0 *h, int nq, const int *iq, int nw, const double *omega, double *chi, double *diag)
+{
+    if (!h) return GW_ERR_ARG;
+    return zd_or_fft(h, [&] { return compute(h, nq, iq, nw, omega, chi, diag); });
+}
+
 gw_status gw_chi0_keep_pair_elements(gw_chi0 *h, int enable)
 {
     if (!h) return GW_ERR_ARG;
@@ -1593,7 +1600,7 @@ gw_status gw_chi0_compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const
         for (int j = 0; j < i; ++j)
             if (iq[j] == iq[i]) return fail(h, GW_ERR_ARG, "slot %d requested twice", iq[i]);
     }
-    return compute_batch(h, nq, iq, nw, omega, om, chi, diag);
+    return zd_or_fft(h, [&] { return compute_batch(h, nq, iq, nw, omega, om, chi, diag); });
 }
 
 int gw_chi0_tuning(const gw_chi0 *h, int *tile_f64, int *waves_f64, int *tile_split)

@@ -4,10 +4,15 @@
 
 using namespace gwapi;
 
-gw_status gw_chi0_adjoint(gw_chi0 *h, int iq, double omega, const double *W, double *L, double *dE_v, double *dE_c,
-                          double *dcoeff_v, double *dcoeff_c)
+// Bytes of the slices of a product's B operand (ka complex inner entries, nout columns)
+static size_t oz_b_bytes(const gw_chi0 *h, int ka, int nout)
 {
-    if (!h) return GW_ERR_ARG;
+    return h->d.prec == GW_PREC_OZAKI_BF16 ? (size_t)gw::oz_slices(h->d.nslices) * 4 * nout * oz_kpad(ka) : 0;
+}
+
+static gw_status adjoint(gw_chi0 *h, int iq, double omega, const double *W, double *L, double *dE_v, double *dE_c,
+                         double *dcoeff_v, double *dcoeff_c)
+{
     gw_status s = check_slot(h, iq);
     if (s) return s;
     if (!W || !dE_v || !dE_c || !dcoeff_v || !dcoeff_c) return fail(h, GW_ERR_ARG, "null pointer");
@@ -74,7 +79,7 @@ gw_status gw_chi0_adjoint(gw_chi0 *h, int iq, double omega, const double *W, dou
     gw::PairPlan pp = pair_plan(h, sp);
     ZdPlan z;
     ZdUse use{h};
-    if ((s = zd_plan(h, sp, nv, nc, true, false, 1, 1, z)) ||
+    if ((s = zd_plan(h, sp, nv, nc, true, false, 1, 1, oz_b_bytes(h, ng, ng), z)) ||
         (z.on && ((s = zd_valence(h, z, sp, v.psi, nv)) || (s = zd_conduction(h, z, c.psi, 0, nc))))) {
         cleanup();
         return s;
@@ -132,6 +137,13 @@ gw_status gw_chi0_adjoint(gw_chi0 *h, int iq, double omega, const double *W, dou
 #undef ACK
     cleanup(); // synchronises: L is valid on return
     return GW_OK;
+}
+
+gw_status gw_chi0_adjoint(gw_chi0 *h, int iq, double omega, const double *W, double *L, double *dE_v, double *dE_c,
+                          double *dcoeff_v, double *dcoeff_c)
+{
+    if (!h) return GW_ERR_ARG;
+    return zd_or_fft(h, [&] { return adjoint(h, iq, omega, W, L, dE_v, dE_c, dcoeff_v, dcoeff_c); });
 }
 
 // ------------------------------------------------------------------ static subspace
@@ -201,10 +213,9 @@ gw_status gw_chi0_subspace_basis(gw_chi0 *h, int ng, const double *chi0, int nei
     return GW_OK;
 }
 
-gw_status gw_chi0_compute_subspace(gw_chi0 *h, int iq, int neig, const double *basis, int nw, const double *omega,
-                                   double *chi_sub)
+static gw_status compute_subspace(gw_chi0 *h, int iq, int neig, const double *basis, int nw, const double *omega,
+                                  double *chi_sub)
 {
-    if (!h) return GW_ERR_ARG;
     if (nw < 1 || nw > gw::kMaxOmega || !omega || !basis || !chi_sub)
         return fail(h, GW_ERR_ARG, "bad arguments (1 <= nw <= %d, non-null pointers)", gw::kMaxOmega);
     gw::OmegaList om;
@@ -223,7 +234,7 @@ gw_status gw_chi0_compute_subspace(gw_chi0 *h, int iq, int neig, const double *b
     const double2 *Mres = resident_for(h, iq); // kept by the last gw_chi0_compute of this slot
     ZdPlan z;
     ZdUse use{h};
-    if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, nw, z)) ||
+    if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, nw, oz_b_bytes(h, ng, neig), z)) ||
                   (z.on && ((s = zd_valence(h, z, sp, v.psi, v.nb)) || (s = zd_conduction(h, z, h->cond.psi, 0, h->cond.nb))))))
         return s;
     const int64_t chunk = z.on ? (int64_t)z.vb * z.cb : std::min<int64_t>(h->d.pair_chunk, P);
@@ -255,6 +266,13 @@ gw_status gw_chi0_compute_subspace(gw_chi0 *h, int iq, int neig, const double *b
     Scope sc(h, "symmetrize");
     CK(h, gw::launch_symmetrize((double2 *)chi_sub, neig, nw, h->st), "symmetrize");
     return GW_OK;
+}
+
+gw_status gw_chi0_compute_subspace(gw_chi0 *h, int iq, int neig, const double *basis, int nw, const double *omega,
+                                   double *chi_sub)
+{
+    if (!h) return GW_ERR_ARG;
+    return zd_or_fft(h, [&] { return compute_subspace(h, iq, neig, basis, nw, omega, chi_sub); });
 }
 
 // ------------------------------------------------------------------ dielectric matrix inverse
@@ -391,9 +409,8 @@ gw_status gw_chi0_epsilon_inverse(gw_chi0 *h, int ng, int nw, const double *chi,
 }
 
 // ------------------------------------------------------------------ real frequencies
-gw_status gw_chi0_compute_real(gw_chi0 *h, int iq, int nw, const double *omega, double eta, double *chi)
+static gw_status compute_real(gw_chi0 *h, int iq, int nw, const double *omega, double eta, double *chi)
 {
-    if (!h) return GW_ERR_ARG;
     if (nw < 1 || 3 * nw > gw::kMaxOmega || !omega || !chi)
         return fail(h, GW_ERR_ARG, "bad arguments (1 <= nw <= %d, non-null pointers)", gw::kMaxOmega / 3);
     if (!(eta > 0.0) || !std::isfinite(eta)) return fail(h, GW_ERR_ARG, "eta must be finite and > 0");
@@ -413,14 +430,15 @@ gw_status gw_chi0_compute_real(gw_chi0 *h, int iq, int nw, const double *omega, 
     const double2 *Mres = resident_for(h, iq); // kept by the last gw_chi0_compute of this slot
     ZdPlan z;
     ZdUse use{h};
-    if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, 3 * nw, z)) ||
+    const size_t parts = sizeof(double2) * 3 * nw * nn, pending = parts > h->realcap ? parts - h->realcap : 0;
+    if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, 3 * nw, pending, z)) ||
                   (z.on && ((s = zd_valence(h, z, sp, v.psi, v.nb)) || (s = zd_conduction(h, z, h->cond.psi, 0, h->cond.nb))))))
         return s;
     const int64_t chunk = z.on ? (int64_t)z.vb * z.cb : std::min<int64_t>(h->d.pair_chunk, P);
-    if ((s = grow(h, (void **)&h->realbuf, &h->realcap, sizeof(double2) * 3 * nw * nn, "real-axis parts")) ||
+    if ((s = grow(h, (void **)&h->realbuf, &h->realcap, parts, "real-axis parts")) ||
         (s = ensure_work(h, (size_t)chunk * ng, (size_t)chunk * 3 * nw)))
         return s;
-    CK(h, cudaMemsetAsync(h->realbuf, 0, sizeof(double2) * 3 * nw * nn, h->st), "zero parts");
+    CK(h, cudaMemsetAsync(h->realbuf, 0, parts, h->st), "zero parts");
     gw::PairPlan pp = pair_plan(h, sp);
     for (int64_t p0 = 0; p0 < P; p0 += chunk) {
         const int64_t cnt = std::min(chunk, P - p0);
@@ -437,6 +455,12 @@ gw_status gw_chi0_compute_real(gw_chi0 *h, int iq, int nw, const double *omega, 
     CK(h, gw::launch_symmetrize(h->realbuf, ng, 3 * nw, h->st), "symmetrize");
     CK(h, gw::launch_combine_real(h->realbuf, nn, nw, (double2 *)chi, h->st), "combine");
     return GW_OK;
+}
+
+gw_status gw_chi0_compute_real(gw_chi0 *h, int iq, int nw, const double *omega, double eta, double *chi)
+{
+    if (!h) return GW_ERR_ARG;
+    return zd_or_fft(h, [&] { return compute_real(h, iq, nw, omega, eta, chi); });
 }
 
 // ------------------------------------------------------------------ forward derivative (JVP)
@@ -458,10 +482,9 @@ static gw_status band_grids(gw_chi0 *h, const BandSet &b, const double *coeff, v
     return GW_OK;
 }
 
-gw_status gw_chi0_jvp(gw_chi0 *h, int iq, int nw, const double *omega, const double *dcoeff_v,
-                      const double *dcoeff_c, const double *dE_v, const double *dE_c, double *dchi)
+static gw_status jvp(gw_chi0 *h, int iq, int nw, const double *omega, const double *dcoeff_v,
+                     const double *dcoeff_c, const double *dE_v, const double *dE_c, double *dchi)
 {
-    if (!h) return GW_ERR_ARG;
     if (nw < 1 || 2 * nw > gw::kMaxOmega || !omega || !dcoeff_v || !dcoeff_c || !dE_v || !dE_c || !dchi)
         return fail(h, GW_ERR_ARG, "bad arguments (1 <= nw <= %d, non-null pointers)", gw::kMaxOmega / 2);
     gw::OmegaList om;
@@ -478,16 +501,17 @@ gw_status gw_chi0_jvp(gw_chi0 *h, int iq, int nw, const double *omega, const dou
     const int ng = sp.ng, nc = c.nb;
     const int64_t nn = (int64_t)ng * ng;
     const int64_t P = (int64_t)v.nb * nc;
+    // work held only for this call
+    const size_t szv = sizeof(double2) * (size_t)v.nb * h->nr, szc = sizeof(double2) * (size_t)nc * h->nr;
+    const size_t szt = sizeof(double2) * 4 * nw * nn;
     ZdPlan z; // side 0: the stored bands, side 1: the tangents
     ZdUse use{h};
-    if ((s = zd_plan(h, sp, v.nb, nc, true, false, 2, 2 * nw, z))) return s;
+    if ((s = zd_plan(h, sp, v.nb, nc, true, false, 2, 2 * nw, szv + szc + szt, z))) return s;
     const int64_t chunk = z.on ? (int64_t)z.vb * z.cb : std::min<int64_t>(h->d.pair_chunk, P);
-    // work held only for this call
     void *gv = nullptr, *gc = nullptr;
     double2 *X1 = nullptr, *X2 = nullptr, *T = nullptr;
     double *wb = nullptr;
-    const size_t szv = sizeof(double2) * (size_t)v.nb * h->nr, szc = sizeof(double2) * (size_t)nc * h->nr;
-    const size_t szx = sizeof(double2) * (size_t)chunk * ng, szt = sizeof(double2) * 4 * nw * nn;
+    const size_t szx = sizeof(double2) * (size_t)chunk * ng;
     const size_t szw = sizeof(double) * 2 * nw * (size_t)chunk;
     auto cleanup = [&]() {
         cudaStreamSynchronize(h->st);
@@ -557,3 +581,9 @@ gw_status gw_chi0_jvp(gw_chi0 *h, int iq, int nw, const double *omega, const dou
     return GW_OK;
 }
 
+gw_status gw_chi0_jvp(gw_chi0 *h, int iq, int nw, const double *omega, const double *dcoeff_v,
+                      const double *dcoeff_c, const double *dE_v, const double *dE_c, double *dchi)
+{
+    if (!h) return GW_ERR_ARG;
+    return zd_or_fft(h, [&] { return jvp(h, iq, nw, omega, dcoeff_v, dcoeff_c, dE_v, dE_c, dchi); });
+}

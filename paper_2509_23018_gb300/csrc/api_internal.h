@@ -173,6 +173,8 @@ struct gw_chi0 {
     float4 *zdS = nullptr;     // cells between the middle- and first-axis kernels, where they are two
     size_t zdScap = 0;         // bytes
     bool zdbusy = false;       // a call has planned with these buffers (ZdUse)
+    bool zdran = false;        // a plan of this call took the route, and
+    bool zdoff = false;        // none may (zd_or_fft)
     int *zdguard = nullptr;    // FP64: set where the slices do not hold and the FFT kernel takes over
     size_t zdguard_cap = 0;
     // scratch slots of the two-float pair kernel (sized in set_gsphere, outside any capture)
@@ -273,9 +275,6 @@ gw_status resident_begin(gw_chi0 *h, int64_t P, int ng, bool *use);
 double2 *resident_for(gw_chi0 *h, int iq);
 // overlapped split-precision streamed compute of one slot (api.cu); Mres: resident output or null
 gw_status compute_overlap(gw_chi0 *h, int iq, const gw::OmegaList &om, double2 *cq, double *dq, double2 *Mres);
-// Stage (a) with the last-axis transform on the tensor cores: whether slot iq takes it, the
-// conduction bands per chunk, the valence slices (once per call), and one chunk's pair
-// elements M[cl nv + v] for the conduction bands c0 .. c0 + cb - 1.
 // Stage (a) on the tensor cores for one call.  zd_plan: blocks of vb x cb pairs (rows: cb = nc, whole
 // valence rows in pair order) and the buffers for `sides` sets of bands; on = false when the route
 // does not take the sphere, would be slower (unless forced) or lacks memory.  zd_valence /
@@ -295,8 +294,21 @@ struct ZdUse {
     gw_chi0 *h;
     ~ZdUse() { h->zdbusy = false; }
 };
+// pending: bytes that the call will still allocate beside its chunk's pair elements, weights and slices
 gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw,
-                  ZdPlan &z);
+                  size_t pending, ZdPlan &z);
+// A call that plans: one that runs out of memory beside the route's buffers is made again without them.
+template <class F>
+gw_status zd_or_fft(gw_chi0 *h, F body)
+{
+    h->zdran = false;
+    gw_status s = body();
+    if (s != GW_ERR_OOM || !h->zdran) return s;
+    h->zdoff = true;
+    s = body();
+    h->zdoff = false;
+    return s;
+}
 bool zd_holds(const gw_chi0 *h, const ZdPlan &z); // side 0 and F as planned (a later plan may have lost them)
 gw_status zd_valence(gw_chi0 *h, ZdPlan &z, const Sphere &sp, const void *psiv, int nv, int side = 0);
 gw_status zd_conduction(gw_chi0 *h, ZdPlan &z, const void *psic, int c0, int cb, int side = 0);

@@ -74,6 +74,36 @@ def test_route_yields_to_the_memory_budget(gw):
     assert h.device_bytes() <= 500 << 20
 
 
+@pytest.mark.parametrize("op", ["jvp", "real", "sub", "adjoint", "chi"])
+def test_more_budget_never_fails(gw, op):
+    """Budgets in steps of 80 MB through the range where the route's buffers begin to fit (slices 0.6 GB, F and
+    cells more): once a call runs, it runs with every larger budget, and gives the same."""
+    p = gwgen.make_problem((40, 40, 40), 12, 300, 3000, 900, seed=4)
+    rng = np.random.default_rng(4)
+    tan = [dev(rng.standard_normal(c.shape) + 1j * rng.standard_normal(c.shape)) * 1e-2 for c in (p.cv, p.cc)]
+    tan += [dev(rng.standard_normal(len(e))) for e in (p.ev, p.ec)]
+    basis = dev(np.linalg.qr(rng.standard_normal((900, 40)) + 1j * rng.standard_normal((900, 40)))[0])
+    W = dev(gwgen.hermitian(rng, 900))
+    run = {"jvp": lambda h: h.jvp(0, [0.0, 2.0], *tan), "real": lambda h: h.compute_real(0, [1.0, 4.0, 8.0], 0.1),
+           "sub": lambda h: h.compute_subspace(0, basis, [0.0]), "adjoint": lambda h: h.adjoint(0, W)[4],
+           "chi": lambda h: h.compute(0, [0.0, 1.0])[0]}[op]
+    kw = dict(prec="ozaki", nslices=7, mtxel="twofloat")
+    ref, ran = run(gw.from_problem(p, **kw)), []
+    for step in range(30):
+        budget = int(0.4e9) + step * (80 << 20)
+        try:
+            h = gw.from_problem(p, mem_budget_bytes=budget, **kw)
+            for _ in range(2):  # the second call finds what the first has left
+                assert rel(run(h), ref) < 5 * TOL
+            h.sync()
+            assert h.device_bytes() <= budget
+            ran.append(True)
+        except gw.GwError as e:
+            assert "OOM" in str(e)
+            ran.append(False)
+    assert ran[-1] and ran == sorted(ran)
+
+
 def test_eight_slices_keep_the_fft_kernel_elsewhere(gw):
     """At eight slices the pair elements' own error would show: other calls than chi on 48^3 keep the FFT
     kernel and stay within its error (bound of the six-slice expansion: 32 * 6 * 2^-54 = 1e-14 a pair)."""
