@@ -454,32 +454,32 @@ gw_status contract_chunk_ozaki(gw_chi0 *h, const double2 *M, int64_t P, int ng, 
     return GW_OK;
 }
 
-// FP64 contraction by slices (oz_gemm_kernel, OzProd::F64) of P pairs for each frequency: *done = false
-// without room for the slices.  The launch of the DMMA kernel behind it returns at once unless the
+// FP64 contraction by slices (oz_gemm_kernel, OzProd::F64) of P pairs for each frequency, in pieces of
+// at most 16384 pairs, smaller ones only where a memory budget or the device has no room for their slices;
+// *done = false where it has none for 1024.  (How much memory happens to be free has no part in it: the pieces
+// decide where the FP64 sums are rounded.)  The launch of the DMMA kernel behind it returns at once unless the
 // slicing kernels found entries that are not finite or column scales beyond 2^+-390.
 static gw_status contract_f64_slices(gw_chi0 *h, const double2 *M, int64_t P, int ng, const double *delta,
                                      int64_t dstride, int nw, double2 *chi, bool *done)
 {
     *done = false;
     const int s = gw::oz_f64_slices();
-    size_t room = 0, total = 0;
-    if (h->d.mem_budget_bytes) {
-        const size_t rest = h->bytes - h->Zcap + (64 << 20);
-        room = rest < h->d.mem_budget_bytes ? h->d.mem_budget_bytes - rest : 0;
-    } else {
-        CK(h, cudaMemGetInfo(&room, &total), "free memory");
-        room = h->Zcap + room / 4;
-    }
     const int64_t per = (int64_t)s * 2 * ng * 2; // bytes of a pair's slices
     int64_t piece = std::min<int64_t>((P + 63) / 64 * 64, 16384);
-    while (piece > 1024 && (size_t)(piece * per) > room) piece = (piece / 2 + 63) / 64 * 64;
-    if ((size_t)(piece * per) > room) return GW_OK;
+    auto halve = [&] { piece = (piece / 2 + 63) / 64 * 64; };
+    if (h->d.mem_budget_bytes) {
+        const size_t rest = h->bytes - h->Zcap + (64 << 20);
+        const size_t room = rest < h->d.mem_budget_bytes ? h->d.mem_budget_bytes - rest : 0;
+        while (piece > 1024 && (size_t)(piece * per) > room) halve();
+        if ((size_t)(piece * per) > room) return GW_OK;
+    }
     const std::string err = h->err;
     const int64_t nt = (ng + gw::oz_box_rows() - 1) / gw::oz_box_rows(), tiles = nt * (nt + 1) / 2;
     gw_status st;
     h->zbusy = true;
-    if ((st = grow(h, &h->Zbuf, &h->Zcap, (size_t)(piece * per), "slice buffer")) ||
-        (st = grow(h, (void **)&h->spbuf, &h->spcap, sizeof(double) * (size_t)nw * dstride, "scale buffer")) ||
+    while ((st = grow(h, &h->Zbuf, &h->Zcap, (size_t)(piece * per), "slice buffer")) == GW_ERR_OOM && piece > 1024)
+        halve();
+    if (st || (st = grow(h, (void **)&h->spbuf, &h->spcap, sizeof(double) * (size_t)nw * dstride, "scale buffer")) ||
         (st = grow(h, (void **)&h->Ebuf, &h->Ecap, sizeof(int) * (size_t)ng, "exponent buffer")) ||
         (st = grow(h, (void **)&h->f64guard, &h->f64guard_cap, sizeof(int), "slice check")) ||
         (st = grow(h, &h->jobbuf, &h->jobcap,
@@ -752,7 +752,7 @@ static bool zd_faster(const gw_chi0 *h, const Sphere &sp, int vb, int cb)
 
 // Room for the route's buffers beside what the call will still take: with a memory budget, what the
 // caller names (pending), the pair elements of a chunk, their slices (for a group of frequencies) and
-// the split tiles' scratch come first; without one, the buffers may grow by a quarter of the free memory.
+// the split tiles' scratch come first; without one, growth by a quarter of the free memory.
 static bool zd_room(const gw_chi0 *h, size_t grow_by, int64_t pairs, int ng, int nw, size_t pending)
 {
     if (grow_by == 0) return true;
@@ -801,11 +801,14 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
     // per valence band: F, and the cells between the two kernels of the other axes
     z.fper = sizeof(float4) * (size_t)lines * z.cb * gw::zd_row_entries(sp.K2);
     z.sper = zd_fused(h) ? 0 : sizeof(float4) * (size_t)n[0] * z.cb * sp.K12;
-    // F of as many valence bands as 5 GB hold (whole tiles), fewer where memory is short
+    // F of as many valence bands as 5 GB hold (whole tiles), fewer where memory is short.  Without a budget
+    // at least one tile's: the size of a sub-block has no part in the results, the route has (2e-13), so
+    // the free memory decides the one and not the other
     int vs = (int)std::min<size_t>(z.vb, std::max<size_t>(1, (size_t)5000000000 / z.fper));
     for (;; vs = vs > ct ? std::max(ct, vs / 2) : vs / 2) {
         if (vs < 1) return GW_OK;
         if (vs > ct) vs -= vs % ct;
+        if (!h->d.mem_budget_bytes && vs <= ct) break;
         size_t by = 0;
         for (int i = 0; i < sides; ++i)
             by += (z.abytes > h->zdAcap[i] ? z.abytes - h->zdAcap[i] : 0) + (z.ebytes > h->zdEcap[i] ? z.ebytes - h->zdEcap[i] : 0);
