@@ -769,11 +769,12 @@ static bool zd_room(const gw_chi0 *h, size_t grow_by, int64_t pairs, int ng, int
     return grow_by <= free_b / 4;
 }
 
-gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw,
-                  size_t pending, ZdPlan &z)
+// Blocks and sub-blocks of a call's plan; false where the route does not take the call or has no room.
+static bool zd_choose(const gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw,
+                      size_t pending, ZdPlan &z)
 {
     z = ZdPlan();
-    if (h->zdoff || !zd_grid(h, sp)) return GW_OK;
+    if (h->zdoff || !zd_grid(h, sp)) return false;
     z.f64 = h->d.mtxel_prec == GW_MTXEL_FP64;
     const int *n = h->d.n, lines = n[0] * n[1];
     const int ct = z.f64 ? gw::zd64_valence_per_tile(sp.K2) : gw::zd_valence_per_tile(n[2], sp.K2);
@@ -782,7 +783,7 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
     // 8e-15.  At up to seven slices the contraction's own error is ten times that and more.  At eight,
     // and with the FP64 contraction, the route serves chi on 48^3 alone (8.7e-14 at eight slices); on
     // the other calls it would raise the error, by up to three times for the gradients.
-    if (!z.f64 && (h->d.prec == GW_PREC_FP64 || h->d.nslices > 7) && !chi48) return GW_OK;
+    if (!z.f64 && (h->d.prec == GW_PREC_FP64 || h->d.nslices > 7) && !chi48) return false;
     if (rows) {
         z.cb = nc;
     } else { // conduction blocks of about 512: four row tiles share a valence tile's columns
@@ -792,10 +793,10 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
         z.cb = (int)std::min<int64_t>(z.cb, h->d.pair_chunk);
     }
     int64_t vb = std::min<int64_t>(nv, h->d.pair_chunk / z.cb);
-    if (vb < 1) return GW_OK;
+    if (vb < 1) return false;
     if (vb >= ct && vb < nv) vb -= vb % ct;
     z.vb = (int)vb;
-    if (!force && !zd_faster(h, sp, z.vb, z.cb)) return GW_OK;
+    if (!force && !zd_faster(h, sp, z.vb, z.cb)) return false;
     z.abytes = z.f64 ? gw::zd64_row_bytes(z.cb, n[2], lines) : gw::zd_row_bytes(z.cb, n[2], lines);
     z.ebytes = sizeof(int) * (size_t)lines * nv;
     // per valence band: F, and the cells between the two kernels of the other axes
@@ -806,7 +807,7 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
     // the free memory decides the one and not the other
     int vs = (int)std::min<size_t>(z.vb, std::max<size_t>(1, (size_t)5000000000 / z.fper));
     for (;; vs = vs > ct ? std::max(ct, vs / 2) : vs / 2) {
-        if (vs < 1) return GW_OK;
+        if (vs < 1) return false;
         if (vs > ct) vs -= vs % ct;
         if (!h->d.mem_budget_bytes && vs <= ct) break;
         size_t by = 0;
@@ -817,6 +818,13 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
         if (force || zd_room(h, by, (int64_t)z.vb * z.cb, sp.ng, nw, pending)) break;
     }
     z.vs = vs;
+    return true;
+}
+
+gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw,
+                  size_t pending, ZdPlan &z)
+{
+    if (!zd_choose(h, sp, nv, nc, rows, force, sides, nw, pending, z)) return GW_OK;
     const std::string err = h->err;
     gw_status s = GW_OK;
     const bool before = h->zdbusy; // an earlier plan of this call
@@ -824,8 +832,8 @@ gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool 
     for (int i = 0; i < sides && !s; ++i)
         if (!(s = grow(h, &h->zdA[i], &h->zdAcap[i], z.abytes, "conduction slices")))
             s = grow(h, (void **)&h->zdE[i], &h->zdEcap[i], z.ebytes, "column exponents");
-    if (!s) s = grow(h, (void **)&h->zdF, &h->zdFcap, z.fper * vs, "last-axis transform");
-    if (!s && z.sper) s = grow(h, (void **)&h->zdS, &h->zdScap, z.sper * vs, "transform cells");
+    if (!s) s = grow(h, (void **)&h->zdF, &h->zdFcap, z.fper * z.vs, "last-axis transform");
+    if (!s && z.sper) s = grow(h, (void **)&h->zdS, &h->zdScap, z.sper * z.vs, "transform cells");
     if (!s && z.f64 && !(s = grow(h, (void **)&h->zdguard, &h->zdguard_cap, sizeof(int), "slice check")))
         CK(h, cudaMemsetAsync(h->zdguard, 0, sizeof(int), h->st), "slice check");
     if (s == GW_ERR_OOM && !force) { // the FFT route needs none of these
@@ -989,6 +997,21 @@ gw_status resident_begin(gw_chi0 *h, int64_t P, int ng, bool *use)
 
 double2 *resident_for(gw_chi0 *h, int iq) { return h->keep_m && h->Mres_iq == iq ? h->Mres : nullptr; }
 
+// The overlapped path's buffers, given back.
+static void drop_overlap(gw_chi0 *h)
+{
+    cudaStreamSynchronize(h->st);
+    if (h->ov_st) cudaStreamSynchronize(h->ov_st);
+    for (int b = 0; b < 2; ++b) {
+        dfree(h, h->ovZ[b], h->ovZcap[b]);
+        dfree(h, h->ovE[b], h->ovEcap[b]);
+        dfree(h, h->ovJ[b], h->ovJcap[b]);
+        h->ovZ[b] = h->ovJ[b] = nullptr;
+        h->ovE[b] = nullptr;
+        h->ovZcap[b] = h->ovEcap[b] = h->ovJcap[b] = 0;
+    }
+}
+
 gw_status compute_overlap(gw_chi0 *h, int iq, const gw::OmegaList &om, double2 *cq, double *dq, double2 *Mres)
 {
     const Sphere &sp = h->sph[iq];
@@ -1149,7 +1172,8 @@ int gw_chi0_streams(gw_chi0 *h, int iq)
     if (!h) return -(int)GW_ERR_ARG;
     gw_status s = check_slot(h, iq);
     if (s) return -(int)s;
-    if (zd_grid(h, h->sph[iq])) return 1; // stage (a) on the tensor cores runs on one stream
+    ZdPlan z; // stage (a) on the tensor cores runs on one stream
+    if (zd_choose(h, h->sph[iq], h->val[iq].nb, h->cond.nb, h->keep_m, false, 1, 1, 0, z)) return 1;
     return overlap_enabled(h, pair_plan(h, h->sph[iq])) ? 2 : 1;
 }
 
@@ -1485,17 +1509,6 @@ static gw_status compute(gw_chi0 *h, int nq, const int *iq, int nw, const double
         gw_status s = resident_begin(h, P, ng, &keep);
         if (s) return s;
         double2 *Mres = keep ? h->Mres : nullptr;
-        // with several frequencies the contractions queue up behind the two slice buffers: one stream
-        if (nw == 1 && overlap_enabled(h, pp) && fault_chunk() < 0 && !zd_grid(h, sp)) {
-            s = compute_overlap(h, iq[i], om, cq, dq, Mres);
-            if (s) return s;
-            Scope sc(h, "symmetrize");
-            CK(h, gw::launch_symmetrize(cq, ng, nw, h->st), "symmetrize");
-            off += (size_t)nw * ng * ng;
-            doff += (size_t)nw * ng;
-            if (keep) h->Mres_iq = iq[i];
-            continue;
-        }
         ZdPlan z;
         ZdUse use{h};
         if (fault_chunk() < 0 && (s = zd_plan(h, sp, v.nb, h->cond.nb, keep, false, 1, nw, 0, z))) return s;
@@ -1531,9 +1544,26 @@ static gw_status compute(gw_chi0 *h, int nq, const int *iq, int nw, const double
             if (keep) h->Mres_iq = iq[i];
             continue;
         }
+        const int64_t fault_at = fault_chunk();
+        // with several frequencies the contractions queue up behind the two slice buffers: one stream
+        if (nw == 1 && overlap_enabled(h, pp) && fault_at < 0) {
+            s = compute_overlap(h, iq[i], om, cq, dq, Mres);
+            if (s && s != GW_ERR_OOM) return s;
+            if (!s) {
+                Scope sc(h, "symmetrize");
+                CK(h, gw::launch_symmetrize(cq, ng, nw, h->st), "symmetrize");
+                off += (size_t)nw * ng * ng;
+                doff += (size_t)nw * ng;
+                if (keep) h->Mres_iq = iq[i];
+                continue;
+            }
+            // no room for a second slice buffer: one stream
+            drop_overlap(h);
+            CK(h, cudaMemsetAsync(cq, 0, sizeof(double2) * (size_t)nw * ng * ng, h->st), "zero chi");
+            if (dq) CK(h, cudaMemsetAsync(dq, 0, sizeof(double) * (size_t)nw * ng, h->st), "zero diag");
+        }
         s = ensure_work(h, (size_t)chunk * ng, (size_t)chunk * nw);
         if (s) return s;
-        const int64_t fault_at = fault_chunk();
         for (int64_t p0 = 0, k = 0; p0 < P; p0 += chunk, ++k) {
             int64_t cnt = std::min(chunk, P - p0);
             if (k == fault_at) return fail(h, GW_ERR_CUDA, "injected host-side fault before chunk %lld", (long long)k);

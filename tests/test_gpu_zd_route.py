@@ -74,7 +74,7 @@ def test_route_yields_to_the_memory_budget(gw):
     assert h.device_bytes() <= 500 << 20
 
 
-@pytest.mark.parametrize("op", ["jvp", "real", "sub", "adjoint", "chi"])
+@pytest.mark.parametrize("op", ["jvp", "real", "sub", "adjoint", "chi", "chi1"])
 def test_more_budget_never_fails(gw, op):
     """Budgets in steps of 80 MB through the range where the route's buffers begin to fit (slices 0.6 GB, F and
     cells more): once a call runs, it runs with every larger budget, and gives the same."""
@@ -86,7 +86,7 @@ def test_more_budget_never_fails(gw, op):
     W = dev(gwgen.hermitian(rng, 900))
     run = {"jvp": lambda h: h.jvp(0, [0.0, 2.0], *tan), "real": lambda h: h.compute_real(0, [1.0, 4.0, 8.0], 0.1),
            "sub": lambda h: h.compute_subspace(0, basis, [0.0]), "adjoint": lambda h: h.adjoint(0, W)[4],
-           "chi": lambda h: h.compute(0, [0.0, 1.0])[0]}[op]
+           "chi": lambda h: h.compute(0, [0.0, 1.0])[0], "chi1": lambda h: h.compute(0, [0.0])[0]}[op]
     kw = dict(prec="ozaki", nslices=7, mtxel="twofloat")
     ref, ran = run(gw.from_problem(p, **kw)), []
     for step in range(30):
@@ -112,3 +112,23 @@ def test_eight_slices_keep_the_fft_kernel_elsewhere(gw):
     h = gw.from_problem(p, prec="ozaki", nslices=8, mtxel="twofloat")
     assert rel(h.compute(0, [0.0])[0], ref) < 4e-14
     h.sync()
+
+
+@pytest.mark.parametrize("chunk", [500, 8192])
+def test_overlap_where_the_route_declines(gw, chunk):
+    """40^3 at eight slices keeps the FFT kernel, and with it the contraction beside it on a second stream: the same
+    bits as on one stream; and a call on one stream where a budget has no room for the second slice buffer."""
+    p = gwgen.make_problem((40, 40, 40), 8, 200, 1500, 300, seed=9)
+    kw = dict(prec="ozaki", nslices=8, mtxel="twofloat", pair_chunk=chunk)
+    one, two = gw.from_problem(p, single_stream=True, **kw), gw.from_problem(p, **kw)
+    assert (one.streams(0), two.streams(0)) == (1, 2)
+    want = one.compute(0, [0.0])[0]
+    one.sync()
+    assert torch.equal(two.compute(0, [0.0])[0], want)
+    two.sync()
+    used = one.device_bytes()
+    for over in (1 << 20, 6 << 20, 64 << 20):
+        h = gw.from_problem(p, mem_budget_bytes=used + over, **kw)
+        assert rel(h.compute(0, [0.0])[0], want) < 4e-14  # tiles in parts may be whole ones here
+        h.sync()
+        assert h.device_bytes() <= used + over
