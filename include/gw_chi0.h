@@ -359,8 +359,8 @@ GW_API gw_status gw_chi0_keep_pair_elements(gw_chi0 *h, int enable);
  * How many streams a single-frequency gw_chi0_compute uses for slot iq as it stands (bands and
  * sphere set): 2 when each chunk's split contraction runs on a second stream beside the next
  * chunk's pair elements (split precision, two-float stage (a) by the grid-specialised FFT pair
- * kernel with blocks of at most 64 KB of shared memory: 24^3, and 40^3 and 48^3 where the
- * tensor-core route of stage (a) does not take the call), else 1 (always 1 on that route, see
+ * kernel with blocks of at most 64 KB of shared memory: 24^3, and 40^3 where the tensor-core
+ * route of stage (a) does not take the call), else 1 (always 1 on that route, see
  * gw_chi0_pair_elements_block).  Calls with several frequencies, and those without room for a second
  * slice buffer, run on one stream.  Negative (a gw_status, negated) on a bad handle or slot.
  */

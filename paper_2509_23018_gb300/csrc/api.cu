@@ -970,8 +970,11 @@ gw_status pair_rows(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::Pai
 // on 40^3, 2 % for 4096 on 24^3, no difference for full chunks.  Slices, exponents and job tables
 // alternate between two buffer sets; job j waits for the contraction of job j - 2.  Taken where
 // the pair kernel's blocks use at most 64 KB of shared memory (24^3 to 48^3).
-bool overlap_enabled(gw_chi0 *h, const gw::PairPlan &pp)
+// 48^3 slots that the route can serve report one stream, and keep it for the calls that its plan leaves (few
+// conduction bands).
+bool overlap_enabled(gw_chi0 *h, const Sphere &sp, const gw::PairPlan &pp, bool keep)
 {
+    if (zd_fused(h) && h->d.n[0] == 48 && !keep && zd_grid(h, sp)) return false;
     if (h->d.prec != GW_PREC_OZAKI_BF16 || h->d.single_stream || h->d.mtxel_prec != GW_MTXEL_TWOFLOAT) return false;
     const size_t ps = gw::pair_tf_ct_smem_bytes(pp);
     return ps > 0 && ps <= 64 * 1024;
@@ -1174,7 +1177,7 @@ int gw_chi0_streams(gw_chi0 *h, int iq)
     if (s) return -(int)s;
     ZdPlan z; // stage (a) on the tensor cores runs on one stream
     if (zd_choose(h, h->sph[iq], h->val[iq].nb, h->cond.nb, h->keep_m, false, 1, 1, 0, z)) return 1;
-    return overlap_enabled(h, pair_plan(h, h->sph[iq])) ? 2 : 1;
+    return overlap_enabled(h, h->sph[iq], pair_plan(h, h->sph[iq]), h->keep_m) ? 2 : 1;
 }
 
 void gw_chi0_destroy(gw_chi0 *h)
@@ -1546,7 +1549,7 @@ static gw_status compute(gw_chi0 *h, int nq, const int *iq, int nw, const double
         }
         const int64_t fault_at = fault_chunk();
         // with several frequencies the contractions queue up behind the two slice buffers: one stream
-        if (nw == 1 && overlap_enabled(h, pp) && fault_at < 0) {
+        if (nw == 1 && overlap_enabled(h, sp, pp, keep) && fault_at < 0) {
             s = compute_overlap(h, iq[i], om, cq, dq, Mres);
             if (s && s != GW_ERR_OOM) return s;
             if (!s) {

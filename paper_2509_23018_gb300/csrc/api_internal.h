@@ -316,7 +316,7 @@ gw_status zd_block(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::Pair
                    int vb, int cb, double2 *M, int64_t sv, int64_t sc);
 gw_status pair_rows(gw_chi0 *h, const ZdPlan &z, const Sphere &sp, const gw::PairPlan &pp, const void *psiv,
                     const void *psic, int nc, int64_t p0, int64_t cnt, double2 *M, int vside = 0, int cside = 0);
-bool overlap_enabled(gw_chi0 *h, const gw::PairPlan &pp);
+bool overlap_enabled(gw_chi0 *h, const Sphere &sp, const gw::PairPlan &pp, bool keep);
 
 // batched path (api_batch.cu)
 gw_status compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const double *omega, const gw::OmegaList &om,
