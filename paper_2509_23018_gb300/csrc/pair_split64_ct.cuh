@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kSplitThreads, split_min_blocks<N>())
     for (int i0 = 0; i0 < n0; i0 += 2, ++nf) {
         const bool late = !bar_wait(&fbar, nf & 1);
         if (__syncthreads_or(late)) { // X complete (or the wait ran out, for every thread alike)
-            if (threadIdx.x == 0) atomicOr(pp.status, kStatusTimeout);
+            pair_give_up(&fbar, nf & 1, pp.status);
             return;
         }
         dstage0_rows<N>(X, Y, K2, K2, ncols, CS, lm);
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kSplitThreads, split_min_blocks<N>())
         const int nbat = K12 - d0 < NB ? K12 - d0 : NB;
         const bool late = !bar_wait(&fbar, nf & 1);
         if (__syncthreads_or(late)) {
-            if (threadIdx.x == 0) atomicOr(pp.status, kStatusTimeout);
+            pair_give_up(&fbar, nf & 1, pp.status);
             return;
         }
         const LMap lm = lmap_lines_fastest(nbat);

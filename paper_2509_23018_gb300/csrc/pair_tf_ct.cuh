@@ -392,6 +392,15 @@ __device__ __forceinline__ void tstage0_rows(const float4 *__restrict__ x, float
 // buffer of a slab pair's columns, in float4, rounded to 128 bytes (TMA destinations)
 __host__ __device__ constexpr int from_f_buf(int ncols, int cs) { return (ncols * cs + 7) / 8 * 8; }
 
+// A wait for a copy ran out: thread 0 records it and gives the copy as long again to land, since the block's
+// shared memory is another's once every thread has left.
+__device__ __forceinline__ void pair_give_up(uint64_t *fbar, unsigned parity, int *status)
+{
+    if (threadIdx.x != 0) return;
+    atomicOr(status, kStatusTimeout);
+    bar_wait(fbar, parity);
+}
+
 template <int N>
 __global__ void __launch_bounds__(pair_threads<N>(), pair_min_blocks<N>())
     pair_kernel_tf_from_f(const __grid_constant__ CUtensorMap tmF, const __grid_constant__ CUtensorMap tmS, int cb,
@@ -452,7 +461,7 @@ __global__ void __launch_bounds__(pair_threads<N>(), pair_min_blocks<N>())
         float4 *X = Xb + b * BUF, *Y = Xb + (b ^ 1) * BUF;
         const bool late = !bar_wait(&fbar, nf & 1);
         if (__syncthreads_or(late)) { // X complete (or the wait ran out, for every thread alike)
-            if (threadIdx.x == 0) atomicOr(pp.status, kStatusTimeout);
+            pair_give_up(&fbar, nf & 1, pp.status);
             return;
         }
         tstage0_rows<N>(X, Y, K2, K2, ncols, CS, lm, kc);
@@ -494,7 +503,7 @@ __global__ void __launch_bounds__(pair_threads<N>(), pair_min_blocks<N>())
         const int nbat = K12 - d0 < NB ? K12 - d0 : NB;
         const bool late = !bar_wait(&fbar, nf & 1);
         if (__syncthreads_or(late)) {
-            if (threadIdx.x == 0) atomicOr(pp.status, kStatusTimeout);
+            pair_give_up(&fbar, nf & 1, pp.status);
             return;
         }
         const LMap lm2 = lmap_lines(nbat);
