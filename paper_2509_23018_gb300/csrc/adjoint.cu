@@ -655,10 +655,12 @@ cudaError_t launch_adj_products(const void *psiv, const void *psic, int v0, int 
                                 int64_t nr, bool tf, double2 *pbv, double2 *pbc, cudaStream_t st)
 {
     if (tf) {
-        // One pass where the grid's points alone fill the GPU and the rows fit the registers.  27000 points:
-        // 0.60 against 0.47 ms (12 x 200 bands, two groups of rows); 110592 points, 8 rows as two groups of
-        // four: 0.80 against 0.79; 64000 points, five rows: 7.1 against 9.2.
-        if (nr >= 60000 && nvc <= 6) {
+        // One pass where the grid's points alone fill the GPU and the rows fit the registers.  Two kernels
+        // against one pass, 300 conduction bands, ms: one row .338 / .375 at 64000 points, .414 / .422 at 91125,
+        // .465 / .434 at 110592; two rows .399 / .352 at 64000; three .469 / .489 at 64000, .719 / .537 at 81000;
+        // four, five and six .693 / .489, .758 / .564 and .811 / .593 at 64000, and less on every larger grid.
+        // 27000 points: one pass slower for any number of rows.
+        if (nvc <= 6 && nr >= (nvc == 1 ? 100000 : nvc == 3 ? 70000 : 60000)) {
             const float4 *pv = (const float4 *)psiv + v0 * nr;
             auto run = [&](auto kern) {
                 kern<<<(unsigned)((nr + 63) / 64), 64, 0, st>>>(pv, (const float4 *)psic, (const float4 *)H, nc, nr,

@@ -21,7 +21,9 @@ def gw():
 
 @pytest.mark.parametrize("n,nv,nc,ngpsi,ng", [(24, 3, 40, 60, 19), (24, 2, 30, 60, 1000), (40, 3, 37, 900, 700),
                                               (48, 2, 40, 2000, 1500), (72, 1, 30, 3000, 2500), (24, 2, 30, 19, 2000),
-                                              (40, 6, 50, 900, 300), (48, 7, 33, 900, 250)])
+                                              (40, 6, 50, 900, 300), (48, 7, 33, 900, 250),
+                                              (40, 1, 30, 900, 300), (40, 4, 30, 900, 300), (40, 5, 30, 900, 300),
+                                              (48, 3, 33, 900, 250)])
 def test_gradients_match_fp64(gw, n, nv, nc, ngpsi, ng):
     p = gwgen.make_problem((n, n, n), nv, nc if nc + nv <= ngpsi else ngpsi - nv, ngpsi, ng, seed=n + ng)
     W = torch.as_tensor(gwgen.hermitian(np.random.default_rng(2), ng), device="cuda")
