@@ -61,8 +61,9 @@ __host__ __device__ __forceinline__ int oz_expo_pos(double a, int no_column)
     return (b - 1ull) < 0x7ff0000000000000ull ? oz_expo_bits(b, no_column) : no_column;
 }
 
-// round(x 2^h), ties to even, h = sh clamped to [-1022, 1023].  The split's exponent bounds
-// |x 2^h| by 2^52, so N is formed by one right shift of the 53-bit significand (k >= 1).
+// round(x 2^h), ties to even, h = sh clamped to [-1022, 1023].  N is formed by one shift of the 53-bit
+// significand.  |x 2^h| < 2^(9 s - 2): up to six slices that is a right shift (k >= 1); seven slices (|N| < 2^61)
+// shift the entries within 2^-8 of their column's largest left, by up to eight bits, which is exact.
 __host__ __device__ __forceinline__ long long oz_round_scaled(double x, int sh)
 {
     const int h = sh < -1022 ? -1022 : (sh > 1023 ? 1023 : sh);
@@ -72,7 +73,7 @@ __host__ __device__ __forceinline__ long long oz_round_scaled(double x, int sh)
     const int k = 1075 - (be != 0 ? be : 1) - h; // |x| 2^h = m 2^-k
     unsigned long long q;
     if (k <= 0) {
-        q = m << (-k < 10 ? -k : 10); // outside the split's range (|x 2^h| >= 2^52); kept defined
+        q = m << (-k < 10 ? -k : 10); // -k <= 8 within the split's range; kept defined beyond it
     } else if (k > 60) {
         q = 0; // |x| 2^h < 2^-7
     } else {

@@ -14,7 +14,7 @@ import pytest
 HERE = os.path.dirname(os.path.abspath(__file__))
 
 
-@pytest.mark.parametrize("s", [3, 4, 5, 6])
+@pytest.mark.parametrize("s", [3, 4, 5, 6, 7])
 def test_nine_bit_digits(s, tmp_path):
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     if not os.path.exists(nvcc):
@@ -29,6 +29,11 @@ def test_nine_bit_digits(s, tmp_path):
         x = rng.choice([c, -c, 0.0, c * rng.uniform(-1, 1), math.ldexp(c, -rng.randrange(60)),
                         -math.ldexp(c * rng.random(), -rng.randrange(60))])
         cases.append((x, c))
+    # up to the largest magnitude that an exponent allows (at seven slices the significand is shifted left there)
+    for e in (-900, 0, 900):
+        c = math.ldexp(1.0 - 2.0 ** -53, e)
+        cases += [(sign * math.ldexp(m, e), c) for sign in (1, -1) for k in range(12)
+                  for m in (math.ldexp(1.0 - 2.0 ** -53, -k), math.ldexp(0.5, -k), math.ldexp(1.0 - rng.random() * 2.0 ** -40, -k))]
     bits = lambda v: struct.unpack("<Q", struct.pack("<d", v))[0]  # noqa: E731
     inp = "".join(f"{bits(x):016x} {bits(c):016x} {s}\n" for x, c in cases)
     out = subprocess.run([exe], input=inp, capture_output=True, text=True, check=True).stdout.splitlines()

@@ -94,24 +94,29 @@ def test_split_ragged(gw, ng):
     assert rel(chi, oracle.chi0(Mo, oracle.delta(p.ev, p.ec, 0.0))) <= TOL_SPLIT
 
 
-@pytest.mark.parametrize("ng", [65, 300, 2000])
-def test_split_tile_widths_agree(gw, ng, monkeypatch):
-    """The split contraction gives the same bits at tile widths 128, 240 and 256 real columns
-    (every entry sums the same slice products in the same K order), on spheres that leave ragged
-    row and column tiles at each width."""
+@pytest.mark.parametrize("ng,P", [(65, 1024), (300, 4099), (1100, 1024), (2000, 8192)])
+def test_split_tiles_in_parts_agree(gw, ng, P):
+    """The last tiles of a launch split their pairs in parts, whose sums are added in FP64; a budget without room for
+    their scratch leaves the tiles whole.  Every tile sums the same slice products: the two differ by the rounding of
+    two-float sums, 2^-46 of a pair's largest product and a K-segment, and both give the same bits in every run."""
     rng = np.random.default_rng(1000 + ng)
-    nv, nc = 8, 40
-    M = rng.standard_normal((nv * nc, ng)) + 1j * rng.standard_normal((nv * nc, ng))
-    ev, ec = -1.0 - rng.random(nv), 1.0 + rng.random(nc)
-    outs = []
-    for width in (128, 240, 256):
-        monkeypatch.setenv("GW_CHI0_SPLIT_TILE", str(width))
-        h = gw.Chi0((8, 8, 8), prec="ozaki", nslices=7)
-        outs.append(h.contract(dev(ev), dev(ec), dev(M), [0.0, 1.5]).cpu().numpy())
-        h.sync()
-    assert np.array_equal(outs[0], outs[1])
-    assert np.array_equal(outs[0], outs[2])
-    assert np.array_equal(outs[0][0], outs[0][0].conj().T)
+    M = rng.standard_normal((P, ng)) + 1j * rng.standard_normal((P, ng))
+    ev, ec = np.full(1, -2.0), np.full(P, 2.0)
+    h = gw.Chi0((8, 8, 8), prec="ozaki", nslices=7)
+    parts = h.contract(dev(ev), dev(ec), dev(M), [0.0]).cpu().numpy()[0]
+    h.sync()
+    assert np.array_equal(parts, h.contract(dev(ev), dev(ec), dev(M), [0.0]).cpu().numpy()[0])
+    # slices, weights, exponents and job table, and 64 KB to spare; a part of one tile takes 256 KB
+    need = 5 * 2 * ng * ((P + 63) // 64 * 64) * 2 + 16 * P + 4 * ng + (1 << 16)
+    hw = gw.Chi0((8, 8, 8), prec="ozaki", nslices=7, mem_budget_bytes=need)
+    whole = hw.contract(dev(ev), dev(ec), dev(M), [0.0]).cpu().numpy()[0]
+    hw.sync()
+    assert hw.device_bytes() < h.device_bytes() - (256 << 10)
+    assert not np.array_equal(parts, whole)
+    assert np.array_equal(whole, whole.conj().T) and np.array_equal(parts, parts.conj().T)
+    mx = np.maximum(np.abs(M.real), np.abs(M.imag)).max(axis=0)
+    segments = 5 * (P // 256 + 1)
+    assert (np.abs(parts - whole) <= 2.0 ** -46 * P * segments * np.outer(mx, mx)).all()
 
 
 def test_streams_query(gw):

@@ -1,7 +1,8 @@
 """Stage (a) on the tensor cores, all callers, on the two grids it is built for: row tiles of 128
 conduction bands (one short, one exact, one over), partial valence tiles, odd and even numbers of kept
 z-frequencies, chunks that hold less than a row of pairs, and a conduction set of several blocks.
-Against the library's FP64 mode (an independent path, 1e-15).  Two-float stage (a) keeps 2e-13 and the
+Against the library's FP64 mode, which shares the digit step and the contraction's kernel with the mode under
+test and is itself held to the FP64 FFT kernel's pair elements contracted on DMMA.  Two-float stage (a) keeps 2e-13 and the
 contraction at seven-slice accuracy, a five-slice expansion, 32 * 5 * 2^-45 = 5e-12 of the product of two
 columns' largest magnitudes per pair: relative to the columns' norms below 2e-11 for these bands."""
 import numpy as np
@@ -47,6 +48,9 @@ def test_route_matches_fp64(gw, n, nv, nc, ngpsi, ng, chunk):
         h = gw.from_problem(p, pair_chunk=chunk, **kw)
         if mode == "split":
             assert h.streams(0) == 1
+        else:  # other kernels from the bands on: the FFT pair kernel and the contraction of given elements
+            dmma = h.contract(dev(p.ev), dev(p.ec), h.pair_elements(0, 0, nv * nc), [0.0, 3.0])
+            assert rel(h.compute(0, [0.0, 3.0])[0], dmma) < 5e-15
         r = {"chi": h.compute(0, [0.0, 3.0])[0], "batch": h.compute_batch([0], [0.0, 3.0])[0],
              "sub": h.compute_subspace(0, basis, [1.0]), "real": h.compute_real(0, [4.0], 0.2),
              "jvp": h.jvp(0, [2.0], *tan)}
