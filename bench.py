@@ -9,7 +9,8 @@ by the 8 N_G^2 P convention).
 
 The headline mode is the split-precision contraction (7 BF16 slices, two-float stage
 (a)) with its error against the oracle stated on sampled entries; the same line carries
-the native FP64 tensor-core path on the same input under "fp64_dmma".
+the FP64 mode on the same input under "fp64", and the same chi from the FP64 FFT kernel's pair
+elements contracted on the native FP64 tensor cores under "fp64_dmma".
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--prec fp64|ozaki] [--impl ours|reference]
     python bench.py --sweep      slice-count sweep on one 72^3 chunk (error and throughput)
@@ -52,7 +53,7 @@ def parse():
                     help="batch: resident M, persistent contraction, CUDA graph (gw_chi0_compute_batch); "
                          "stream: chunk-by-chunk launches (gw_chi0_compute)")
     ap.add_argument("--no-fp64-compare", action="store_true",
-                    help="skip the native FP64 DMMA run on the same input (split-precision mode only)")
+                    help="skip the FP64 runs on the same input (split-precision mode only)")
     ap.add_argument("--mtxel", default=None, choices=["fp64", "twofloat"],
                     help="stage (a) arithmetic; default fp64 with --prec fp64, twofloat with --prec ozaki")
     ap.add_argument("--config", default="c2_48cube", choices=sorted(gwgen.CONFIGS))
@@ -773,18 +774,19 @@ def roofline_for(cfg, prec, nslices, res, single_stream=False):
     kname = "contract_f64" if prec == "fp64" else "ozaki_gemm"
     tkey = kname + ("_single_stream" if single_stream and prec != "fp64" else "")
     kms, kn = res["timing"].get(kname, (0.0, 0))
-    nchunk = -(-cfg.npairs // cfg.pair_chunk)
-    # low-precision flops of the kept slice pairs, each 4 N_G^2 P per chunk and frequency.  FP64 by slices:
+    # low-precision flops of the kept slice pairs, each 4 N_G^2 P per step and frequency.  FP64 by slices:
     # 28 products, and each launch has a second behind it that returns at once (the DMMA kernel, for
     # what the slices do not hold); FP64 on DMMA (batches): the upper triangle's FP64 flops
     sliced = prec == "fp64" and "oz_split" in res["timing"]
     if prec == "fp64" and not sliced:
-        per_launch_flops = 4.0 * cfg.ng * (cfg.ng + 1) * cfg.npairs / nchunk
+        step_flops = 4.0 * cfg.ng * (cfg.ng + 1) * cfg.npairs
     else:
         prods = OZ_F64_PRODUCTS if sliced else oz_products(nslices)
-        per_launch_flops = prods * 4.0 * cfg.ng ** 2 * cfg.npairs / nchunk
+        step_flops = prods * 4.0 * cfg.ng ** 2 * cfg.npairs
     if sliced:
         kn //= 2
+    # a step's blocks need not be whole pair chunks: the launches are counted
+    per_launch_flops = step_flops * round(res["total_ms"] / res["ms_per_step"]) / kn if kn else None
     peak, peak_src = peak_for("ozaki" if sliced else prec)
     achieved = per_launch_flops / (kms / kn * 1e-3) * 1e-12 if kn else None
     return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
@@ -794,6 +796,35 @@ def roofline_for(cfg, prec, nslices, res, single_stream=False):
             "peak_source": peak_src, "share_of_step": kms / res["total_ms"] if res["total_ms"] else None,
             "traffic_source": traffic_for(tkey, cfg)[1],
             "probe_peaks_tops": {k: v for k, v in LIVE_PEAKS.items() if not k.startswith("_")}}
+
+
+def run_dmma(cfg, prob, dev):
+    """One pass on the native FP64 units: all pair elements by the FP64 FFT kernel (gw_chi0_pair_elements),
+    contracted on DMMA (gw_chi0_contract).  Returns chi and the times of the two."""
+    import torch
+    import paper_2509_23018_gb300 as gw
+    h = gw.from_problem(prob, prec="fp64", pair_chunk=cfg.pair_chunk)
+    ev, ec = torch.as_tensor(prob.ev, device=dev), torch.as_tensor(prob.ec, device=dev)
+    M = torch.empty((cfg.npairs, cfg.ng), dtype=torch.complex128, device=dev)
+    h.pair_elements(0, 0, min(cfg.npairs, cfg.pair_chunk), out=M)  # warm-up of both kernels
+    h.contract(ev[:1], ec[:min(cfg.nc, 64)], M[:min(cfg.nc, 64)], [0.0])
+    h.sync()
+    e = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
+    e[0].record()
+    h.pair_elements(0, 0, cfg.npairs, out=M)
+    e[1].record()
+    chi = h.contract(ev, ec, M, [0.0])
+    e[2].record()
+    h.sync()
+    pair, con = e[0].elapsed_time(e[1]), e[1].elapsed_time(e[2])
+    flops = 4.0 * cfg.ng * (cfg.ng + 1) * cfg.npairs  # upper triangle
+    peak, src = peak_for("fp64")
+    tf = flops / (con * 1e-3) * 1e-12
+    h.destroy()
+    return chi[0].cpu().numpy(), {
+        "pair_ms": pair, "contract_ms": con, "value": conv_flops(cfg) / ((pair + con) * 1e-3) * 1e-12, "unit": "TFLOP/s",
+        "roofline": {"bound": "tensor", "achieved": tf, "peak": peak, "unit": "TFLOP/s", "frac": tf / peak,
+                     "kernel": "contract_f64", "peak_source": src, "flops": flops}}
 
 
 def ours(args):
@@ -839,8 +870,8 @@ def ours(args):
     if rank == 0 and not args.no_cpu_baseline and not args.no_check:
         blk = oracle_block(cfg, prob)
         err = block_error(main["chi"], blk)
-    # the native FP64 tensor-core path on the same input, for the FP64-vs-split comparison
-    other = None
+    # the FP64 mode and the native FP64 tensor-core path on the same input, for the FP64-vs-split comparison
+    other = dmma = None
     if args.prec == "ozaki" and not args.no_fp64_compare:
         f = run_mode(args, cfg, prob, dev, "fp64", 0, "fp64", max(1, min(2, args.steps)), 1, False, world)
         other = {"value": f["value"], "unit": "TFLOP/s", "ms_per_q": f["ms_per_step"], "mtxel": "fp64",
@@ -849,10 +880,17 @@ def ours(args):
         if blk is not None:
             other["error"] = block_error(f["chi"], blk)
         if err is not None:
-            # the whole matrix against the library's FP64 mode (seven slices, whole-number sums; itself
-            # within 1e-15 of the oracle's block)
             d = main["chi"] - f["chi"]
             err["rel_frobenius_full_vs_fp64_mode"] = float(np.linalg.norm(d) / np.linalg.norm(f["chi"]))
+        if cfg.npairs * cfg.ng * 16 < 40e9:
+            # every pair element at once: the FFT kernel and DMMA, which the modes above do not run
+            chi_d, dmma = run_dmma(cfg, prob, dev)
+            if blk is not None:
+                dmma["error"] = block_error(chi_d, blk)
+            norm = float(np.linalg.norm(chi_d))
+            dmma["fp64_mode_rel_frobenius_full"] = float(np.linalg.norm(f["chi"] - chi_d)) / norm
+            if err is not None:
+                err["rel_frobenius_full_vs_fp64_dmma"] = float(np.linalg.norm(main["chi"] - chi_d)) / norm
     cpu = None
     if rank == 0 and not args.no_cpu_baseline:
         cpu = cpu_baseline(cfg, prob, args.cpu_sample_pairs)
@@ -870,7 +908,7 @@ def ours(args):
                            "parallelism": f"replicas x{world} (independent q-points)",
                            "streams": main.get("streams", 1)},
                 "error": err, "roofline": roofline, "roofline_contraction": roofline_other, "rooflines": rooflines,
-                "single_stream": alone, "fp64_dmma": other, "cpu_baseline": cpu, "e2e": main["e2e"],
+                "single_stream": alone, "fp64": other, "fp64_dmma": dmma, "cpu_baseline": cpu, "e2e": main["e2e"],
                 "gpu_launches": main["launches"], "kernel_ms": main["kernel_ms"], "clocks": main["clocks"]}
         print(json.dumps(line), flush=True)
     if world > 1:
@@ -917,9 +955,9 @@ def sweep(args):
         r = run_mode(args, cfg, prob, dev, "fp64", 0, "fp64", 1, 1 if not full else 0, False, 1)
         e = block_error(r["chi"], blk)
         rf = roofline_for(cfg, "fp64", 0, r)
-        out["fp64_dmma"] = {"rel_err": e["rel_frobenius_vs_oracle"],
-                            "contract_tflops": rf["achieved"], "contract_ms": rf["ms_per_launch"],
-                            "ms_per_q": r["ms_per_step"], "value": r["value"], "roofline": rf}
+        out["fp64"] = {"rel_err": e["rel_frobenius_vs_oracle"],
+                       "contract_tflops": rf["achieved"], "contract_ms": rf["ms_per_launch"],
+                       "ms_per_q": r["ms_per_step"], "value": r["value"], "roofline": rf}
     if not args.no_cpu_baseline:
         # at N_G = 6000 the oracle takes about 47 ms a pair on 16 cores: 512 pairs stay near 25 s
         cpu = cpu_baseline(cfg, prob, min(args.cpu_sample_pairs, 512))
