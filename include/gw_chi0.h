@@ -76,7 +76,13 @@ typedef enum {
     GW_PREC_FP64 = 0,      /* FP64 FFT + contraction to FP64 accuracy: of computed pair elements by seven
                               nine-bit slices on the BF16 tensor cores (62 bits of a column's largest
                               entry, whole-number sums), otherwise on the FP64 tensor cores (DMMA);
-                              a budget without room for the slices leaves all of it to DMMA */
+                              a budget without room for the slices leaves all of it to DMMA, some
+                              forty times slower.  The slices' error is relative to the columns' norms
+                              (1e-18 of them an entry; below a double sum's over the matrix), a double
+                              sum's to each term: where two columns have their weight on different
+                              pairs, their entry of chi is far below the norms and keeps fewer digits
+                              than a double sum of its terms.  gw_chi0_pair_elements with
+                              gw_chi0_contract, and gw_chi0_compute_batch, contract on DMMA. */
     GW_PREC_OZAKI_BF16 = 1 /* FP64 FFT + split-precision contraction on BF16 tensor cores */
 } gw_prec;
 
@@ -169,7 +175,9 @@ GW_API gw_status gw_chi0_compute(gw_chi0 *h, int nq, const int *iq, int nw, cons
  * sizes, frequencies, output pointers) into a CUDA graph and replayed on later calls.
  * On the first call of a problem shape in FP64 mode an autotuner times the contraction's
  * launch-shape candidates (tile edge 32/64 and wave count) and keeps the fastest for the handle
- * (see gw_chi0_tuning); the split contraction has one tile shape.  The first call
+ * (see gw_chi0_tuning); the split contraction has one tile shape.  FP64 batches contract on DMMA, which takes
+ * far longer than the slices of gw_chi0_compute (8192 pairs, N_G = 2000: 138 ms against 3.5): in FP64 mode
+ * a loop of gw_chi0_compute over the slots is faster from a few dozen pairs on.  The first call
  * synchronises the stream; replays are asynchronous.  Slots must be distinct.
  * Errors: as gw_chi0_compute; GW_ERR_OOM when the resident buffers do not fit.
  */

@@ -525,8 +525,8 @@ static gw_status contract_f64_slices(gw_chi0 *h, const double2 *M, int64_t P, in
 }
 
 // FP64: computed pair elements go by slices from 32 pairs on (16 pairs: 72 to 86 us against 82 to 85 of
-// the DMMA kernel for N_G = 40 to 500; 32: 72 to 87 against 158; 1024: 131 to 135 against 1200; 8192 pairs
-// at N_G = 2000: 2.9 ms against 138).  Elements that the caller passes in stay on the DMMA kernel, whose
+// the DMMA kernel for N_G = 40 to 500; 32: 72 to 87 against 158; 1024: 130 to 149 against 1200; 8192 pairs
+// at N_G = 2000: 3.5 ms against 138).  Elements that the caller passes in stay on the DMMA kernel, whose
 // error is relative to each term of a sum where the slices' is relative to the columns' norms.
 gw_status contract_chunk(gw_chi0 *h, const double2 *M, int64_t P, int ng, const double *delta, int64_t dstride,
                          int nw, double2 *chi, bool given)

@@ -92,9 +92,9 @@ cudaError_t launch_pair_split2(const CUtensorMap &tmS, int64_t R, int cb, int64_
 cudaError_t launch_pair_tf_from_f(const CUtensorMap &tmF, const CUtensorMap &tmS, int64_t R, int cb, int64_t sv,
                                   int64_t sc, const PairPlan &pp, double2 *M, cudaStream_t st);
 
-// ---- the same in FP64 (zdft64.cu, pair_split64.cu): seven nine-bit slices per operand, double2 grids, F
+// ---- the same in FP64 (zdft64.cu, pair_split64_ct.cuh): seven nine-bit slices per operand, double2 grids, F
 // and cells.  Lines of 24 to 56 points.  guard: set by the slicing kernels where an entry is not finite
-// or a line is scaled by more than 2^+-400; the product returns at once where it is set.
+// or a line is scaled by more than 2^+-390; the product returns at once where it is set.
 size_t zd64_row_bytes(int nr, int n, int lines); // row slices and exponents
 cudaError_t launch_zd64_rows(const void *psi, int nr, int n, int lines, void *A, int *guard, cudaStream_t st);
 cudaError_t launch_zd64_colexp(const void *psi, int nb, int n, int lines, int *E, int *guard, cudaStream_t st);
