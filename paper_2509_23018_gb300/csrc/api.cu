@@ -726,28 +726,45 @@ static bool zd_grid(const gw_chi0 *h, const Sphere &sp)
     return !small_cube && gw::pair_split_supported(n[0]) && gw::pair_split_supported(n[1]);
 }
 
-// Whether a block of vb x cb pairs takes less time this way, from microseconds measured on one GB300:
-// the FFT kernel 1.04 a pair on 48^3, 0.84 on 40^3, 5.1 on 72^3, 28e-6 a grid point where it is not
-// grid-specialised, and no less than for the 600 pairs that fill the GPU; here 5.2e-3 per line, stage
-// of 8 points and tile of 128 conduction bands x CT valence bands, however few of its rows and columns
-// hold bands, and for the other two axes 7.2e-6 per line and kept frequency of a pair.
-// FP64: the FFT kernel 61e-6 a grid point (48^3; 79e-6 on 24^3) and no less than for one pair an SM; here
-// 14e-3 and 34e-6.
-static bool zd_faster(const gw_chi0 *h, const Sphere &sp, int vb, int cb)
+// Whether a call of nv x nc pairs in blocks of z.vb x z.cb takes less time this way than with the FFT kernel in
+// launches of `launch` pairs.  From microseconds measured on one GB300 for 1 x 1 to 64 x 32 and 16 x 128 bands on
+// thirteen grids, two-float:
+//  the FFT kernel 1.12 a pair on 48^3, 0.84 on 40^3, 5.2 on 72^3, about 28e-6 a grid point where it is not
+//  grid-specialised, a launch for its pairs rounded up to one an SM (its time is a staircase), and no less
+//  than for 280, 300, 215 and 210;
+//  here 11e-3 per line, stage of 8 points and tile of 128 conduction bands x CT valence bands, however few of its
+//  rows and columns hold bands (8e-3 with four row tiles to a column tile), 8.2e-6 per line and kept frequency of a
+//  pair for the other two axes, no less than for 300 pairs, and 20 + the row slices' bytes at 4.3 TB/s per
+//  conduction block.
+// FP64: the FFT kernel 64e-6 a grid point (57e-6 on 32^3 to 75e-6 on 45^3) and no less than for 176 pairs; here 19e-3, 36e-6
+// for at least 230 pairs, and 2.9 TB/s.
+// Few conduction bands and many valence bands are what loses: 40 x 2 bands on 48^3 take 1.53 ms here and 0.31 there,
+// on 72^3 7.7 and 1.1, 64 x 32 3.0 and 2.3; 8 x 128 0.74 and 1.17, 3.3 and 5.6.  Over the measured cases the rule's
+// choice is at most 6 % slower than the better one.
+static bool zd_faster(const gw_chi0 *h, const Sphere &sp, int nv, int nc, int64_t launch, const ZdPlan &z)
 {
-    const bool f64 = h->d.mtxel_prec == GW_MTXEL_FP64;
-    const int *n = h->d.n, ct = f64 ? gw::zd64_valence_per_tile(sp.K2) : gw::zd_valence_per_tile(n[2], sp.K2);
+    const int *n = h->d.n, ct = z.f64 ? gw::zd64_valence_per_tile(sp.K2) : gw::zd_valence_per_tile(n[2], sp.K2);
     const bool cube = n[0] == n[1] && n[1] == n[2];
-    const double lines = (double)n[0] * n[1], pairs = (double)vb * cb;
-    const double tiles = (double)((cb + 127) / 128) * ((vb + ct - 1) / ct);
-    if (f64)
-        return tiles * lines * ((n[2] + 7) / 8) * 14e-3 + 34e-6 * lines * sp.K2 * pairs <
-               61e-6 * lines * n[2] * std::max(pairs, 152.0);
-    const double fft = cube && n[0] == 48   ? 1.04
-                       : cube && n[0] == 40 ? 0.84
-                       : cube && n[0] == 72 ? 5.1
-                                            : 28e-6 * lines * n[2];
-    return tiles * lines * ((n[2] + 7) / 8) * 5.2e-3 + 7.2e-6 * lines * sp.K2 * pairs < fft * std::max(pairs, 600.0);
+    const double lines = (double)n[0] * n[1], blocks = (double)((nv + z.vb - 1) / z.vb) * ((nc + z.cb - 1) / z.cb);
+    const double pairs = (double)z.vb * z.cb, stages = (n[2] + 7) / 8;
+    const double tiles = (double)((z.cb + 127) / 128) * ((z.vb + ct - 1) / ct);
+    const double row_us = 20.0 + (z.f64 ? gw::zd64_row_bytes(z.cb, n[2], (int)lines) / 2.9e6
+                                        : gw::zd_row_bytes(z.cb, n[2], (int)lines) / 4.3e6);
+    const double here = blocks * (tiles * lines * stages * (z.f64 ? 19e-3 : 11e-3) +
+                                  lines * sp.K2 * (z.f64 ? 36e-6 * std::max(pairs, 230.0) : 8.2e-6 * std::max(pairs, 300.0))) +
+                        ((nc + z.cb - 1) / z.cb) * row_us;
+    double per = 28e-6 * lines * n[2], least = 210.0; // the FFT kernel: a pair, and pairs that a launch costs at least
+    if (z.f64) {
+        per = 64e-6 * lines * n[2];
+        least = 176.0;
+    } else if (cube && (n[0] == 40 || n[0] == 48 || n[0] == 72)) {
+        per = n[0] == 40 ? 0.84 : n[0] == 48 ? 1.12 : 5.2;
+        least = n[0] == 40 ? 300.0 : n[0] == 48 ? 280.0 : 215.0;
+    }
+    const int64_t P = (int64_t)nv * nc, sms = num_sms();
+    auto fft = [&](int64_t pairs) { return per * std::max((double)((pairs + sms - 1) / sms * sms), least); };
+    const double there = P / launch * fft(launch) + (P % launch ? fft(P % launch) : 0.0);
+    return here < there;
 }
 
 // Room for the route's buffers beside what the call will still take: with a memory budget, what the
@@ -771,7 +788,7 @@ static bool zd_room(const gw_chi0 *h, size_t grow_by, int64_t pairs, int ng, int
 
 // Blocks and sub-blocks of a call's plan; false where the route does not take the call or has no room.
 static bool zd_choose(const gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw,
-                      size_t pending, ZdPlan &z)
+                      size_t pending, int64_t launch, ZdPlan &z)
 {
     z = ZdPlan();
     if (h->zdoff || !zd_grid(h, sp)) return false;
@@ -796,7 +813,7 @@ static bool zd_choose(const gw_chi0 *h, const Sphere &sp, int nv, int nc, bool r
     if (vb < 1) return false;
     if (vb >= ct && vb < nv) vb -= vb % ct;
     z.vb = (int)vb;
-    if (!force && !zd_faster(h, sp, z.vb, z.cb)) return false;
+    if (!force && !zd_faster(h, sp, nv, nc, launch, z)) return false;
     z.abytes = z.f64 ? gw::zd64_row_bytes(z.cb, n[2], lines) : gw::zd_row_bytes(z.cb, n[2], lines);
     z.ebytes = sizeof(int) * (size_t)lines * nv;
     // per valence band: F, and the cells between the two kernels of the other axes
@@ -822,9 +839,9 @@ static bool zd_choose(const gw_chi0 *h, const Sphere &sp, int nv, int nc, bool r
 }
 
 gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw,
-                  size_t pending, ZdPlan &z)
+                  size_t pending, int64_t launch, ZdPlan &z)
 {
-    if (!zd_choose(h, sp, nv, nc, rows, force, sides, nw, pending, z)) return GW_OK;
+    if (!zd_choose(h, sp, nv, nc, rows, force, sides, nw, pending, launch, z)) return GW_OK;
     const std::string err = h->err;
     gw_status s = GW_OK;
     const bool before = h->zdbusy; // an earlier plan of this call
@@ -1176,7 +1193,9 @@ int gw_chi0_streams(gw_chi0 *h, int iq)
     gw_status s = check_slot(h, iq);
     if (s) return -(int)s;
     ZdPlan z; // stage (a) on the tensor cores runs on one stream
-    if (zd_choose(h, h->sph[iq], h->val[iq].nb, h->cond.nb, h->keep_m, false, 1, 1, 0, z)) return 1;
+    const int nv = h->val[iq].nb, nc = h->cond.nb;
+    const int64_t chunk = std::min<int64_t>(h->d.pair_chunk, (int64_t)nv * nc);
+    if (zd_choose(h, h->sph[iq], nv, nc, h->keep_m, false, 1, 1, 0, chunk, z)) return 1;
     return overlap_enabled(h, h->sph[iq], pair_plan(h, h->sph[iq]), h->keep_m) ? 2 : 1;
 }
 
@@ -1452,7 +1471,7 @@ gw_status gw_chi0_pair_elements_block(gw_chi0 *h, int iq, int c0, int cb, double
     if (cb == 0) return GW_OK;
     ZdPlan z;
     ZdUse use{h};
-    if ((s = zd_plan(h, sp, nv, cb, false, true, 1, 1, 0, z))) return s;
+    if ((s = zd_plan(h, sp, nv, cb, false, true, 1, 1, 0, 1, z))) return s;
     const gw::PairPlan pp = pair_plan(h, sp);
     if ((s = zd_valence(h, z, sp, v.psi, nv))) return s;
     for (int b0 = 0; b0 < cb; b0 += z.cb) {
@@ -1514,7 +1533,7 @@ static gw_status compute(gw_chi0 *h, int nq, const int *iq, int nw, const double
         double2 *Mres = keep ? h->Mres : nullptr;
         ZdPlan z;
         ZdUse use{h};
-        if (fault_chunk() < 0 && (s = zd_plan(h, sp, v.nb, h->cond.nb, keep, false, 1, nw, 0, z))) return s;
+        if (fault_chunk() < 0 && (s = zd_plan(h, sp, v.nb, h->cond.nb, keep, false, 1, nw, 0, chunk, z))) return s;
         if (z.on) {
             const int nc = h->cond.nb;
             if ((s = ensure_work(h, keep ? 0 : (size_t)z.vb * z.cb * ng, (size_t)z.vb * z.cb * nw)) ||

@@ -220,7 +220,7 @@ gw_status compute_batch(gw_chi0 *h, int nq, const int *iq, int nw, const double 
     std::vector<ZdPlan> zd(nq);
     ZdUse use{h};
     for (int i = 0; i < nq; ++i)
-        if ((s = zd_plan(h, h->sph[iq[i]], h->val[iq[i]].nb, h->cond.nb, true, false, 1, 1, 0, zd[i]))) return s;
+        if ((s = zd_plan(h, h->sph[iq[i]], h->val[iq[i]].nb, h->cond.nb, true, false, 1, 1, 0, L.P[i], zd[i]))) return s;
     for (auto &z : zd) z.on = z.on && zd_holds(h, z);
     if ((s = batch_autotune(h, nq, iq, nw, om, L, (double2 *)chi, zd))) return s;
 

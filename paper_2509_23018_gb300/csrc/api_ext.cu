@@ -79,7 +79,7 @@ static gw_status adjoint(gw_chi0 *h, int iq, double omega, const double *W, doub
     gw::PairPlan pp = pair_plan(h, sp);
     ZdPlan z;
     ZdUse use{h};
-    if ((s = zd_plan(h, sp, nv, nc, true, false, 1, 1, oz_b_bytes(h, ng, ng), z)) ||
+    if ((s = zd_plan(h, sp, nv, nc, true, false, 1, 1, oz_b_bytes(h, ng, ng), cmax, z)) ||
         (z.on && ((s = zd_valence(h, z, sp, v.psi, nv)) || (s = zd_conduction(h, z, c.psi, 0, nc))))) {
         cleanup();
         return s;
@@ -234,7 +234,8 @@ static gw_status compute_subspace(gw_chi0 *h, int iq, int neig, const double *ba
     const double2 *Mres = resident_for(h, iq); // kept by the last gw_chi0_compute of this slot
     ZdPlan z;
     ZdUse use{h};
-    if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, nw, oz_b_bytes(h, ng, neig), z)) ||
+    if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, nw, oz_b_bytes(h, ng, neig),
+                              std::min<int64_t>(h->d.pair_chunk, P), z)) ||
                   (z.on && ((s = zd_valence(h, z, sp, v.psi, v.nb)) || (s = zd_conduction(h, z, h->cond.psi, 0, h->cond.nb))))))
         return s;
     const int64_t chunk = z.on ? (int64_t)z.vb * z.cb : std::min<int64_t>(h->d.pair_chunk, P);
@@ -431,7 +432,8 @@ static gw_status compute_real(gw_chi0 *h, int iq, int nw, const double *omega, d
     ZdPlan z;
     ZdUse use{h};
     const size_t parts = sizeof(double2) * 3 * nw * nn, pending = parts > h->realcap ? parts - h->realcap : 0;
-    if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, 3 * nw, pending, z)) ||
+    if (!Mres && ((s = zd_plan(h, sp, v.nb, h->cond.nb, true, false, 1, 3 * nw, pending,
+                              std::min<int64_t>(h->d.pair_chunk, P), z)) ||
                   (z.on && ((s = zd_valence(h, z, sp, v.psi, v.nb)) || (s = zd_conduction(h, z, h->cond.psi, 0, h->cond.nb))))))
         return s;
     const int64_t chunk = z.on ? (int64_t)z.vb * z.cb : std::min<int64_t>(h->d.pair_chunk, P);
@@ -506,7 +508,8 @@ static gw_status jvp(gw_chi0 *h, int iq, int nw, const double *omega, const doub
     const size_t szt = sizeof(double2) * 4 * nw * nn;
     ZdPlan z; // side 0: the stored bands, side 1: the tangents
     ZdUse use{h};
-    if ((s = zd_plan(h, sp, v.nb, nc, true, false, 2, 2 * nw, szv + szc + szt, z))) return s;
+    if ((s = zd_plan(h, sp, v.nb, nc, true, false, 2, 2 * nw, szv + szc + szt,
+                     std::min<int64_t>(h->d.pair_chunk, P), z))) return s;
     const int64_t chunk = z.on ? (int64_t)z.vb * z.cb : std::min<int64_t>(h->d.pair_chunk, P);
     void *gv = nullptr, *gc = nullptr;
     double2 *X1 = nullptr, *X2 = nullptr, *T = nullptr;

@@ -294,9 +294,10 @@ struct ZdUse {
     gw_chi0 *h;
     ~ZdUse() { h->zdbusy = false; }
 };
-// pending: bytes that the call will still allocate beside its chunk's pair elements, weights and slices
+// pending: bytes that the call will still allocate beside its chunk's pair elements, weights and slices;
+// launch: pairs that the FFT kernel would take at once
 gw_status zd_plan(gw_chi0 *h, const Sphere &sp, int nv, int nc, bool rows, bool force, int sides, int nw,
-                  size_t pending, ZdPlan &z);
+                  size_t pending, int64_t launch, ZdPlan &z);
 // A call that plans: one that runs out of memory beside the route's buffers is made again without them.
 template <class F>
 gw_status zd_or_fft(gw_chi0 *h, F body)

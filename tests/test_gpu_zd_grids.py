@@ -28,7 +28,7 @@ SHAPES = [((30, 36, 40), 13, 147, 700, 333, 8192), ((25, 32, 27), 9, 150, 500, 2
           ((32, 60, 36), 11, 200, 900, 500, 8192), ((50, 64, 60), 4, 130, 2000, 1100, 300),
           ((60, 54, 72), 5, 129, 2500, 1500, 8192), ((48, 40, 24), 6, 150, 600, 250, 8192),
           ((24, 30, 32), 12, 140, 600, 250, 8192), ((40, 48, 48), 9, 130, 1500, 600, 8192),
-          ((72, 72, 72), 3, 140, 8000, 6000, 8192), ((36, 36, 36), 11, 130, 900, 450, 8192)]
+          ((72, 72, 72), 9, 140, 8000, 6000, 8192), ((36, 36, 36), 11, 130, 900, 450, 8192)]
 
 
 @pytest.mark.parametrize("grid,nv,nc,ngpsi,ng,chunk", SHAPES)

@@ -136,3 +136,34 @@ def test_overlap_where_the_route_declines(gw, chunk):
         assert rel(h.compute(0, [0.0])[0], want) < 4e-14  # tiles in parts may be whole ones here
         h.sync()
         assert h.device_bytes() <= used + over
+
+
+@pytest.mark.parametrize("op", ["chi", "batch", "real"])
+@pytest.mark.parametrize("n,nv,nc,chunk,route", [(48, 40, 2, 8192, False), (48, 8, 128, 8192, True), (40, 40, 2, 8192, False),
+                                                 (72, 13, 1, 8192, False), (72, 8, 128, 8192, True)])
+def test_small_calls_take_the_faster_kernel(gw, n, nv, nc, chunk, route, op):
+    """Few conduction bands fill little of a tile of 128 rows, and each tile of valence bands costs as much as a
+    full one: those calls keep the FFT kernel, and both give the same."""
+    p = gwgen.make_problem((n, n, n), nv, nc, 5 * n * n // 6, n * n // 3, seed=n + nc)
+    run = {"chi": lambda h: h.compute(0, [0.0, 2.0])[0], "batch": lambda h: h.compute_batch([0], [0.0, 2.0])[0],
+           "real": lambda h: h.compute_real(0, [1.0], 0.1)}[op]
+    h = gw.from_problem(p, prec="ozaki", nslices=7, mtxel="twofloat", pair_chunk=chunk, single_stream=True)
+    got = run(h)
+    h.sync()
+    if op != "batch":  # (captured: no times)
+        h.set_timing(True)
+        run(h)
+        h.sync()
+        assert ("zdft" in h.timing(reset=True)) == route
+    assert rel(got, run(gw.from_problem(p, prec="fp64"))) < 5 * TOL
+
+
+@pytest.mark.parametrize("prec,mtxel", [("ozaki", "twofloat"), ("fp64", "fp64")])
+def test_batch_of_chunks_below_a_tile(gw, prec, mtxel):
+    """A batch's blocks follow the pair chunk, its FFT launch does not: 40 x 7 bands in chunks of 100 pairs stay on
+    the FFT kernel, and match the streamed call."""
+    p = gwgen.make_problem((48, 48, 48), 40, 7, 2000, 400, seed=3)
+    h = gw.from_problem(p, prec=prec, nslices=7, mtxel=mtxel, pair_chunk=100)
+    a, b = h.compute_batch([0], [0.0, 2.0])[0], h.compute(0, [0.0, 2.0])[0]
+    h.sync()
+    assert rel(a, b) < (TOL if prec == "ozaki" else 5e-15)
