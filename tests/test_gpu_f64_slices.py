@@ -136,3 +136,21 @@ def test_slices_make_room_for_what_a_call_needs(gw):
         if (iq, ran) == (0, True):
             seen = True
     assert seen
+
+
+@pytest.mark.parametrize("nv,nc,ng,nw,sliced", [(8, 7, 40, 9, False), (4, 8, 40, 1, True), (8, 7, 40, 1, True),
+                                                (16, 64, 300, 9, True), (3, 30, 300, 9, False), (8, 127, 7, 9, False)])
+def test_few_pairs_at_many_frequencies_stay_on_dmma(gw, nv, nc, ng, nw, sliced):
+    """The slices cost a few launches a frequency, the DMMA kernel one for all: which of them runs, and the result."""
+    p = problem(nv, nc, ng)
+    h = gw.from_problem(p, prec="fp64", pair_chunk=100 if ng == 7 else 8192)
+    om = [2.0 * k for k in range(nw)]
+    h.set_timing(True)
+    chi = h.compute(0, om)[0]
+    h.sync()
+    assert ("oz_split" in h.timing(reset=True)) == sliced
+    M = h.pair_elements(0, 0, nv * nc)
+    for i, w in enumerate(om):
+        ref = reference(p, M, w)
+        assert float(torch.linalg.vector_norm(chi[i] - ref) / torch.linalg.vector_norm(ref)) < TOL
+    h.destroy()
