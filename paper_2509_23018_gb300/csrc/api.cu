@@ -526,9 +526,10 @@ static gw_status contract_f64_slices(gw_chi0 *h, const double2 *M, int64_t P, in
 
 // FP64: computed pair elements go by slices where that takes less time, from 32 pairs on (16 pairs: 72 to 86
 // us against 82 to 85 of the DMMA kernel for N_G = 40 to 500; 32: 72 to 87 against 158; 1024: 130 to 149
-// against 1200; 8192 pairs at N_G = 2000: 3.5 ms against 138).  The slices cost five launches a frequency, about 75
-// us, where one DMMA launch serves them all: 4.8 us a pair of an item while each has an SM of its own, 8.6 with two
-// to an SM.  (56 pairs, N_G = 40, 27 weights: 1.84 ms by slices, 0.37 on DMMA.)  Elements that the caller passes in
+// against 1200; 8192 pairs at N_G = 2000: 3.5 ms against 138).  The slices cost five launches a frequency, 72 us
+// and .055 a pair up to 1024 (.0135 beyond) beside their products, where one DMMA launch serves them all: 4.8 us a
+// pair of an item while each has an SM of its own, 8.6 with two to an SM.  (56 pairs, N_G = 40, 27 weights: 1.84 ms
+// by slices, .37 on DMMA; 1677 pairs, N_G = 40, 9 weights: 1.35 against 1.12.)  Elements that the caller passes in
 // stay on the DMMA kernel, whose error is relative to each term of a sum where the slices' is relative to the
 // columns' norms.
 static bool f64_slices_faster(const gw_chi0 *h, int64_t P, int ng, int nw)
@@ -537,9 +538,11 @@ static bool f64_slices_faster(const gw_chi0 *h, int64_t P, int ng, int nw)
     const int64_t nt = (ng + h->tuned_bt - 1) / h->tuned_bt, tiles = nt * (nt + 1) / 2 * nw;
     const int64_t want = (int64_t)h->tuned_waves * 2 * num_sms(); // f64_schedule's split
     const int64_t ks = std::min<int64_t>(std::max<int64_t>(1, (want + tiles - 1) / tiles), std::max<int64_t>(1, (P + 255) / 256));
-    const double items = (double)tiles * ks, per = (double)P / ks;
-    const double dmma = items <= num_sms() ? 4.8 * per : 8.6 * per * std::max(1.0, items / (2 * num_sms()));
-    return nw * (75.0 + 1.07e-7 * ng * ng * P) < dmma;
+    const double items = (double)tiles * ks / num_sms(), per = (double)P / ks; // items an SM
+    const double dmma = per * (items <= 1.0 ? 4.8 : items <= 2.0 ? 4.8 + 3.8 * (items - 1.0) : 4.3 * items);
+    const double slices = 72.0 + 0.055 * std::min<int64_t>(P, 1024) + 0.0135 * std::max<int64_t>(P - 1024, 0) +
+                          1e-7 * ng * ng * P;
+    return nw * slices < dmma;
 }
 
 gw_status contract_chunk(gw_chi0 *h, const double2 *M, int64_t P, int ng, const double *delta, int64_t dstride,

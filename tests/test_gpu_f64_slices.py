@@ -139,7 +139,8 @@ def test_slices_make_room_for_what_a_call_needs(gw):
 
 
 @pytest.mark.parametrize("nv,nc,ng,nw,sliced", [(8, 7, 40, 9, False), (4, 8, 40, 1, True), (8, 7, 40, 1, True),
-                                                (16, 64, 300, 9, True), (3, 30, 300, 9, False), (8, 127, 7, 9, False)])
+                                                (16, 64, 300, 9, True), (3, 30, 300, 9, False), (8, 127, 7, 9, False), (13, 129, 40, 27, False),
+                                                (16, 512, 200, 9, True)])
 def test_few_pairs_at_many_frequencies_stay_on_dmma(gw, nv, nc, ng, nw, sliced):
     """The slices cost a few launches a frequency, the DMMA kernel one for all: which of them runs, and the result."""
     p = problem(nv, nc, ng)
