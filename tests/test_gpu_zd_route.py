@@ -158,6 +158,19 @@ def test_small_calls_take_the_faster_kernel(gw, n, nv, nc, chunk, route, op):
     assert rel(got, run(gw.from_problem(p, prec="fp64"))) < 5 * TOL
 
 
+@pytest.mark.parametrize("nv,nc", [(2, 1), (2, 32), (16, 30)])
+def test_sphere_of_few_vectors_takes_the_faster_kernel(gw, nv, nc):
+    """The FFT kernel takes less time the fewer frequencies a sphere keeps along the last axis; 27 vectors on 48^3 stay
+    on it, and match FP64."""
+    p = gwgen.make_problem((48, 48, 48), nv, nc, 2000, 27, seed=nc)
+    h = gw.from_problem(p, prec="ozaki", nslices=7, mtxel="twofloat")
+    h.set_timing(True)
+    got = h.compute(0, [0.0, 2.0])[0]
+    h.sync()
+    assert "zdft" not in h.timing(reset=True)
+    assert rel(got, gw.from_problem(p, prec="fp64").compute(0, [0.0, 2.0])[0]) < 5 * TOL
+
+
 @pytest.mark.parametrize("prec,mtxel", [("ozaki", "twofloat"), ("fp64", "fp64")])
 def test_batch_of_chunks_below_a_tile(gw, prec, mtxel):
     """A batch's blocks follow the pair chunk, its FFT launch does not: 40 x 7 bands in chunks of 100 pairs stay on
