@@ -758,7 +758,7 @@ static bool zd_grid(const gw_chi0 *h, const Sphere &sp)
 // for at least 230 pairs, and 2.9 TB/s.
 // Few conduction bands and many valence bands are what loses: 40 x 2 bands on 48^3 take 1.53 ms here and 0.31 there,
 // on 72^3 7.7 and 1.1, 64 x 32 3.0 and 2.3; 8 x 128 0.74 and 1.17, 3.3 and 5.6.  Over the measured cases the rule's
-// choice is at most 8 % slower than the better one (17 % for a sphere of few vectors).
+// choice is at most 6 % slower than the better one (17 % for a sphere of few vectors).
 static bool zd_faster(const gw_chi0 *h, const Sphere &sp, int nv, int nc, int64_t launch, const ZdPlan &z)
 {
     const int *n = h->d.n, ct = z.f64 ? gw::zd64_valence_per_tile(sp.K2) : gw::zd_valence_per_tile(n[2], sp.K2);
@@ -779,7 +779,7 @@ static bool zd_faster(const gw_chi0 *h, const Sphere &sp, int nv, int nc, int64_
         per = n[0] == 40 ? 0.84 : n[0] == 48 ? 1.12 : 5.2;
         least = n[0] == 40 ? 300.0 : n[0] == 48 ? 280.0 : 215.0;
     }
-    if (!z.f64) per *= std::min(1.0, 0.66 + 0.78 * sp.K2 / n[2]);
+    if (!z.f64) per *= std::min(1.0, 0.62 + 1.2 * sp.K2 / n[2]);
     const int64_t P = (int64_t)nv * nc, sms = num_sms();
     auto fft = [&](int64_t pairs) { return per * std::max((double)((pairs + sms - 1) / sms * sms), least); };
     const double there = P / launch * fft(launch) + (P % launch ? fft(P % launch) : 0.0);
