@@ -758,7 +758,8 @@ static bool zd_grid(const gw_chi0 *h, const Sphere &sp)
 // for at least 230 pairs, and 2.9 TB/s.
 // Few conduction bands and many valence bands are what loses: 40 x 2 bands on 48^3 take 1.53 ms here and 0.31 there,
 // on 72^3 7.7 and 1.1, 64 x 32 3.0 and 2.3; 8 x 128 0.74 and 1.17, 3.3 and 5.6.  Over the measured cases the rule's
-// choice is at most 6 % slower than the better one (17 % for a sphere of few vectors).
+// choice is at most 6 % slower than the better one; over thin boxes of 3 to 29 kept frequencies 17 % (36^3, 8 x 1
+// bands, 298 us for 255), FP64 60 % (36^3, 2 x 1 bands, 29 kept, the FFT kernel's 727 us for 455).
 static bool zd_faster(const gw_chi0 *h, const Sphere &sp, int nv, int nc, int64_t launch, const ZdPlan &z)
 {
     const int *n = h->d.n, ct = z.f64 ? gw::zd64_valence_per_tile(sp.K2) : gw::zd_valence_per_tile(n[2], sp.K2);
